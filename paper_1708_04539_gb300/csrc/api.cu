@@ -55,7 +55,8 @@ enum StepKind {
   ST_SMALL_LEVEL,
   ST_GSLICE,
   ST_OUTMAX,
-  ST_MIRROR
+  ST_MIRROR,
+  ST_UNPACK_PIVOTS
 };
 
 struct Step {
@@ -136,6 +137,10 @@ struct pselinv_ctx {
   char* lu = nullptr;
   char* nf = nullptr;
   char* ainv = nullptr;
+  char* winv = nullptr;    // triangular inverses of the diagonal blocks (SymDev::w_off)
+  char* piv = nullptr;     // factored pivot blocks of the diagonal LU
+  std::vector<int64_t> w_off;
+  int64_t w_stride = 0;
   char* scratch = nullptr;
   size_t scratch_bytes = 0;
   size_t scratch_high = 0;  // plan building: highest scratch byte a step uses
@@ -254,6 +259,16 @@ int upload_structure(pselinv_ctx* h) {
     upload(host, o_rr, rr);
     upload(host, o_rs, rs);
   }
+  // supernode of every column, offsets of the triangular inverses
+  size_t o_snof = 0, o_woff = 0;
+  h->w_off.resize((size_t)H.ns);
+  h->w_stride = 0;
+  for (int64_t k = 0; k < H.ns; k++) {
+    h->w_off[(size_t)k] = h->w_stride;
+    h->w_stride += 2 * H.sn_width[k] * H.sn_width[k];
+  }
+  upload(host, o_snof, narrow<int32_t>(H.sup_of));
+  upload(host, o_woff, h->w_off);
   // the global index of every position of R_L(K) (R_K)
   size_t o_lrows = 0;
   upload(host, o_lrows, narrow<int32_t>(H.rows));
@@ -308,6 +323,9 @@ int upload_structure(pselinv_ctx* h) {
   S.lrows = (const int32_t*)(b + o_lrows);
   S.urows = S.lrows;
   S.n = H.n;
+  S.sn_of = (const int32_t*)(b + o_snof);
+  S.w_off = (const int64_t*)(b + o_woff);
+  S.w_stride = h->w_stride;
   if (H.general) {
     S.sn_cu = (const int32_t*)(b + o_cu);
     S.urows_ptr = (const int64_t*)(b + o_urptr);
@@ -650,6 +668,79 @@ void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& pr
 void add_ozaki_schur(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
                      size_t base, bool lower);
 
+// tile of the diagonal blocks' small products: 16 x 16 while 32 x 32 tiles
+// would leave SMs without a CTA (a 32 x 32 x 32 product takes an SM's FP64
+// pipe about 9 us), 32 x 32 beyond
+int choose_small_tile(int dtype, const std::vector<GemmDesc>& descs) {
+  int64_t tiles = 0;
+  for (const GemmDesc& g : descs)
+    tiles += (int64_t)ceil_div(g.M, gemm_tile_m(dtype, GEMM_32x32)) *
+             ceil_div(g.N, gemm_tile_n(dtype, GEMM_32x32));
+  return tiles < 2 * 152 ? GEMM_16x16 : GEMM_32x32;
+}
+
+// One launch of panel tasks (32 lines each).  More than two per SM: tasks of
+// 32 kLuGroups lines, so that the pivot block is factored less often.
+void add_panel_step(Plan& P, const std::vector<LuTask>& tasks, int level) {
+  if (tasks.empty()) return;
+  Step d;
+  d.kind = ST_LU_PANEL;
+  d.cfg = tasks.size() > 2 * 152 ? kLuGroups : 1;
+  d.level = level;
+  if (d.cfg == 1) {
+    d.n = (int)tasks.size();
+    d.tasks = P.push(tasks);
+  } else {
+    std::vector<LuTask> grouped;
+    for (const LuTask& t : tasks)
+      if (t.line0 % (32 * kLuGroups) == 0) grouped.push_back(t);
+    d.n = (int)grouped.size();
+    d.tasks = P.push(grouped);
+  }
+  P.steps.push_back(d);
+}
+
+// The triangular inverses of the wide supernodes from those of their 32 x 32
+// pivot blocks (written by the panel steps), doubling the block size b: for
+// neighbouring blocks 1, 2 of one triangle
+//   (L^{-1})_21 = -(L_22)^{-1} (L_21 (L_11)^{-1}),
+//   (U^{-1})_12 = -(U_11)^{-1} (U_12 (U_22)^{-1}),
+// two launches per doubling for both triangles of every supernode.
+// mofs: scratch offset (s^2 / 2 scalars) of each one's inner products.
+void add_inverse_merges(pselinv_ctx* h, Plan& P, const std::vector<SnTask>& wide,
+                        const std::vector<int64_t>& mofs, int level) {
+  const HostSym& H = h->H;
+  const size_t es = h->esize;
+  for (int64_t b = kLuPanel; b < 256; b *= 2) {
+    std::vector<GemmDesc> inner, outer;
+    for (size_t t = 0; t < wide.size(); t++) {
+      const int64_t K = wide[t].K, s = H.sn_width[K];
+      const char* D = h->lu + ((size_t)wide[t].inst * H.storage + H.sn_offset[K]) * es;
+      char* Linv = h->winv + (size_t)(wide[t].inst * h->w_stride + h->w_off[K]) * es;
+      char* Uinv = Linv + (size_t)s * s * es;
+      char* T = h->scratch + (size_t)mofs[t] * es;
+      auto at = [&](auto* M, int64_t i, int64_t j) { return M + (size_t)(i + j * s) * es; };
+      for (int64_t i0 = 0; i0 + b < s; i0 += 2 * b) {
+        const int64_t i1 = i0 + b;
+        const int n1 = (int)b, n2 = (int)std::min<int64_t>(b, s - i1), ld = (int)s;
+        char* TU = T + (size_t)(n1 * n2) * es;
+        inner.push_back(make_desc(at(D, i1, i0), at(Linv, i0, i0), T, n2, n1, n1, ld, ld, n2, 0, 0,
+                                  1.0, 0.0, 0, 1, GEMM_TRI_LOWER_B));
+        outer.push_back(make_desc(at(Linv, i1, i1), T, at(Linv, i1, i0), n2, n1, n2, ld, n2, ld, 0,
+                                  0, -1.0, 0.0, 0, 1, GEMM_TRI_LOWER_A));
+        inner.push_back(make_desc(at(D, i0, i1), at(Uinv, i1, i1), TU, n1, n2, n2, ld, ld, n1, 0, 0,
+                                  1.0, 0.0, 0, 1, GEMM_TRI_UPPER_B));
+        outer.push_back(make_desc(at(Uinv, i0, i0), TU, at(Uinv, i0, i1), n1, n2, n1, ld, n1, ld, 0,
+                                  0, -1.0, 0.0, 0, 1, GEMM_TRI_UPPER_A));
+        T = TU + (size_t)(n1 * n2) * es;
+      }
+    }
+    if (inner.empty()) break;
+    add_gemm_step(P, h->dtype, choose_small_tile(h->dtype, inner), inner, level);
+    add_gemm_step(P, h->dtype, choose_small_tile(h->dtype, outer), outer, level);
+  }
+}
+
 int build_factor_plan(pselinv_ctx* h) {
   const HostSym& H = h->H;
   Plan& P = h->factor_plan;
@@ -673,72 +764,104 @@ int build_factor_plan(pselinv_ctx* h) {
   // upper triangle is mirrored from its lower one before its LU
   const bool ldlt = h->opts.symmetric != 0 && !H.general;
   for (size_t lev = 0; lev + 1 < H.hlevel_ptr.size(); lev++) {
-    std::vector<SnTask> diag, gt;
-    std::vector<TriBlock> tri;
+    std::vector<SnTask> wide, gt;  // wide: more than one panel
+    std::vector<LuTask> panels;    // first panels of every supernode, 32 lines per task
     std::vector<int64_t> gofs;
     std::vector<GemmDesc> trsm, schur;
-    std::vector<SchurProduct> sprods;
+    std::vector<SchurProduct> sprods, solves;
     std::vector<CopySeg> segs;
+    const int64_t l0 = H.hlevel_ptr[lev], l1 = H.hlevel_ptr[lev + 1];
+    // split precision: the triangular solves of wide supernodes and the Schur
+    // products of levels with enough Schur work as sliced tensor-core products
+    // (their operands sliced from the level's scratch after its FP64 region);
+    // otherwise FP64 row panels, which beat 64 x 64 tiles on these products
+    // at every width (40^3 factorisation 61.9 -> 57.1 ms)
+    double sflops = 0;
+    for (int64_t i = l0; i < l1; i++) {
+      const int64_t K = H.hlevel_sn[i];
+      sflops += 2.0 * (double)cK(H, K) * (double)cU(H, K) * (double)H.sn_width[K] * (double)nb;
+    }
+    const double min_flops = h->opts.factor_split_mflops < 0    ? 0.0
+                             : h->opts.factor_split_mflops == 0 ? 2e8
+                                                                : 1e6 * h->opts.factor_split_mflops;
+    const bool split = h->opts.factor_precision == PSELINV_PREC_OZAKI_FP16 && sflops > 0 &&
+                       sflops >= min_flops;
     int64_t off = 0;  // scalars into scratch
+    int64_t smax = 0;
+    std::vector<int64_t> mofs;  // scratch of the wide supernodes' inverse merges
     for (int64_t b = 0; b < nb; b++)
-      for (int64_t i = H.hlevel_ptr[lev]; i < H.hlevel_ptr[lev + 1]; i++) {
+      for (int64_t i = l0; i < l1; i++) {
         // c: rows of the L panel (R_K, or R_L(K) for a general pattern),
         // cu: rows of the U^T panel (c, or R_U(K))
         const int64_t K = H.hlevel_sn[i], s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
-        const int64_t w0 = off, t0 = w0 + 2 * s * s, s0 = t0 + (c + cu) * s;
-        off = s0 + c * cu;
-        diag.push_back({(int)b, (int)K, 0, 0});
-        if (c == 0 && cu == 0) continue;
-        tri.push_back({b, K, w0});
+        smax = std::max(smax, s);
+        const bool narrow = s <= kLuPanel;
+        const int64_t lines =
+            (narrow ? c + (ldlt ? 0 : cu) : 2 * (s - kLuPanel)) + 2 * std::min<int64_t>(s, kLuPanel);
+        for (int64_t l = 0; l < lines; l += 32) panels.push_back({(int)b, (int)K, 0, (int)l});
         char* base = h->lu + ((size_t)b * H.storage + H.sn_offset[K]) * es;
         char* Lp = base + (size_t)s * s * es;
         char* Up = Lp + (size_t)c * s * es;
-        char* Linv = h->scratch + (size_t)w0 * es;
+        char* Linv = h->winv + (size_t)(b * h->w_stride + h->w_off[K]) * es;
         char* Uinv = Linv + (size_t)s * s * es;
-        char* TL = h->scratch + (size_t)t0 * es;
-        char* TU = TL + (size_t)c * s * es;
+        // TL, TU: the solved panels, in place (narrow: by the panel step; split:
+        // the sliced products read copies), else in scratch and copied back
+        char *TL = Lp, *TU = Up;
+        if (!narrow) {
+          wide.push_back({(int)b, (int)K, 0, 0});
+          mofs.push_back(off);
+          off += s * s / 2;
+          if (!(split && c > 0 && cu > 0) && (c > 0 || cu > 0)) {
+            TL = h->scratch + (size_t)off * es;
+            TU = TL + (size_t)c * s * es;
+            off += (c + cu) * s;
+            // L = A U^-1, U^T = A^T L^-T: both B operands upper triangular
+            if (c > 0)
+              trsm.push_back(make_desc(Lp, Uinv, TL, c, s, s, c, s, c, 0, 0, 1.0, 0.0, 0, 1,
+                                       GEMM_TRI_UPPER_B));
+            if (cu > 0)
+              trsm.push_back(make_desc(ldlt ? Lp : Up, Linv, TU, cu, s, s, cu, s, cu, 0, 1, 1.0,
+                                       0.0, 0, 1, GEMM_TRI_UPPER_B));
+            segs.push_back({TL, Lp, (c + cu) * s});
+          }
+        }
+        const int64_t s0 = off;
+        off += c * cu;
         char* Sc = h->scratch + (size_t)s0 * es;
-        // L = A U^-1, U^T = A^T L^-T: both B operands upper triangular
-        if (c > 0)
-          trsm.push_back(make_desc(Lp, Uinv, TL, c, s, s, c, s, c, 0, 0, 1.0, 0.0, 0, 1,
-                                   GEMM_TRI_UPPER_B));
-        if (cu > 0)
-          trsm.push_back(make_desc(ldlt ? Lp : Up, Linv, TU, cu, s, s, cu, s, cu, 0, 1, 1.0, 0.0,
-                                   0, 1, GEMM_TRI_UPPER_B));
+        const SchurProduct q{TL, TU, Sc, (int)c, (int)cu, (int)s, Lp, ldlt ? Lp : Up, Uinv, Linv};
         if (c > 0 && cu > 0) {
+          if (!narrow && split) solves.push_back(q);
           schur.push_back(make_desc(TL, TU, Sc, c, cu, s, c, cu, c, 0, 1, 1.0, 0.0));
-          sprods.push_back({TL, TU, Sc, (int)c, (int)cu, (int)s, Lp, ldlt ? Lp : Up, Uinv, Linv});
+          sprods.push_back(q);
           for (int tq = 0; tq < ceil_div(cu, 32); tq++)
             for (int tp = ldlt ? tq : 0; tp < ceil_div(c, 32); tp++) {
               gt.push_back({(int)b, (int)K, tp, tq});
               gofs.push_back(s0);
             }
         }
-        segs.push_back({TL, Lp, (c + cu) * s});
       }
-    // blocked LU of the diagonal blocks: panels of 32 columns, each a panel
-    // launch (pivot block, L21 rows, U12 columns) and a trailing-update GEMM,
-    // batched over the level's supernodes
-    int64_t smax = 0;
-    for (const SnTask& t : diag) smax = std::max<int64_t>(smax, H.sn_width[t.K]);
-    if (ldlt && !diag.empty()) {
+    h->scratch_high = std::max(h->scratch_high, (size_t)off * es);
+    if (ldlt && !wide.empty()) {
       Step mr;
       mr.kind = ST_MIRROR;
-      mr.n = (int)diag.size();
-      mr.tasks = P.push(diag);
+      mr.n = (int)wide.size();
+      mr.tasks = P.push(wide);
       mr.level = (int)lev;
       P.steps.push_back(mr);
     }
-    for (int64_t j0 = 0; j0 < smax; j0 += 32) {
-      std::vector<SnTask> piv, pan;
+    // blocked LU of the diagonal blocks: per panel of 32 columns one panel
+    // launch and (wide supernodes) one trailing-update GEMM, batched over the
+    // level's supernodes; a narrow supernode is done after its panel
+    for (int64_t j0 = 0; j0 < smax; j0 += kLuPanel) {
       std::vector<GemmDesc> upd;
-      for (const SnTask& t : diag) {
+      if (j0 > 0) panels.clear();
+      for (const SnTask& t : wide) {
         const int64_t s = H.sn_width[t.K];
         if (s <= j0) continue;
-        const int64_t w = std::min<int64_t>(32, s - j0), rest = s - j0 - w;
-        const int nbk = (int)ceil_div(rest, 32);
-        piv.push_back({t.inst, t.K, (int)j0, 0});
-        for (int blk = 1; blk <= 2 * nbk; blk++) pan.push_back({t.inst, t.K, (int)j0, blk});
+        const int64_t w = std::min<int64_t>(kLuPanel, s - j0), rest = s - j0 - w;
+        if (j0 > 0)
+          for (int64_t l = 0; l < 2 * rest + 2 * w; l += 32)
+            panels.push_back({t.inst, t.K, (int)j0, (int)l});
         if (rest > 0) {
           char* D = h->lu + ((size_t)t.inst * H.storage + H.sn_offset[t.K]) * es;
           upd.push_back(make_desc(D + (size_t)(j0 + w + j0 * s) * es, D + (size_t)(j0 + (j0 + w) * s) * es,
@@ -746,39 +869,17 @@ int build_factor_plan(pselinv_ctx* h) {
                                   (int)w, (int)s, (int)s, (int)s, 0, 0, -1.0, 1.0));
         }
       }
-      for (const auto* list : {&piv, &pan}) {
-        if (list->empty()) continue;
-        Step d;
-        d.kind = ST_LU_PANEL;
-        d.n = (int)list->size();
-        d.tasks = P.push(*list);
-        d.level = (int)lev;
-        P.steps.push_back(d);
-      }
-      add_gemm_step(P, dt, kLuUpdateCfg, upd, (int)lev);
+      add_panel_step(P, panels, (int)lev);
+      add_gemm_step(P, dt, choose_small_tile(dt, upd), upd, (int)lev);
     }
-    // split precision: the triangular solves and the Schur products of
-    // levels with enough Schur work as sliced tensor-core products (their
-    // operands sliced from the level's scratch after its FP64 region);
-    // otherwise FP64 row panels, which beat 64 x 64 tiles on these products
-    // at every width (40^3 factorisation 61.9 -> 57.1 ms)
-    double sflops = 0;
-    for (const SchurProduct& q : sprods) sflops += 2.0 * q.c * q.cu * q.s;
-    const double min_flops = h->opts.factor_split_mflops < 0    ? 0.0
-                             : h->opts.factor_split_mflops == 0 ? 2e8
-                                                                : 1e6 * h->opts.factor_split_mflops;
-    const bool split = h->opts.factor_precision == PSELINV_PREC_OZAKI_FP16 && !sprods.empty() &&
-                       sflops >= min_flops;
-    add_tri_step(P, H, tri, (int)lev, 0);
-    if (split && sprods.size() * 2 == trsm.size()) {
-      add_ozaki_trsm(h, P, sprods, (int)lev, align256((size_t)off * es));
-    } else {
-      add_gemm_step(P, dt, GEMM_ROWS, trsm, (int)lev);
-    }
-    if (split)
+    add_inverse_merges(h, P, wide, mofs, (int)lev);
+    add_gemm_step(P, dt, GEMM_ROWS, trsm, (int)lev);
+    if (split) {
+      add_ozaki_trsm(h, P, solves, (int)lev, align256((size_t)off * es));
       add_ozaki_schur(h, P, sprods, (int)lev, align256((size_t)off * es), ldlt);
-    else
+    } else {
       add_gemm_step(P, dt, GEMM_ROWS, schur, (int)lev, -1, ldlt);
+    }
     if (!gt.empty()) {
       Step sc;
       sc.kind = ST_SCATTER_SUB;
@@ -790,6 +891,12 @@ int build_factor_plan(pselinv_ctx* h) {
       P.steps.push_back(sc);
     }
     add_copy_step(P, segs, (int)lev, es);
+  }
+  if (H.n > 0) {
+    Step up;
+    up.kind = ST_UNPACK_PIVOTS;
+    up.n = (int)H.ns;
+    P.steps.push_back(up);
   }
   if (h->scratch_high > h->scratch_bytes) return PSELINV_ERR_CHECK;
   CK(cudaMalloc(&P.arena, P.host.size() + 256));
@@ -1039,6 +1146,7 @@ struct OzBuilder {
 // and its slices serve both products.  Scratch from `base`.
 void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
                     size_t base) {
+  if (prods.empty()) return;
   OzBuilder ob(h, base);
   int64_t nmax = 0;
   for (const SchurProduct& q : prods) nmax += q.c + q.cu + 2 * q.s;
@@ -1689,7 +1797,11 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
                      (const SnTask*)(a + s.tasks), s.n, h->max_width, s.cfg, st);
       break;
     case ST_LU_PANEL:
-      launch_lu_panel(h->dtype, h->S, h->lu, (const SnTask*)(a + s.tasks), s.n, st);
+      launch_lu_panel(h->dtype, h->S, h->lu, h->winv, h->piv, (const LuTask*)(a + s.tasks), s.n,
+                      s.cfg, h->opts.symmetric != 0 && !h->H.general, st);
+      break;
+    case ST_UNPACK_PIVOTS:
+      launch_unpack_pivots(h->dtype, h->S, h->lu, h->piv, (int)h->nbatch, st);
       break;
     case ST_GATHER:
       if (h->H.general)
@@ -1834,12 +1946,15 @@ void free_numeric(pselinv_ctx* h) {
   cudaFree(h->nf);
   cudaFree(h->ainv);
   cudaFree(h->scratch);
+  cudaFree(h->winv);
+  cudaFree(h->piv);
   cudaFree(h->staging);
   cudaFree(h->outstage);
   cudaFree(h->cbuf);
   cudaFree(h->rcmax);
   h->lu = h->nf = h->ainv = h->scratch = h->staging = h->outstage = h->cbuf = nullptr;
   h->rcmax = nullptr;
+  h->winv = h->piv = nullptr;
   h->dtype = 0;
   h->nbatch = 0;
   h->factored = h->inverted = false;
@@ -2047,6 +2162,10 @@ int pselinv_factor(pselinv_t h, int dtype, int64_t nbatch, const void* values, v
     CK(cudaMalloc(&h->nf, sbytes));
     CK(cudaMalloc(&h->ainv, sbytes));
     CK(cudaMemset(h->nf, 0, sbytes));
+    // zeros outside the triangles, which are never written
+    CK(cudaMalloc(&h->winv, (size_t)nbatch * h->w_stride * es + 256));
+    CK(cudaMemset(h->winv, 0, (size_t)nbatch * h->w_stride * es + 256));
+    CK(cudaMalloc(&h->piv, (size_t)nbatch * h->H.n * kLuPanel * es + 256));
     h->scratch_bytes = scratch_need(h->H, nbatch, es);
     CK(cudaMalloc(&h->scratch, h->scratch_bytes));
     CK(cudaMalloc(&h->staging, (size_t)nbatch * h->H.nnz * es + 256));
@@ -2363,7 +2482,7 @@ int pselinv_profile(pselinv_t h, int which, void* stream, pselinv_step_stat* out
                                 PSELINV_STEP_SLICE,   PSELINV_STEP_OZAKI_GEMM, PSELINV_STEP_MEMSET,
                                 PSELINV_STEP_DIAG_LU, PSELINV_STEP_SMALL_LEVEL,
                                 PSELINV_STEP_GATHER_SLICE, PSELINV_STEP_OUTPUT_MAXIMA,
-                                PSELINV_STEP_COPY};
+                                PSELINV_STEP_COPY, PSELINV_STEP_COPY};
     out[i].kind = kinds[s.kind];
     out[i].level = s.level;
     out[i].tasks = s.n;

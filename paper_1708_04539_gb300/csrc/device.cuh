@@ -97,6 +97,11 @@ struct SymDev {
   const int32_t* lrows;
   const int32_t* urows;
   int64_t n;
+  const int32_t* sn_of;  // supernode of every (permuted) column
+  // triangular inverses of the diagonal blocks: L_KK^{-1} (s x s) and behind
+  // it U_KK^{-1} at winv + inst * w_stride + w_off[K]
+  const int64_t* w_off;
+  int64_t w_stride;
   // general patterns (general = 1; null for structurally symmetric
   // handles): sn_c, rows_ptr, rows_blk and blk_* describe R_L(K) (the L
   // panel's rows), sn_cu, urows_ptr, urows_blk and ublk_* R_U(K) (the U^T
@@ -166,6 +171,9 @@ constexpr int GEMM_TRI_LOWER_B = 1;
 constexpr int GEMM_TRI_UPPER_A = 2;
 // op(B)(k, n) = 0 for k > n (upper triangular B): a tile needs k < n0 + BN
 constexpr int GEMM_TRI_UPPER_B = 4;
+// op(A)(m, k) = 0 for k > m (lower triangular A): a tile needs k < m0 + BM
+// (tile kernels only)
+constexpr int GEMM_TRI_LOWER_A = 8;
 struct GemmTask {
   int d, tm, tn, ks;
 };
@@ -173,6 +181,14 @@ struct GemmTask {
 // per-supernode work item (instance, supernode, extra)
 struct SnTask {
   int inst, K, a, b;
+};
+
+// panel step of the diagonal LU: 32-column panels, tasks of 32 or
+// 32 kLuGroups lines (see lu_panel_kernel)
+constexpr int kLuPanel = 32;
+constexpr int kLuGroups = 3;
+struct LuTask {
+  int inst, K, j0, line0;
 };
 
 // contiguous copy segment
@@ -279,14 +295,15 @@ enum DType { DT_F64 = 1, DT_C128 = 2 };
 // and the zero triangle of a triangular op(B) skipped exactly).  Its tasks
 // are {d, row block, column chunk, NW + 16 x K chunk}, NW in {4, 8} the
 // width the kernel computes for the chunk.
-enum GemmCfg { GEMM_64x64 = 0, GEMM_32x32 = 1, GEMM_128x64 = 2, GEMM_ROWS = 3, GEMM_NCFG = 4 };
+enum GemmCfg { GEMM_64x64 = 0, GEMM_32x32 = 1, GEMM_128x64 = 2, GEMM_ROWS = 3, GEMM_NCFG = 4,
+               GEMM_16x16 = 4 };  // 16 x 16: small factorisation products, not tunable
 constexpr int kRowsBlock = 64;
 constexpr int kRowsChunk = 8;
 // a triangular op(B) (at most one of LOWER_B / UPPER_B) must be square; an
 // upper op(A) only goes with a lower op(B)
 inline bool rows_eligible(const GemmDesc& d) {
   const int t = d.tri & (GEMM_TRI_LOWER_B | GEMM_TRI_UPPER_B);
-  if (t == (GEMM_TRI_LOWER_B | GEMM_TRI_UPPER_B)) return false;
+  if (t == (GEMM_TRI_LOWER_B | GEMM_TRI_UPPER_B) || (d.tri & GEMM_TRI_LOWER_A)) return false;
   if (t != 0 && d.N != d.K) return false;
   return !(d.tri & GEMM_TRI_UPPER_A) || t == GEMM_TRI_LOWER_B;
 }
@@ -306,10 +323,13 @@ size_t trace_partial_bytes();
 // value scatter (A's entries into the storage of every instance)
 void launch_scatter_values(int dtype, const SymDev& S, const void* values, void* store,
                            int nbatch, cudaStream_t st);
-// one panel step of the blocked diagonal LU: tasks {inst, K, j0, blk}
-// (blk 0: pivot block, 1..nb: rows of L21, nb+1..2nb: columns of U12)
-void launch_lu_panel(int dtype, const SymDev& S, void* store, const SnTask* tasks, int ntasks,
-                     cudaStream_t st);
+// one panel step of the blocked diagonal LU (one CTA per task; groups = 1 or
+// kLuGroups: 32 or 32 kLuGroups lines per task; sym: symmetric values), and
+// the factored pivot blocks into the storage
+void launch_lu_panel(int dtype, const SymDev& S, void* store, void* winv, void* piv,
+                     const LuTask* tasks, int ntasks, int groups, bool sym, cudaStream_t st);
+void launch_unpack_pivots(int dtype, const SymDev& S, void* store, const void* piv, int nbatch,
+                          cudaStream_t st);
 // triangular inverses of the diagonal blocks of `store`:
 // tasks {inst, K, which (0 = L unit lower, 1 = U upper), first column of a
 // panel of 8 columns}; small = 1: blocks of width <= 32, one task per

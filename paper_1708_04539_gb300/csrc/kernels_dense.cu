@@ -8,6 +8,8 @@
 // 4 flop/clk/SM), so the FP64 GEMM is a register-tiled SIMT DFMA kernel:
 // it saturates the FP64 pipe with a 16x16 thread grid and 4x4 (real) or
 // 2x2 (complex) outputs per thread.
+#include <algorithm>
+
 #include "device.cuh"
 
 namespace pselinv {
@@ -43,6 +45,7 @@ gemm_kernel(const GemmDesc* __restrict__ descs, const GemmTask* __restrict__ tas
     if (d.tri & GEMM_TRI_LOWER_B) kb = max(kb, n0);
     if (d.tri & GEMM_TRI_UPPER_A) kb = max(kb, m0);
     if (d.tri & GEMM_TRI_UPPER_B) ke = min(ke, n0 + BN);
+    if (d.tri & GEMM_TRI_LOWER_A) ke = min(ke, m0 + BM);
     T acc[TM][TN];
 #pragma unroll
     for (int i = 0; i < TM; i++)
@@ -126,106 +129,260 @@ gemm_kernel(const GemmDesc* __restrict__ descs, const GemmTask* __restrict__ tas
   }
 }
 
-// Panel step of the blocked LU without pivoting of the s x s diagonal
-// block of a supernode (right-looking, panels of 32 columns; the trailing
-// update A22 -= L21 U12 is a GEMM launch of its own).  Task {inst, K, j0,
-// blk} with w = min(32, s - j0) and nb = number of 32-blocks below the
-// pivot block: blk = 0 factors the w x w pivot block at (j0, j0) in shared
-// memory and writes it back (a launch of its own, before the others read
-// it); blk in [1, nb] solves the 32 rows j0 + w + 32 (blk - 1) .. of
-// L21 = A21 U11^{-1}, blk in [nb + 1, 2 nb] the 32 columns of
-// U12 = L11^{-1} A12.  One division per pivot and CTA.
+// Panel step of the blocked LU without pivoting of the supernodes' diagonal
+// blocks (right-looking, panels of 32 columns; the trailing update A22 -=
+// L21 U12 is a GEMM launch of its own).  A task {inst, K, j0, line0} factors
+// the w x w pivot block at (j0, j0), w = min(32, s - j0), in registers and
+// eliminates 32 G "lines" beside it.  The lines of a panel, in order:
+//   nl rows of L21 (X U11 = A21), nl columns of U12 (L11 Y = A12): the rest of
+//      the diagonal block (s > 32: nl = s - j0 - w, in place);
+//   for a narrow supernode (s <= 32, one panel) instead the c rows of its L
+//      panel and the cu rows of its U^T panel, so that its triangular solves
+//      need no inverse and no launch of their own (symmetric values: no U^T
+//      lines, an L line's unscaled entries are the row of U^T);
+//   w unit rows and w unit columns: U11^{-1} and L11^{-1} into winv.
+// Every task of a panel factors the pivot block again (the FP64 pipe takes
+// 64 cycles per warp instruction whatever the mask, so the pivot block's
+// chain, not its work, is what a panel waits for, and a second launch would
+// wait for it twice).  The task with line0 = 0 stores the factored block in
+// `piv` (column j of the matrix at piv + 32 (inst n + j)); unpack_pivots moves
+// it into the storage once nobody reads the unfactored block any more.
+// Threads: warp 0 runs the pivot chain alone on its scheduler: an FP64
+// instruction of a chain takes 64 cycles on an idle SM, 133 while the other
+// three schedulers keep the pipe full and 366 when its own does too.  Warps
+// 1-3 hold the pivot block (row = lane, columns 3 jj + (warp & 3) - 1),
+// warps 4 g + 1 .. 4 g + 3 the lines 32 (g - 1) .. of the task (line = lane,
+// entries along the panel in registers).  Step k, one block barrier: warp 0
+// updates column k + 1, computes its reciprocal and the scaled column of L;
+// the others apply step k to the columns behind it and publish row k + 1,
+// column k + 2 and the lines' entries k + 1.
+// Bound: the pivot chain (five dependent FP64 operations and a barrier per
+// column) and, about as long, the FP64 pipe.
+template <typename T>
+__device__ __forceinline__ T shfl_t(T v, int src);
+template <>
+__device__ __forceinline__ double shfl_t(double v, int src) {
+  return __shfl_sync(0xffffffffu, v, src);
+}
+template <>
+__device__ __forceinline__ cdouble shfl_t(cdouble v, int src) {
+  return {__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src)};
+}
+// 1 / d: the approximate reciprocal (relative error e below 2^-19) and one
+// third-order step r (1 + e + e^2) of the Householder family, three dependent
+// operations against about nine of a division; within 2^-52 of 1 / d over
+// 10^8 random mantissas.  Numbers near the ends of the range, zeros and
+// non-finite ones take the division.
+__device__ __forceinline__ double rcp_s(double d) {
+  const int e = (__double2hiint(d) >> 20) & 0x7FF;
+  if (e < 64 || e > 1982) return 1.0 / d;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  const double h = fma(-d, r, 1.0);
+  return fma(r, fma(h, h, h), r);
+}
+__device__ __forceinline__ cdouble rcp_s(cdouble b) {
+  const int ex = (__double2hiint(b.x) >> 20) & 0x7FF, ey = (__double2hiint(b.y) >> 20) & 0x7FF;
+  const int e = max(ex, ey);
+  if (e < 640 || e > 1400) return div_s(sc_one(cdouble()), b);  // |b|^2 could leave the range
+  const double r = rcp_s(fma(b.x, b.x, b.y * b.y));
+  return {b.x * r, -b.y * r};
+}
+__device__ __forceinline__ double fnma_s(double a, double b, double c) { return fma(-a, b, c); }
+__device__ __forceinline__ cdouble fnma_s(cdouble a, cdouble b, cdouble c) {
+  return {fma(-a.x, b.x, fma(a.y, b.y, c.x)), fma(-a.x, b.y, fma(-a.y, b.x, c.y))};
+}
+
+constexpr int kLuW = kLuPanel;  // panel width
+template <typename T, int G>
+__global__ void __launch_bounds__(128 * (G + 1))
+lu_panel_kernel(SymDev S, T* store, T* winv, T* piv, const LuTask* __restrict__ tasks, int sym) {
+  constexpr int kThr = 128 * (G + 1);
+  extern __shared__ __align__(16) unsigned char lu_smem[];
+  T(*Dd)[kLuW + 1] = reinterpret_cast<T(*)[kLuW + 1]>(lu_smem);  // A11, then the rows of U11
+  T(*Ls)[kLuW + 1] = Dd + kLuW;                                  // scaled columns of L11
+  T(*X)[kLuW + 1] = Ls + kLuW;                                   // lines (unscaled)
+  T* R = reinterpret_cast<T*>(X + 32 * G);                       // reciprocals of the pivots
+  T(*Cn)[kLuW] = reinterpret_cast<T(*)[kLuW]>(R + kLuW);         // the chain's next column
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int team = warp >> 2, q = (warp & 3) - 1;  // q = -1: the chain (warp 0) or idle
+  const LuTask task = tasks[blockIdx.x];
+  const int K = task.K, j0 = task.j0, s = S.sn_width[K], c = S.sn_c[K];
+  const int w = min(kLuW, s - j0), rest = s - j0 - w;
+  const bool narrow = s <= kLuW;
+  T* D = store + (int64_t)task.inst * S.storage + S.sn_off[K];
+  T* W = winv + (int64_t)task.inst * S.w_stride + S.w_off[K];
+  // line ranges and addresses: entry k of L line i at Lb[i + k ldl], of U line i
+  // at Ub[i us + k uk]
+  const int cu = S.general ? S.sn_cu[K] : c;
+  const int nl = narrow ? c : rest, nu = narrow ? (sym ? 0 : cu) : rest;
+  T* Lb = narrow ? D + s * s : D + (j0 + w) + (int64_t)j0 * s;
+  const int64_t ldl = narrow ? c : s;
+  T* Ub = narrow ? D + s * s + (int64_t)c * s : D + j0 + (int64_t)(j0 + w) * s;
+  const int64_t us = narrow ? 1 : s, uk = narrow ? cu : 1;
+  const int nlines = nl + nu + 2 * w;
+
+  for (int e = tid; e < kLuW * kLuW; e += kThr) {
+    const int i = e & (kLuW - 1), j = e / kLuW;
+    // symmetric values: a narrow block's upper triangle is its lower one's
+    const int si = sym && narrow && i < j ? j : i, sj = sym && narrow && i < j ? i : j;
+    Dd[i][j] = i < w && j < w ? D[(j0 + si) + (int64_t)(j0 + sj) * s] : sc_zero(T());
+    Ls[i][j] = sc_zero(T());
+  }
+  // lines: lanes along the lines (contiguous), except the columns of U12 of a
+  // wide block, contiguous along k
+  for (int e = tid; e < 32 * G * kLuW; e += kThr) {
+    const int i = e % (32 * G), k = e / (32 * G), l = task.line0 + i;
+    if (l >= nlines || k >= w) {
+      X[i][k] = sc_zero(T());
+    } else if (l < nl) {
+      X[i][k] = Lb[l + k * ldl];
+    } else if (l < nl + nu) {
+      if (narrow) X[i][k] = Ub[(l - nl) * us + k * uk];
+    } else {
+      const int u = l - nl - nu;  // unit row u, or unit column u - w
+      X[i][k] = (u < w ? u : u - w) == k ? sc_one(T()) : sc_zero(T());
+    }
+  }
+  if (!narrow)
+    for (int e = tid; e < 32 * G * kLuW; e += kThr) {
+      const int k = e & 31, i = e >> 5, l = task.line0 + i;
+      if (l >= nl && l < nl + nu && k < w) X[i][k] = Ub[(l - nl) * us + k * uk];
+    }
+  __syncthreads();
+  const int row = team == 0 ? lane : 32 * (team - 1) + lane;  // row of Dd or of X
+  // a line's multiplier and coefficients: L lines (and unit rows) x_k r_k and
+  // row k of U11, U lines (and unit columns) x_k and column k of L11
+  const int line = task.line0 + row;
+  const bool is_l = team > 0 && (line < nl || (line >= nl + nu && line < nl + nu + w));
+  if (warp == 0) {
+    T v = Dd[lane][0], l = sc_zero(T());
+    for (int k = 0; k < w; k++) {
+      // column k is final (rows >= k): its reciprocal and column of L11
+      if (k > 0) v = fnma_s(l, Dd[k - 1][k], k == 1 ? Dd[lane][1] : Cn[k & 1][lane]);
+      const T p = shfl_t(v, k);
+      const T r = rcp_s(p);
+      l = mul_s(v, r);
+      Ls[lane][k] = l;
+      if (lane == 0) {
+        R[k] = r;
+        Dd[k][k] = p;
+        if (is_zero(p)) set_error(S.err, DEV_ZERO_PIVOT, S.sn_first[K] + j0 + k);
+      }
+      __syncthreads();
+    }
+  } else if (q < 0) {
+    for (int k = 0; k < w; k++) __syncthreads();
+  } else {
+    constexpr int kCols = (kLuW + 2) / 3;
+    const T* sm = reinterpret_cast<const T*>(lu_smem);
+    const bool from_u = team == 0 || is_l;  // coefficients from the rows of U11
+    const int cbase = from_u ? 0 : kLuW * (kLuW + 1);
+    const int cj = from_u ? 1 : kLuW + 1, ck = from_u ? kLuW + 1 : 1;  // strides along j and k
+    const bool warp_l = __any_sync(0xffffffffu, is_l);
+    // a[jj] holds column 3 (t + jj) + q in round t (columns past the panel hold
+    // values nobody uses)
+    T a[kCols];
+#pragma unroll
+    for (int jj = 0; jj < kCols; jj++) {
+      const int j = min(3 * jj + q, kLuW - 1);
+      a[jj] = team == 0 ? Dd[row][j] : X[row][j];
+    }
+    const int nr = (w + 2) / 3;
+    for (int t = 0; t < nr; t++) {
+      const int nj = nr - t;  // columns of this warp still in the panel
+#pragma unroll
+      for (int kk = 0; kk < 3; kk++) {
+        const int k = 3 * t + kk;
+        if (k >= w) break;
+        __syncthreads();  // row k of U11, column k of L11, r_k and x_k are in place
+        // (rows <= k of the pivot block are final and published: their lanes run along)
+        T m = team == 0 ? Ls[lane][k] : X[row][k];
+        if (warp_l) {
+          const T ml = mul_s(m, R[k]);
+          if (is_l) m = ml;
+        }
+        const T* cp = sm + cbase + (3 * t + q) * cj + k * ck;
+        // team 0 publishes column k + 2 for the chain (which has column k + 1
+        // itself), the lines their entry k + 1
+        const int ahead = team == 0 ? 2 : 1;
+        if (q - kk >= ahead) {
+          a[0] = fnma_s(m, cp[0], a[0]);
+          if (q - kk == ahead) {
+            if (team == 0) Cn[k & 1][lane] = a[0];
+            else X[row][k + 1] = a[0];
+          }
+        }
+        if (nj > 1 && q + 3 - kk >= ahead) {
+          a[1] = fnma_s(m, cp[3 * cj], a[1]);
+          if (q + 3 - kk == ahead) {
+            if (team == 0) Cn[k & 1][lane] = a[1];
+            else X[row][k + 1] = a[1];
+          }
+        }
+        // (jumps out: a predicated-off FP64 instruction still takes its 64 cycles)
+#pragma unroll
+        for (int jj = 2; jj < kCols; jj++) {
+          if (jj >= nj) break;
+          a[jj] = fnma_s(m, cp[3 * jj * cj], a[jj]);
+        }
+        if (team == 0 && lane == k + 1) {  // row k + 1 of U11 right of its diagonal is final
+#pragma unroll
+          for (int jj = 0; jj < kCols; jj++) {
+            const int j = 3 * (t + jj) + q;
+            if (jj < nj && j > k + 1) Dd[k + 1][j] = a[jj];
+          }
+        }
+      }
+#pragma unroll
+      for (int jj = 0; jj + 1 < kCols; jj++) a[jj] = a[jj + 1];
+    }
+  }
+  __syncthreads();
+  if (task.line0 == 0) {
+    T* P = piv + ((int64_t)task.inst * S.n + S.sn_first[K] + j0) * kLuW;
+    for (int e = tid; e < w * w; e += kThr) {
+      const int i = e % w, j = e / w;
+      P[i + j * kLuW] = i <= j ? Dd[i][j] : Ls[i][j];
+    }
+  }
+  for (int e = tid; e < 32 * G * kLuW; e += kThr) {
+    const int i = e % (32 * G), k = e / (32 * G), l = task.line0 + i;
+    if (l >= nlines || k >= w) continue;
+    const T x = X[i][k];
+    if (l < nl) {
+      Lb[l + k * ldl] = mul_s(x, R[k]);
+      if (sym && narrow) D[s * s + (int64_t)c * s + l + (int64_t)k * c] = x;
+    } else if (l < nl + nu) {
+      if (narrow) Ub[(l - nl) * us + k * uk] = x;
+    } else {
+      const int u = l - nl - nu;
+      if (u < w)  // row u of U11^{-1}
+        W[(int64_t)s * s + (j0 + u) + (int64_t)(j0 + k) * s] = k < u ? sc_zero(T()) : mul_s(x, R[k]);
+      else  // column u - w of L11^{-1}
+        W[(j0 + k) + (int64_t)(j0 + u - w) * s] = k < u - w ? sc_zero(T()) : x;
+    }
+  }
+  if (!narrow)
+    for (int e = tid; e < 32 * G * kLuW; e += kThr) {
+      const int k = e & 31, i = e >> 5, l = task.line0 + i;
+      if (l >= nl && l < nl + nu && k < w) Ub[(l - nl) * us + k * uk] = X[i][k];
+    }
+}
+
+// The factored pivot blocks (piv, see lu_panel_kernel) into the diagonal
+// blocks of the storage: one thread per entry.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-lu_panel_kernel(SymDev S, T* store, const SnTask* __restrict__ tasks, int ntasks) {
-  __shared__ T Dd[32][33];
-  __shared__ T R[32];
-  __shared__ T X[32][33];
-  const int tid = threadIdx.x;
-  for (int t = blockIdx.x; t < ntasks; t += gridDim.x) {
-    const SnTask task = tasks[t];
-    const int K = task.K;
-    const int s = S.sn_width[K];
-    const int j0 = task.a, blk = task.b;
-    const int w = min(32, s - j0);
-    T* D = store + (int64_t)task.inst * S.storage + S.sn_off[K];
-    for (int e = tid; e < w * w; e += kThreads) {
-      const int i = e % w, j = e / w;
-      Dd[i][j] = D[(j0 + i) + (int64_t)(j0 + j) * s];
-    }
-    __syncthreads();
-    const int nb = (s - j0 - w + 31) / 32;
-    if (blk == 0) {
-      for (int k = 0; k < w; k++) {
-        if (tid == 0) {
-          const T piv = Dd[k][k];
-          if (is_zero(piv)) set_error(S.err, DEV_ZERO_PIVOT, S.sn_first[K] + j0 + k);
-          R[k] = div_s(sc_one(T()), piv);
-        }
-        __syncthreads();
-        for (int i = k + 1 + tid; i < w; i += kThreads) Dd[i][k] = mul_s(Dd[i][k], R[k]);
-        __syncthreads();
-        const int m = w - k - 1;
-        for (int e = tid; e < m * m; e += kThreads) {
-          const int i = k + 1 + e % m, j = k + 1 + e / m;
-          Dd[i][j] = sub_s(Dd[i][j], mul_s(Dd[i][k], Dd[k][j]));
-        }
-        __syncthreads();
-      }
-      for (int e = tid; e < w * w; e += kThreads) {
-        const int i = e % w, j = e / w;
-        D[(j0 + i) + (int64_t)(j0 + j) * s] = Dd[i][j];
-      }
-      __syncthreads();
-      continue;
-    }
-    // the pivot block is factored already: L11 below, U11 on and above
-    if (tid < w) R[tid] = div_s(sc_one(T()), Dd[tid][tid]);
-    __syncthreads();
-    if (blk <= nb) {
-      // rows of L21: X U11 = A21, one column of X at a time
-      const int r0 = j0 + w + 32 * (blk - 1), nr = min(32, s - r0);
-      for (int e = tid; e < nr * w; e += kThreads) {
-        const int i = e % nr, j = e / nr;
-        X[i][j] = D[(r0 + i) + (int64_t)(j0 + j) * s];
-      }
-      __syncthreads();
-      for (int j = 0; j < w; j++) {
-        for (int i = tid; i < nr; i += kThreads) X[i][j] = mul_s(X[i][j], R[j]);
-        __syncthreads();
-        const int m = w - j - 1;
-        for (int e = tid; e < nr * m; e += kThreads) {
-          const int i = e % nr, kk = j + 1 + e / nr;
-          X[i][kk] = sub_s(X[i][kk], mul_s(X[i][j], Dd[j][kk]));
-        }
-        __syncthreads();
-      }
-      for (int e = tid; e < nr * w; e += kThreads) {
-        const int i = e % nr, j = e / nr;
-        D[(r0 + i) + (int64_t)(j0 + j) * s] = X[i][j];
-      }
-    } else {
-      // columns of U12: L11 Y = A12 (unit lower), one row of Y at a time
-      const int c0 = j0 + w + 32 * (blk - nb - 1), nc = min(32, s - c0);
-      for (int e = tid; e < w * nc; e += kThreads) {
-        const int i = e % w, j = e / w;
-        X[i][j] = D[(j0 + i) + (int64_t)(c0 + j) * s];
-      }
-      __syncthreads();
-      for (int k = 0; k < w - 1; k++) {
-        const int m = w - k - 1;
-        for (int e = tid; e < m * nc; e += kThreads) {
-          const int i = k + 1 + e % m, j = e / m;
-          X[i][j] = sub_s(X[i][j], mul_s(Dd[i][k], X[k][j]));
-        }
-        __syncthreads();
-      }
-      for (int e = tid; e < w * nc; e += kThreads) {
-        const int i = e % w, j = e / w;
-        D[(j0 + i) + (int64_t)(c0 + j) * s] = X[i][j];
-      }
-    }
-    __syncthreads();
+unpack_pivots_kernel(SymDev S, T* store, const T* __restrict__ piv, int64_t total) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t g = e / kLuW, b = g / S.n;
+    const int i = (int)(e - g * kLuW), col = (int)(g - b * S.n);
+    const int K = S.sn_of[col], s = S.sn_width[K], j = col - S.sn_first[K];
+    const int j0 = j & ~(kLuW - 1);
+    if (i < min(kLuW, s - j0))
+      store[b * S.storage + S.sn_off[K] + (j0 + i) + (int64_t)j * s] = piv[e];
   }
 }
 
@@ -515,11 +672,13 @@ void gemm_launch_t(const GemmDesc* descs, const GemmTask* tasks, int ntasks, int
 }  // namespace
 
 int gemm_tile_m(int dtype, int cfg) {
+  if (cfg == GEMM_16x16) return 16;
   if (cfg == GEMM_128x64) return dtype == DT_F64 ? 128 : 64;
   if (cfg == GEMM_32x32) return 32;
   return dtype == DT_F64 ? 64 : 32;
 }
 int gemm_tile_n(int dtype, int cfg) {
+  if (cfg == GEMM_16x16) return 16;
   if (cfg == GEMM_128x64) return dtype == DT_F64 ? 64 : 32;
   if (cfg == GEMM_32x32) return dtype == DT_F64 ? 32 : 16;
   return dtype == DT_F64 ? 64 : 32;
@@ -537,12 +696,14 @@ void launch_gemm(int dtype, int cfg, const GemmDesc* descs, const GemmTask* task
   }
   if (dtype == DT_F64) {
     switch (cfg) {
+      case GEMM_16x16: gemm_launch_t<double, 16, 16, 32>(descs, tasks, ntasks, grid, st); break;
       case GEMM_32x32: gemm_launch_t<double, 32, 32, 16>(descs, tasks, ntasks, grid, st); break;
       case GEMM_128x64: gemm_launch_t<double, 128, 64, 8>(descs, tasks, ntasks, grid, st); break;
       default: gemm_launch_t<double, 64, 64, 16>(descs, tasks, ntasks, grid, st); break;
     }
   } else {
     switch (cfg) {
+      case GEMM_16x16: gemm_launch_t<cdouble, 16, 16, 32>(descs, tasks, ntasks, grid, st); break;
       case GEMM_32x32: gemm_launch_t<cdouble, 32, 16, 16>(descs, tasks, ntasks, grid, st); break;
       case GEMM_128x64: gemm_launch_t<cdouble, 64, 32, 8>(descs, tasks, ntasks, grid, st); break;
       default: gemm_launch_t<cdouble, 32, 32, 16>(descs, tasks, ntasks, grid, st); break;
@@ -550,16 +711,53 @@ void launch_gemm(int dtype, int cfg, const GemmDesc* descs, const GemmTask* task
   }
 }
 
-void launch_lu_panel(int dtype, const SymDev& S, void* store, const SnTask* tasks, int ntasks,
-                     cudaStream_t st) {
+namespace {
+template <typename T, int G>
+constexpr int lu_smem_bytes() {
+  return (int)sizeof(T) * ((2 + G) * kLuW * (kLuW + 1) + 3 * kLuW);
+}
+template <typename T, int G>
+void lu_launch_t(const SymDev& S, void* store, void* winv, void* piv, const LuTask* tasks,
+                 int ntasks, bool sym, cudaStream_t st) {
+  lu_panel_kernel<T, G><<<ntasks, 128 * (G + 1), lu_smem_bytes<T, G>(), st>>>(
+      S, (T*)store, (T*)winv, (T*)piv, tasks, sym ? 1 : 0);
+}
+}  // namespace
+
+void launch_lu_panel(int dtype, const SymDev& S, void* store, void* winv, void* piv,
+                     const LuTask* tasks, int ntasks, int groups, bool sym, cudaStream_t st) {
   if (ntasks <= 0) return;
-  if (dtype == DT_F64)
-    lu_panel_kernel<double><<<ntasks, kThreads, 0, st>>>(S, (double*)store, tasks, ntasks);
-  else
-    lu_panel_kernel<cdouble><<<ntasks, kThreads, 0, st>>>(S, (cdouble*)store, tasks, ntasks);
+  if (dtype == DT_F64) {
+    if (groups == 1) lu_launch_t<double, 1>(S, store, winv, piv, tasks, ntasks, sym, st);
+    else lu_launch_t<double, kLuGroups>(S, store, winv, piv, tasks, ntasks, sym, st);
+  } else {
+    if (groups == 1) lu_launch_t<cdouble, 1>(S, store, winv, piv, tasks, ntasks, sym, st);
+    else lu_launch_t<cdouble, kLuGroups>(S, store, winv, piv, tasks, ntasks, sym, st);
+  }
 }
 
-cudaError_t prepare_dense_kernels(int, int) { return cudaSuccess; }
+void launch_unpack_pivots(int dtype, const SymDev& S, void* store, const void* piv, int nbatch,
+                          cudaStream_t st) {
+  const int64_t total = (int64_t)nbatch * S.n * kLuW;
+  if (total == 0) return;
+  const int grid = (int)std::min<int64_t>((total + kThreads - 1) / kThreads, 152 * 16);
+  if (dtype == DT_F64)
+    unpack_pivots_kernel<double><<<grid, kThreads, 0, st>>>(S, (double*)store, (const double*)piv,
+                                                            total);
+  else
+    unpack_pivots_kernel<cdouble><<<grid, kThreads, 0, st>>>(S, (cdouble*)store,
+                                                             (const cdouble*)piv, total);
+}
+
+cudaError_t prepare_dense_kernels(int, int) {
+  const cudaError_t e = cudaFuncSetAttribute(lu_panel_kernel<cdouble, 1>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             lu_smem_bytes<cdouble, 1>());
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(lu_panel_kernel<cdouble, kLuGroups>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              lu_smem_bytes<cdouble, kLuGroups>());
+}
 
 namespace {
 // FP64 pipe throughput: kPeakChains independent fused multiply-add chains
