@@ -1436,6 +1436,31 @@ constexpr int kNormMaxKsplit = 8;
 constexpr int64_t kTriSideTasks = 4 * 152;
 constexpr int64_t kTriThirdTasks = 8 * 152;
 
+// K split of FP64 products: a task's chain of multiply-adds (row panels: 8 per
+// k, 64 cycles each) should not outlast a quarter of the launch's work spread
+// over the chip (16 cycles per warp operation and SM), so that a few tasks
+// more or less per scheduler do not show, down to chunks of 32.  Returns
+// whether any product is split (its chunks then add atomically).  24^3 upwind
+// sweep: step 4 of level 7 (24 MFLOP, K up to 500) 160 -> 41 us, steps 3 and 5
+// of level 2 (110 MFLOP, 384 tasks unsplit) 150 -> 119 us.
+bool split_fp64_products(std::vector<GemmDesc>& descs, int dtype) {
+  const double cplx = dtype == DT_F64 ? 1.0 : 4.0;
+  double ops = 0;
+  for (const GemmDesc& g : descs) ops += (double)ceil_div(g.M, 32) * g.N * (double)g.K * cplx;
+  const double least = 32.0 * kRowsChunk * 64.0 * cplx;
+  const double target = std::max(ops * 4.0 / 152.0, least);
+  bool any = false;
+  for (GemmDesc& g : descs) {
+    const int ks = (int)std::min(std::ceil(g.K * kRowsChunk * 64.0 * cplx / target),
+                                 std::max(1.0, g.K / 32.0));
+    if (ks <= 1) continue;
+    g.ksplit = ks;
+    g.atomic = 1;
+    any = true;
+  }
+  return any;
+}
+
 // An FP64 level of narrow supernodes as one fused launch (gather and steps
 // 3-5 in shared memory), each supernode's output columns split into tasks
 // of at most kSmallLevelTaskFma multiply-adds, when every supernode fits
@@ -1655,6 +1680,7 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
       for (int64_t i = H.level_ptr[lev]; i < H.level_ptr[lev + 1]; i++)
         if (in_set(H.level_sn[i])) groups.push_back({H.level_sn[i]});
     }
+    std::vector<CopySeg> zmain;  // outputs of steps 3 and 5 that are accumulated
     const int slot_main = precision == PSELINV_PREC_OZAKI_FP16 ? 4 : 1;
     const int slot_diag = precision == PSELINV_PREC_OZAKI_FP16 ? 5 : 2;
     for (const auto& grp : groups) {
@@ -1689,7 +1715,6 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
           const size_t so = ((size_t)b * H.storage + H.sn_offset[K]) * es;
           const size_t lo = so + (size_t)s * s * es, uo = lo + (size_t)c * s * es;
           char* G = h->scratch + (size_t)g0 * es;
-          const int ksplit = std::max(1, (int)std::min<int64_t>(cu / 256, 64));
           if (H.general) {
             // G = Ainv(R_U, R_L) (cu x c).  Step 3: Ainv(R_U, K) = -G Lhat into
             // the U^T panel; step 5: Ainv(K, R_L)^T = -G^T Uhat^T into the L
@@ -1702,7 +1727,7 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
             main.push_back(make_desc(G, h->nf + lo, h->ainv + uo, cu, s, c, cu, c, cu, 0, 0, -1.0, 0.0));
             main.push_back(make_desc(G, h->nf + uo, h->ainv + lo, c, s, cu, cu, cu, c, 1, 0, -1.0, 0.0));
             dg.push_back(make_desc(h->nf + uo, h->ainv + uo, h->ainv + so, s, s, cu, cu, cu, s, 1, 0,
-                                   -1.0, 1.0, 1, ksplit));
+                                   -1.0, 1.0, 1));
             continue;
           }
           for (int tq = 0; tq < ceil_div(c, 32); tq++)
@@ -1717,7 +1742,7 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
           else
             main.push_back(make_desc(G, h->nf + uo, h->ainv + uo, c, s, c, c, c, c, 1, 0, -1.0, 0.0));
           dg.push_back(make_desc(h->nf + (sym ? lo : uo), h->ainv + lo, h->ainv + so, s, s, c, c, c,
-                                 s, 1, 0, -1.0, 1.0, 1, ksplit));
+                                 s, 1, 0, -1.0, 1.0, 1));
         }
       add_zero_step(P, zsegs, (int)lev);
       if (gt.empty()) continue;
@@ -1729,6 +1754,10 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
       g.offs = P.push(gofs);
       g.level = (int)lev;
       P.steps.push_back(g);
+      if (split_fp64_products(main, dt))
+        for (const GemmDesc& m : main)
+          if (m.atomic) zmain.push_back({nullptr, m.C, (int64_t)m.M * m.N * (int64_t)(es / 8)});
+      split_fp64_products(dg, dt);
       add_gemm_step(P, dt, tuned_value(h, precision, (int)lev, slot_main, cfg), main, (int)lev,
                     slot_main);
       add_copy_step(P, mirror, (int)lev, es);
@@ -1741,7 +1770,19 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
         if (in_set(H.level_sn[i])) sns.push_back(H.level_sn[i]);
       add_outmax_step(h, P, sns, (int)lev);
     }
-    if (P.steps.size() > first_main) P.steps[first_main].wait = EV_LEVEL + (int)lev;
+    size_t main_at = first_main;
+    if (!zmain.empty()) {  // zeroed on the side stream, behind the level's normalisation
+      add_zero_step(P, zmain, (int)lev);
+      Step z = P.steps.back();
+      P.steps.pop_back();
+      z.side = 1;
+      z.signal = EV_LEVEL + (int)lev;
+      if (first_main > 0 && P.steps[first_main - 1].signal == z.signal)
+        P.steps[first_main - 1].signal = -1;
+      P.steps.insert(P.steps.begin() + (std::ptrdiff_t)first_main, z);
+      main_at++;
+    }
+    if (P.steps.size() > main_at) P.steps[main_at].wait = EV_LEVEL + (int)lev;
   }
   if (last_split >= 0) {
     // a partitioned sweep starts from imported blocks G_r = Ainv(R_U(r),
