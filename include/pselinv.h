@@ -330,10 +330,8 @@ typedef struct pselinv_step_stat {
   double ms;      /* device time from CUDA events around the launch */
   int32_t param;  /* GEMM: kernel config (0 64x64, 1 32x32, 2 128x64 tiles, 3 row
                      panels); OZAKI_GEMM: K split;
-                     TRI_INV: 0 wide blocks (a warp per column), 1 blocks <= 32 wide;
                      else -1 */
-  int32_t side;   /* stream of the launch in a sweep: 0 main, 1 normalisation side stream,
-                     2 third stream (triangular inverses of the deeper levels) */
+  int32_t side;   /* stream of the launch in a sweep: 0 main, 1 normalisation side stream */
   double start_ms; /* which = 2: time from the start of the sweep until the launch's stream
                       reached it (its wait included); else 0 */
 } pselinv_step_stat;

@@ -42,7 +42,6 @@ int cuda_status(cudaError_t e) {
 
 enum StepKind {
   ST_GEMM,
-  ST_TRI_INV,
   ST_GATHER,
   ST_SCATTER_SUB,
   ST_COPY,
@@ -61,7 +60,7 @@ enum StepKind {
 
 struct Step {
   StepKind kind;
-  int cfg = 0;    // GEMM: kernel config; TRI_INV: 1 small blocks; SLICE: 1 maxima pass;
+  int cfg = 0;    // GEMM: kernel config; LU_PANEL: line groups of a task; SLICE: 1 maxima pass;
                   // OZGEMM: slices; SMALL_LEVEL: shared-memory bytes of a CTA
   int n = 0;      // tasks / segments
   int n2 = 0;     // GSLICE: ordinary slice tasks after the n G tiles
@@ -73,7 +72,7 @@ struct Step {
   double flops = 0;                       // useful flops of a GEMM step
   int level = -1;
   int slot = -1;      // tunable step: 0 normalisation, 1 steps 3+5, 2 step 4
-  int side = 0;       // 1: side stream (normalisation, one level ahead); 2: third stream
+  int side = 0;       // 1: side stream (normalisation, one level ahead)
   int wait = -1;      // event index waited on before the launch
   int signal = -1;    // event index recorded after the launch
   int param = 0;      // tuned parameter in use (GEMM tile config or K split)
@@ -82,8 +81,7 @@ struct Step {
 
 // events of a multi-stream plan
 enum PlanEvent {
-  EV_FORK = 0, EV_SIDE_JOIN = 1, EV_THIRD_JOIN = 2, EV_THIRD_DONE = 3, EV_MAIN_JOIN = 4,
-  EV_THIRD_DONE2 = 5, EV_LEVEL = 6
+  EV_FORK = 0, EV_SIDE_JOIN = 1, EV_MAIN_JOIN = 2, EV_LEVEL = 3
 };
 
 struct Plan {
@@ -129,7 +127,6 @@ struct pselinv_ctx {
   void* dsym = nullptr;
   SymDev S{};
   int* derr = nullptr;
-  int max_width = 1;
   // numeric state
   int dtype = 0;
   int64_t nbatch = 0;
@@ -166,7 +163,6 @@ struct pselinv_ctx {
   cudaStream_t cap_stream = nullptr;
   cudaStream_t main_stream = nullptr;   // sweep launches (highest priority)
   cudaStream_t side_stream = nullptr;   // normalisation one level ahead
-  cudaStream_t third_stream = nullptr;  // triangular inverses of the deeper levels (lowest)
   int64_t last_info = -1;
   int last_status = 0;
   // supernodes the selected-inversion plan covers (empty = all): one
@@ -499,20 +495,17 @@ size_t ozaki_norm_bytes(const HostSym& H, int64_t nb, int S, size_t es) {
 }
 
 // scratch of the selected-inversion sweep before the normalisation region:
-// W (2 s^2 for every supernode) and the largest level's G (FP64 levels) or
-// split-level operands
+// the largest level's G (FP64 levels) or split-level operands
 size_t selinv_main_bytes(const HostSym& H, int64_t nb, size_t es) {
-  int64_t w = 0, gmax = 0;
-  for (int64_t k = 0; k < H.ns; k++) w += 2 * H.sn_width[k] * H.sn_width[k];
+  int64_t gmax = 0;
   for (size_t d = 0; d + 1 < H.level_ptr.size(); d++) {
     int64_t g = 0;
-    for (int64_t i = H.level_ptr[d]; i < H.level_ptr[d + 1]; i++) {
+    for (int64_t i = H.level_ptr[d]; i < H.level_ptr[d + 1]; i++)
       g += cK(H, H.level_sn[i]) * cU(H, H.level_sn[i]);
-    }
     gmax = std::max(gmax, g);
   }
-  return align256(std::max((size_t)((w + gmax) * nb) * es + 256,
-                           (size_t)(w * nb) * es + ozaki_level_bytes(H, nb, 6, es) + 4096));
+  return align256(
+      std::max((size_t)(gmax * nb) * es + 256, ozaki_level_bytes(H, nb, 6, es) + 4096));
 }
 
 // row and column maxima of the split levels' operands, a region of their
@@ -530,8 +523,8 @@ size_t maxima_bytes(const HostSym& H, int64_t nb) {
 // split normalisation (side stream) has its own region after the sweep's,
 // the maxima theirs after that
 size_t scratch_need(const HostSym& H, int64_t nb, size_t es) {
-  // factorisation levels: W, the panels and the Schur product in FP64, then
-  // the slices of a split level's operands (counted for every level)
+  // factorisation levels: the inverse merges, the panels and the Schur product
+  // in FP64, then the slices of a split level's operands (counted for every level)
   size_t fmax = 0;
   const size_t parts = es / 8;
   for (size_t d = 0; d + 1 < H.hlevel_ptr.size(); d++) {
@@ -539,7 +532,7 @@ size_t scratch_need(const HostSym& H, int64_t nb, size_t es) {
     size_t oz = 512;
     for (int64_t i = H.hlevel_ptr[d]; i < H.hlevel_ptr[d + 1]; i++) {
       const int64_t K = H.hlevel_sn[i], s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
-      f += 2 * s * s + (c + cu) * s + c * cu;
+      f += (s * s + 1) / 2 + (c + cu) * s + c * cu;
       if (c > 0 && cu > 0)  // A_{C,K}, A_{K,C}^T, Uinv, Linv (the solves; then TL, TU)
         oz += parts * (slice_bytes(c, s, 6) + slice_bytes(cu, s, 6) + 2 * slice_bytes(s, s, 6)) +
               exps_bytes(c) + exps_bytes(cu) + 2 * exps_bytes(s) + 2048 +
@@ -600,46 +593,6 @@ void gemm_features<GemmDesc>(Step& st, const std::vector<GemmDesc>& descs, doubl
   }
   const double v[8] = {n, fl, mm, mn, mk, n ? sm / n : 0, n ? sn / n : 0, n ? sk / n : 0};
   for (int i = 0; i < 8; i++) st.feat[i] = (float)std::log2(1.0 + v[i]);
-}
-
-// Triangular-inverse launches over blocks {instance, supernode, W offset}:
-// blocks of width <= 32 one warp per triangle (cfg 1), wider ones in panels
-// of 8 columns, one warp per column (cfg 0).
-struct TriBlock {
-  int64_t b, K, w0;
-};
-void add_tri_step(Plan& P, const HostSym& H, const std::vector<TriBlock>& blocks, int level,
-                  int stream, bool allow_small = true) {
-  std::vector<SnTask> wide, small;
-  std::vector<int64_t> wofs_wide, wofs_small;
-  for (const TriBlock& t : blocks) {
-    const int64_t s = H.sn_width[t.K];
-    for (int which = 0; which < 2; which++) {
-      if (s <= 32 && allow_small) {
-        small.push_back({(int)t.b, (int)t.K, which, 0});
-        wofs_small.push_back(t.w0 + which * s * s);
-        continue;
-      }
-      for (int64_t j = 0; j < s; j += 8) {
-        wide.push_back({(int)t.b, (int)t.K, which, (int)j});
-        wofs_wide.push_back(t.w0 + which * s * s);
-      }
-    }
-  }
-  auto push = [&](const std::vector<SnTask>& tasks, const std::vector<int64_t>& wofs, int cfg) {
-    if (tasks.empty()) return;
-    Step st;
-    st.kind = ST_TRI_INV;
-    st.cfg = cfg;
-    st.n = (int)tasks.size();
-    st.tasks = P.push(tasks);
-    st.offs = P.push(wofs);
-    st.level = level;
-    st.side = stream;
-    P.steps.push_back(st);
-  };
-  push(wide, wofs_wide, 0);
-  push(small, wofs_small, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -907,9 +860,9 @@ int build_factor_plan(pselinv_ctx* h) {
 
 // ---------------------------------------------------------------------------
 // selected-inversion plan (FP64 / complex128 products):
-//   normalise (all supernodes at once): Linv, Uinv; Lhat = L Linv,
-//   Uhat^T = U^T Uinv^T, D = Uinv Linv (-> Ainv_KK);
-//   then for every depth level (roots first): gather G = Ainv_CC,
+//   normalise (level by level): Lhat = L Linv, Uhat^T = U^T Uinv^T,
+//   D = Uinv Linv (-> Ainv_KK);
+//   for every depth level (roots first): gather G = Ainv_CC,
 //   Ainv_CK = -G Lhat, (Ainv_KC)^T = -G^T Uhat^T, Ainv_KK += -Uhat Ainv_CK.
 // schedule = PER_SUPERNODE issues the three level launches per supernode.
 // ---------------------------------------------------------------------------
@@ -1227,8 +1180,7 @@ void add_ozaki_schur(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& p
 // operands (Linv and Uinv serve two products each).  Linv and Uinv hold
 // exact zeros outside their triangles, so the full products are the
 // triangular ones.  Steps go to the side stream; scratch from `base`.
-void add_ozaki_normalize(pselinv_ctx* h, Plan& P, int lev, int64_t nb,
-                         const std::vector<int64_t>& wbase, size_t base) {
+void add_ozaki_normalize(pselinv_ctx* h, Plan& P, int lev, int64_t nb, size_t base) {
   const HostSym& H = h->H;
   const size_t es = h->esize;
   OzBuilder ob(h, base);
@@ -1249,7 +1201,7 @@ void add_ozaki_normalize(pselinv_ctx* h, Plan& P, int lev, int64_t nb,
       const int s = (int)H.sn_width[K], c = (int)cK(H, K);
       const size_t so = ((size_t)b * H.storage + H.sn_offset[K]) * es;
       const size_t lo = so + (size_t)s * s * es, uo = lo + (size_t)c * s * es;
-      const char* Linv = h->scratch + (size_t)wbase[b * H.ns + K] * es;
+      const char* Linv = h->winv + (size_t)(b * h->w_stride + h->w_off[K]) * es;
       const char* Uinv = Linv + (size_t)s * s * es;
       SliceDesc lb = ob.slice(Linv, s, SLICE_COLS, s, s);  // Linv(k, n)
       SliceDesc ub = ob.slice(Uinv, s, SLICE_ROWS, s, s);  // Uinv(n, k) = Uinv(m, k)
@@ -1325,7 +1277,7 @@ void add_outmax_step(pselinv_ctx* h, Plan& P, const std::vector<int64_t>& sns, i
 // steps 3 and 5, slice Ainv(C,K), sliced product for step 4 accumulated onto
 // D_K.  Scratch layout after the W region (byte offsets).
 void add_ozaki_level(pselinv_ctx* h, Plan& P, const std::vector<int64_t>& grp, int64_t nb,
-                     int64_t gbase_scalars, int lev, size_t& max_cursor) {
+                     int lev, size_t& max_cursor) {
   const HostSym& H = h->H;
   const int S = h->slices;
   const size_t es = h->esize;
@@ -1336,7 +1288,7 @@ void add_ozaki_level(pselinv_ctx* h, Plan& P, const std::vector<int64_t>& grp, i
   std::vector<OzDesc> main, dg;
   std::vector<CopySeg> zero, mirror;
   const bool sym = h->opts.symmetric != 0;
-  OzBuilder ob(h, (size_t)gbase_scalars * es);
+  OzBuilder ob(h, 0);
   // column maxima of every panel operand of the level (the sweep's maxima
   // region, zeroed at its start); G's exponents come from the running
   // row / column maxima of Ainv instead
@@ -1431,10 +1383,6 @@ void add_ozaki_level(pselinv_ctx* h, Plan& P, const std::vector<int64_t>& grp, i
 
 // largest K split of the normalisation's products
 constexpr int kNormMaxKsplit = 8;
-// triangular-inverse tasks (8 columns each) of the levels whose inverses
-// the side stream computes itself, and of the first third-stream launch
-constexpr int64_t kTriSideTasks = 4 * 152;
-constexpr int64_t kTriThirdTasks = 8 * 152;
 
 // K split of FP64 products: a task's chain of multiply-adds (row panels: 8 per
 // k, 64 cycles each) should not outlast a quarter of the launch's work spread
@@ -1535,64 +1483,15 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
   const int dt = h->dtype;
   const int64_t nb = h->nbatch;
   const int cfg = choose_cfg(schedule);
-  // W region: Linv | Uinv per (instance, supernode)
-  std::vector<int64_t> wbase((size_t)(nb * H.ns));
-  int64_t off = 0;
-  for (int64_t b = 0; b < nb; b++)
-    for (int64_t K = 0; K < H.ns; K++) {
-      wbase[b * H.ns + K] = off;
-      off += 2 * H.sn_width[K] * H.sn_width[K];
-    }
-  const int64_t gbase = off;
   // Normalisation (Algorithm 1 step 2 and D_K) on the side stream, one
   // depth level ahead of the sweep so that it overlaps the previous level's
-  // products.  Triangular inverses first: the blocks of the levels nearest
-  // the roots (needed first, few and wide) in one launch on the side
-  // stream; the next levels' in a launch on a third stream that runs beside
-  // the first levels, and the deep levels' in a second one behind it; the
-  // first normalisation that needs either waits for it.
+  // products, from the triangular inverses that the factorisation kept.
   const int nlev = (int)H.level_ptr.size() - 1;
   // a partitioned sweep covers a subset of the supernodes
   auto in_set = [&](int64_t K) { return h->subset.empty() || h->subset[(size_t)K] != 0; };
-  int lev_a = -1, lev_b = -1;
-  {
-    auto level_tasks = [&](int l) {
-      int64_t t = 0;
-      for (int64_t i = H.level_ptr[l]; i < H.level_ptr[l + 1]; i++)
-        t += 2 * ((H.sn_width[H.level_sn[i]] + 7) / 8);
-      return t * nb;
-    };
-    int64_t tasks = 0;
-    for (int l = 0; l < nlev; l++) {
-      if (l > 0 && tasks + level_tasks(l) > kTriSideTasks) break;
-      tasks += level_tasks(l);
-      lev_a = l;
-    }
-    tasks = 0;
-    lev_b = lev_a;
-    for (int l = lev_a + 1; l < nlev; l++) {
-      if (l > lev_a + 1 && tasks + level_tasks(l) > kTriThirdTasks) break;
-      tasks += level_tasks(l);
-      lev_b = l;
-    }
-    std::vector<TriBlock> ta, tb, tc;
-    for (int64_t b = 0; b < nb; b++)
-      for (int l = 0; l < nlev; l++)
-        for (int64_t i = H.level_ptr[l]; i < H.level_ptr[l + 1]; i++) {
-          const int64_t K = H.level_sn[i];
-          if (!in_set(K)) continue;
-          (l <= lev_a ? ta : l <= lev_b ? tb : tc).push_back({b, K, wbase[b * H.ns + K]});
-        }
-    add_tri_step(P, H, ta, -1, 1, false);  // one launch: the first normalisation waits for it
-    add_tri_step(P, H, tb, -1, 2);
-    if (!tb.empty()) P.steps.back().signal = EV_THIRD_DONE;
-    add_tri_step(P, H, tc, -1, 2);
-    if (!tc.empty()) P.steps.back().signal = EV_THIRD_DONE2;
-  }
   const size_t norm_base = selinv_main_bytes(H, nb, es);
   const size_t max_base = norm_base + ozaki_norm_bytes(H, nb, 6, es);
   size_t max_cursor = max_base;
-  bool third_waited = false, third_waited2 = false;
   // split = true: Lhat, Uhat^T and D_K as sliced products
   auto add_normalize = [&](int lev, bool split) {
     std::vector<GemmDesc> norm;
@@ -1600,10 +1499,10 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
       for (int64_t i = H.level_ptr[lev]; i < H.level_ptr[lev + 1]; i++) {
         const int64_t K = H.level_sn[i];
         if (!in_set(K)) continue;
-        const int64_t s = H.sn_width[K], c = cK(H, K), cu = cU(H, K), w0 = wbase[b * H.ns + K];
+        const int64_t s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
         const size_t so = ((size_t)b * H.storage + H.sn_offset[K]) * es;
-        char* Linv = h->scratch + (size_t)w0 * es;
-        char* Uinv = Linv + (size_t)s * s * es;
+        const char* Linv = h->winv + (size_t)(b * h->w_stride + h->w_off[K]) * es;
+        const char* Uinv = Linv + (size_t)s * s * es;
         if (split) continue;  // all three as sliced products
         // D_K = Uinv Linv (upper x lower), Lhat = L Linv, Uhat^T = U^T Uinv^T (lower B)
         norm.push_back(make_desc(Uinv, Linv, h->ainv + so, s, s, s, s, s, s, 0, 0, 1.0, 0.0, 0, 1,
@@ -1637,18 +1536,9 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
       add_zero_step(P, zero, lev);
     }
     add_gemm_step(P, dt, tuned_value(h, precision, lev, 0, GEMM_ROWS), norm, lev, 0);
-    if (split) add_ozaki_normalize(h, P, lev, nb, wbase, norm_base);
+    if (split) add_ozaki_normalize(h, P, lev, nb, norm_base);
     for (size_t i = first; i < P.steps.size(); i++) P.steps[i].side = 1;
-    if (P.steps.size() > first) {
-      if (lev > lev_b && !third_waited2) {
-        P.steps[first].wait = EV_THIRD_DONE2;  // after EV_THIRD_DONE on the same stream
-        third_waited = third_waited2 = true;
-      } else if (lev > lev_a && !third_waited) {
-        P.steps[first].wait = EV_THIRD_DONE;
-        third_waited = true;
-      }
-      P.steps.back().signal = EV_LEVEL + lev;
-    }
+    if (P.steps.size() > first) P.steps.back().signal = EV_LEVEL + lev;
   };
   P.two_streams = true;
   P.ev.assign(EV_LEVEL + std::max(nlev, 0), nullptr);
@@ -1685,7 +1575,7 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
     const int slot_diag = precision == PSELINV_PREC_OZAKI_FP16 ? 5 : 2;
     for (const auto& grp : groups) {
       if (split_level) {
-        add_ozaki_level(h, P, grp, nb, gbase, (int)lev, max_cursor);
+        add_ozaki_level(h, P, grp, nb, (int)lev, max_cursor);
         continue;
       }
       if (schedule == PSELINV_SCHED_LEVEL && !H.general && add_small_level(h, P, grp, nb, (int)lev))
@@ -1694,7 +1584,7 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
       std::vector<int64_t> gofs;
       std::vector<GemmDesc> main, dg;
       std::vector<CopySeg> mirror, zsegs;
-      int64_t goff = gbase;
+      int64_t goff = 0;
       for (int64_t b = 0; b < nb; b++)
         for (int64_t K : grp) {
           const int64_t s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
@@ -1748,7 +1638,7 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
       if (gt.empty()) continue;
       Step g;
       g.kind = ST_GATHER;
-      g.bytes = (size_t)((goff - gbase) * (int64_t)es * 2);
+      g.bytes = (size_t)(goff * (int64_t)es * 2);
       g.n = (int)gt.size();
       g.tasks = P.push(gt);
       g.offs = P.push(gofs);
@@ -1833,10 +1723,6 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
       launch_gemm(h->dtype, s.cfg, (const GemmDesc*)(a + s.descs), (const GemmTask*)(a + s.tasks),
                   s.n, s.grid, st);
       break;
-    case ST_TRI_INV:
-      launch_tri_inv(h->dtype, h->S, h->lu, h->scratch, (const int64_t*)(a + s.offs),
-                     (const SnTask*)(a + s.tasks), s.n, h->max_width, s.cfg, st);
-      break;
     case ST_LU_PANEL:
       launch_lu_panel(h->dtype, h->S, h->lu, h->winv, h->piv, (const LuTask*)(a + s.tasks), s.n,
                       s.cfg, h->opts.symmetric != 0 && !h->H.general, st);
@@ -1902,10 +1788,9 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
 
 // The streams of a multi-stream sweep (created on first use): the sweep's
 // own launches at the highest priority, the normalisation one level ahead
-// below it, the triangular inverses of the deeper levels lowest, so that
-// pending CTAs of the critical path are scheduled first.
+// below it, so that pending CTAs of the critical path are scheduled first.
 struct SweepStreams {
-  cudaStream_t main, side, third;
+  cudaStream_t main, side;
 };
 int sweep_streams(pselinv_ctx* h, SweepStreams* out) {
   int least = 0, greatest = 0;
@@ -1915,9 +1800,7 @@ int sweep_streams(pselinv_ctx* h, SweepStreams* out) {
     CK(cudaStreamCreateWithPriority(&h->main_stream, cudaStreamNonBlocking, greatest));
   if (!h->side_stream)
     CK(cudaStreamCreateWithPriority(&h->side_stream, cudaStreamNonBlocking, middle));
-  if (!h->third_stream)
-    CK(cudaStreamCreateWithPriority(&h->third_stream, cudaStreamNonBlocking, least));
-  *out = {h->main_stream, h->side_stream, h->third_stream};
+  *out = {h->main_stream, h->side_stream};
   return PSELINV_OK;
 }
 
@@ -1935,19 +1818,16 @@ int run_steps(pselinv_ctx* h, Plan& P, cudaStream_t st) {
   CK(cudaEventRecord(P.ev[EV_FORK], st));
   CK(cudaStreamWaitEvent(q3.main, P.ev[EV_FORK], 0));
   CK(cudaStreamWaitEvent(q3.side, P.ev[EV_FORK], 0));
-  CK(cudaStreamWaitEvent(q3.third, P.ev[EV_FORK], 0));
   for (const Step& s : P.steps) {
-    cudaStream_t q = s.side == 1 ? q3.side : s.side == 2 ? q3.third : q3.main;
+    cudaStream_t q = s.side == 1 ? q3.side : q3.main;
     if (s.wait >= 0) CK(cudaStreamWaitEvent(q, P.ev[s.wait], 0));
     launch_step(h, P, s, q);
     if (s.signal >= 0) CK(cudaEventRecord(P.ev[s.signal], q));
   }
   CK(cudaEventRecord(P.ev[EV_MAIN_JOIN], q3.main));
   CK(cudaEventRecord(P.ev[EV_SIDE_JOIN], q3.side));
-  CK(cudaEventRecord(P.ev[EV_THIRD_JOIN], q3.third));
   CK(cudaStreamWaitEvent(st, P.ev[EV_MAIN_JOIN], 0));
   CK(cudaStreamWaitEvent(st, P.ev[EV_SIDE_JOIN], 0));
-  CK(cudaStreamWaitEvent(st, P.ev[EV_THIRD_JOIN], 0));
   CK(cudaGetLastError());
   return PSELINV_OK;
 }
@@ -2001,11 +1881,10 @@ void free_numeric(pselinv_ctx* h) {
   h->factored = h->inverted = false;
 }
 
-// Common tail of the analyses: widest supernode, the input pattern (for
-// the consumers), and the device copy of the structure.
+// Common tail of the analyses: the input pattern (for the consumers), and
+// the device copy of the structure.
 int finish_analyze(pselinv_ctx* h, int64_t n, const int64_t* colptr, const int64_t* rowind,
                    pselinv_t* out) {
-  for (int64_t k = 0; k < h->H.ns; k++) h->max_width = std::max<int>(h->max_width, (int)h->H.sn_width[k]);
   h->colptr_h.assign(colptr, colptr + n + 1);
   h->rowind_h.assign(rowind, rowind + colptr[n]);
   if (!h->opts.host_only) {
@@ -2212,7 +2091,7 @@ int pselinv_factor(pselinv_t h, int dtype, int64_t nbatch, const void* values, v
     CK(cudaMalloc(&h->staging, (size_t)nbatch * h->H.nnz * es + 256));
     CK(cudaMalloc(&h->outstage, (size_t)h->H.nnz * es + 256));
     CK(cudaMalloc(&h->rcmax, (size_t)nbatch * 2 * h->H.n * 8 + 256));
-    CK(prepare_dense_kernels(dtype, h->max_width));
+    CK(prepare_dense_kernels());
     CK(prepare_map_kernels());
     CK(prepare_ozaki_kernels());
     h->slices = h->opts.slices <= 0 ? 6 : std::min(6, std::max(4, (int)h->opts.slices));
@@ -2476,10 +2355,9 @@ int pselinv_profile(pselinv_t h, int which, void* stream, pselinv_step_stat* out
     if (rc != PSELINV_OK) return rc;
     CK(cudaStreamWaitEvent(q3.main, ev[0], 0));
     CK(cudaStreamWaitEvent(q3.side, ev[0], 0));
-    CK(cudaStreamWaitEvent(q3.third, ev[0], 0));
     for (size_t i = 0; i < ns; i++) {
       const Step& s = P.steps[i];
-      cudaStream_t q = s.side == 1 ? q3.side : s.side == 2 ? q3.third : q3.main;
+      cudaStream_t q = s.side == 1 ? q3.side : q3.main;
       if (s.wait >= 0) CK(cudaStreamWaitEvent(q, P.ev[s.wait], 0));
       CK(cudaEventRecord(ev[2 * i + 1], q));
       launch_step(h, P, s, q);
@@ -2488,10 +2366,8 @@ int pselinv_profile(pselinv_t h, int which, void* stream, pselinv_step_stat* out
     }
     CK(cudaEventRecord(P.ev[EV_MAIN_JOIN], q3.main));
     CK(cudaEventRecord(P.ev[EV_SIDE_JOIN], q3.side));
-    CK(cudaEventRecord(P.ev[EV_THIRD_JOIN], q3.third));
     CK(cudaStreamWaitEvent(st, P.ev[EV_MAIN_JOIN], 0));
     CK(cudaStreamWaitEvent(st, P.ev[EV_SIDE_JOIN], 0));
-    CK(cudaStreamWaitEvent(st, P.ev[EV_THIRD_JOIN], 0));
   } else if (which == 2) {
     for (size_t i = 0; i < ns; i++) {
       CK(cudaEventRecord(ev[2 * i + 1], st));
@@ -2517,8 +2393,8 @@ int pselinv_profile(pselinv_t h, int which, void* stream, pselinv_step_stat* out
     }
     out[i].start_ms = t0;
     const Step& s = P.steps[i];
-    static const int kinds[] = {PSELINV_STEP_GEMM,    PSELINV_STEP_TRI_INV,
-                                PSELINV_STEP_GATHER,  PSELINV_STEP_SCATTER_SUB, PSELINV_STEP_COPY,
+    static const int kinds[] = {PSELINV_STEP_GEMM,    PSELINV_STEP_GATHER,
+                                 PSELINV_STEP_SCATTER_SUB, PSELINV_STEP_COPY,
                                 PSELINV_STEP_MEMSET,  PSELINV_STEP_SCATTER_VALUES,
                                 PSELINV_STEP_SLICE,   PSELINV_STEP_OZAKI_GEMM, PSELINV_STEP_MEMSET,
                                 PSELINV_STEP_DIAG_LU, PSELINV_STEP_SMALL_LEVEL,
@@ -2530,9 +2406,7 @@ int pselinv_profile(pselinv_t h, int which, void* stream, pselinv_step_stat* out
     out[i].flops = s.flops;
     out[i].bytes = (double)s.bytes;
     out[i].ms = ms;
-    out[i].param = (s.kind == ST_GEMM || s.kind == ST_OZGEMM) ? s.param
-                   : s.kind == ST_TRI_INV                  ? s.cfg
-                                                           : -1;
+    out[i].param = (s.kind == ST_GEMM || s.kind == ST_OZGEMM) ? s.param : -1;
     out[i].side = s.side;
   }
   for (auto& e : ev) cudaEventDestroy(e);
@@ -3045,7 +2919,6 @@ void pselinv_free(pselinv_t h) {
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->main_stream) cudaStreamDestroy(h->main_stream);
     if (h->side_stream) cudaStreamDestroy(h->side_stream);
-    if (h->third_stream) cudaStreamDestroy(h->third_stream);
     cudaFree(h->dsym);
     cudaFree(h->derr);
     cudaFree(h->tslot);

@@ -330,19 +330,12 @@ void launch_lu_panel(int dtype, const SymDev& S, void* store, void* winv, void* 
                      const LuTask* tasks, int ntasks, int groups, bool sym, cudaStream_t st);
 void launch_unpack_pivots(int dtype, const SymDev& S, void* store, const void* piv, int nbatch,
                           cudaStream_t st);
-// triangular inverses of the diagonal blocks of `store`:
-// tasks {inst, K, which (0 = L unit lower, 1 = U upper), first column of a
-// panel of 8 columns}; small = 1: blocks of width <= 32, one task per
-// triangle (first column 0); result (s x s) at out + wofs[task]
-void launch_tri_inv(int dtype, const SymDev& S, const void* store, void* out,
-                    const int64_t* wofs, const SnTask* tasks, int ntasks, int max_width,
-                    int small, cudaStream_t st);
 // FP64 peak loop (the FP64 roofline's denominator): grid for `sms` SMs;
 // the launch returns its flops (out: grid * 256 doubles of device scratch)
 int fp64_peak_grid(int sms);
 double launch_fp64_peak(double* out, int grid, int iters, cudaStream_t st);
-// one-time kernel attributes (dynamic shared memory of tri_inv for max_width)
-cudaError_t prepare_dense_kernels(int dtype, int max_width);
+// one-time kernel attributes
+cudaError_t prepare_dense_kernels();
 // G_K = Ainv(R_K, R_K) gathered from `store` into out + gofs[task]
 // tasks {inst, K, tile_p, tile_q} (32 x 32 tiles).  With mofs != null
 // (real data only), the row and column maxima of |G_K| are also accumulated
