@@ -83,10 +83,12 @@ typedef struct pselinv_opts {
   int32_t host_only;     /* 1: pselinv_analyze makes no CUDA call (structure inspection only;
                             the handle then refuses pselinv_factor) */
   int32_t split_normalise; /* PREC_OZAKI_FP16 only.  0 (default): the normalisation (Lhat,
-                            Uhat^T, Algorithm 1 step 2) and D_K = U_KK^{-1} L_KK^{-1} stay in
-                            FP64 like the triangular inverses and the final Ainv_KK
-                            combination; 1: in split levels they are sliced products too
-                            (faster, one more rounding stage) */
+                            Uhat^T, Algorithm 1 step 2) has FP64 accuracy (FP64 products, or
+                            on split levels products of eight slices of 8 bits for supernodes
+                            wider than 32 columns), and D_K = U_KK^{-1} L_KK^{-1} stays in FP64
+                            like the triangular inverses and the final Ainv_KK combination; 1:
+                            in split levels all three are products of opts.slices slices (one
+                            more rounding stage) */
   int32_t symmetric;     /* 1: the values satisfy A = A^T (real symmetric or complex
                             symmetric, not Hermitian).  Then Uhat = Lhat^T and
                             Ainv(K, C) = Ainv(C, K)^T: the sweep skips the normalisation
@@ -204,7 +206,7 @@ int pselinv_analyze(int64_t n, const int64_t* colptr, const int64_t* rowind,
  * (A^{-1})_{x,y} (Eq. sel_entries: the transposed position), and
  * pselinv_trace / pselinv_weighted_sum use the same entries.  Both
  * precisions are available; with PSELINV_PREC_OZAKI_FP16 the normalisation
- * stays FP64 (opts->split_normalise is ignored) and G_K = Ainv(R_U, R_L) is
+ * keeps its FP64 accuracy (opts->split_normalise is ignored) and G_K = Ainv(R_U, R_L) is
  * gathered and sliced for steps 3 and 5 as for the other handles.
  * opts->symmetric must be 0; pselinv_group, pselinv_partition and the block
  * transfers return PSELINV_ERR_UNSUPPORTED for these handles.  Other errors

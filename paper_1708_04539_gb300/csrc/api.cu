@@ -55,7 +55,9 @@ enum StepKind {
   ST_GSLICE,
   ST_OUTMAX,
   ST_MIRROR,
-  ST_UNPACK_PIVOTS
+  ST_UNPACK_PIVOTS,
+  ST_NORM_SLICE,
+  ST_NORM_GEMM
 };
 
 struct Step {
@@ -478,14 +480,21 @@ size_t ozaki_level_bytes(const HostSym& H, int64_t nb, int S, size_t es) {
   return mx;
 }
 
+// slices of the normalisation's operands on split levels, and the narrowest
+// supernode whose normalisation is sliced (a narrower one's operands would be
+// mostly padding: K blocks of 32 and column tiles of 64)
+constexpr int kNormSlices = 8;
+constexpr int64_t kNormMinWidth = 33;
+
 // bytes of the split normalisation of the largest level
-size_t ozaki_norm_bytes(const HostSym& H, int64_t nb, int S, size_t es) {
+size_t ozaki_norm_bytes(const HostSym& H, int64_t nb, size_t es) {
+  const int S = kNormSlices;
   const size_t parts = es / 8;
   size_t mx = 0;
   for (size_t d = 0; d + 1 < H.level_ptr.size(); d++) {
     size_t b = 512;
     for (int64_t i = H.level_ptr[d]; i < H.level_ptr[d + 1]; i++) {
-      const int64_t K = H.level_sn[i], s = H.sn_width[K], c = cK(H, K);
+      const int64_t K = H.level_sn[i], s = H.sn_width[K], c = std::max(cK(H, K), cU(H, K));
       b += 2 * (parts * slice_bytes(s, s, S) + exps_bytes(s) + 512) + (size_t)(2 * c + 2 * s) * 8;
       if (c > 0) b += 2 * (parts * slice_bytes(c, s, S) + exps_bytes(c) + 512);
     }
@@ -541,7 +550,7 @@ size_t scratch_need(const HostSym& H, int64_t nb, size_t es) {
     fmax = std::max(fmax, align256((size_t)(f * nb) * es) + oz * (size_t)nb + 512);
   }
   return std::max(fmax + 256,
-                  selinv_main_bytes(H, nb, es) + ozaki_norm_bytes(H, nb, 6, es) +
+                  selinv_main_bytes(H, nb, es) + ozaki_norm_bytes(H, nb, es) +
                       maxima_bytes(H, nb));
 }
 
@@ -1040,8 +1049,9 @@ struct OzBuilder {
   pselinv_ctx* h;
   size_t off;  // next free byte of the scratch arena
   int S, cplx;
-  OzBuilder(pselinv_ctx* h_, size_t off_)
-      : h(h_), off(off_), S(h_->slices), cplx(h_->dtype == PSELINV_C128 ? 1 : 0) {}
+  OzBuilder(pselinv_ctx* h_, size_t off_, int slices = 0)
+      : h(h_), off(off_), S(slices ? slices : h_->slices),
+        cplx(h_->dtype == PSELINV_C128 ? 1 : 0) {}
   char* take(size_t bytes) {
     off = align256(off);
     const size_t o = off;
@@ -1062,6 +1072,7 @@ struct OzBuilder {
     d.R64 = (int)r64(R);
     d.K32 = (int)k32(Kd) * (cplx ? 2 : 1);
     d.cplx = cplx;
+    d.tri = 0;
     d.out = (__half*)take(slice_bytes(R, Kd, S) * (cplx ? 2 : 1));
     d.exps = (int*)take(exps_bytes(R));
     d.maxbits = nullptr;
@@ -1235,6 +1246,87 @@ void add_ozaki_normalize(pselinv_ctx* h, Plan& P, int lev, int64_t nb, size_t ba
   add_slice_step(P, sl, lev, false);
   add_ozgemm_step(P, prods, h->slices, lev, false, 1, -1);
   for (size_t i = first; i < P.steps.size(); i++) P.steps[i].side = 1;
+}
+
+// The normalisation of the supernodes {instance, K} of a split level as
+// eight-slice products (K = s; FP64 accuracy, see norm_gemm_kernel): the
+// panels and the triangular inverses sliced in one launch, then Lhat = L Linv
+// and Uhat^T = U^T Uinv^T in another.  Scratch from `base`.
+void add_sliced_normalize(pselinv_ctx* h, Plan& P, const std::vector<std::pair<int64_t, int64_t>>& sns,
+                          int lev, size_t base) {
+  if (sns.empty()) return;
+  const HostSym& H = h->H;
+  const size_t es = h->esize;
+  OzBuilder ob(h, base, kNormSlices);
+  std::vector<SliceDesc> sl;
+  std::vector<OzDesc> prods;
+  for (const auto& bk : sns) {
+    const int64_t b = bk.first, K = bk.second;
+    const int s = (int)H.sn_width[K], c = (int)cK(H, K), cu = (int)cU(H, K);
+    const size_t so = ((size_t)b * H.storage + H.sn_offset[K]) * es;
+    const size_t lo = so + (size_t)s * s * es, uo = lo + (size_t)c * s * es;
+    const char* Linv = h->winv + (size_t)(b * h->w_stride + h->w_off[K]) * es;
+    const char* Uinv = Linv + (size_t)s * s * es;
+    if (c > 0) {
+      SliceDesc lb = ob.slice(Linv, s, SLICE_COLS, s, s);  // Linv(k, n)
+      lb.tri = 1;
+      const SliceDesc la = ob.slice(h->lu + lo, c, SLICE_ROWS, c, s);
+      sl.push_back(lb);
+      sl.push_back(la);
+      ob.product(prods, la, lb, h->nf + lo, c, c, s, 1.0);
+    }
+    if (cu > 0 && !h->opts.symmetric) {  // symmetric A: Uhat = Lhat^T, not needed
+      SliceDesc ub = ob.slice(Uinv, s, SLICE_ROWS, s, s);  // Uinv(n, k)
+      ub.tri = 1;
+      const SliceDesc ua = ob.slice(h->lu + uo, cu, SLICE_ROWS, cu, s);
+      sl.push_back(ub);
+      sl.push_back(ua);
+      ob.product(prods, ua, ub, h->nf + uo, cu, cu, s, 1.0);
+    }
+  }
+  if (prods.empty()) return;
+  // few row blocks: their K range is spread over CTAs too
+  int64_t blocks = 0;
+  for (const SliceDesc& d : sl) blocks += d.R64;
+  const int span = blocks >= 4 * 152 ? 16 : 2;
+  std::vector<SliceTask> st;
+  double bytes = 0;
+  for (size_t d = 0; d < sl.size(); d++) {
+    for (int rb = 0; rb < sl[d].R64; rb++)
+      for (int kc = 0; kc < sl[d].K32; kc += span) st.push_back({(int)d, rb, kc});
+    bytes += (double)es * sl[d].R * sl[d].Kd + 2.0 * kNormSlices * 64.0 * sl[d].R64 * 32 * sl[d].K32;
+  }
+  Step a;
+  a.kind = ST_NORM_SLICE;
+  a.cfg = span;
+  a.n = (int)st.size();
+  a.descs = P.push(sl);
+  a.tasks = P.push(st);
+  a.bytes = (size_t)bytes;
+  a.level = lev;
+  P.steps.push_back(a);
+  std::vector<OzTask> tasks;
+  double flops = 0;
+  bytes = 0;
+  for (size_t d = 0; d < prods.size(); d++) {
+    const OzDesc& g = prods[d];
+    for (int tm = 0; tm < ceil_div(g.M, 128); tm++)  // longest K range first
+      for (int tn = 0; tn < ceil_div(g.N, 64); tn++) tasks.push_back({(int)d, tm, tn, 0});
+    flops += (double)g.M * g.N * (g.N + 1) * g.cscale;
+    bytes += 2.0 * kNormSlices * ((double)g.M + g.N / 2.0) * g.K32 * 32 + 8.0 * g.M * g.N;
+  }
+  std::stable_sort(tasks.begin(), tasks.end(), [&](const OzTask& x, const OzTask& y) {
+    return prods[x.d].K32 - 2 * x.tn > prods[y.d].K32 - 2 * y.tn;
+  });
+  Step m;
+  m.kind = ST_NORM_GEMM;
+  m.n = (int)tasks.size();
+  m.descs = P.push(prods);
+  m.tasks = P.push(tasks);
+  m.flops = flops;
+  m.bytes = (size_t)bytes;
+  m.level = lev;
+  P.steps.push_back(m);
 }
 
 // Merge the finished blocks of the supernodes `sns` (diagonal block, L and
@@ -1490,11 +1582,13 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
   // a partitioned sweep covers a subset of the supernodes
   auto in_set = [&](int64_t K) { return h->subset.empty() || h->subset[(size_t)K] != 0; };
   const size_t norm_base = selinv_main_bytes(H, nb, es);
-  const size_t max_base = norm_base + ozaki_norm_bytes(H, nb, 6, es);
+  const size_t max_base = norm_base + ozaki_norm_bytes(H, nb, es);
   size_t max_cursor = max_base;
-  // split = true: Lhat, Uhat^T and D_K as sliced products
-  auto add_normalize = [&](int lev, bool split) {
+  // sliced: Lhat and Uhat^T of wide supernodes as eight-slice products; split:
+  // Lhat, Uhat^T and D_K all as sliced products (opts.split_normalise)
+  auto add_normalize = [&](int lev, bool sliced, bool split) {
     std::vector<GemmDesc> norm;
+    std::vector<std::pair<int64_t, int64_t>> wide;  // {instance, supernode}
     for (int64_t b = 0; b < nb; b++)
       for (int64_t i = H.level_ptr[lev]; i < H.level_ptr[lev + 1]; i++) {
         const int64_t K = H.level_sn[i];
@@ -1508,6 +1602,10 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
         norm.push_back(make_desc(Uinv, Linv, h->ainv + so, s, s, s, s, s, s, 0, 0, 1.0, 0.0, 0, 1,
                                  GEMM_TRI_UPPER_A | GEMM_TRI_LOWER_B));
         const size_t lo = so + (size_t)s * s * es, uo = lo + (size_t)c * s * es;
+        if (sliced && s >= kNormMinWidth) {
+          wide.push_back({b, K});
+          continue;
+        }
         if (c > 0)
           norm.push_back(make_desc(h->lu + lo, Linv, h->nf + lo, c, s, s, c, s, c, 0, 0, 1.0, 0.0,
                                    0, 1, GEMM_TRI_LOWER_B));
@@ -1516,6 +1614,7 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
                                    0.0, 0, 1, GEMM_TRI_LOWER_B));
       }
     const size_t first = P.steps.size();
+    add_sliced_normalize(h, P, wide, lev, norm_base);
     // levels of few wide supernodes (near the roots): split K so that the
     // launch has tasks for every SM, its K loops being the level's latency;
     // the outputs are then zeroed and accumulated
@@ -1557,7 +1656,8 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
   }
   for (size_t lev = 0; lev + 1 < H.level_ptr.size(); lev++) {
     const bool split_level = split_lv[lev] != 0;
-    add_normalize((int)lev, split_level && h->opts.split_normalise != 0 && !H.general);
+    const bool split_norm = split_level && h->opts.split_normalise != 0 && !H.general;
+    add_normalize((int)lev, split_level && !split_norm, split_norm);
     const size_t first_main = P.steps.size();
     // groups: the whole level, or one supernode at a time
     std::vector<std::vector<int64_t>> groups;
@@ -1726,6 +1826,13 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
     case ST_LU_PANEL:
       launch_lu_panel(h->dtype, h->S, h->lu, h->winv, h->piv, (const LuTask*)(a + s.tasks), s.n,
                       s.cfg, h->opts.symmetric != 0 && !h->H.general, st);
+      break;
+    case ST_NORM_SLICE:
+      launch_norm_slice((const SliceDesc*)(a + s.descs), (const SliceTask*)(a + s.tasks), s.n, s.cfg,
+                        st);
+      break;
+    case ST_NORM_GEMM:
+      launch_norm_gemm((const OzDesc*)(a + s.descs), (const OzTask*)(a + s.tasks), s.n, h->derr, st);
       break;
     case ST_UNPACK_PIVOTS:
       launch_unpack_pivots(h->dtype, h->S, h->lu, h->piv, (int)h->nbatch, st);
@@ -2399,7 +2506,8 @@ int pselinv_profile(pselinv_t h, int which, void* stream, pselinv_step_stat* out
                                 PSELINV_STEP_SLICE,   PSELINV_STEP_OZAKI_GEMM, PSELINV_STEP_MEMSET,
                                 PSELINV_STEP_DIAG_LU, PSELINV_STEP_SMALL_LEVEL,
                                 PSELINV_STEP_GATHER_SLICE, PSELINV_STEP_OUTPUT_MAXIMA,
-                                PSELINV_STEP_COPY, PSELINV_STEP_COPY};
+                                PSELINV_STEP_COPY, PSELINV_STEP_COPY,
+                                PSELINV_STEP_SLICE, PSELINV_STEP_OZAKI_GEMM};
     out[i].kind = kinds[s.kind];
     out[i].level = s.level;
     out[i].tasks = s.n;

@@ -213,6 +213,7 @@ enum SliceMode { SLICE_ROWS = 0, SLICE_COLS = 1 };
 struct SliceDesc {
   const double* src;
   int ld, mode, R, Kd, S, R64, K32, cplx;
+  int tri;  // X(r, k) = 0 for k < r (the normalisation's triangular operands)
   __half* out;
   int* exps;
   unsigned long long* maxbits;  // max_k |X(r,k)| as bit patterns (from the gather or a maxima pass)
@@ -279,6 +280,13 @@ void launch_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, bo
 // half) instead of shared memory
 void launch_ozaki_gemm(int S, const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
                        bool persistent, bool a_tmem, cudaStream_t st);
+// The normalisation's products at eight slices (K <= 256; op(B) lower
+// triangular): slices with their own row maxima, `span` K blocks per task
+// {d, row block, first K block}; products C = A op(B), tasks {d, tm, tn, 0}
+void launch_norm_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, int span,
+                       cudaStream_t st);
+void launch_norm_gemm(const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
+                      cudaStream_t st);
 void launch_zero(const CopySeg* segs, int nseg, int per_seg, cudaStream_t st);
 // a kernel whose only wait never completes: it gives up after budget_ns and
 // records DEV_TIMEOUT in err[0]

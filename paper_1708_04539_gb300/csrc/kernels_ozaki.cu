@@ -196,6 +196,94 @@ __device__ __forceinline__ void write_digits(const double (&x)[8], int e, int S,
     write_digits_s<4>(x, e, dst, slice_stride);
 }
 
+// The eight balanced base-256 digits of the normalisation's operands, Q =
+// rint(x 2^{63 - e}), |Q| <= 2^63, from four exact floats of two digits each
+// (|a_s| <= 128).
+__device__ __forceinline__ void write_digits8(const double (&x)[8], int e, __half* dst,
+                                              int64_t slice_stride) {
+  float p[4][8];
+#pragma unroll
+  for (int j = 0; j < 8; j++) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x[j]);
+    const int E = (int)((b >> 52) & 0x7FF);
+    const int r = 1012 + e - E;  // |x| 2^{63 - e} = M 2^{-r}, r >= -10
+    unsigned long long q = 0;
+    if (E != 0 && r < 54) {
+      const unsigned long long M = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+      q = r <= 0 ? M << -r : (M + (1ull << (r - 1))) >> r;
+    }
+    const float sg = (long long)b < 0 ? -1.0f : 1.0f;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const uint32_t k = (uint32_t)(q >> (16 * i)) & 0xFFFFu;
+      p[i][j] = __fmaf_rn(__uint_as_float(0x4B000000u | k), sg, -8388608.0f * sg);
+    }
+  }
+#pragma unroll
+  for (int s = 7; s >= 0; s--) {  // slices 6-7 from p[0], 4-5 from p[1], ...
+    const int i = (7 - s) / 2;
+    float a[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+      a[j] = p[i][j];
+      if (s > 0) {  // one digit: v = 256 t + a, t = rint(v / 256), exact
+        constexpr float kRound = 12582912.0f;
+        const float t = __fsub_rn(__fmaf_rn(a[j], 0.00390625f, kRound), kRound);
+        a[j] = __fmaf_rn(-256.0f, t, a[j]);
+        p[i][j] = t;
+      }
+      if (s > 0 && s % 2 == 0) p[i + 1][j] += p[i][j];  // carry (exact)
+    }
+    uint4 w;
+    __half2 h0 = __floats2half2_rn(a[0], a[1]), h1 = __floats2half2_rn(a[2], a[3]);
+    __half2 h2 = __floats2half2_rn(a[4], a[5]), h3 = __floats2half2_rn(a[6], a[7]);
+    w.x = *reinterpret_cast<uint32_t*>(&h0);
+    w.y = *reinterpret_cast<uint32_t*>(&h1);
+    w.z = *reinterpret_cast<uint32_t*>(&h2);
+    w.w = *reinterpret_cast<uint32_t*>(&h3);
+    *reinterpret_cast<uint4*>(dst + s * slice_stride) = w;
+  }
+}
+
+// Eight-digit slices of operands with K <= 256 (the normalisation): a task is
+// a 64-row block and `span` K blocks from kc; every task finds its rows'
+// maxima itself over the whole K (a row is read by four lanes of one warp, and
+// comes from L1 / L2 the second time), so no maxima pass, no zeroed buffer and
+// one launch instead of three.  d.tri: X(r, k) = 0 for k < r, and nobody reads
+// the K blocks left of the row block's diagonal.
+__global__ void __launch_bounds__(kSliceThreads)
+norm_slice_kernel(const SliceDesc* __restrict__ descs, const SliceTask* __restrict__ tasks,
+                  int ntasks, int span) {
+  const int tid = threadIdx.x, ci = tid >> 3, rr = tid & 7;
+  const int rl = (ci >> 2) * 8 + rr, kg = ci & 3;
+  for (int t = blockIdx.x; t < ntasks; t += gridDim.x) {
+    const SliceTask task = tasks[t];
+    const SliceDesc& d = descs[task.d];
+    const int r = task.rb * 64 + rl;
+    unsigned long long m = 0;
+    for (int kb = 0; kb < d.K32; kb++) {
+      double x[8];
+      load8(d, r, kb * 32 + kg * 8, x);
+#pragma unroll
+      for (int j = 0; j < 8; j++) m = max(m, abs_bits(x[j]));
+    }
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 8));
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    const int e = r < d.R ? exp_of_max(m) : 0;
+    if (task.kc == 0 && kg == 0 && r < d.R) d.exps[r] = e;
+    const int64_t slice_stride = (int64_t)d.R64 * d.K32 * (kTileBytes / 2);
+    const int half = d.cplx ? d.K32 / 2 : d.K32;
+    const int kb1 = min(d.K32, task.kc + span);
+    for (int kb = task.kc; kb < kb1; kb++) {
+      if (d.tri && (kb >= half ? kb - half : kb) < 2 * task.rb) continue;
+      double x[8];
+      load8(d, r, kb * 32 + kg * 8, x);
+      write_digits8(x, e, d.out + ((int64_t)task.rb * d.K32 + kb) * (kTileBytes / 2) + tid * 8,
+                    slice_stride);
+    }
+  }
+}
+
 // Slices of one task (see the work item above); exponents from d.maxbits.
 __device__ __forceinline__ void slice_task(const SliceDesc& d, const SliceTask& task, int tid) {
   const int ci = tid >> 3, rr = tid & 7;
@@ -959,6 +1047,250 @@ constexpr int gemm_smem() {
   return oz_stages<S, ATMEM>() * S * 3 * kTileBytes + (ATMEM ? kOzDrainWarps * 32 * 32 * 8 : 0);
 }
 
+// ---------------------------------------------------------------------------
+// The normalisation Lhat = L L_KK^{-1}, Uhat^T = U^T U_KK^{-T} as products of
+// eight base-256 slices: 63 bits below each row's and column's power of two
+// and the 36 slice pairs with s + t <= 7, so an output is off by some 2^-60 of
+// its row's and column's largest products.  Against correctly rounded exact
+// products of panels of 3D, 2D and DG matrices (s = 128) the relative error in
+// norm is 2e-18 to 2e-17; an FP64 sum's is 1.5e-16 to 2.8e-16.  (Base 128, 56
+// bits: up to 6e-16, from columns of Lhat far below their rows' largest
+// entries.)
+// K = s <= 256 (real and imaginary parts: 2 x 256).  A chunk of 4 K blocks adds
+// at most 128 x 8 x 2^14 = 2^24 to an accumulator, exact; its 8 x 64
+// accumulators take all of tensor memory, and its sum goes straight to the
+// output, rounded once; later chunks are added in FP64.  op(B)(k, n) = 0 for k
+// < n: K blocks left of a column tile's diagonal are skipped.
+// Roles and ring as in ozaki_gemm_kernel (two stages of 96 KB).  The FP64
+// pipe needs c s^2 multiply-adds at 2 per cycle and SM for what is here 20
+// MMAs per 128 x 64 x 16.
+// ---------------------------------------------------------------------------
+constexpr int kNormS = 8;
+constexpr int kNormChunk = 4;  // K blocks per exact chunk
+constexpr int kNormStage = kNormS * 3 * kTileBytes;
+constexpr int kNormStages = 2;
+
+// K blocks of a task: sequence position i -> K block
+struct NormRange {
+  int k0, n1, n;  // first block of a part, blocks per part, blocks in all
+  __device__ __forceinline__ NormRange(const OzDesc* d, int tn) {
+    const int part = d->half ? d->half : d->K32;
+    k0 = 2 * tn;
+    n1 = part - k0;
+    n = d->half ? 2 * n1 : n1;
+  }
+  __device__ __forceinline__ int block(int i, int half) const {
+    return i < n1 ? k0 + i : half + k0 + i - n1;
+  }
+};
+
+__global__ void __launch_bounds__(kOzThreads, 1)
+norm_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ tasks, int ntasks,
+                 int* err) {
+  constexpr int S = kNormS;
+  constexpr int kAB = S * 2 * kTileBytes;
+  constexpr uint32_t kTmemCols = 512;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t bar_full[kNormStages], bar_free[kNormStages], bar_acc_full,
+      bar_acc_empty;
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int abort_flag;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int i = 0; i < kNormStages; i++) {
+      mbar_init(smem_u32(&bar_full[i]), 1);
+      mbar_init(smem_u32(&bar_free[i]), 1);
+    }
+    mbar_init(smem_u32(&bar_acc_full), 1);
+    mbar_init(smem_u32(&bar_acc_empty), kOzDrainWarps);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_slot)),
+                 "r"(kTmemCols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = tmem_slot;
+  bool ok = true;
+
+  if (warp == kOzDrainWarps) {
+    // ---- producer ----
+    if (lane == 0) {
+      uint32_t g = 0;
+      for (int t = blockIdx.x; t < ntasks && ok; t += gridDim.x) {
+        const OzTask task = tasks[t];
+        const OzDesc* dp = descs + task.d;
+        const int K32 = dp->K32, half = dp->half, swap_b = dp->swap_b;
+        const NormRange kr(dp, task.tn);
+        const bool a_second = 2 * task.tm + 1 < dp->A_R64;
+        const uint32_t bytes = (uint32_t)(S * (a_second ? 3 : 2) * kTileBytes);
+        const int64_t a_sl = (int64_t)dp->A_R64 * K32 * kTileBytes;
+        const int64_t b_sl = (int64_t)dp->B_R64 * K32 * kTileBytes;
+        const unsigned char* A = reinterpret_cast<const unsigned char*>(dp->A);
+        const unsigned char* B = reinterpret_cast<const unsigned char*>(dp->B);
+        for (int i = 0; i < kr.n; i++, g++) {
+          const int stg = (int)(g % kNormStages);
+          const uint32_t u = g / kNormStages;
+          if ((u > 0 && !mbar_wait(smem_u32(&bar_free[stg]), (u - 1) & 1)) || abort_flag) {
+            ok = false;
+            break;
+          }
+          unsigned char* st = smem + stg * kNormStage;
+          const uint32_t fb = smem_u32(&bar_full[stg]);
+          mbar_expect_tx(fb, bytes);
+          const int kb = kr.block(i, half);
+          const int kbb = swap_b ? (kb < half ? kb + half : kb - half) : kb;
+          for (int sl = 0; sl < S; sl++) {
+            const unsigned char* a0 = A + sl * a_sl + ((int64_t)(2 * task.tm) * K32 + kb) * kTileBytes;
+            bulk_load(smem_u32(st + sl * 2 * kTileBytes), a0, kTileBytes, fb);
+            if (a_second)
+              bulk_load(smem_u32(st + sl * 2 * kTileBytes + kTileBytes), a0 + (int64_t)K32 * kTileBytes,
+                        kTileBytes, fb);
+            bulk_load(smem_u32(st + kAB + sl * kTileBytes),
+                      B + sl * b_sl + ((int64_t)task.tn * K32 + kbb) * kTileBytes, kTileBytes, fb);
+          }
+        }
+      }
+      if (!ok) {
+        abort_flag = 1;
+        // let the copies already issued land before the CTA exits (bounded)
+        for (uint32_t k = g > (uint32_t)kNormStages ? g - kNormStages : 0u; k < g; k++)
+          mbar_wait(smem_u32(&bar_full[k % kNormStages]), (k / kNormStages) & 1);
+      }
+    }
+  } else if (warp == kOzDrainWarps + 1) {
+    // ---- MMA issue ----
+    if (lane == 0) {
+      uint32_t g = 0, q = 0;
+      for (int t = blockIdx.x; t < ntasks && ok; t += gridDim.x) {
+        const OzTask task = tasks[t];
+        const OzDesc* dp = descs + task.d;
+        const int half = dp->half, neg_half = dp->neg_half;
+        const NormRange kr(dp, task.tn);
+        for (int i = 0; i < kr.n; i++, g++) {
+          const int stg = (int)(g % kNormStages);
+          const bool first = i % kNormChunk == 0;
+          const bool last = i % kNormChunk == kNormChunk - 1 || i == kr.n - 1;
+          if (first && q > 0 && !mbar_wait(smem_u32(&bar_acc_empty), (q - 1) & 1)) {
+            ok = false;
+            break;
+          }
+          if (!mbar_wait(smem_u32(&bar_full[stg]), (g / kNormStages) & 1) || abort_flag) {
+            ok = false;
+            break;
+          }
+          fence_after();
+          const uint32_t st = smem_u32(smem + stg * kNormStage);
+          const bool neg_a = neg_half && kr.block(i, half) >= half;
+          const uint32_t idesc = neg_a ? kIdescNegA : kIdesc;
+          const uint32_t idesc2 = neg_a ? kIdescN128NegA : kIdescN128;
+          const uint64_t a0 = smem_desc(st), b0 = smem_desc(st + kAB);
+#pragma unroll
+          for (int sa = 0; sa < S; sa++)
+#pragma unroll
+            for (int tb = 0; tb < S - sa; tb += 2) {
+              const uint32_t dt = tmem + (uint32_t)((sa + tb) * 64);
+              const uint64_t ad = a0 + (uint64_t)((sa * 2 * kTileBytes) >> 4);
+              const uint64_t bd = b0 + (uint64_t)((tb * kTileBytes) >> 4);
+              const uint32_t id = tb + 1 < S - sa ? idesc2 : idesc;
+              mma_f16(dt, ad, bd, (sa == 0 && first) ? 0u : 1u, id);
+              mma_f16(dt, ad + (256 >> 4), bd + (256 >> 4), 1u, id);
+            }
+          mma_commit(smem_u32(&bar_free[stg]));
+          if (last) {
+            mma_commit(smem_u32(&bar_acc_full));
+            q++;
+          }
+        }
+      }
+      if (!ok) {
+        abort_flag = 1;
+        if (g > 0)
+          mbar_wait(smem_u32(&bar_free[(g - 1) % kNormStages]), ((g - 1) / kNormStages) & 1);
+      }
+    }
+  } else {
+    // ---- drain and epilogue (warps 0-7) ----
+    const int quarter = warp & 3, hcol = warp >> 2;
+    const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(hcol * 32);
+    uint32_t q = 0;
+    for (int t = blockIdx.x; t < ntasks && ok; t += gridDim.x) {
+      const OzTask task = tasks[t];
+      const OzDesc* dp = descs + task.d;
+      const NormRange kr(dp, task.tn);
+      const int dM = dp->M, dN = dp->N, ldc = dp->ldc, cscale = dp->cscale, coff = dp->coff;
+      const int* __restrict__ eB = dp->eB;
+      double* __restrict__ Cp = dp->C;
+      const int nchunks = (kr.n + kNormChunk - 1) / kNormChunk;
+      const int r = task.tm * 128 + quarter * 32 + lane;
+      const int nb = task.tn * 64 + hcol * 32;
+      const int ea = r < dM ? dp->eA[r] : 0;
+      for (int c = 0; c < nchunks; c++, q++) {
+        if (!mbar_wait(smem_u32(&bar_acc_full), q & 1) || abort_flag) {
+          ok = false;
+          break;
+        }
+        fence_after();
+#pragma unroll 1
+        for (int g2 = 0; g2 < 2; g2++) {
+          // sum_d P_d 256^{7-d} = hi 2^32 + lo, |hi| < 2^46, |lo| < 2^49
+          long long hi[16], lo[16];
+#pragma unroll
+          for (int j = 0; j < 16; j++) hi[j] = lo[j] = 0;
+#pragma unroll
+          for (int dd = 0; dd < S; dd++) {
+            uint32_t v[16];
+            tmem_ld16(trow + (uint32_t)(dd * 64 + g2 * 16), v);
+            const int shift = 8 * (dd < 4 ? 3 - dd : 7 - dd);
+#pragma unroll
+            for (int j = 0; j < 16; j++) {
+              const long long p = (long long)__float2int_rn(__uint_as_float(v[j])) << shift;
+              if (dd < 4) hi[j] += p; else lo[j] += p;
+            }
+          }
+          if (g2 == 1) {  // every accumulator read: the next chunk's MMAs may start
+            fence_before();
+            __syncwarp();
+            if (lane == 0)
+              asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_acc_empty))
+                           : "memory");
+          }
+          if (r < dM) {
+#pragma unroll
+            for (int j = 0; j < 16; j++) {
+              const int n = nb + g2 * 16 + j;
+              if (n < dN) {
+                const int eb = eB[n];
+                // the sum's top 63 bits, the rest as a sticky bit
+                const long long top = hi[j] + (lo[j] >> 32);
+                const uint32_t rem = (uint32_t)lo[j];
+                const long long u = (top << 16) | (long long)(rem >> 16) | ((rem & 0xFFFFu) != 0);
+                double v = scaled_int_to_double(u, ea + eb - 70 + 16, false);
+                // exponent 1025: an infinity or a NaN in the row
+                if (ea > 1024 || eb > 1024) v = __longlong_as_double(0x7FF8000000000000ll);
+                double* cp = Cp + (r + (int64_t)n * ldc) * cscale + coff;
+                *cp = c == 0 ? v : *cp + v;
+              }
+            }
+          }
+          __syncwarp();  // converged again for the next tensor-memory load
+        }
+      }
+    }
+    if (!ok) abort_flag = 1;
+  }
+  if (!ok && lane == 0) atomicExch(err, DEV_TIMEOUT);
+  fence_before();
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
+}
+
 // Failure-path check: wait on an mbarrier that nothing will complete, with a
 // short budget, and record the timeout like any other bounded wait.
 __global__ void wait_selftest_kernel(int* err, unsigned long long budget_ns) {
@@ -1002,7 +1334,23 @@ cudaError_t prepare_ozaki_kernels() {
   PSELINV_OZ_ATTR(5, true)
   PSELINV_OZ_ATTR(6, true)
 #undef PSELINV_OZ_ATTR
-  return cudaSuccess;
+  return cudaFuncSetAttribute(norm_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              kNormStages * kNormStage);
+}
+
+void launch_norm_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, int span,
+                       cudaStream_t st) {
+  if (ntasks <= 0) return;
+  const int grid = ntasks < 152 * 16 ? ntasks : 152 * 16;
+  norm_slice_kernel<<<grid, kSliceThreads, 0, st>>>(descs, tasks, ntasks, span);
+}
+
+void launch_norm_gemm(const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
+                      cudaStream_t st) {
+  if (ntasks <= 0) return;
+  // one task per CTA (one CTA fits an SM): the launch runs beside the sweep's
+  // own, whose CTAs take the SMs that finish
+  norm_gemm_kernel<<<ntasks, kOzThreads, kNormStages * kNormStage, st>>>(descs, tasks, ntasks, err);
 }
 
 void launch_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, bool maxima,
