@@ -56,7 +56,7 @@ enum StepKind {
   ST_OUTMAX,
   ST_MIRROR,
   ST_UNPACK_PIVOTS,
-  ST_NORM_SLICE,
+  ST_PANEL_SLICE,
   ST_NORM_GEMM
 };
 
@@ -65,7 +65,7 @@ struct Step {
   int cfg = 0;    // GEMM: kernel config; LU_PANEL: line groups of a task; SLICE: 1 maxima pass;
                   // OZGEMM: slices; SMALL_LEVEL: shared-memory bytes of a CTA
   int n = 0;      // tasks / segments
-  int n2 = 0;     // GSLICE: ordinary slice tasks after the n G tiles
+  int n2 = 0;     // GSLICE: ordinary slice tasks after the n G tiles; LU_PANEL: 1 panel solves
   int grid = 0;
   size_t tasks = 0, descs = 0, offs = 0, offs2 = 0;  // byte offsets into the plan arena
   void* ptr = nullptr;                    // memset target / store
@@ -642,11 +642,13 @@ int choose_small_tile(int dtype, const std::vector<GemmDesc>& descs) {
 }
 
 // One launch of panel tasks (32 lines each).  More than two per SM: tasks of
-// 32 kLuGroups lines, so that the pivot block is factored less often.
-void add_panel_step(Plan& P, const std::vector<LuTask>& tasks, int level) {
+// 32 kLuGroups lines, so that the pivot block is factored less often (from one
+// per SM on: 40^3 upwind factorisation 12.45 against 12.1 ms).
+void add_panel_step(Plan& P, const std::vector<LuTask>& tasks, int level, bool solve) {
   if (tasks.empty()) return;
   Step d;
   d.kind = ST_LU_PANEL;
+  d.n2 = solve ? 1 : 0;  // narrow supernodes: their panels' rows are among the lines
   d.cfg = tasks.size() > 2 * 152 ? kLuGroups : 1;
   d.level = level;
   if (d.cfg == 1) {
@@ -727,6 +729,7 @@ int build_factor_plan(pselinv_ctx* h) {
   const bool ldlt = h->opts.symmetric != 0 && !H.general;
   for (size_t lev = 0; lev + 1 < H.hlevel_ptr.size(); lev++) {
     std::vector<SnTask> wide, gt;  // wide: more than one panel
+    std::vector<SnTask> mirrored;  // symmetric values: blocks whose upper triangle is filled in
     std::vector<LuTask> panels;    // first panels of every supernode, 32 lines per task
     std::vector<int64_t> gofs;
     std::vector<GemmDesc> trsm, schur;
@@ -757,9 +760,10 @@ int build_factor_plan(pselinv_ctx* h) {
         // cu: rows of the U^T panel (c, or R_U(K))
         const int64_t K = H.hlevel_sn[i], s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
         smax = std::max(smax, s);
-        const bool narrow = s <= kLuPanel;
-        const int64_t lines =
-            (narrow ? c + (ldlt ? 0 : cu) : 2 * (s - kLuPanel)) + 2 * std::min<int64_t>(s, kLuPanel);
+        const bool oz = split && c > 0 && cu > 0;  // panel solves as sliced products
+        const bool narrow = s <= kLuPanel && !split;  // panel solves in the panel launch
+        const int64_t w = std::min<int64_t>(s, kLuPanel);
+        const int64_t lines = (narrow ? c + (ldlt ? 0 : cu) : 2 * (s - w)) + 2 * w;
         for (int64_t l = 0; l < lines; l += 32) panels.push_back({(int)b, (int)K, 0, (int)l});
         char* base = h->lu + ((size_t)b * H.storage + H.sn_offset[K]) * es;
         char* Lp = base + (size_t)s * s * es;
@@ -769,11 +773,15 @@ int build_factor_plan(pselinv_ctx* h) {
         // TL, TU: the solved panels, in place (narrow: by the panel step; split:
         // the sliced products read copies), else in scratch and copied back
         char *TL = Lp, *TU = Up;
-        if (!narrow) {
+        if (s > kLuPanel) {
           wide.push_back({(int)b, (int)K, 0, 0});
           mofs.push_back(off);
           off += s * s / 2;
-          if (!(split && c > 0 && cu > 0) && (c > 0 || cu > 0)) {
+        } else if (ldlt && split) {
+          mirrored.push_back({(int)b, (int)K, 0, 0});
+        }
+        if (!narrow) {
+          if (!oz && (c > 0 || cu > 0)) {
             TL = h->scratch + (size_t)off * es;
             TU = TL + (size_t)c * s * es;
             off += (c + cu) * s;
@@ -792,7 +800,7 @@ int build_factor_plan(pselinv_ctx* h) {
         char* Sc = h->scratch + (size_t)s0 * es;
         const SchurProduct q{TL, TU, Sc, (int)c, (int)cu, (int)s, Lp, ldlt ? Lp : Up, Uinv, Linv};
         if (c > 0 && cu > 0) {
-          if (!narrow && split) solves.push_back(q);
+          if (oz) solves.push_back(q);
           schur.push_back(make_desc(TL, TU, Sc, c, cu, s, c, cu, c, 0, 1, 1.0, 0.0));
           sprods.push_back(q);
           for (int tq = 0; tq < ceil_div(cu, 32); tq++)
@@ -803,11 +811,12 @@ int build_factor_plan(pselinv_ctx* h) {
         }
       }
     h->scratch_high = std::max(h->scratch_high, (size_t)off * es);
-    if (ldlt && !wide.empty()) {
+    if (ldlt) mirrored.insert(mirrored.end(), wide.begin(), wide.end());
+    if (!mirrored.empty()) {
       Step mr;
       mr.kind = ST_MIRROR;
-      mr.n = (int)wide.size();
-      mr.tasks = P.push(wide);
+      mr.n = (int)mirrored.size();
+      mr.tasks = P.push(mirrored);
       mr.level = (int)lev;
       P.steps.push_back(mr);
     }
@@ -831,7 +840,7 @@ int build_factor_plan(pselinv_ctx* h) {
                                   (int)w, (int)s, (int)s, (int)s, 0, 0, -1.0, 1.0));
         }
       }
-      add_panel_step(P, panels, (int)lev);
+      add_panel_step(P, panels, (int)lev, !split);
       add_gemm_step(P, dt, choose_small_tile(dt, upd), upd, (int)lev);
     }
     add_inverse_merges(h, P, wide, mofs, (int)lev);
@@ -920,6 +929,33 @@ void add_slice_step(Plan& P, const std::vector<SliceDesc>& descs, int level, boo
   Step st;
   st.cfg = maxima ? 1 : 0;
   st.kind = ST_SLICE;
+  st.n = (int)tasks.size();
+  st.descs = P.push(descs);
+  st.tasks = P.push(tasks);
+  st.bytes = (size_t)bytes;
+  st.level = level;
+  P.steps.push_back(st);
+}
+
+// Slices of operands with K <= 256, each task finding its rows' maxima: one
+// launch (see panel_slice_kernel).  Few row blocks: their K range is spread
+// over CTAs too.
+void add_panel_slice_step(Plan& P, const std::vector<SliceDesc>& descs, int level) {
+  if (descs.empty()) return;
+  int64_t blocks = 0;
+  for (const SliceDesc& d : descs) blocks += d.R64;
+  const int span = blocks >= 4 * 152 ? 16 : 2;
+  std::vector<SliceTask> tasks;
+  double bytes = 0;
+  for (size_t d = 0; d < descs.size(); d++) {
+    const SliceDesc& g = descs[d];
+    for (int rb = 0; rb < g.R64; rb++)
+      for (int kc = 0; kc < g.K32; kc += span) tasks.push_back({(int)d, rb, kc});
+    bytes += 8.0 * g.R * g.Kd * (g.cplx ? 2 : 1) + 2.0 * g.S * g.R64 * 64.0 * g.K32 * 32;
+  }
+  Step st;
+  st.kind = ST_PANEL_SLICE;
+  st.cfg = span;
   st.n = (int)tasks.size();
   st.descs = P.push(descs);
   st.tasks = P.push(tasks);
@@ -1112,74 +1148,44 @@ void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& pr
                     size_t base) {
   if (prods.empty()) return;
   OzBuilder ob(h, base);
-  int64_t nmax = 0;
-  for (const SchurProduct& q : prods) nmax += q.c + q.cu + 2 * q.s;
-  unsigned long long* maxbase = (unsigned long long*)ob.take((size_t)nmax * 8 + 8);
   std::vector<SliceDesc> sl;
   std::vector<OzDesc> out;
-  int64_t moff = 0;
   for (const SchurProduct& q : prods) {
-    SliceDesc al = ob.slice(q.AL, q.c, SLICE_ROWS, q.c, q.s);
-    al.maxbits = maxbase + moff;
-    SliceDesc ub = ob.slice(q.Uinv, q.s, SLICE_COLS, q.s, q.s);
-    ub.maxbits = maxbase + moff + q.c;
-    SliceDesc lb = ob.slice(q.Linv, q.s, SLICE_ROWS, q.s, q.s);
-    lb.maxbits = maxbase + moff + q.c + q.s;
+    const SliceDesc al = ob.slice(q.AL, q.c, SLICE_ROWS, q.c, q.s);
+    const SliceDesc ub = ob.slice(q.Uinv, q.s, SLICE_COLS, q.s, q.s);
+    const SliceDesc lb = ob.slice(q.Linv, q.s, SLICE_ROWS, q.s, q.s);
     SliceDesc au = al;
     if (q.AU != q.AL) {
       au = ob.slice(q.AU, q.cu, SLICE_ROWS, q.cu, q.s);
-      au.maxbits = maxbase + moff + q.c + 2 * q.s;
       sl.push_back(au);
     }
-    moff += q.c + q.cu + 2 * q.s;
     sl.push_back(al);
     sl.push_back(ub);
     sl.push_back(lb);
     ob.product(out, al, ub, q.TL, q.c, q.c, q.s, 1.0);
     ob.product(out, au, lb, q.TU, q.cu, q.cu, q.s, 1.0);
   }
-  Step ms;
-  ms.kind = ST_MEMSET;
-  ms.ptr = maxbase;
-  ms.bytes = (size_t)nmax * 8;
-  ms.level = lev;
-  P.steps.push_back(ms);
-  add_slice_step(P, sl, lev, true);
-  add_slice_step(P, sl, lev, false);
+  add_panel_slice_step(P, sl, lev);
   add_ozgemm_step(P, out, h->slices, lev, false, 1, 0);
 }
 
-// Schur products of one factorisation level as sliced products: row maxima
-// and slices of TL and TU (both by rows: A = TL, B = TU with K = s), then
-// the products into the FP64 Sc blocks the scatter subtracts.  Scratch from
+// Schur products of one factorisation level as sliced products: slices of TL
+// and TU (both by rows: A = TL, B = TU with K = s), then the products into the
+// FP64 Sc blocks the scatter subtracts.  Scratch from
 // `base` (bytes), after the level's FP64 region.
 void add_ozaki_schur(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
                      size_t base, bool lower) {
   OzBuilder ob(h, base);
-  int64_t nmax = 0;
-  for (const SchurProduct& q : prods) nmax += q.c + q.cu;
-  unsigned long long* maxbase = (unsigned long long*)ob.take((size_t)nmax * 8 + 8);
   std::vector<SliceDesc> sl;
   std::vector<OzDesc> out;
-  int64_t moff = 0;
   for (const SchurProduct& q : prods) {
-    SliceDesc a = ob.slice(q.TL, q.c, SLICE_ROWS, q.c, q.s);
-    a.maxbits = maxbase + moff;
-    SliceDesc b = ob.slice(q.TU, q.cu, SLICE_ROWS, q.cu, q.s);
-    b.maxbits = maxbase + moff + q.c;
-    moff += q.c + q.cu;
+    const SliceDesc a = ob.slice(q.TL, q.c, SLICE_ROWS, q.c, q.s);
+    const SliceDesc b = ob.slice(q.TU, q.cu, SLICE_ROWS, q.cu, q.s);
     sl.push_back(a);
     sl.push_back(b);
     ob.product(out, a, b, q.Sc, q.c, q.c, q.cu, 1.0);
   }
-  Step ms;
-  ms.kind = ST_MEMSET;
-  ms.ptr = maxbase;
-  ms.bytes = (size_t)nmax * 8;
-  ms.level = lev;
-  P.steps.push_back(ms);
-  add_slice_step(P, sl, lev, true);
-  add_slice_step(P, sl, lev, false);
+  add_panel_slice_step(P, sl, lev);
   // K = s <= 256 is one exact chunk: no K split, no accumulation
   add_ozgemm_step(P, out, h->slices, lev, false, 1, 0, lower);
 }
@@ -1285,29 +1291,9 @@ void add_sliced_normalize(pselinv_ctx* h, Plan& P, const std::vector<std::pair<i
     }
   }
   if (prods.empty()) return;
-  // few row blocks: their K range is spread over CTAs too
-  int64_t blocks = 0;
-  for (const SliceDesc& d : sl) blocks += d.R64;
-  const int span = blocks >= 4 * 152 ? 16 : 2;
-  std::vector<SliceTask> st;
-  double bytes = 0;
-  for (size_t d = 0; d < sl.size(); d++) {
-    for (int rb = 0; rb < sl[d].R64; rb++)
-      for (int kc = 0; kc < sl[d].K32; kc += span) st.push_back({(int)d, rb, kc});
-    bytes += (double)es * sl[d].R * sl[d].Kd + 2.0 * kNormSlices * 64.0 * sl[d].R64 * 32 * sl[d].K32;
-  }
-  Step a;
-  a.kind = ST_NORM_SLICE;
-  a.cfg = span;
-  a.n = (int)st.size();
-  a.descs = P.push(sl);
-  a.tasks = P.push(st);
-  a.bytes = (size_t)bytes;
-  a.level = lev;
-  P.steps.push_back(a);
+  add_panel_slice_step(P, sl, lev);
   std::vector<OzTask> tasks;
-  double flops = 0;
-  bytes = 0;
+  double flops = 0, bytes = 0;
   for (size_t d = 0; d < prods.size(); d++) {
     const OzDesc& g = prods[d];
     for (int tm = 0; tm < ceil_div(g.M, 128); tm++)  // longest K range first
@@ -1825,10 +1811,10 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
       break;
     case ST_LU_PANEL:
       launch_lu_panel(h->dtype, h->S, h->lu, h->winv, h->piv, (const LuTask*)(a + s.tasks), s.n,
-                      s.cfg, h->opts.symmetric != 0 && !h->H.general, st);
+                      s.cfg, s.n2 != 0, h->opts.symmetric != 0 && !h->H.general, st);
       break;
-    case ST_NORM_SLICE:
-      launch_norm_slice((const SliceDesc*)(a + s.descs), (const SliceTask*)(a + s.tasks), s.n, s.cfg,
+    case ST_PANEL_SLICE:
+      launch_panel_slice((const SliceDesc*)(a + s.descs), (const SliceTask*)(a + s.tasks), s.n, s.cfg,
                         st);
       break;
     case ST_NORM_GEMM:

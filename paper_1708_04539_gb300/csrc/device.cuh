@@ -280,10 +280,11 @@ void launch_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, bo
 // half) instead of shared memory
 void launch_ozaki_gemm(int S, const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
                        bool persistent, bool a_tmem, cudaStream_t st);
-// The normalisation's products at eight slices (K <= 256; op(B) lower
-// triangular): slices with their own row maxima, `span` K blocks per task
-// {d, row block, first K block}; products C = A op(B), tasks {d, tm, tn, 0}
-void launch_norm_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, int span,
+// Slices of operands with K <= 256 with their own row maxima (desc.maxbits
+// unused), `span` K blocks per task {d, row block, first K block}; and the
+// normalisation's products at eight slices (K <= 256; op(B) lower
+// triangular): C = A op(B), tasks {d, tm, tn, 0}
+void launch_panel_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, int span,
                        cudaStream_t st);
 void launch_norm_gemm(const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
                       cudaStream_t st);
@@ -332,10 +333,12 @@ size_t trace_partial_bytes();
 void launch_scatter_values(int dtype, const SymDev& S, const void* values, void* store,
                            int nbatch, cudaStream_t st);
 // one panel step of the blocked diagonal LU (one CTA per task; groups = 1 or
-// kLuGroups: 32 or 32 kLuGroups lines per task; sym: symmetric values), and
-// the factored pivot blocks into the storage
+// kLuGroups: 32 or 32 kLuGroups lines per task; solve: narrow supernodes'
+// panels too; sym: symmetric values), and the factored pivot blocks into the
+// storage
 void launch_lu_panel(int dtype, const SymDev& S, void* store, void* winv, void* piv,
-                     const LuTask* tasks, int ntasks, int groups, bool sym, cudaStream_t st);
+                     const LuTask* tasks, int ntasks, int groups, bool solve, bool sym,
+                     cudaStream_t st);
 void launch_unpack_pivots(int dtype, const SymDev& S, void* store, const void* piv, int nbatch,
                           cudaStream_t st);
 // FP64 peak loop (the FP64 roofline's denominator): grid for `sms` SMs;

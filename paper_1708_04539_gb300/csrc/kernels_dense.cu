@@ -136,10 +136,13 @@ gemm_kernel(const GemmDesc* __restrict__ descs, const GemmTask* __restrict__ tas
 // eliminates 32 G "lines" beside it.  The lines of a panel, in order:
 //   nl rows of L21 (X U11 = A21), nl columns of U12 (L11 Y = A12): the rest of
 //      the diagonal block (s > 32: nl = s - j0 - w, in place);
-//   for a narrow supernode (s <= 32, one panel) instead the c rows of its L
-//      panel and the cu rows of its U^T panel, so that its triangular solves
-//      need no inverse and no launch of their own (symmetric values: no U^T
-//      lines, an L line's unscaled entries are the row of U^T);
+//   for a narrow supernode (s <= 32, one panel; solve = 1) instead the c rows
+//      of its L panel and the cu rows of its U^T panel, so that its triangular
+//      solves need no inverse and no launch of their own (symmetric values: no
+//      U^T lines, an L line's unscaled entries are the row of U^T).  Levels with
+//      sliced panel solves leave them to those (solve = 0): 64 lines a block
+//      instead of 64 + c + cu (20 complex shifts of a 16^3 operator, a level of
+//      660 tasks: 352 -> 242 us);
 //   w unit rows and w unit columns: U11^{-1} and L11^{-1} into winv.
 // Every task of a panel factors the pivot block again (the FP64 pipe takes
 // 64 cycles per warp instruction whatever the mask, so the pivot block's
@@ -196,7 +199,8 @@ __device__ __forceinline__ cdouble fnma_s(cdouble a, cdouble b, cdouble c) {
 constexpr int kLuW = kLuPanel;  // panel width
 template <typename T, int G>
 __global__ void __launch_bounds__(128 * (G + 1))
-lu_panel_kernel(SymDev S, T* store, T* winv, T* piv, const LuTask* __restrict__ tasks, int sym) {
+lu_panel_kernel(SymDev S, T* store, T* winv, T* piv, const LuTask* __restrict__ tasks, int solve,
+                int sym) {
   constexpr int kThr = 128 * (G + 1);
   extern __shared__ __align__(16) unsigned char lu_smem[];
   T(*Dd)[kLuW + 1] = reinterpret_cast<T(*)[kLuW + 1]>(lu_smem);  // A11, then the rows of U11
@@ -209,7 +213,7 @@ lu_panel_kernel(SymDev S, T* store, T* winv, T* piv, const LuTask* __restrict__ 
   const LuTask task = tasks[blockIdx.x];
   const int K = task.K, j0 = task.j0, s = S.sn_width[K], c = S.sn_c[K];
   const int w = min(kLuW, s - j0), rest = s - j0 - w;
-  const bool narrow = s <= kLuW;
+  const bool narrow = s <= kLuW && solve;
   T* D = store + (int64_t)task.inst * S.storage + S.sn_off[K];
   T* W = winv + (int64_t)task.inst * S.w_stride + S.w_off[K];
   // line ranges and addresses: entry k of L line i at Lb[i + k ldl], of U line i
@@ -271,8 +275,8 @@ lu_panel_kernel(SymDev S, T* store, T* winv, T* piv, const LuTask* __restrict__ 
       }
       __syncthreads();
     }
-  } else if (q < 0) {
-    for (int k = 0; k < w; k++) __syncthreads();
+  } else if (q < 0 || (team > 0 && task.line0 + 32 * (team - 1) >= nlines)) {
+    for (int k = 0; k < w; k++) __syncthreads();  // a scheduler's spare warp, or no lines left
   } else {
     constexpr int kCols = (kLuW + 2) / 3;
     const T* sm = reinterpret_cast<const T*>(lu_smem);
@@ -558,21 +562,22 @@ constexpr int lu_smem_bytes() {
 }
 template <typename T, int G>
 void lu_launch_t(const SymDev& S, void* store, void* winv, void* piv, const LuTask* tasks,
-                 int ntasks, bool sym, cudaStream_t st) {
+                 int ntasks, bool solve, bool sym, cudaStream_t st) {
   lu_panel_kernel<T, G><<<ntasks, 128 * (G + 1), lu_smem_bytes<T, G>(), st>>>(
-      S, (T*)store, (T*)winv, (T*)piv, tasks, sym ? 1 : 0);
+      S, (T*)store, (T*)winv, (T*)piv, tasks, solve ? 1 : 0, sym ? 1 : 0);
 }
 }  // namespace
 
 void launch_lu_panel(int dtype, const SymDev& S, void* store, void* winv, void* piv,
-                     const LuTask* tasks, int ntasks, int groups, bool sym, cudaStream_t st) {
+                     const LuTask* tasks, int ntasks, int groups, bool solve, bool sym,
+                     cudaStream_t st) {
   if (ntasks <= 0) return;
   if (dtype == DT_F64) {
-    if (groups == 1) lu_launch_t<double, 1>(S, store, winv, piv, tasks, ntasks, sym, st);
-    else lu_launch_t<double, kLuGroups>(S, store, winv, piv, tasks, ntasks, sym, st);
+    if (groups == 1) lu_launch_t<double, 1>(S, store, winv, piv, tasks, ntasks, solve, sym, st);
+    else lu_launch_t<double, kLuGroups>(S, store, winv, piv, tasks, ntasks, solve, sym, st);
   } else {
-    if (groups == 1) lu_launch_t<cdouble, 1>(S, store, winv, piv, tasks, ntasks, sym, st);
-    else lu_launch_t<cdouble, kLuGroups>(S, store, winv, piv, tasks, ntasks, sym, st);
+    if (groups == 1) lu_launch_t<cdouble, 1>(S, store, winv, piv, tasks, ntasks, solve, sym, st);
+    else lu_launch_t<cdouble, kLuGroups>(S, store, winv, piv, tasks, ntasks, solve, sym, st);
   }
 }
 

@@ -248,14 +248,14 @@ __device__ __forceinline__ void write_digits8(const double (&x)[8], int e, __hal
   }
 }
 
-// Eight-digit slices of operands with K <= 256 (the normalisation): a task is
-// a 64-row block and `span` K blocks from kc; every task finds its rows'
-// maxima itself over the whole K (a row is read by four lanes of one warp, and
-// comes from L1 / L2 the second time), so no maxima pass, no zeroed buffer and
-// one launch instead of three.  d.tri: X(r, k) = 0 for k < r, and nobody reads
-// the K blocks left of the row block's diagonal.
+// Slices of operands with K = s <= 256 (the normalisation's, the
+// factorisation's): a task is a 64-row block and `span` K blocks from kc;
+// every task finds its rows' maxima itself over the whole K (a row is read by
+// four lanes of one warp, and comes from L1 / L2 the second time), so no maxima
+// pass, no zeroed buffer and one launch instead of three.  d.tri: X(r, k) = 0
+// for k < r, and nobody reads the K blocks left of the row block's diagonal.
 __global__ void __launch_bounds__(kSliceThreads)
-norm_slice_kernel(const SliceDesc* __restrict__ descs, const SliceTask* __restrict__ tasks,
+panel_slice_kernel(const SliceDesc* __restrict__ descs, const SliceTask* __restrict__ tasks,
                   int ntasks, int span) {
   const int tid = threadIdx.x, ci = tid >> 3, rr = tid & 7;
   const int rl = (ci >> 2) * 8 + rr, kg = ci & 3;
@@ -281,8 +281,11 @@ norm_slice_kernel(const SliceDesc* __restrict__ descs, const SliceTask* __restri
       if (d.tri && (kb >= half ? kb - half : kb) < 2 * task.rb) continue;
       double x[8];
       load8(d, r, kb * 32 + kg * 8, x);
-      write_digits8(x, e, d.out + ((int64_t)task.rb * d.K32 + kb) * (kTileBytes / 2) + tid * 8,
-                    slice_stride);
+      __half* out = d.out + ((int64_t)task.rb * d.K32 + kb) * (kTileBytes / 2) + tid * 8;
+      if (d.S == 8)
+        write_digits8(x, e, out, slice_stride);
+      else
+        write_digits(x, e, d.S, out, slice_stride);
     }
   }
 }
@@ -1341,11 +1344,11 @@ cudaError_t prepare_ozaki_kernels() {
                               kNormStages * kNormStage);
 }
 
-void launch_norm_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, int span,
+void launch_panel_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, int span,
                        cudaStream_t st) {
   if (ntasks <= 0) return;
   const int grid = ntasks < 152 * 16 ? ntasks : 152 * 16;
-  norm_slice_kernel<<<grid, kSliceThreads, 0, st>>>(descs, tasks, ntasks, span);
+  panel_slice_kernel<<<grid, kSliceThreads, 0, st>>>(descs, tasks, ntasks, span);
 }
 
 void launch_norm_gemm(const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
