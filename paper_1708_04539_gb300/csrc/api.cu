@@ -57,7 +57,8 @@ enum StepKind {
   ST_MIRROR,
   ST_UNPACK_PIVOTS,
   ST_PANEL_SLICE,
-  ST_NORM_GEMM
+  ST_NORM_GEMM,
+  ST_SCHUR_SCATTER
 };
 
 struct Step {
@@ -664,6 +665,50 @@ void add_panel_step(Plan& P, const std::vector<LuTask>& tasks, int level, bool s
   P.steps.push_back(d);
 }
 
+// FP64 Schur complements of one level, scattered as they are computed.  Tile
+// and K split by the level's work over the chip (FP64 pipe, 16 cycles per warp
+// operation and SM): less than 40 us of it (four waves of 32 x 32 x 32 tasks):
+// 16 x 16 tiles, else 32 x 32 (28 MFLOP of complex grids 41 against 60 us; 24^3
+// upwind, 62 MFLOP: 66 us at 32 x 32); a task's K range short enough to last no
+// longer than half the level's work, in steps of 32.
+void add_schur_scatter(pselinv_ctx* h, Plan& P, const std::vector<SchurDesc>& descs, int level,
+                       bool lower) {
+  if (descs.empty()) return;
+  const double cplx = h->dtype == DT_F64 ? 1.0 : 4.0;
+  double ops = 0, bytes = 0;
+  for (const SchurDesc& d : descs) {
+    const double e = (double)d.c * d.cu * (lower ? 0.5 : 1.0), s = (double)h->H.sn_width[d.K];
+    ops += e * s / 32 * cplx;
+    bytes += (double)h->esize * (2.0 * e + s * (d.c + d.cu));
+  }
+  const double cycles = ops * 16.0 / 152.0;
+  const int tile = cycles < 80e3 ? 16 : 32;
+  const double per_k = tile * tile / 32.0 * 19.0 * cplx;  // cycles of a task per k
+  const int kmax = std::max(32, (int)(std::max(cycles / 2, per_k * 32) / per_k) / 32 * 32);
+  std::vector<SchurTask> tasks;
+  for (size_t d = 0; d < descs.size(); d++) {
+    const int s = (int)h->H.sn_width[descs[d].K];
+    for (int k = 0; k < s; k += kmax)
+      for (int tq = 0; tq < ceil_div(descs[d].cu, tile); tq++)
+        for (int tp = lower ? tq : 0; tp < ceil_div(descs[d].c, tile); tp++)
+          tasks.push_back({(int)d, tp, tq, k, std::min(s, k + kmax)});
+  }
+  // longest K ranges first
+  std::stable_sort(tasks.begin(), tasks.end(), [](const SchurTask& a, const SchurTask& b) {
+    return a.k1 - a.k0 > b.k1 - b.k0;
+  });
+  Step st;
+  st.kind = ST_SCHUR_SCATTER;
+  st.cfg = tile;
+  st.n = (int)tasks.size();
+  st.descs = P.push(descs);
+  st.tasks = P.push(tasks);
+  st.flops = 64.0 * ops;
+  st.bytes = (size_t)bytes;
+  st.level = level;
+  P.steps.push_back(st);
+}
+
 // The triangular inverses of the wide supernodes from those of their 32 x 32
 // pivot blocks (written by the panel steps), doubling the block size b: for
 // neighbouring blocks 1, 2 of one triangle
@@ -732,15 +777,14 @@ int build_factor_plan(pselinv_ctx* h) {
     std::vector<SnTask> mirrored;  // symmetric values: blocks whose upper triangle is filled in
     std::vector<LuTask> panels;    // first panels of every supernode, 32 lines per task
     std::vector<int64_t> gofs;
-    std::vector<GemmDesc> trsm, schur;
+    std::vector<GemmDesc> trsm;
+    std::vector<SchurDesc> schur;
     std::vector<SchurProduct> sprods, solves;
     std::vector<CopySeg> segs;
     const int64_t l0 = H.hlevel_ptr[lev], l1 = H.hlevel_ptr[lev + 1];
-    // split precision: the triangular solves of wide supernodes and the Schur
-    // products of levels with enough Schur work as sliced tensor-core products
-    // (their operands sliced from the level's scratch after its FP64 region);
-    // otherwise FP64 row panels, which beat 64 x 64 tiles on these products
-    // at every width (40^3 factorisation 61.9 -> 57.1 ms)
+    // split precision: the triangular solves and the Schur products of levels
+    // with enough Schur work as sliced tensor-core products (their operands
+    // sliced from the level's scratch after its FP64 region)
     double sflops = 0;
     for (int64_t i = l0; i < l1; i++) {
       const int64_t K = H.hlevel_sn[i];
@@ -796,12 +840,15 @@ int build_factor_plan(pselinv_ctx* h) {
           }
         }
         const int64_t s0 = off;
-        off += c * cu;
+        if (split) off += c * cu;
         char* Sc = h->scratch + (size_t)s0 * es;
         const SchurProduct q{TL, TU, Sc, (int)c, (int)cu, (int)s, Lp, ldlt ? Lp : Up, Uinv, Linv};
         if (c > 0 && cu > 0) {
           if (oz) solves.push_back(q);
-          schur.push_back(make_desc(TL, TU, Sc, c, cu, s, c, cu, c, 0, 1, 1.0, 0.0));
+          if (!split) {
+            schur.push_back({TL, TU, (int)b, (int)K, (int)c, (int)cu});
+            continue;
+          }
           sprods.push_back(q);
           for (int tq = 0; tq < ceil_div(cu, 32); tq++)
             for (int tp = ldlt ? tq : 0; tp < ceil_div(c, 32); tp++) {
@@ -844,12 +891,15 @@ int build_factor_plan(pselinv_ctx* h) {
       add_gemm_step(P, dt, choose_small_tile(dt, upd), upd, (int)lev);
     }
     add_inverse_merges(h, P, wide, mofs, (int)lev);
-    add_gemm_step(P, dt, GEMM_ROWS, trsm, (int)lev);
+    // few solves: small tiles (a row panel's 8 columns per thread are a chain of
+    // 8 s multiply-adds, 65 us for s = 64 complex; a 16 x 16 tile's 2 s)
+    add_gemm_step(P, dt, choose_small_tile(dt, trsm) == GEMM_16x16 ? GEMM_16x16 : GEMM_ROWS, trsm,
+                  (int)lev);
     if (split) {
       add_ozaki_trsm(h, P, solves, (int)lev, align256((size_t)off * es));
       add_ozaki_schur(h, P, sprods, (int)lev, align256((size_t)off * es), ldlt);
     } else {
-      add_gemm_step(P, dt, GEMM_ROWS, schur, (int)lev, -1, ldlt);
+      add_schur_scatter(h, P, schur, (int)lev, ldlt);
     }
     if (!gt.empty()) {
       Step sc;
@@ -1813,6 +1863,11 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
       launch_lu_panel(h->dtype, h->S, h->lu, h->winv, h->piv, (const LuTask*)(a + s.tasks), s.n,
                       s.cfg, s.n2 != 0, h->opts.symmetric != 0 && !h->H.general, st);
       break;
+    case ST_SCHUR_SCATTER:
+      launch_schur_scatter(h->dtype, h->S, h->lu, (const SchurDesc*)(a + s.descs),
+                           (const SchurTask*)(a + s.tasks), s.n, s.cfg,
+                           h->opts.symmetric != 0 && !h->H.general, st);
+      break;
     case ST_PANEL_SLICE:
       launch_panel_slice((const SliceDesc*)(a + s.descs), (const SliceTask*)(a + s.tasks), s.n, s.cfg,
                         st);
@@ -2493,7 +2548,8 @@ int pselinv_profile(pselinv_t h, int which, void* stream, pselinv_step_stat* out
                                 PSELINV_STEP_DIAG_LU, PSELINV_STEP_SMALL_LEVEL,
                                 PSELINV_STEP_GATHER_SLICE, PSELINV_STEP_OUTPUT_MAXIMA,
                                 PSELINV_STEP_COPY, PSELINV_STEP_COPY,
-                                PSELINV_STEP_SLICE, PSELINV_STEP_OZAKI_GEMM};
+                                PSELINV_STEP_SLICE, PSELINV_STEP_OZAKI_GEMM,
+                                PSELINV_STEP_GEMM};
     out[i].kind = kinds[s.kind];
     out[i].level = s.level;
     out[i].tasks = s.n;

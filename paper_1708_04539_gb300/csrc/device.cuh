@@ -191,6 +191,17 @@ struct LuTask {
   int inst, K, j0, line0;
 };
 
+// one supernode's FP64 Schur complement TL TU^T (TL: c x s, TU: cu x s,
+// column-major) and a tile of it over K range [k0, k1)
+struct SchurDesc {
+  const void* TL;
+  const void* TU;
+  int inst, K, c, cu;
+};
+struct SchurTask {
+  int d, tp, tq, k0, k1;
+};
+
 // contiguous copy segment
 struct CopySeg {
   const void* src;
@@ -385,6 +396,11 @@ void launch_scatter_set(int dtype, const SymDev& S, void* store, const void* src
 void launch_scatter_sub(int dtype, const SymDev& S, void* store, const void* src,
                         const int64_t* sofs, const SnTask* tasks, int ntasks, bool lower,
                         cudaStream_t st);
+// store(R_L, R_U) -= TL TU^T in one launch (tile: 16 or 32; lower: entries on
+// or below the diagonal)
+void launch_schur_scatter(int dtype, const SymDev& S, void* store, const SchurDesc* descs,
+                          const SchurTask* tasks, int ntasks, int tile, bool lower,
+                          cudaStream_t st);
 // upper triangle of each task's diagonal block := its lower one, transposed
 void launch_mirror_lower(int dtype, const SymDev& S, void* store, const SnTask* tasks, int ntasks,
                          cudaStream_t st);

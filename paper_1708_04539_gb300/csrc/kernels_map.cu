@@ -193,11 +193,35 @@ gather_general_kernel(SymDev S, const T* __restrict__ store, T* out,
   }
 }
 
+// Slot of the Schur update of entry (i, m), i = R_L(K)[p] in supernode I, m =
+// R_U(K)[q] in J: the diagonal block (I == J), the L panel of J (I > J: position
+// of i in R_L(J) from the map of R_U(K)'s block) or the U^T panel of I (I < J:
+// position of m in R_U(I)).  ok = false when a checked map read is out of range.
+__device__ __forceinline__ int64_t schur_slot_general(const SymDev& S, int64_t rbL, int64_t rbU, int p,
+                                                      int q, bool& ok) {
+  const int bp = S.rows_blk[rbL + p], bq = S.urows_blk[rbU + q];
+  const int I = S.blk_sn[bp], J = S.ublk_sn[bq];
+  const int i = S.lrows[rbL + p], m = S.urows[rbU + q];
+  if (I == J) {
+    const int sI = S.sn_width[I], f = S.sn_first[I];
+    return S.sn_off[I] + (i - f) + (int64_t)(m - f) * sI;
+  }
+  const int64_t ri = I > J ? S.ublk_rel[bq] - S.ublk_q0[bq] + p : S.blk_rel[bp] - S.blk_q0[bp] + q;
+  if (S.check && (ri < 0 || ri >= S.relidx_size)) {
+    ok = false;
+    return 0;
+  }
+  if (I > J) {
+    const int sJ = S.sn_width[J];
+    return S.sn_off[J] + (int64_t)sJ * sJ + S.relidx[ri] + (int64_t)(m - S.sn_first[J]) * S.sn_c[J];
+  }
+  const int sI = S.sn_width[I];
+  return S.sn_off[I] + (int64_t)sI * sI + (int64_t)S.sn_c[I] * sI + S.relidx[ri] +
+         (int64_t)(i - S.sn_first[I]) * S.sn_cu[I];
+}
+
 // store(R_L(K), R_U(K)) -= Sc (c_L x c_U, column-major; atomic: supernodes
-// of one level may update the same ancestors).  Entry (i, m), i = R_L[p] in
-// supernode I, m = R_U[q] in J, goes to the diagonal block (I == J), the L
-// panel of J (I > J: position of i in R_L(J) from the map of R_U(K)'s block)
-// or the U^T panel of I (I < J: position of m in R_U(I)).
+// of one level may update the same ancestors); slots as above.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 scatter_sub_general_kernel(SymDev S, T* store, const T* __restrict__ src,
@@ -215,29 +239,8 @@ scatter_sub_general_kernel(SymDev S, T* store, const T* __restrict__ src,
     for (int r = ly; r < kTile; r += kThreads / 32) {
       const int p = p0 + lx, q = q0 + r;
       if (p >= cl || q >= cu) continue;
-      const int bp = S.rows_blk[rbL + p], bq = S.urows_blk[rbU + q];
-      const int I = S.blk_sn[bp], J = S.ublk_sn[bq];
-      const int i = S.lrows[rbL + p], m = S.urows[rbU + q];
-      int64_t slot;
       bool ok = true;
-      if (I == J) {
-        const int sI = S.sn_width[I], f = S.sn_first[I];
-        slot = S.sn_off[I] + (i - f) + (int64_t)(m - f) * sI;
-      } else if (I > J) {
-        const int64_t ri = S.ublk_rel[bq] - S.ublk_q0[bq] + p;
-        if (S.check && (ri < 0 || ri >= S.relidx_size)) ok = false;
-        const int sJ = S.sn_width[J];
-        slot = ok ? S.sn_off[J] + (int64_t)sJ * sJ + S.relidx[ri] +
-                        (int64_t)(m - S.sn_first[J]) * S.sn_c[J]
-                  : 0;
-      } else {
-        const int64_t ri = S.blk_rel[bp] - S.blk_q0[bp] + q;
-        if (S.check && (ri < 0 || ri >= S.relidx_size)) ok = false;
-        const int sI = S.sn_width[I];
-        slot = ok ? S.sn_off[I] + (int64_t)sI * sI + (int64_t)S.sn_c[I] * sI + S.relidx[ri] +
-                        (int64_t)(i - S.sn_first[I]) * S.sn_cu[I]
-                  : 0;
-      }
+      const int64_t slot = schur_slot_general(S, rbL, rbU, p, q, ok);
       if (S.check && (slot < 0 || slot >= S.storage)) ok = false;
       if (!ok) {
         set_error(S.err, DEV_CHECK, K);
@@ -309,6 +312,119 @@ scatter_sub_kernel(SymDev S, T* store, const T* __restrict__ src, const int64_t*
       else
         atomic_add_s(dst + slot, scale_s(v, -1.0));
     }
+    __syncthreads();
+  }
+}
+
+// Schur complement of one supernode's FP64 panels subtracted straight from
+// the ancestors: a task computes the TS x TS tile (tp, tq) of TL TU^T over K
+// range [k0, k1) and subtracts it atomically (so a K split costs nothing but
+// atomics), the storage bases of the tile's rows and columns staged as in
+// scatter_sub_kernel.  The product is never stored, and a level needs one
+// launch for what were a product and a scatter.  256 threads, (TS / 16)^2
+// outputs each; the FP64 pipe (19 cycles per warp operation and SM) is the
+// bound of a task: 32 x 32 x 32 takes it 10 us, 16 x 16 x 32 2.5 us, so levels
+// of little work use the small tile (see add_schur_scatter).
+template <typename T, int TS, bool LOWER, bool GENERAL>
+__global__ void __launch_bounds__(kThreads)
+schur_scatter_kernel(SymDev S, T* store, const SchurDesc* __restrict__ descs,
+                     const SchurTask* __restrict__ tasks, int ntasks) {
+  constexpr int TM = TS / 16, BK = 32, NL = TS * BK / kThreads;
+  __shared__ T sa[BK][TS], sb[BK][TS];
+  __shared__ int64_t cdiag[TS], cpan[TS], crel[TS], rpan[TS], rrel[TS];
+  __shared__ int csn[TS], rsn[TS];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  for (int t = blockIdx.x; t < ntasks; t += gridDim.x) {
+    const SchurTask task = tasks[t];
+    const SchurDesc d = descs[task.d];
+    const T* __restrict__ A = (const T*)d.TL;
+    const T* __restrict__ B = (const T*)d.TU;
+    const int K = d.K, c = d.c, cu = d.cu;
+    const int p0 = task.tp * TS, q0 = task.tq * TS;
+    const int64_t rbL = S.rows_ptr[K], rbU = GENERAL ? S.urows_ptr[K] : rbL;
+    T ra[NL], rb[NL];
+    auto load = [&](int k0) {
+#pragma unroll
+      for (int i = 0; i < NL; i++) {
+        const int e = tid + i * kThreads, m = e % TS, k = k0 + e / TS;
+        const bool in = k < task.k1;
+        ra[i] = in && p0 + m < c ? A[p0 + m + (int64_t)k * c] : sc_zero(T());
+        rb[i] = in && q0 + m < cu ? B[q0 + m + (int64_t)k * cu] : sc_zero(T());
+      }
+    };
+    load(task.k0);
+    if (!GENERAL) {
+      if (tid < TS) {
+        if (q0 + tid < c) {
+          cdiag[tid] = S.col_diag[rbL + q0 + tid];
+          cpan[tid] = S.col_pan[rbL + q0 + tid];
+          crel[tid] = S.col_rel[rbL + q0 + tid];
+          csn[tid] = S.col_sn[rbL + q0 + tid];
+        }
+      } else if (tid < 2 * TS) {
+        const int m = tid - TS;
+        if (p0 + m < c) {
+          rpan[m] = S.row_pan[rbL + p0 + m];
+          rrel[m] = S.row_rel[rbL + p0 + m];
+          rsn[m] = S.row_sn[rbL + p0 + m];
+        }
+      }
+    }
+    T acc[TM][TM];
+#pragma unroll
+    for (int i = 0; i < TM; i++)
+#pragma unroll
+      for (int j = 0; j < TM; j++) acc[i][j] = sc_zero(T());
+    for (int k0 = task.k0; k0 < task.k1; k0 += BK) {
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < NL; i++) {
+        const int e = tid + i * kThreads;
+        sa[e / TS][e % TS] = ra[i];
+        sb[e / TS][e % TS] = rb[i];
+      }
+      __syncthreads();
+      if (k0 + BK < task.k1) load(k0 + BK);
+      const int kn = min(BK, task.k1 - k0);
+#pragma unroll 4
+      for (int k = 0; k < kn; k++) {
+        T a[TM], b[TM];
+#pragma unroll
+        for (int i = 0; i < TM; i++) a[i] = sa[k][tx + 16 * i];
+#pragma unroll
+        for (int j = 0; j < TM; j++) b[j] = sb[k][ty + 16 * j];
+#pragma unroll
+        for (int i = 0; i < TM; i++)
+#pragma unroll
+          for (int j = 0; j < TM; j++) acc[i][j] = fma_s(a[i], b[j], acc[i][j]);
+      }
+    }
+    T* dst = store + (int64_t)d.inst * S.storage;
+#pragma unroll
+    for (int i = 0; i < TM; i++)
+#pragma unroll
+      for (int j = 0; j < TM; j++) {
+        const int pl = tx + 16 * i, ql = ty + 16 * j, p = p0 + pl, q = q0 + ql;
+        if (p >= c || q >= cu || (LOWER && p < q)) continue;
+        int64_t slot = 0;
+        bool ok = true;
+        if (GENERAL) {
+          slot = schur_slot_general(S, rbL, rbU, p, q, ok);
+        } else {
+          const bool col_side = rsn[pl] >= csn[ql];
+          const int64_t ri = col_side ? crel[ql] + p : rrel[pl] + q;
+          if (S.check && (ri < 0 || ri >= S.relidx_size)) ok = false;
+          if (ok)
+            slot = (col_side ? (rsn[pl] == csn[ql] ? cdiag[ql] : cpan[ql]) : rpan[pl]) +
+                   S.relidx[ri];
+        }
+        if (S.check && (slot < 0 || slot >= S.storage)) ok = false;
+        if (!ok) {
+          set_error(S.err, DEV_CHECK, K);
+          continue;
+        }
+        atomic_add_s(dst + slot, scale_s(acc[i][j], -1.0));
+      }
     __syncthreads();
   }
 }
@@ -605,6 +721,35 @@ void launch_scatter_sub(int dtype, const SymDev& S, void* store, const void* src
     else
       scatter_sub_kernel<cdouble><<<grid, kThreads, 0, st>>>(
           S, (cdouble*)store, (const cdouble*)src, sofs, tasks, ntasks);
+  }
+}
+
+namespace {
+template <typename T, int TS>
+void schur_launch_t(const SymDev& S, void* store, const SchurDesc* descs, const SchurTask* tasks,
+                    int ntasks, bool lower, cudaStream_t st) {
+  if (S.general)
+    schur_scatter_kernel<T, TS, false, true><<<ntasks, kThreads, 0, st>>>(S, (T*)store, descs, tasks,
+                                                                          ntasks);
+  else if (lower)
+    schur_scatter_kernel<T, TS, true, false><<<ntasks, kThreads, 0, st>>>(S, (T*)store, descs, tasks,
+                                                                          ntasks);
+  else
+    schur_scatter_kernel<T, TS, false, false><<<ntasks, kThreads, 0, st>>>(S, (T*)store, descs,
+                                                                           tasks, ntasks);
+}
+}  // namespace
+
+void launch_schur_scatter(int dtype, const SymDev& S, void* store, const SchurDesc* descs,
+                          const SchurTask* tasks, int ntasks, int tile, bool lower,
+                          cudaStream_t st) {
+  if (ntasks <= 0) return;
+  if (dtype == DT_F64) {
+    if (tile == 16) schur_launch_t<double, 16>(S, store, descs, tasks, ntasks, lower, st);
+    else schur_launch_t<double, 32>(S, store, descs, tasks, ntasks, lower, st);
+  } else {
+    if (tile == 16) schur_launch_t<cdouble, 16>(S, store, descs, tasks, ntasks, lower, st);
+    else schur_launch_t<cdouble, 32>(S, store, descs, tasks, ntasks, lower, st);
   }
 }
 

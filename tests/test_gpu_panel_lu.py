@@ -77,3 +77,34 @@ def test_many_instances(torch, s, complex_values):
     h.selinv()
     check(p, h, [0, 77, nb - 1])
     h.close()
+
+
+@pytest.mark.parametrize("kind", ["real", "complex", "symmetric"])
+def test_large_schur_tiles(torch, kind):
+    """Levels with enough Schur work for 32 x 32 tiles and a K split: ragged
+    tiles (133 rows) over supernodes of 90 columns, 24 instances."""
+    import paper_1708_04539_gb300 as ps
+    n, nb = 90 + 133, 24
+    ii, jj = np.meshgrid(np.arange(n), np.arange(n), indexing="ij")
+    p = gen.problems._finish_small(n, ii.reshape(-1), jj.reshape(-1), 990, kind == "complex",
+                                   f"dense_{n}", 90, symmetric_values=kind == "symmetric")
+    p.values = np.ascontiguousarray(p.values[None, :] * np.linspace(0.5, 2.0, nb)[:, None])
+    h = ps.SelInv.from_problem(p, symmetric=kind == "symmetric", check_level=1)
+    h.factor(torch.from_numpy(p.values).cuda())
+    h.selinv()
+    check(p, h, [0, nb - 1])
+    h.close()
+
+
+@pytest.mark.parametrize("density,max_sn", [(0.02, 16), (0.3, 64)])
+def test_general_schur(torch, density, max_sn):
+    """C_L != C_U: the Schur tiles through the two row structures' maps."""
+    import paper_1708_04539_gb300 as ps
+    p = gen.general_random(300, density, 77, max_sn=max_sn)
+    h = ps.SelInv.from_general_problem(p, check_level=1)
+    h.factor(torch.from_numpy(p.values).cuda())
+    h.selinv()
+    got = h.get_selected()
+    ref = oracle.gextract(oracle.general_selected_inverse(p), p.colptr, p.rowind)
+    assert np.abs(got - ref).max() < 1e-10 * np.abs(ref).max()
+    h.close()
