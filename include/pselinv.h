@@ -103,8 +103,9 @@ typedef struct pselinv_opts {
                             A_{K,C}^T L_KK^{-T} and the Schur-complement products
                             L_{C,K} U_{K,C} of pselinv_factor as sliced FP16 tensor-core
                             products (exact FP32 accumulation, FP64 result) on the levels
-                            whose Schur products reach factor_split_mflops; the diagonal
-                            LU, the triangular inverses and the scatter into the
+                            whose Schur products reach factor_split_mflops (smaller levels
+                            keep FP64 accuracy: FP64 products, or products of eight slices
+                            where the FP64 pipe would take longer); the diagonal LU, the triangular inverses and the scatter into the
                             ancestors stay FP64 */
   int32_t factor_split_mflops; /* factor_precision = OZAKI_FP16: smallest Schur-product work
                             (MFLOP) of a level that goes split; 0 = default (200); < 0:

@@ -57,7 +57,7 @@ enum StepKind {
   ST_MIRROR,
   ST_UNPACK_PIVOTS,
   ST_PANEL_SLICE,
-  ST_NORM_GEMM,
+  ST_GEMM8,
   ST_SCHUR_SCATTER
 };
 
@@ -484,12 +484,12 @@ size_t ozaki_level_bytes(const HostSym& H, int64_t nb, int S, size_t es) {
 // slices of the normalisation's operands on split levels, and the narrowest
 // supernode whose normalisation is sliced (a narrower one's operands would be
 // mostly padding: K blocks of 32 and column tiles of 64)
-constexpr int kNormSlices = 8;
+constexpr int kSlices8 = 8;
 constexpr int64_t kNormMinWidth = 33;
 
 // bytes of the split normalisation of the largest level
 size_t ozaki_norm_bytes(const HostSym& H, int64_t nb, size_t es) {
-  const int S = kNormSlices;
+  const int S = kSlices8;
   const size_t parts = es / 8;
   size_t mx = 0;
   for (size_t d = 0; d + 1 < H.level_ptr.size(); d++) {
@@ -544,7 +544,7 @@ size_t scratch_need(const HostSym& H, int64_t nb, size_t es) {
       const int64_t K = H.hlevel_sn[i], s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
       f += (s * s + 1) / 2 + (c + cu) * s + c * cu;
       if (c > 0 && cu > 0)  // A_{C,K}, A_{K,C}^T, Uinv, Linv (the solves; then TL, TU)
-        oz += parts * (slice_bytes(c, s, 6) + slice_bytes(cu, s, 6) + 2 * slice_bytes(s, s, 6)) +
+        oz += parts * (slice_bytes(c, s, 8) + slice_bytes(cu, s, 8) + 2 * slice_bytes(s, s, 8)) +
               exps_bytes(c) + exps_bytes(cu) + 2 * exps_bytes(s) + 2048 +
               (size_t)(c + cu + 2 * s) * 8;
     }
@@ -627,9 +627,9 @@ struct SchurProduct {
   const char *AL, *AU, *Uinv, *Linv;
 };
 void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
-                    size_t base);
+                    size_t base, bool eight);
 void add_ozaki_schur(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
-                     size_t base, bool lower);
+                     size_t base, bool lower, bool eight);
 
 // tile of the diagonal blocks' small products: 16 x 16 while 32 x 32 tiles
 // would leave SMs without a CTA (a 32 x 32 x 32 product takes an SM's FP64
@@ -750,6 +750,8 @@ void add_inverse_merges(pselinv_ctx* h, Plan& P, const std::vector<SnTask>& wide
   }
 }
 
+constexpr double kEightMinFlops = 2e8;
+
 int build_factor_plan(pselinv_ctx* h) {
   const HostSym& H = h->H;
   Plan& P = h->factor_plan;
@@ -785,16 +787,22 @@ int build_factor_plan(pselinv_ctx* h) {
     // split precision: the triangular solves and the Schur products of levels
     // with enough Schur work as sliced tensor-core products (their operands
     // sliced from the level's scratch after its FP64 region)
-    double sflops = 0;
+    double sflops = 0, fp64 = 0;  // Schur flops; FP64 operations of the level's products
     for (int64_t i = l0; i < l1; i++) {
       const int64_t K = H.hlevel_sn[i];
-      sflops += 2.0 * (double)cK(H, K) * (double)cU(H, K) * (double)H.sn_width[K] * (double)nb;
+      const double c = (double)cK(H, K), cu = (double)cU(H, K), s = (double)H.sn_width[K];
+      sflops += 2.0 * c * cu * s * (double)nb;
+      fp64 += (2.0 * c * cu * s + (c + cu) * s * s) * (double)nb * (dt == DT_F64 ? 1.0 : 4.0) *
+              (ldlt ? 0.5 : 1.0);
     }
     const double min_flops = h->opts.factor_split_mflops < 0    ? 0.0
                              : h->opts.factor_split_mflops == 0 ? 2e8
                                                                 : 1e6 * h->opts.factor_split_mflops;
-    const bool split = h->opts.factor_precision == PSELINV_PREC_OZAKI_FP16 && sflops > 0 &&
-                       sflops >= min_flops;
+    const bool ozaki = h->opts.factor_precision == PSELINV_PREC_OZAKI_FP16 && sflops > 0;
+    // smaller levels keep FP64 accuracy, as products of eight slices where the
+    // FP64 pipe would take longer than their four launches (200 MFLOP: 160 us)
+    const bool eight = ozaki && sflops < min_flops && fp64 >= kEightMinFlops;
+    const bool split = (ozaki && sflops >= min_flops) || eight;
     int64_t off = 0;  // scalars into scratch
     int64_t smax = 0;
     std::vector<int64_t> mofs;  // scratch of the wide supernodes' inverse merges
@@ -896,8 +904,8 @@ int build_factor_plan(pselinv_ctx* h) {
     add_gemm_step(P, dt, choose_small_tile(dt, trsm) == GEMM_16x16 ? GEMM_16x16 : GEMM_ROWS, trsm,
                   (int)lev);
     if (split) {
-      add_ozaki_trsm(h, P, solves, (int)lev, align256((size_t)off * es));
-      add_ozaki_schur(h, P, sprods, (int)lev, align256((size_t)off * es), ldlt);
+      add_ozaki_trsm(h, P, solves, (int)lev, align256((size_t)off * es), eight);
+      add_ozaki_schur(h, P, sprods, (int)lev, align256((size_t)off * es), ldlt, eight);
     } else {
       add_schur_scatter(h, P, schur, (int)lev, ldlt);
     }
@@ -1173,6 +1181,7 @@ struct OzBuilder {
     d.B = b.out; d.eB = b.exps; d.B_R64 = b.R64;
     d.C = (double*)C; d.ldc = ldc; d.M = M; d.N = N;
     d.K32 = a.K32;
+    d.tri = b.tri;
     d.cscale = cplx ? 2 : 1;
     if (!cplx) {
       out.push_back(d);
@@ -1189,21 +1198,56 @@ struct OzBuilder {
   }
 };
 
+// Products of eight slices (see gemm8_kernel), longest K ranges first;
+// lower_c: the tiles of C on or below its diagonal only
+void add_gemm8_step(Plan& P, const std::vector<OzDesc>& prods, int lev, bool lower_c) {
+  std::vector<OzTask> tasks;
+  double flops = 0, bytes = 0;
+  for (size_t d = 0; d < prods.size(); d++) {
+    const OzDesc& g = prods[d];
+    for (int tm = 0; tm < ceil_div(g.M, 128); tm++)
+      for (int tn = 0; tn < ceil_div(g.N, 64); tn++)
+        if (!lower_c || (tm + 1) * 128 > tn * 64) tasks.push_back({(int)d, tm, tn, 0});
+    const double half = g.tri || lower_c ? 0.5 : 1.0;
+    flops += 2.0 * half * g.M * g.N * (double)g.K32 * 32;
+    bytes += 2.0 * kSlices8 * ((double)g.M + g.N) * g.K32 * 32 + 8.0 * g.M * g.N;
+  }
+  if (tasks.empty()) return;
+  auto blocks = [&](const OzTask& t) {
+    const OzDesc& g = prods[t.d];
+    const int part = g.half ? g.half : g.K32;
+    return (g.tri == 1 ? part - 2 * t.tn : g.tri == 2 ? std::min(part, 2 * t.tn + 2) : part) *
+           (g.half ? 2 : 1);
+  };
+  std::stable_sort(tasks.begin(), tasks.end(),
+                   [&](const OzTask& x, const OzTask& y) { return blocks(x) > blocks(y); });
+  Step m;
+  m.kind = ST_GEMM8;
+  m.n = (int)tasks.size();
+  m.descs = P.push(prods);
+  m.tasks = P.push(tasks);
+  m.flops = flops;
+  m.bytes = (size_t)bytes;
+  m.level = lev;
+  P.steps.push_back(m);
+}
+
 // Triangular solves of one factorisation level as sliced products (K = s):
 // TL = AL Uinv (B(n, k) = Uinv(k, n)) and TU = AU Linv^T (B(n, k) =
 // Linv(n, k)); Uinv and Linv hold exact zeros outside their triangles, so
 // the full products are the triangular ones.  For symmetric values AU is AL
 // and its slices serve both products.  Scratch from `base`.
 void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
-                    size_t base) {
+                    size_t base, bool eight) {
   if (prods.empty()) return;
-  OzBuilder ob(h, base);
+  OzBuilder ob(h, base, eight ? kSlices8 : 0);
   std::vector<SliceDesc> sl;
   std::vector<OzDesc> out;
   for (const SchurProduct& q : prods) {
     const SliceDesc al = ob.slice(q.AL, q.c, SLICE_ROWS, q.c, q.s);
-    const SliceDesc ub = ob.slice(q.Uinv, q.s, SLICE_COLS, q.s, q.s);
-    const SliceDesc lb = ob.slice(q.Linv, q.s, SLICE_ROWS, q.s, q.s);
+    SliceDesc ub = ob.slice(q.Uinv, q.s, SLICE_COLS, q.s, q.s);
+    SliceDesc lb = ob.slice(q.Linv, q.s, SLICE_ROWS, q.s, q.s);
+    if (eight) ub.tri = lb.tri = 2;
     SliceDesc au = al;
     if (q.AU != q.AL) {
       au = ob.slice(q.AU, q.cu, SLICE_ROWS, q.cu, q.s);
@@ -1216,7 +1260,10 @@ void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& pr
     ob.product(out, au, lb, q.TU, q.cu, q.cu, q.s, 1.0);
   }
   add_panel_slice_step(P, sl, lev);
-  add_ozgemm_step(P, out, h->slices, lev, false, 1, 0);
+  if (eight)
+    add_gemm8_step(P, out, lev, false);
+  else
+    add_ozgemm_step(P, out, h->slices, lev, false, 1, 0);
 }
 
 // Schur products of one factorisation level as sliced products: slices of TL
@@ -1224,8 +1271,8 @@ void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& pr
 // FP64 Sc blocks the scatter subtracts.  Scratch from
 // `base` (bytes), after the level's FP64 region.
 void add_ozaki_schur(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
-                     size_t base, bool lower) {
-  OzBuilder ob(h, base);
+                     size_t base, bool lower, bool eight) {
+  OzBuilder ob(h, base, eight ? kSlices8 : 0);
   std::vector<SliceDesc> sl;
   std::vector<OzDesc> out;
   for (const SchurProduct& q : prods) {
@@ -1236,8 +1283,11 @@ void add_ozaki_schur(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& p
     ob.product(out, a, b, q.Sc, q.c, q.c, q.cu, 1.0);
   }
   add_panel_slice_step(P, sl, lev);
-  // K = s <= 256 is one exact chunk: no K split, no accumulation
-  add_ozgemm_step(P, out, h->slices, lev, false, 1, 0, lower);
+  // K = s <= 256 is one exact chunk of six slices: no K split, no accumulation
+  if (eight)
+    add_gemm8_step(P, out, lev, lower);
+  else
+    add_ozgemm_step(P, out, h->slices, lev, false, 1, 0, lower);
 }
 
 // Split-precision normalisation of one depth level (Algorithm 1 step 2 and
@@ -1305,7 +1355,7 @@ void add_ozaki_normalize(pselinv_ctx* h, Plan& P, int lev, int64_t nb, size_t ba
 }
 
 // The normalisation of the supernodes {instance, K} of a split level as
-// eight-slice products (K = s; FP64 accuracy, see norm_gemm_kernel): the
+// eight-slice products (K = s; FP64 accuracy, see gemm8_kernel): the
 // panels and the triangular inverses sliced in one launch, then Lhat = L Linv
 // and Uhat^T = U^T Uinv^T in another.  Scratch from `base`.
 void add_sliced_normalize(pselinv_ctx* h, Plan& P, const std::vector<std::pair<int64_t, int64_t>>& sns,
@@ -1313,7 +1363,7 @@ void add_sliced_normalize(pselinv_ctx* h, Plan& P, const std::vector<std::pair<i
   if (sns.empty()) return;
   const HostSym& H = h->H;
   const size_t es = h->esize;
-  OzBuilder ob(h, base, kNormSlices);
+  OzBuilder ob(h, base, kSlices8);
   std::vector<SliceDesc> sl;
   std::vector<OzDesc> prods;
   for (const auto& bk : sns) {
@@ -1340,29 +1390,8 @@ void add_sliced_normalize(pselinv_ctx* h, Plan& P, const std::vector<std::pair<i
       ob.product(prods, ua, ub, h->nf + uo, cu, cu, s, 1.0);
     }
   }
-  if (prods.empty()) return;
   add_panel_slice_step(P, sl, lev);
-  std::vector<OzTask> tasks;
-  double flops = 0, bytes = 0;
-  for (size_t d = 0; d < prods.size(); d++) {
-    const OzDesc& g = prods[d];
-    for (int tm = 0; tm < ceil_div(g.M, 128); tm++)  // longest K range first
-      for (int tn = 0; tn < ceil_div(g.N, 64); tn++) tasks.push_back({(int)d, tm, tn, 0});
-    flops += (double)g.M * g.N * (g.N + 1) * g.cscale;
-    bytes += 2.0 * kNormSlices * ((double)g.M + g.N / 2.0) * g.K32 * 32 + 8.0 * g.M * g.N;
-  }
-  std::stable_sort(tasks.begin(), tasks.end(), [&](const OzTask& x, const OzTask& y) {
-    return prods[x.d].K32 - 2 * x.tn > prods[y.d].K32 - 2 * y.tn;
-  });
-  Step m;
-  m.kind = ST_NORM_GEMM;
-  m.n = (int)tasks.size();
-  m.descs = P.push(prods);
-  m.tasks = P.push(tasks);
-  m.flops = flops;
-  m.bytes = (size_t)bytes;
-  m.level = lev;
-  P.steps.push_back(m);
+  add_gemm8_step(P, prods, lev, false);
 }
 
 // Merge the finished blocks of the supernodes `sns` (diagonal block, L and
@@ -1872,8 +1901,8 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
       launch_panel_slice((const SliceDesc*)(a + s.descs), (const SliceTask*)(a + s.tasks), s.n, s.cfg,
                         st);
       break;
-    case ST_NORM_GEMM:
-      launch_norm_gemm((const OzDesc*)(a + s.descs), (const OzTask*)(a + s.tasks), s.n, h->derr, st);
+    case ST_GEMM8:
+      launch_gemm8((const OzDesc*)(a + s.descs), (const OzTask*)(a + s.tasks), s.n, h->derr, st);
       break;
     case ST_UNPACK_PIVOTS:
       launch_unpack_pivots(h->dtype, h->S, h->lu, h->piv, (int)h->nbatch, st);

@@ -224,7 +224,7 @@ enum SliceMode { SLICE_ROWS = 0, SLICE_COLS = 1 };
 struct SliceDesc {
   const double* src;
   int ld, mode, R, Kd, S, R64, K32, cplx;
-  int tri;  // X(r, k) = 0 for k < r (the normalisation's triangular operands)
+  int tri;  // 1: X(r, k) = 0 for k < r, 2: for k > r (gemm8's triangular operands), else 0
   __half* out;
   int* exps;
   unsigned long long* maxbits;  // max_k |X(r,k)| as bit patterns (from the gather or a maxima pass)
@@ -246,6 +246,7 @@ struct OzDesc {
   double* C;
   int A_R64, B_R64, K32, M, N, ldc, ksplit, atomic;
   int half, swap_b, neg_half, cscale, coff;
+  int tri;  // gemm8: op(B)(k, n) = 0 for k < n (1) or k > n (2)
   double alpha;
 };
 struct OzTask {
@@ -292,12 +293,11 @@ void launch_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, bo
 void launch_ozaki_gemm(int S, const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
                        bool persistent, bool a_tmem, cudaStream_t st);
 // Slices of operands with K <= 256 with their own row maxima (desc.maxbits
-// unused), `span` K blocks per task {d, row block, first K block}; and the
-// normalisation's products at eight slices (K <= 256; op(B) lower
-// triangular): C = A op(B), tasks {d, tm, tn, 0}
+// unused), `span` K blocks per task {d, row block, first K block}; and
+// products of eight slices, C = A op(B), tasks {d, tm, tn, 0}
 void launch_panel_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, int span,
                        cudaStream_t st);
-void launch_norm_gemm(const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
+void launch_gemm8(const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
                       cudaStream_t st);
 void launch_zero(const CopySeg* segs, int nseg, int per_seg, cudaStream_t st);
 // a kernel whose only wait never completes: it gives up after budget_ns and

@@ -252,8 +252,9 @@ __device__ __forceinline__ void write_digits8(const double (&x)[8], int e, __hal
 // factorisation's): a task is a 64-row block and `span` K blocks from kc;
 // every task finds its rows' maxima itself over the whole K (a row is read by
 // four lanes of one warp, and comes from L1 / L2 the second time), so no maxima
-// pass, no zeroed buffer and one launch instead of three.  d.tri: X(r, k) = 0
-// for k < r, and nobody reads the K blocks left of the row block's diagonal.
+// pass, no zeroed buffer and one launch instead of three.  d.tri = 1 / 2:
+// X(r, k) = 0 for k < r / k > r, and nobody reads the K blocks left / right of
+// the row block's diagonal.
 __global__ void __launch_bounds__(kSliceThreads)
 panel_slice_kernel(const SliceDesc* __restrict__ descs, const SliceTask* __restrict__ tasks,
                   int ntasks, int span) {
@@ -278,7 +279,8 @@ panel_slice_kernel(const SliceDesc* __restrict__ descs, const SliceTask* __restr
     const int half = d.cplx ? d.K32 / 2 : d.K32;
     const int kb1 = min(d.K32, task.kc + span);
     for (int kb = task.kc; kb < kb1; kb++) {
-      if (d.tri && (kb >= half ? kb - half : kb) < 2 * task.rb) continue;
+      const int kp = kb >= half ? kb - half : kb;
+      if ((d.tri == 1 && kp < 2 * task.rb) || (d.tri == 2 && kp > 2 * task.rb + 1)) continue;
       double x[8];
       load8(d, r, kb * 32 + kg * 8, x);
       __half* out = d.out + ((int64_t)task.rb * d.K32 + kb) * (kTileBytes / 2) + tid * 8;
@@ -1054,9 +1056,12 @@ constexpr int gemm_smem() {
 }
 
 // ---------------------------------------------------------------------------
-// The normalisation Lhat = L L_KK^{-1}, Uhat^T = U^T U_KK^{-T} as products of
-// eight base-256 slices: 63 bits below each row's and column's power of two
-// and the 36 slice pairs with s + t <= 7, so an output is off by some 2^-60 of
+// Products with K = s <= 256 at FP64 accuracy: the normalisation Lhat = L
+// L_KK^{-1}, Uhat^T = U^T U_KK^{-T} of split levels, and the panel solves and
+// Schur products of the split factorisation's levels that are too small for
+// opts.slices slices.  Eight base-256 slices: 63 bits below each row's and
+// column's power of two and the 36 slice pairs with s + t <= 7, so an output
+// is off by some 2^-60 of
 // its row's and column's largest products.  Against correctly rounded exact
 // products of panels of 3D, 2D and DG matrices (s = 128) the relative error in
 // norm is 2e-18 to 2e-17; an FP64 sum's is 1.5e-16 to 2.8e-16.  (Base 128, 56
@@ -1065,24 +1070,24 @@ constexpr int gemm_smem() {
 // K = s <= 256 (real and imaginary parts: 2 x 256).  A chunk of 4 K blocks adds
 // at most 128 x 8 x 2^14 = 2^24 to an accumulator, exact; its 8 x 64
 // accumulators take all of tensor memory, and its sum goes straight to the
-// output, rounded once; later chunks are added in FP64.  op(B)(k, n) = 0 for k
-// < n: K blocks left of a column tile's diagonal are skipped.
+// output, rounded once; later chunks are added in FP64.  A triangular op(B)
+// (d.tri) skips the K blocks beyond a column tile's diagonal.
 // Roles and ring as in ozaki_gemm_kernel (two stages of 96 KB).  The FP64
 // pipe needs c s^2 multiply-adds at 2 per cycle and SM for what is here 20
 // MMAs per 128 x 64 x 16.
 // ---------------------------------------------------------------------------
-constexpr int kNormS = 8;
-constexpr int kNormChunk = 4;  // K blocks per exact chunk
-constexpr int kNormStage = kNormS * 3 * kTileBytes;
-constexpr int kNormStages = 2;
+constexpr int k8Slices = 8;
+constexpr int k8Chunk = 4;  // K blocks per exact chunk
+constexpr int k8Stage = k8Slices * 3 * kTileBytes;
+constexpr int k8Stages = 2;
 
 // K blocks of a task: sequence position i -> K block
-struct NormRange {
+struct Range8 {
   int k0, n1, n;  // first block of a part, blocks per part, blocks in all
-  __device__ __forceinline__ NormRange(const OzDesc* d, int tn) {
+  __device__ __forceinline__ Range8(const OzDesc* d, int tn) {
     const int part = d->half ? d->half : d->K32;
-    k0 = 2 * tn;
-    n1 = part - k0;
+    k0 = d->tri == 1 ? 2 * tn : 0;
+    n1 = (d->tri == 2 ? min(part, 2 * tn + 2) : part) - k0;
     n = d->half ? 2 * n1 : n1;
   }
   __device__ __forceinline__ int block(int i, int half) const {
@@ -1091,19 +1096,19 @@ struct NormRange {
 };
 
 __global__ void __launch_bounds__(kOzThreads, 1)
-norm_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ tasks, int ntasks,
+gemm8_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ tasks, int ntasks,
                  int* err) {
-  constexpr int S = kNormS;
+  constexpr int S = k8Slices;
   constexpr int kAB = S * 2 * kTileBytes;
   constexpr uint32_t kTmemCols = 512;
   extern __shared__ __align__(1024) unsigned char smem[];
-  __shared__ __align__(8) uint64_t bar_full[kNormStages], bar_free[kNormStages], bar_acc_full,
+  __shared__ __align__(8) uint64_t bar_full[k8Stages], bar_free[k8Stages], bar_acc_full,
       bar_acc_empty;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
-    for (int i = 0; i < kNormStages; i++) {
+    for (int i = 0; i < k8Stages; i++) {
       mbar_init(smem_u32(&bar_full[i]), 1);
       mbar_init(smem_u32(&bar_free[i]), 1);
     }
@@ -1132,7 +1137,7 @@ norm_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ ta
         const OzTask task = tasks[t];
         const OzDesc* dp = descs + task.d;
         const int K32 = dp->K32, half = dp->half, swap_b = dp->swap_b;
-        const NormRange kr(dp, task.tn);
+        const Range8 kr(dp, task.tn);
         const bool a_second = 2 * task.tm + 1 < dp->A_R64;
         const uint32_t bytes = (uint32_t)(S * (a_second ? 3 : 2) * kTileBytes);
         const int64_t a_sl = (int64_t)dp->A_R64 * K32 * kTileBytes;
@@ -1140,13 +1145,13 @@ norm_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ ta
         const unsigned char* A = reinterpret_cast<const unsigned char*>(dp->A);
         const unsigned char* B = reinterpret_cast<const unsigned char*>(dp->B);
         for (int i = 0; i < kr.n; i++, g++) {
-          const int stg = (int)(g % kNormStages);
-          const uint32_t u = g / kNormStages;
+          const int stg = (int)(g % k8Stages);
+          const uint32_t u = g / k8Stages;
           if ((u > 0 && !mbar_wait(smem_u32(&bar_free[stg]), (u - 1) & 1)) || abort_flag) {
             ok = false;
             break;
           }
-          unsigned char* st = smem + stg * kNormStage;
+          unsigned char* st = smem + stg * k8Stage;
           const uint32_t fb = smem_u32(&bar_full[stg]);
           mbar_expect_tx(fb, bytes);
           const int kb = kr.block(i, half);
@@ -1165,8 +1170,8 @@ norm_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ ta
       if (!ok) {
         abort_flag = 1;
         // let the copies already issued land before the CTA exits (bounded)
-        for (uint32_t k = g > (uint32_t)kNormStages ? g - kNormStages : 0u; k < g; k++)
-          mbar_wait(smem_u32(&bar_full[k % kNormStages]), (k / kNormStages) & 1);
+        for (uint32_t k = g > (uint32_t)k8Stages ? g - k8Stages : 0u; k < g; k++)
+          mbar_wait(smem_u32(&bar_full[k % k8Stages]), (k / k8Stages) & 1);
       }
     }
   } else if (warp == kOzDrainWarps + 1) {
@@ -1177,21 +1182,21 @@ norm_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ ta
         const OzTask task = tasks[t];
         const OzDesc* dp = descs + task.d;
         const int half = dp->half, neg_half = dp->neg_half;
-        const NormRange kr(dp, task.tn);
+        const Range8 kr(dp, task.tn);
         for (int i = 0; i < kr.n; i++, g++) {
-          const int stg = (int)(g % kNormStages);
-          const bool first = i % kNormChunk == 0;
-          const bool last = i % kNormChunk == kNormChunk - 1 || i == kr.n - 1;
+          const int stg = (int)(g % k8Stages);
+          const bool first = i % k8Chunk == 0;
+          const bool last = i % k8Chunk == k8Chunk - 1 || i == kr.n - 1;
           if (first && q > 0 && !mbar_wait(smem_u32(&bar_acc_empty), (q - 1) & 1)) {
             ok = false;
             break;
           }
-          if (!mbar_wait(smem_u32(&bar_full[stg]), (g / kNormStages) & 1) || abort_flag) {
+          if (!mbar_wait(smem_u32(&bar_full[stg]), (g / k8Stages) & 1) || abort_flag) {
             ok = false;
             break;
           }
           fence_after();
-          const uint32_t st = smem_u32(smem + stg * kNormStage);
+          const uint32_t st = smem_u32(smem + stg * k8Stage);
           const bool neg_a = neg_half && kr.block(i, half) >= half;
           const uint32_t idesc = neg_a ? kIdescNegA : kIdesc;
           const uint32_t idesc2 = neg_a ? kIdescN128NegA : kIdescN128;
@@ -1217,7 +1222,7 @@ norm_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ ta
       if (!ok) {
         abort_flag = 1;
         if (g > 0)
-          mbar_wait(smem_u32(&bar_free[(g - 1) % kNormStages]), ((g - 1) / kNormStages) & 1);
+          mbar_wait(smem_u32(&bar_free[(g - 1) % k8Stages]), ((g - 1) / k8Stages) & 1);
       }
     }
   } else {
@@ -1228,11 +1233,11 @@ norm_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ ta
     for (int t = blockIdx.x; t < ntasks && ok; t += gridDim.x) {
       const OzTask task = tasks[t];
       const OzDesc* dp = descs + task.d;
-      const NormRange kr(dp, task.tn);
+      const Range8 kr(dp, task.tn);
       const int dM = dp->M, dN = dp->N, ldc = dp->ldc, cscale = dp->cscale, coff = dp->coff;
       const int* __restrict__ eB = dp->eB;
       double* __restrict__ Cp = dp->C;
-      const int nchunks = (kr.n + kNormChunk - 1) / kNormChunk;
+      const int nchunks = (kr.n + k8Chunk - 1) / k8Chunk;
       const int r = task.tm * 128 + quarter * 32 + lane;
       const int nb = task.tn * 64 + hcol * 32;
       const int ea = r < dM ? dp->eA[r] : 0;
@@ -1340,8 +1345,8 @@ cudaError_t prepare_ozaki_kernels() {
   PSELINV_OZ_ATTR(5, true)
   PSELINV_OZ_ATTR(6, true)
 #undef PSELINV_OZ_ATTR
-  return cudaFuncSetAttribute(norm_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kNormStages * kNormStage);
+  return cudaFuncSetAttribute(gemm8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              k8Stages * k8Stage);
 }
 
 void launch_panel_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, int span,
@@ -1351,12 +1356,12 @@ void launch_panel_slice(const SliceDesc* descs, const SliceTask* tasks, int ntas
   panel_slice_kernel<<<grid, kSliceThreads, 0, st>>>(descs, tasks, ntasks, span);
 }
 
-void launch_norm_gemm(const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
+void launch_gemm8(const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
                       cudaStream_t st) {
   if (ntasks <= 0) return;
   // one task per CTA (one CTA fits an SM): the launch runs beside the sweep's
   // own, whose CTAs take the SMs that finish
-  norm_gemm_kernel<<<ntasks, kOzThreads, kNormStages * kNormStage, st>>>(descs, tasks, ntasks, err);
+  gemm8_kernel<<<ntasks, kOzThreads, k8Stages * k8Stage, st>>>(descs, tasks, ntasks, err);
 }
 
 void launch_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, bool maxima,

@@ -108,3 +108,27 @@ def test_general_schur(torch, density, max_sn):
     ref = oracle.gextract(oracle.general_selected_inverse(p), p.colptr, p.rowind)
     assert np.abs(got - ref).max() < 1e-10 * np.abs(ref).max()
     h.close()
+
+
+@pytest.mark.parametrize("kind,nb", [("real", 40), ("complex", 12), ("symmetric", 80)])
+@pytest.mark.parametrize("s", [30, 96])
+def test_eight_slice_levels(torch, kind, nb, s):
+    """Split factorisation, levels below its threshold of Schur work but with
+    more FP64 work than a few launches: products of eight slices, held to the
+    FP64 tolerance."""
+    import paper_1708_04539_gb300 as ps
+    n = s + 133
+    nb = nb * (5 if s == 30 else 1)
+    ii, jj = np.meshgrid(np.arange(n), np.arange(n), indexing="ij")
+    p = gen.problems._finish_small(n, ii.reshape(-1), jj.reshape(-1), 995, kind == "complex",
+                                   f"dense_{n}", s, symmetric_values=kind == "symmetric")
+    p.values = np.ascontiguousarray(p.values[None, :] * np.linspace(0.5, 2.0, nb)[:, None])
+    h = ps.SelInv.from_problem(p, symmetric=kind == "symmetric",
+                               factor_precision=ps.PREC_OZAKI_FP16, factor_split_mflops=100000)
+    h.factor(torch.from_numpy(p.values).cuda())
+    h.selinv()
+    assert any(r["kind"] == "ozaki_gemm" for r in h.profile(1))
+    h.factor(torch.from_numpy(p.values).cuda())
+    h.selinv()
+    check(p, h, [0, nb - 1])
+    h.close()
