@@ -709,48 +709,53 @@ void add_schur_scatter(pselinv_ctx* h, Plan& P, const std::vector<SchurDesc>& de
   P.steps.push_back(st);
 }
 
-// The triangular inverses of the wide supernodes from those of their 32 x 32
-// pivot blocks (written by the panel steps), doubling the block size b: for
-// neighbouring blocks 1, 2 of one triangle
-//   (L^{-1})_21 = -(L_22)^{-1} (L_21 (L_11)^{-1}),
-//   (U^{-1})_12 = -(U_11)^{-1} (U_12 (U_22)^{-1}),
-// two launches per doubling for both triangles of every supernode.
-// mofs: scratch offset (s^2 / 2 scalars) of each one's inner products.
-void add_inverse_merges(pselinv_ctx* h, Plan& P, const std::vector<SnTask>& wide,
-                        const std::vector<int64_t>& mofs, int level) {
+// The triangular inverses of the wide supernodes, one block row of L^{-1} and
+// one block column of U^{-1} behind each panel p (32 columns):
+//   TL = L[p, 0:p] L^{-1}[0:p, 0:p],   L^{-1}[p, 0:p] = -(L_pp)^{-1} TL,
+//   TU = U^{-1}[0:p, 0:p] U[0:p, p],   U^{-1}[0:p, p] = -TU (U_pp)^{-1};
+// the diagonal blocks' inverses come from the panel launches.  All of it runs
+// on the side stream beside the next panels (TL and TU of panel p need panels
+// < p only), so that after the last panel one launch of K = 32 products
+// remains; merging doubled blocks after the LU instead took 72 us of a 256
+// wide level's 340.
+// inner: the products TL, TU of panel p (once block row p - 1 is there), else
+// the second ones.  mofs: scratch offset (s^2 / 2 scalars) of each supernode.
+void add_inverse_row(pselinv_ctx* h, Plan& P, const std::vector<SnTask>& wide,
+                     const std::vector<int64_t>& mofs, int64_t p, bool inner, int level) {
   const HostSym& H = h->H;
   const size_t es = h->esize;
-  for (int64_t b = kLuPanel; b < 256; b *= 2) {
-    std::vector<GemmDesc> inner, outer;
-    for (size_t t = 0; t < wide.size(); t++) {
-      const int64_t K = wide[t].K, s = H.sn_width[K];
-      const char* D = h->lu + ((size_t)wide[t].inst * H.storage + H.sn_offset[K]) * es;
-      char* Linv = h->winv + (size_t)(wide[t].inst * h->w_stride + h->w_off[K]) * es;
-      char* Uinv = Linv + (size_t)s * s * es;
-      char* T = h->scratch + (size_t)mofs[t] * es;
-      auto at = [&](auto* M, int64_t i, int64_t j) { return M + (size_t)(i + j * s) * es; };
-      for (int64_t i0 = 0; i0 + b < s; i0 += 2 * b) {
-        const int64_t i1 = i0 + b;
-        const int n1 = (int)b, n2 = (int)std::min<int64_t>(b, s - i1), ld = (int)s;
-        char* TU = T + (size_t)(n1 * n2) * es;
-        inner.push_back(make_desc(at(D, i1, i0), at(Linv, i0, i0), T, n2, n1, n1, ld, ld, n2, 0, 0,
-                                  1.0, 0.0, 0, 1, GEMM_TRI_LOWER_B));
-        outer.push_back(make_desc(at(Linv, i1, i1), T, at(Linv, i1, i0), n2, n1, n2, ld, n2, ld, 0,
-                                  0, -1.0, 0.0, 0, 1, GEMM_TRI_LOWER_A));
-        inner.push_back(make_desc(at(D, i0, i1), at(Uinv, i1, i1), TU, n1, n2, n2, ld, ld, n1, 0, 0,
-                                  1.0, 0.0, 0, 1, GEMM_TRI_UPPER_B));
-        outer.push_back(make_desc(at(Uinv, i0, i0), TU, at(Uinv, i0, i1), n1, n2, n1, ld, n1, ld, 0,
-                                  0, -1.0, 0.0, 0, 1, GEMM_TRI_UPPER_A));
-        T = TU + (size_t)(n1 * n2) * es;
-      }
+  std::vector<GemmDesc> prods;
+  for (size_t t = 0; t < wide.size(); t++) {
+    const int64_t K = wide[t].K, s = H.sn_width[K], i = p * kLuPanel;
+    if (i >= s) continue;
+    const char* D = h->lu + ((size_t)wide[t].inst * H.storage + H.sn_offset[K]) * es;
+    char* Linv = h->winv + (size_t)(wide[t].inst * h->w_stride + h->w_off[K]) * es;
+    char* Uinv = Linv + (size_t)s * s * es;
+    const int n = (int)i, w = (int)std::min<int64_t>(kLuPanel, s - i), ld = (int)s;
+    char* TL = h->scratch + (size_t)mofs[t] * es;
+    char* TU = TL + (size_t)(n * w) * es;
+    auto at = [&](auto* M, int64_t r, int64_t c) { return M + (size_t)(r + c * s) * es; };
+    if (inner) {
+      prods.push_back(make_desc(at(D, i, 0), Linv, TL, w, n, n, ld, ld, w, 0, 0, 1.0, 0.0, 0, 1,
+                                GEMM_TRI_LOWER_B));
+      prods.push_back(make_desc(Uinv, at(D, 0, i), TU, n, w, n, ld, ld, n, 0, 0, 1.0, 0.0, 0, 1,
+                                GEMM_TRI_UPPER_A));
+    } else {
+      prods.push_back(make_desc(at(Linv, i, i), TL, at(Linv, i, 0), w, n, w, ld, w, ld, 0, 0, -1.0,
+                                0.0, 0, 1, GEMM_TRI_LOWER_A));
+      prods.push_back(make_desc(TU, at(Uinv, i, i), at(Uinv, 0, i), n, w, w, n, ld, ld, 0, 0, -1.0,
+                                0.0, 0, 1, GEMM_TRI_UPPER_B));
     }
-    if (inner.empty()) break;
-    add_gemm_step(P, h->dtype, choose_small_tile(h->dtype, inner), inner, level);
-    add_gemm_step(P, h->dtype, choose_small_tile(h->dtype, outer), outer, level);
   }
+  const size_t first = P.steps.size();
+  add_gemm_step(P, h->dtype, choose_small_tile(h->dtype, prods), prods, level);
+  for (size_t k = first; k < P.steps.size(); k++) P.steps[k].side = 1;
 }
 
 constexpr double kEightMinFlops = 2e8;
+// events of a height level of the factorisation: one per panel (8 of 32
+// columns at most), one for its inverses
+constexpr int kPanelEvents = 9;
 
 int build_factor_plan(pselinv_ctx* h) {
   const HostSym& H = h->H;
@@ -774,6 +779,17 @@ int build_factor_plan(pselinv_ctx* h) {
   // work) and U^T panels are solved from the L panels; each diagonal block's
   // upper triangle is mirrored from its lower one before its LU
   const bool ldlt = h->opts.symmetric != 0 && !H.general;
+  // the next step of the main stream after the level's last panel waits for
+  // its inverses (the solves read them, and the scratch of their products is
+  // free again then)
+  int inverse_ready = -1;
+  auto wait_inverse = [&](size_t from) {
+    for (size_t i = from; i < P.steps.size() && inverse_ready >= 0; i++)
+      if (P.steps[i].side == 0) {
+        P.steps[i].wait = inverse_ready;
+        inverse_ready = -1;
+      }
+  };
   for (size_t lev = 0; lev + 1 < H.hlevel_ptr.size(); lev++) {
     std::vector<SnTask> wide, gt;  // wide: more than one panel
     std::vector<SnTask> mirrored;  // symmetric values: blocks whose upper triangle is filled in
@@ -878,6 +894,7 @@ int build_factor_plan(pselinv_ctx* h) {
     // blocked LU of the diagonal blocks: per panel of 32 columns one panel
     // launch and (wide supernodes) one trailing-update GEMM, batched over the
     // level's supernodes; a narrow supernode is done after its panel
+    size_t at = P.steps.size();
     for (int64_t j0 = 0; j0 < smax; j0 += kLuPanel) {
       std::vector<GemmDesc> upd;
       if (j0 > 0) panels.clear();
@@ -896,9 +913,25 @@ int build_factor_plan(pselinv_ctx* h) {
         }
       }
       add_panel_step(P, panels, (int)lev, !split);
+      wait_inverse(at);
+      at = P.steps.size();
+      if (!wide.empty()) {  // side stream: block row p of the inverses, inner products of p + 1
+        const int64_t p = j0 / kLuPanel;
+        const int ev = EV_LEVEL + (int)lev * kPanelEvents + (int)p;
+        P.steps.back().signal = ev;
+        if (p > 0) add_inverse_row(h, P, wide, mofs, p, false, (int)lev);
+        const size_t last_row = P.steps.size();
+        add_inverse_row(h, P, wide, mofs, p + 1, true, (int)lev);
+        if (P.steps.size() > at) P.steps[at].wait = ev;
+        if (j0 + kLuPanel >= smax && last_row > at) {  // the last block row
+          inverse_ready = EV_LEVEL + (int)lev * kPanelEvents + kPanelEvents - 1;
+          P.steps[last_row - 1].signal = inverse_ready;
+        }
+        at = P.steps.size();
+      }
       add_gemm_step(P, dt, choose_small_tile(dt, upd), upd, (int)lev);
     }
-    add_inverse_merges(h, P, wide, mofs, (int)lev);
+    at = P.steps.size();
     // few solves: small tiles (a row panel's 8 columns per thread are a chain of
     // 8 s multiply-adds, 65 us for s = 64 complex; a 16 x 16 tile's 2 s)
     add_gemm_step(P, dt, choose_small_tile(dt, trsm) == GEMM_16x16 ? GEMM_16x16 : GEMM_ROWS, trsm,
@@ -920,13 +953,20 @@ int build_factor_plan(pselinv_ctx* h) {
       P.steps.push_back(sc);
     }
     add_copy_step(P, segs, (int)lev, es);
+    wait_inverse(at);
   }
+  const size_t at = P.steps.size();
   if (H.n > 0) {
     Step up;
     up.kind = ST_UNPACK_PIVOTS;
     up.n = (int)H.ns;
     P.steps.push_back(up);
   }
+  wait_inverse(at);
+  P.two_streams = true;
+  P.ev.assign(EV_LEVEL + (H.hlevel_ptr.empty() ? 0 : (H.hlevel_ptr.size() - 1) * kPanelEvents),
+              nullptr);
+  for (auto& e : P.ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   if (h->scratch_high > h->scratch_bytes) return PSELINV_ERR_CHECK;
   CK(cudaMalloc(&P.arena, P.host.size() + 256));
   CK(cudaMemcpy(P.arena, P.host.data(), P.host.size(), cudaMemcpyHostToDevice));
