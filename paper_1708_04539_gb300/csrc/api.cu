@@ -15,6 +15,7 @@
 #include <tuple>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <vector>
 
@@ -75,16 +76,16 @@ struct Step {
   double flops = 0;                       // useful flops of a GEMM step
   int level = -1;
   int slot = -1;      // tunable step: 0 normalisation, 1 steps 3+5, 2 step 4
-  int side = 0;       // 1: side stream (normalisation, one level ahead)
-  int wait = -1;      // event index waited on before the launch
-  int signal = -1;    // event index recorded after the launch
+  int side = 0;       // 1: side stream (normalisation, inverses), 2: bulk stream (Schur products)
+  int wait = -1, wait2 = -1;      // event indices waited on before the launch
+  int signal = -1, signal2 = -1;  // event indices recorded after the launch
   int param = 0;      // tuned parameter in use (GEMM tile config or K split)
   float feat[8] = {}; // shape features of the step (cost model input)
 };
 
 // events of a multi-stream plan
 enum PlanEvent {
-  EV_FORK = 0, EV_SIDE_JOIN = 1, EV_MAIN_JOIN = 2, EV_LEVEL = 3
+  EV_FORK = 0, EV_SIDE_JOIN = 1, EV_MAIN_JOIN = 2, EV_BULK_JOIN = 3, EV_LEVEL = 4
 };
 
 struct Plan {
@@ -165,7 +166,8 @@ struct pselinv_ctx {
   std::vector<pselinv_tune_record> records;
   cudaStream_t cap_stream = nullptr;
   cudaStream_t main_stream = nullptr;   // sweep launches (highest priority)
-  cudaStream_t side_stream = nullptr;   // normalisation one level ahead
+  cudaStream_t side_stream = nullptr;   // normalisation one level ahead; inverses
+  cudaStream_t bulk_stream = nullptr;   // Schur products off the critical path (lowest)
   int64_t last_info = -1;
   int last_status = 0;
   // supernodes the selected-inversion plan covers (empty = all): one
@@ -529,6 +531,22 @@ size_t maxima_bytes(const HostSym& H, int64_t nb) {
   return b;
 }
 
+// scalars (one instance) of the inner products of the largest height level's
+// inverses (add_inverse_row), in front of the levels' scratch: a level's LU
+// runs while the one below still uses its own
+int64_t inverse_scratch(const HostSym& H) {
+  int64_t mx = 0;
+  for (size_t d = 0; d + 1 < H.hlevel_ptr.size(); d++) {
+    int64_t t = 0;
+    for (int64_t i = H.hlevel_ptr[d]; i < H.hlevel_ptr[d + 1]; i++) {
+      const int64_t s = H.sn_width[H.hlevel_sn[i]];
+      if (s > kLuPanel) t += s * s / 2;
+    }
+    mx = std::max(mx, t);
+  }
+  return mx;
+}
+
 // scratch needed (bytes) by the factor and selected-inversion plans; the
 // split normalisation (side stream) has its own region after the sweep's,
 // the maxima theirs after that
@@ -537,12 +555,13 @@ size_t scratch_need(const HostSym& H, int64_t nb, size_t es) {
   // in FP64, then the slices of a split level's operands (counted for every level)
   size_t fmax = 0;
   const size_t parts = es / 8;
+  const int64_t t = inverse_scratch(H);
   for (size_t d = 0; d + 1 < H.hlevel_ptr.size(); d++) {
-    int64_t f = 0;
+    int64_t f = t;
     size_t oz = 512;
     for (int64_t i = H.hlevel_ptr[d]; i < H.hlevel_ptr[d + 1]; i++) {
       const int64_t K = H.hlevel_sn[i], s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
-      f += (s * s + 1) / 2 + (c + cu) * s + c * cu;
+      f += (c + cu) * s + c * cu;
       if (c > 0 && cu > 0)  // A_{C,K}, A_{K,C}^T, Uinv, Linv (the solves; then TL, TU)
         oz += parts * (slice_bytes(c, s, 8) + slice_bytes(cu, s, 8) + 2 * slice_bytes(s, s, 8)) +
               exps_bytes(c) + exps_bytes(cu) + 2 * exps_bytes(s) + 2048 +
@@ -628,8 +647,13 @@ struct SchurProduct {
 };
 void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
                     size_t base, bool eight);
-void add_ozaki_schur(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
-                     size_t base, bool lower, bool eight);
+void add_ozaki_schur_slices(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
+                            size_t base, bool eight, std::vector<OzDesc>& out);
+using TileFilter = std::function<bool(int, int, int)>;  // (descriptor, tile row, tile column)
+void add_ozgemm_step(Plan& P, std::vector<OzDesc>& descs, int S, int level, bool force_atomic,
+                     int ks, int slot, bool lower_c, const TileFilter& keep);
+void add_gemm8_step(Plan& P, const std::vector<OzDesc>& prods, int lev, bool lower_c,
+                    const TileFilter& keep);
 
 // tile of the diagonal blocks' small products: 16 x 16 while 32 x 32 tiles
 // would leave SMs without a CTA (a 32 x 32 x 32 product takes an SM's FP64
@@ -671,8 +695,9 @@ void add_panel_step(Plan& P, const std::vector<LuTask>& tasks, int level, bool s
 // 16 x 16 tiles, else 32 x 32 (28 MFLOP of complex grids 41 against 60 us; 24^3
 // upwind, 62 MFLOP: 66 us at 32 x 32); a task's K range short enough to last no
 // longer than half the level's work, in steps of 32.
+// keep: which entries (tile origins) the launch covers (null: all).
 void add_schur_scatter(pselinv_ctx* h, Plan& P, const std::vector<SchurDesc>& descs, int level,
-                       bool lower) {
+                       bool lower, const TileFilter& keep) {
   if (descs.empty()) return;
   const double cplx = h->dtype == DT_F64 ? 1.0 : 4.0;
   double ops = 0, bytes = 0;
@@ -686,13 +711,17 @@ void add_schur_scatter(pselinv_ctx* h, Plan& P, const std::vector<SchurDesc>& de
   const double per_k = tile * tile / 32.0 * 19.0 * cplx;  // cycles of a task per k
   const int kmax = std::max(32, (int)(std::max(cycles / 2, per_k * 32) / per_k) / 32 * 32);
   std::vector<SchurTask> tasks;
+  double all = 0;
   for (size_t d = 0; d < descs.size(); d++) {
     const int s = (int)h->H.sn_width[descs[d].K];
     for (int k = 0; k < s; k += kmax)
       for (int tq = 0; tq < ceil_div(descs[d].cu, tile); tq++)
-        for (int tp = lower ? tq : 0; tp < ceil_div(descs[d].c, tile); tp++)
-          tasks.push_back({(int)d, tp, tq, k, std::min(s, k + kmax)});
+        for (int tp = lower ? tq : 0; tp < ceil_div(descs[d].c, tile); tp++, all++)
+          if (!keep || keep((int)d, tp * tile, tq * tile))
+            tasks.push_back({(int)d, tp, tq, k, std::min(s, k + kmax)});
   }
+  if (tasks.empty()) return;
+  const double share = (double)tasks.size() / all;
   // longest K ranges first
   std::stable_sort(tasks.begin(), tasks.end(), [](const SchurTask& a, const SchurTask& b) {
     return a.k1 - a.k0 > b.k1 - b.k0;
@@ -703,8 +732,8 @@ void add_schur_scatter(pselinv_ctx* h, Plan& P, const std::vector<SchurDesc>& de
   st.n = (int)tasks.size();
   st.descs = P.push(descs);
   st.tasks = P.push(tasks);
-  st.flops = 64.0 * ops;
-  st.bytes = (size_t)bytes;
+  st.flops = 64.0 * ops * share;
+  st.bytes = (size_t)(bytes * share);
   st.level = level;
   P.steps.push_back(st);
 }
@@ -754,8 +783,9 @@ void add_inverse_row(pselinv_ctx* h, Plan& P, const std::vector<SnTask>& wide,
 
 constexpr double kEightMinFlops = 2e8;
 // events of a height level of the factorisation: one per panel (8 of 32
-// columns at most), one for its inverses
-constexpr int kPanelEvents = 9;
+// columns at most), and for its inverses, the operands and the bulk of its
+// Schur products, and the solves of narrow supernodes on the bulk stream
+constexpr int kEvInverse = 8, kEvOperands = 9, kEvBulk = 10, kEvSolved = 11, kPanelEvents = 12;
 
 int build_factor_plan(pselinv_ctx* h) {
   const HostSym& H = h->H;
@@ -779,32 +809,16 @@ int build_factor_plan(pselinv_ctx* h) {
   // work) and U^T panels are solved from the L panels; each diagonal block's
   // upper triangle is mirrored from its lower one before its LU
   const bool ldlt = h->opts.symmetric != 0 && !H.general;
-  // the next step of the main stream after the level's last panel waits for
-  // its inverses (the solves read them, and the scratch of their products is
-  // free again then)
-  int inverse_ready = -1;
-  auto wait_inverse = [&](size_t from) {
-    for (size_t i = from; i < P.steps.size() && inverse_ready >= 0; i++)
-      if (P.steps[i].side == 0) {
-        P.steps[i].wait = inverse_ready;
-        inverse_ready = -1;
-      }
-  };
-  for (size_t lev = 0; lev + 1 < H.hlevel_ptr.size(); lev++) {
-    std::vector<SnTask> wide, gt;  // wide: more than one panel
-    std::vector<SnTask> mirrored;  // symmetric values: blocks whose upper triangle is filled in
-    std::vector<LuTask> panels;    // first panels of every supernode, 32 lines per task
-    std::vector<int64_t> gofs;
-    std::vector<GemmDesc> trsm;
-    std::vector<SchurDesc> schur;
-    std::vector<SchurProduct> sprods, solves;
-    std::vector<CopySeg> segs;
-    const int64_t l0 = H.hlevel_ptr[lev], l1 = H.hlevel_ptr[lev + 1];
-    // split precision: the triangular solves and the Schur products of levels
-    // with enough Schur work as sliced tensor-core products (their operands
-    // sliced from the level's scratch after its FP64 region)
+  const int nlev = (int)H.hlevel_ptr.size() - 1;
+  // precision of each level's products.  Split: opts.slices slices where the
+  // Schur work pays for them; smaller levels keep FP64 accuracy, as products of
+  // eight slices where the FP64 pipe would take longer than their four launches
+  // (200 MFLOP: 160 us)
+  enum { LV_FP64, LV_SPLIT, LV_EIGHT };
+  std::vector<int> mode((size_t)std::max(nlev, 0) + 1, LV_FP64);
+  for (int lev = 0; lev < nlev && h->opts.factor_precision == PSELINV_PREC_OZAKI_FP16; lev++) {
     double sflops = 0, fp64 = 0;  // Schur flops; FP64 operations of the level's products
-    for (int64_t i = l0; i < l1; i++) {
+    for (int64_t i = H.hlevel_ptr[lev]; i < H.hlevel_ptr[lev + 1]; i++) {
       const int64_t K = H.hlevel_sn[i];
       const double c = (double)cK(H, K), cu = (double)cU(H, K), s = (double)H.sn_width[K];
       sflops += 2.0 * c * cu * s * (double)nb;
@@ -814,14 +828,54 @@ int build_factor_plan(pselinv_ctx* h) {
     const double min_flops = h->opts.factor_split_mflops < 0    ? 0.0
                              : h->opts.factor_split_mflops == 0 ? 2e8
                                                                 : 1e6 * h->opts.factor_split_mflops;
-    const bool ozaki = h->opts.factor_precision == PSELINV_PREC_OZAKI_FP16 && sflops > 0;
-    // smaller levels keep FP64 accuracy, as products of eight slices where the
-    // FP64 pipe would take longer than their four launches (200 MFLOP: 160 us)
-    const bool eight = ozaki && sflops < min_flops && fp64 >= kEightMinFlops;
-    const bool split = (ozaki && sflops >= min_flops) || eight;
-    int64_t off = 0;  // scalars into scratch
-    int64_t smax = 0;
-    std::vector<int64_t> mofs;  // scratch of the wide supernodes' inverse merges
+    if (sflops > 0)
+      mode[(size_t)lev] = sflops >= min_flops ? LV_SPLIT : fp64 >= kEightMinFlops ? LV_EIGHT : LV_FP64;
+  }
+  // A level's diagonal blocks are complete once the level below has updated
+  // them, long before the rest of its Schur products are: where there is enough
+  // of that rest, the updates of the parents' diagonal blocks ("corner") come
+  // first and the next level's LU runs beside the rest on the bulk stream.
+  //   inverse_ready: this level's inverses; bulk_ready: the level below's rest.
+  // Both are waited for by the next main-stream step that is not an LU panel
+  // (a later event of the same stream stands for an earlier one).
+  int inverse_ready = -1, bulk_ready = -1;
+  auto wait_pending = [&](size_t from) {
+    for (size_t i = from; i < P.steps.size() && (inverse_ready >= 0 || bulk_ready >= 0); i++)
+      if (P.steps[i].side == 0) {
+        P.steps[i].wait = inverse_ready;
+        P.steps[i].wait2 = bulk_ready;
+        inverse_ready = bulk_ready = -1;
+      }
+  };
+  auto event = [&](int lev, int k) { return EV_LEVEL + lev * kPanelEvents + k; };
+  // the rows of R_K in a parent one level up whose LU does not wait for the
+  // bulk stream (it solves no panels): K's corner
+  auto corner_rows = [&](int lev, int64_t K) -> int {
+    const int64_t J = H.sn_parent[K];
+    if (J < 0 || H.sn_height[J] != lev + 1) return 0;
+    if (H.sn_width[J] <= kLuPanel && mode[(size_t)lev + 1] == LV_FP64) return 0;
+    return H.blk_pe[H.sn_blk[K]];
+  };
+  const int64_t tbase = nb * inverse_scratch(H);
+  for (size_t lev = 0; lev + 1 < H.hlevel_ptr.size(); lev++) {
+    std::vector<SnTask> wide, sns;  // more than one panel; supernodes of sliced Schur products
+    std::vector<SnTask> mirrored;  // symmetric values: blocks whose upper triangle is filled in
+    // first panels, 32 lines per task: blocks alone, and narrow supernodes with
+    // their panel solves
+    std::vector<LuTask> panels, solving;
+    std::vector<int> corner;  // corner rows of every Schur product
+    std::vector<GemmDesc> trsm;
+    std::vector<SchurDesc> schur;
+    std::vector<SchurProduct> sprods, solves;
+    std::vector<CopySeg> segs;
+    const int64_t l0 = H.hlevel_ptr[lev], l1 = H.hlevel_ptr[lev + 1];
+    // sliced solves and Schur products: operands sliced from the level's scratch
+    // after its FP64 region
+    const bool split = mode[lev] != LV_FP64, eight = mode[lev] == LV_EIGHT;
+    int64_t off = tbase, toff = 0;  // scalars into scratch
+    int64_t smax = 0, entries = 0;
+    double ops = 0;                 // FP64 warp operations of the Schur products
+    std::vector<int64_t> mofs, sofs;  // scratch of the wide supernodes' inverses; of Sc
     for (int64_t b = 0; b < nb; b++)
       for (int64_t i = l0; i < l1; i++) {
         // c: rows of the L panel (R_K, or R_L(K) for a general pattern),
@@ -832,7 +886,8 @@ int build_factor_plan(pselinv_ctx* h) {
         const bool narrow = s <= kLuPanel && !split;  // panel solves in the panel launch
         const int64_t w = std::min<int64_t>(s, kLuPanel);
         const int64_t lines = (narrow ? c + (ldlt ? 0 : cu) : 2 * (s - w)) + 2 * w;
-        for (int64_t l = 0; l < lines; l += 32) panels.push_back({(int)b, (int)K, 0, (int)l});
+        for (int64_t l = 0; l < lines; l += 32)
+          (narrow ? solving : panels).push_back({(int)b, (int)K, 0, (int)l});
         char* base = h->lu + ((size_t)b * H.storage + H.sn_offset[K]) * es;
         char* Lp = base + (size_t)s * s * es;
         char* Up = Lp + (size_t)c * s * es;
@@ -843,8 +898,8 @@ int build_factor_plan(pselinv_ctx* h) {
         char *TL = Lp, *TU = Up;
         if (s > kLuPanel) {
           wide.push_back({(int)b, (int)K, 0, 0});
-          mofs.push_back(off);
-          off += s * s / 2;
+          mofs.push_back(toff);
+          toff += s * s / 2;
         } else if (ldlt && split) {
           mirrored.push_back({(int)b, (int)K, 0, 0});
         }
@@ -869,16 +924,16 @@ int build_factor_plan(pselinv_ctx* h) {
         const SchurProduct q{TL, TU, Sc, (int)c, (int)cu, (int)s, Lp, ldlt ? Lp : Up, Uinv, Linv};
         if (c > 0 && cu > 0) {
           if (oz) solves.push_back(q);
+          corner.push_back(H.general ? 0 : corner_rows((int)lev, K));
+          entries += c * cu;
+          ops += (double)c * cu * s / 32 * (dt == DT_F64 ? 1.0 : 4.0) * (ldlt ? 0.5 : 1.0);
           if (!split) {
             schur.push_back({TL, TU, (int)b, (int)K, (int)c, (int)cu});
-            continue;
+          } else {
+            sprods.push_back(q);
+            sofs.push_back(s0);
+            sns.push_back({(int)b, (int)K, 0, 0});
           }
-          sprods.push_back(q);
-          for (int tq = 0; tq < ceil_div(cu, 32); tq++)
-            for (int tp = ldlt ? tq : 0; tp < ceil_div(c, 32); tp++) {
-              gt.push_back({(int)b, (int)K, tp, tq});
-              gofs.push_back(s0);
-            }
         }
       }
     h->scratch_high = std::max(h->scratch_high, (size_t)off * es);
@@ -895,6 +950,19 @@ int build_factor_plan(pselinv_ctx* h) {
     // launch and (wide supernodes) one trailing-update GEMM, batched over the
     // level's supernodes; a narrow supernode is done after its panel
     size_t at = P.steps.size();
+    if (bulk_ready >= 0 && !panels.empty()) {
+      // panels of narrow supernodes take updates of the rest: behind it
+      const size_t first = P.steps.size();
+      add_panel_step(P, solving, (int)lev, true);
+      if (P.steps.size() > first) {
+        P.steps.back().side = 2;
+        bulk_ready = event((int)lev, kEvSolved);
+        P.steps.back().signal = bulk_ready;
+      }
+      at = P.steps.size();
+    } else {
+      panels.insert(panels.end(), solving.begin(), solving.end());
+    }
     for (int64_t j0 = 0; j0 < smax; j0 += kLuPanel) {
       std::vector<GemmDesc> upd;
       if (j0 > 0) panels.clear();
@@ -913,18 +981,18 @@ int build_factor_plan(pselinv_ctx* h) {
         }
       }
       add_panel_step(P, panels, (int)lev, !split);
-      wait_inverse(at);
+      if (wide.empty()) wait_pending(at);  // (panel solves among them)
       at = P.steps.size();
       if (!wide.empty()) {  // side stream: block row p of the inverses, inner products of p + 1
         const int64_t p = j0 / kLuPanel;
-        const int ev = EV_LEVEL + (int)lev * kPanelEvents + (int)p;
+        const int ev = event((int)lev, (int)p);
         P.steps.back().signal = ev;
         if (p > 0) add_inverse_row(h, P, wide, mofs, p, false, (int)lev);
         const size_t last_row = P.steps.size();
         add_inverse_row(h, P, wide, mofs, p + 1, true, (int)lev);
         if (P.steps.size() > at) P.steps[at].wait = ev;
         if (j0 + kLuPanel >= smax && last_row > at) {  // the last block row
-          inverse_ready = EV_LEVEL + (int)lev * kPanelEvents + kPanelEvents - 1;
+          inverse_ready = event((int)lev, kEvInverse);
           P.steps[last_row - 1].signal = inverse_ready;
         }
         at = P.steps.size();
@@ -936,13 +1004,43 @@ int build_factor_plan(pselinv_ctx* h) {
     // 8 s multiply-adds, 65 us for s = 64 complex; a 16 x 16 tile's 2 s)
     add_gemm_step(P, dt, choose_small_tile(dt, trsm) == GEMM_16x16 ? GEMM_16x16 : GEMM_ROWS, trsm,
                   (int)lev);
+    std::vector<OzDesc> prods;
     if (split) {
       add_ozaki_trsm(h, P, solves, (int)lev, align256((size_t)off * es), eight);
-      add_ozaki_schur(h, P, sprods, (int)lev, align256((size_t)off * es), ldlt, eight);
-    } else {
-      add_schur_scatter(h, P, schur, (int)lev, ldlt);
+      add_ozaki_schur_slices(h, P, sprods, (int)lev, align256((size_t)off * es), eight, prods);
     }
-    if (!gt.empty()) {
+    wait_pending(at);
+    // Schur products and their scatter, of the corner tiles (part 1), of the
+    // others (2) or all (0)
+    auto in_part = [&](int part, int i, int64_t p0, int64_t q0) {
+      return part == 0 || (part == 1) == (p0 < corner[(size_t)i] && q0 < corner[(size_t)i]);
+    };
+    auto add_schur = [&](int part) {
+      const int per = dt == DT_F64 ? 1 : 2;  // real and imaginary products
+      if (!split) {
+        add_schur_scatter(h, P, schur, (int)lev, ldlt,
+                          [&](int d, int p0, int q0) { return in_part(part, d, p0, q0); });
+        return;
+      }
+      const TileFilter keep = [&](int d, int tm, int tn) {
+        return in_part(part, d / per, tm * 128, tn * 64);
+      };
+      if (eight)
+        add_gemm8_step(P, prods, (int)lev, ldlt, keep);
+      else  // K = s <= 256 is one exact chunk of six slices: no K split, no accumulation
+        add_ozgemm_step(P, prods, h->slices, (int)lev, false, 1, 0, ldlt, keep);
+      std::vector<SnTask> gt;
+      std::vector<int64_t> gofs;
+      for (size_t i = 0; i < sns.size(); i++) {
+        const int64_t c = cK(H, sns[i].K), cu = cU(H, sns[i].K);
+        for (int tq = 0; tq < ceil_div(cu, 32); tq++)
+          for (int tp = ldlt ? tq : 0; tp < ceil_div(c, 32); tp++)
+            if (in_part(part, (int)i, tp * 32, tq * 32)) {
+              gt.push_back({sns[i].inst, sns[i].K, tp, tq});
+              gofs.push_back(sofs[i]);
+            }
+      }
+      if (gt.empty()) return;
       Step sc;
       sc.kind = ST_SCATTER_SUB;
       sc.cfg = ldlt ? 1 : 0;
@@ -951,9 +1049,35 @@ int build_factor_plan(pselinv_ctx* h) {
       sc.offs = P.push(gofs);
       sc.level = (int)lev;
       P.steps.push_back(sc);
+    };
+    // enough Schur work to hide behind the next level's LU (a wide block's takes
+    // 34 us a panel): 2 M entries of sliced products are about 36 us with their
+    // scatter; the corner's own launches cost the critical path about 15
+    bool wide_next = false;
+    if ((int)lev + 1 < nlev)
+      for (int64_t i = l1; i < H.hlevel_ptr[lev + 2]; i++)
+        wide_next = wide_next || H.sn_width[H.hlevel_sn[i]] > 2 * kLuPanel;
+    const double bulk = split ? (double)entries * (dt == DT_F64 ? 1.0 : 2.0) * (ldlt ? 0.5 : 1.0) / 2e6
+                              : ops * 16.0 / 152.0 / 72e3;
+    if (!H.general && wide_next && bulk >= 1.0) {
+      size_t last = P.steps.size() - 1;  // the operands are there after the last main step
+      while (last > 0 && P.steps[last].side != 0) last--;
+      P.steps[last].signal2 = event((int)lev, kEvOperands);
+      add_schur(1);
+      wait_pending(at);
+      const size_t first = P.steps.size();
+      add_schur(2);
+      for (size_t i = first; i < P.steps.size(); i++) P.steps[i].side = 2;
+      if (P.steps.size() > first) {
+        P.steps[first].wait = event((int)lev, kEvOperands);
+        bulk_ready = event((int)lev, kEvBulk);
+        P.steps.back().signal = bulk_ready;
+      }
+    } else {
+      add_schur(0);
+      wait_pending(at);
     }
     add_copy_step(P, segs, (int)lev, es);
-    wait_inverse(at);
   }
   const size_t at = P.steps.size();
   if (H.n > 0) {
@@ -962,7 +1086,7 @@ int build_factor_plan(pselinv_ctx* h) {
     up.n = (int)H.ns;
     P.steps.push_back(up);
   }
-  wait_inverse(at);
+  wait_pending(at);
   P.two_streams = true;
   P.ev.assign(EV_LEVEL + (H.hlevel_ptr.empty() ? 0 : (H.hlevel_ptr.size() - 1) * kPanelEvents),
               nullptr);
@@ -1133,11 +1257,12 @@ bool set_ozaki_ksplit(std::vector<OzDesc>& descs, int ks, bool force_atomic) {
   return any;
 }
 
+// keep: which tiles of the products the launch covers (null: all)
 void add_ozgemm_step(Plan& P, std::vector<OzDesc>& descs, int S, int level, bool force_atomic,
-                     int ks, int slot, bool lower_c = false) {
+                     int ks, int slot, bool lower_c, const TileFilter& keep) {
   if (descs.empty()) return;
   std::vector<OzTask> tasks;
-  double flops = 0, bytes = 0;
+  double flops = 0, bytes = 0, all = 0;
   set_ozaki_ksplit(descs, ks, force_atomic);
   for (size_t d = 0; d < descs.size(); d++) {
     OzDesc& g = descs[d];
@@ -1146,14 +1271,16 @@ void add_ozgemm_step(Plan& P, std::vector<OzDesc>& descs, int S, int level, bool
     // DRAM once and from L2 for the others
     for (int k = 0; k < g.ksplit; k++)
       for (int tm = 0; tm < ceil_div(g.M, 128); tm++)
-        for (int tn = 0; tn < ceil_div(g.N, 64); tn++)
-          if (!lower_c || (tm + 1) * 128 > tn * 64) tasks.push_back({(int)d, tm, tn, k});
+        for (int tn = 0; tn < ceil_div(g.N, 64); tn++, all++)
+          if ((!lower_c || (tm + 1) * 128 > tn * 64) && (!keep || keep((int)d, tm, tn)))
+            tasks.push_back({(int)d, tm, tn, k});
     flops += (lower_c ? 1.0 : 2.0) * g.M * g.N * (double)g.K32 * 32;
     // slices of both operands read once, the FP64 result written (read too
     // when accumulated)
     bytes += 2.0 * S * ((double)g.M + g.N) * g.K32 * 32 +
              8.0 * g.M * g.N * (g.atomic ? 2.0 : 1.0) * g.cscale;
   }
+  if (tasks.empty()) return;
   // longest tasks (most K blocks) first
   auto kblocks = [&](const OzTask& t) {
     const OzDesc& g = descs[t.d];
@@ -1166,11 +1293,12 @@ void add_ozgemm_step(Plan& P, std::vector<OzDesc>& descs, int S, int level, bool
   Step st;
   st.kind = ST_OZGEMM;
   st.cfg = S;
-  st.bytes = (size_t)bytes;
+  const double share = keep ? (double)tasks.size() / all : 1.0;
+  st.bytes = (size_t)(bytes * share);
   st.n = (int)tasks.size();
   st.descs = P.push(descs);
   st.tasks = P.push(tasks);
-  st.flops = flops;
+  st.flops = flops * share;
   st.level = level;
   st.slot = slot;
   st.param = ks;
@@ -1240,14 +1368,16 @@ struct OzBuilder {
 
 // Products of eight slices (see gemm8_kernel), longest K ranges first;
 // lower_c: the tiles of C on or below its diagonal only
-void add_gemm8_step(Plan& P, const std::vector<OzDesc>& prods, int lev, bool lower_c) {
+void add_gemm8_step(Plan& P, const std::vector<OzDesc>& prods, int lev, bool lower_c,
+                    const TileFilter& keep) {
   std::vector<OzTask> tasks;
-  double flops = 0, bytes = 0;
+  double flops = 0, bytes = 0, all = 0;
   for (size_t d = 0; d < prods.size(); d++) {
     const OzDesc& g = prods[d];
     for (int tm = 0; tm < ceil_div(g.M, 128); tm++)
-      for (int tn = 0; tn < ceil_div(g.N, 64); tn++)
-        if (!lower_c || (tm + 1) * 128 > tn * 64) tasks.push_back({(int)d, tm, tn, 0});
+      for (int tn = 0; tn < ceil_div(g.N, 64); tn++, all++)
+        if ((!lower_c || (tm + 1) * 128 > tn * 64) && (!keep || keep((int)d, tm, tn)))
+          tasks.push_back({(int)d, tm, tn, 0});
     const double half = g.tri || lower_c ? 0.5 : 1.0;
     flops += 2.0 * half * g.M * g.N * (double)g.K32 * 32;
     bytes += 2.0 * kSlices8 * ((double)g.M + g.N) * g.K32 * 32 + 8.0 * g.M * g.N;
@@ -1266,8 +1396,8 @@ void add_gemm8_step(Plan& P, const std::vector<OzDesc>& prods, int lev, bool low
   m.n = (int)tasks.size();
   m.descs = P.push(prods);
   m.tasks = P.push(tasks);
-  m.flops = flops;
-  m.bytes = (size_t)bytes;
+  m.flops = flops * (keep ? (double)tasks.size() / all : 1.0);
+  m.bytes = (size_t)(bytes * (keep ? (double)tasks.size() / all : 1.0));
   m.level = lev;
   P.steps.push_back(m);
 }
@@ -1301,20 +1431,18 @@ void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& pr
   }
   add_panel_slice_step(P, sl, lev);
   if (eight)
-    add_gemm8_step(P, out, lev, false);
+    add_gemm8_step(P, out, lev, false, nullptr);
   else
-    add_ozgemm_step(P, out, h->slices, lev, false, 1, 0);
+    add_ozgemm_step(P, out, h->slices, lev, false, 1, 0, false, nullptr);
 }
 
-// Schur products of one factorisation level as sliced products: slices of TL
-// and TU (both by rows: A = TL, B = TU with K = s), then the products into the
-// FP64 Sc blocks the scatter subtracts.  Scratch from
-// `base` (bytes), after the level's FP64 region.
-void add_ozaki_schur(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
-                     size_t base, bool lower, bool eight) {
+// Operands of the Schur products of one factorisation level: slices of TL and
+// TU (both by rows: A = TL, B = TU with K = s) in one launch, and the products
+// into the FP64 Sc blocks that the scatter subtracts.
+void add_ozaki_schur_slices(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
+                            size_t base, bool eight, std::vector<OzDesc>& out) {
   OzBuilder ob(h, base, eight ? kSlices8 : 0);
   std::vector<SliceDesc> sl;
-  std::vector<OzDesc> out;
   for (const SchurProduct& q : prods) {
     const SliceDesc a = ob.slice(q.TL, q.c, SLICE_ROWS, q.c, q.s);
     const SliceDesc b = ob.slice(q.TU, q.cu, SLICE_ROWS, q.cu, q.s);
@@ -1323,11 +1451,6 @@ void add_ozaki_schur(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& p
     ob.product(out, a, b, q.Sc, q.c, q.c, q.cu, 1.0);
   }
   add_panel_slice_step(P, sl, lev);
-  // K = s <= 256 is one exact chunk of six slices: no K split, no accumulation
-  if (eight)
-    add_gemm8_step(P, out, lev, lower);
-  else
-    add_ozgemm_step(P, out, h->slices, lev, false, 1, 0, lower);
 }
 
 // Split-precision normalisation of one depth level (Algorithm 1 step 2 and
@@ -1390,7 +1513,7 @@ void add_ozaki_normalize(pselinv_ctx* h, Plan& P, int lev, int64_t nb, size_t ba
   P.steps.push_back(ms);
   add_slice_step(P, sl, lev, true);
   add_slice_step(P, sl, lev, false);
-  add_ozgemm_step(P, prods, h->slices, lev, false, 1, -1);
+  add_ozgemm_step(P, prods, h->slices, lev, false, 1, -1, false, nullptr);
   for (size_t i = first; i < P.steps.size(); i++) P.steps[i].side = 1;
 }
 
@@ -1431,7 +1554,7 @@ void add_sliced_normalize(pselinv_ctx* h, Plan& P, const std::vector<std::pair<i
     }
   }
   add_panel_slice_step(P, sl, lev);
-  add_gemm8_step(P, prods, lev, false);
+  add_gemm8_step(P, prods, lev, false, nullptr);
 }
 
 // Merge the finished blocks of the supernodes `sns` (diagonal block, L and
@@ -1571,11 +1694,11 @@ void add_ozaki_level(pselinv_ctx* h, Plan& P, const std::vector<int64_t>& grp, i
   // outputs of products split along K (requested, or forced by the exact
   // chunk limit) are accumulated: zero them first
   if (set_ozaki_ksplit(main, ks_main, false)) add_zero_step(P, zero, lev);
-  add_ozgemm_step(P, main, S, lev, false, ks_main, 1);
+  add_ozgemm_step(P, main, S, lev, false, ks_main, 1, false, nullptr);
   add_copy_step(P, mirror, lev, es);
   add_slice_step(P, sl2, lev, true);
   add_slice_step(P, sl2, lev, false);
-  add_ozgemm_step(P, dg, S, lev, true, ks_diag, 2);
+  add_ozgemm_step(P, dg, S, lev, true, ks_diag, 2, false, nullptr);
 }
 
 // largest K split of the normalisation's products
@@ -1921,6 +2044,12 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
   return PSELINV_OK;
 }
 
+// SMs that the bulk stream's sliced products take (one CTA of 216 KB shared
+// memory each): the others are free for the LU panels beside them (factorisation
+// of 8^3 x 64 / 10^3 x 64 DG, ms: 96 SMs 24.6 / 83.5, 120: 23.8 / 75.1, 140: 24.0 /
+// 71.1, one CTA per task: 27.2 / 90.6)
+constexpr int kBulkSms = 136;
+
 void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) {
   char* a = P.arena;
   switch (s.kind) {
@@ -1980,7 +2109,8 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
       break;
     case ST_OZGEMM:
       launch_ozaki_gemm(s.cfg, (const OzDesc*)(a + s.descs), (const OzTask*)(a + s.tasks), s.n,
-                        h->derr, s.side == 0, h->opts.ozaki_a_tmem != 0, st);
+                        h->derr, s.side == 0 ? 152 : s.side == 2 ? kBulkSms : s.n,
+                        h->opts.ozaki_a_tmem != 0, st);
       break;
     case ST_ZERO:
       launch_zero((const CopySeg*)(a + s.tasks), s.n, s.grid, st);
@@ -2005,9 +2135,11 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
 
 // The streams of a multi-stream sweep (created on first use): the sweep's
 // own launches at the highest priority, the normalisation one level ahead
-// below it, so that pending CTAs of the critical path are scheduled first.
+// below it, the factorisation's bulk Schur products lowest, so that pending
+// CTAs of the critical path are scheduled first.
 struct SweepStreams {
-  cudaStream_t main, side;
+  cudaStream_t main, side, bulk;
+  cudaStream_t of(const Step& s) const { return s.side == 1 ? side : s.side == 2 ? bulk : main; }
 };
 int sweep_streams(pselinv_ctx* h, SweepStreams* out) {
   int least = 0, greatest = 0;
@@ -2017,7 +2149,9 @@ int sweep_streams(pselinv_ctx* h, SweepStreams* out) {
     CK(cudaStreamCreateWithPriority(&h->main_stream, cudaStreamNonBlocking, greatest));
   if (!h->side_stream)
     CK(cudaStreamCreateWithPriority(&h->side_stream, cudaStreamNonBlocking, middle));
-  *out = {h->main_stream, h->side_stream};
+  if (!h->bulk_stream)
+    CK(cudaStreamCreateWithPriority(&h->bulk_stream, cudaStreamNonBlocking, least));
+  *out = {h->main_stream, h->side_stream, h->bulk_stream};
   return PSELINV_OK;
 }
 
@@ -2035,16 +2169,21 @@ int run_steps(pselinv_ctx* h, Plan& P, cudaStream_t st) {
   CK(cudaEventRecord(P.ev[EV_FORK], st));
   CK(cudaStreamWaitEvent(q3.main, P.ev[EV_FORK], 0));
   CK(cudaStreamWaitEvent(q3.side, P.ev[EV_FORK], 0));
+  CK(cudaStreamWaitEvent(q3.bulk, P.ev[EV_FORK], 0));
   for (const Step& s : P.steps) {
-    cudaStream_t q = s.side == 1 ? q3.side : q3.main;
-    if (s.wait >= 0) CK(cudaStreamWaitEvent(q, P.ev[s.wait], 0));
+    cudaStream_t q = q3.of(s);
+    for (int e : {s.wait, s.wait2})
+      if (e >= 0) CK(cudaStreamWaitEvent(q, P.ev[e], 0));
     launch_step(h, P, s, q);
-    if (s.signal >= 0) CK(cudaEventRecord(P.ev[s.signal], q));
+    for (int e : {s.signal, s.signal2})
+      if (e >= 0) CK(cudaEventRecord(P.ev[e], q));
   }
   CK(cudaEventRecord(P.ev[EV_MAIN_JOIN], q3.main));
   CK(cudaEventRecord(P.ev[EV_SIDE_JOIN], q3.side));
+  CK(cudaEventRecord(P.ev[EV_BULK_JOIN], q3.bulk));
   CK(cudaStreamWaitEvent(st, P.ev[EV_MAIN_JOIN], 0));
   CK(cudaStreamWaitEvent(st, P.ev[EV_SIDE_JOIN], 0));
+  CK(cudaStreamWaitEvent(st, P.ev[EV_BULK_JOIN], 0));
   CK(cudaGetLastError());
   return PSELINV_OK;
 }
@@ -2574,7 +2713,7 @@ int pselinv_profile(pselinv_t h, int which, void* stream, pselinv_step_stat* out
     CK(cudaStreamWaitEvent(q3.side, ev[0], 0));
     for (size_t i = 0; i < ns; i++) {
       const Step& s = P.steps[i];
-      cudaStream_t q = s.side == 1 ? q3.side : q3.main;
+      cudaStream_t q = q3.of(s);
       if (s.wait >= 0) CK(cudaStreamWaitEvent(q, P.ev[s.wait], 0));
       CK(cudaEventRecord(ev[2 * i + 1], q));
       launch_step(h, P, s, q);
@@ -3138,6 +3277,7 @@ void pselinv_free(pselinv_t h) {
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->main_stream) cudaStreamDestroy(h->main_stream);
     if (h->side_stream) cudaStreamDestroy(h->side_stream);
+    if (h->bulk_stream) cudaStreamDestroy(h->bulk_stream);
     cudaFree(h->dsym);
     cudaFree(h->derr);
     cudaFree(h->tslot);

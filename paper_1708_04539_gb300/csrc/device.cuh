@@ -288,10 +288,11 @@ cudaError_t prepare_ozaki_kernels();
 // maxima = true: accumulate row maxima into desc.maxbits; false: write the slices
 void launch_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, bool maxima,
                   cudaStream_t st);
-// a_tmem: the MMAs read A from tensor memory (copied from the stage per K
+// max_grid: most CTAs of the launch (persistent beyond); a_tmem: the MMAs read
+// A from tensor memory (copied from the stage per K
 // half) instead of shared memory
 void launch_ozaki_gemm(int S, const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
-                       bool persistent, bool a_tmem, cudaStream_t st);
+                       int max_grid, bool a_tmem, cudaStream_t st);
 // Slices of operands with K <= 256 with their own row maxima (desc.maxbits
 // unused), `span` K blocks per task {d, row block, first K block}; and
 // products of eight slices, C = A op(B), tasks {d, tm, tn, 0}

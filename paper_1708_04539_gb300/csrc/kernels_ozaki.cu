@@ -1470,12 +1470,13 @@ void launch_gslice(int dtype, const SymDev& S, const void* store, const SliceDes
 }
 
 void launch_ozaki_gemm(int S, const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
-                       bool persistent, bool a_tmem, cudaStream_t st) {
+                       int max_grid, bool a_tmem, cudaStream_t st) {
   if (ntasks <= 0) return;
-  // one CTA fits an SM (shared memory and tensor memory): a persistent grid
-  // on the sweep's stream; one task per CTA on the normalisation stream, so
-  // that its CTAs leave SMs to the sweep between tasks
-  const int grid = persistent && ntasks > 152 ? 152 : ntasks;
+  // one CTA fits an SM (shared memory and tensor memory): a persistent grid on
+  // the critical stream (all SMs) and for the factorisation's bulk (most of
+  // them); one task per CTA on the normalisation stream, so that its CTAs leave
+  // SMs to the sweep between tasks
+  const int grid = ntasks < max_grid ? ntasks : max_grid;
 #define PSELINV_OZ_LAUNCH(SS, AT)                                                        \
   ozaki_gemm_kernel<SS, AT><<<grid, kOzThreads, gemm_smem<SS, AT>(), st>>>(descs, tasks, \
                                                                           ntasks, err)
