@@ -1729,46 +1729,48 @@ bool split_fp64_products(std::vector<GemmDesc>& descs, int dtype) {
   return any;
 }
 
-// An FP64 level of narrow supernodes as one fused launch (gather and steps
-// 3-5 in shared memory), each supernode's output columns split into tasks
-// of at most kSmallLevelTaskFma multiply-adds, when every supernode fits
-// and the estimated time (multiply-adds at 2 per cycle and SM) is below
-// that of the gather and two GEMM launches (about 15 us each plus the
-// level's flops at 1 TFLOP/s).  Returns false to leave
-// the level to those launches.
-constexpr double kSmallLevelTaskFma = 65536;
+// An FP64 level as one fused launch (gather and steps 3-5,
+// small_level_kernel); false for a level without off-diagonal blocks.  Every
+// FP64 level of the level schedule runs this way: against the gather and the
+// two K-split products it measured 8 / 27 us (a level of 0.01 Mflop), 37 / 76
+// (15), 171 / 162 (141), 739 / 837 (785), 6440 / 6700 (7600), over whole sweeps
+// 0.52 / 1.72 ms (one-way 90^2), 2.4 / 4.7 (five 2D grids), 3.8 / 4.7 (24^3 upwind),
+// 76.5 / 80.4 (40^3); only levels whose tasks just exceed a wave of 760 lose (up
+// to 14%, dif 30^3 level 4).  The longest tasks go first, so that the last wave
+// is short (24^3 complex stencil: 3.25 -> 2.99 ms).
 bool add_small_level(pselinv_ctx* h, Plan& P, const std::vector<int64_t>& grp, int64_t nb, int lev) {
   const HostSym& H = h->H;
-  const bool sym = h->opts.symmetric != 0;
+  const bool sym = h->opts.symmetric != 0 && !H.general;
   const double cplx = h->dtype == DT_F64 ? 1.0 : 4.0;
-  std::vector<SnTask> tasks;
+  std::vector<LevelTask> tasks;
   size_t smem = 0;
-  double fma_max = 0, flops = 0, bytes = 0;
+  double flops = 0, bytes = 0;
   for (int64_t K : grp) {
-    const int64_t s = H.sn_width[K], c = cK(H, K);
-    if (c == 0) continue;
-    if (c > kSmallLevelMaxC) return false;
-    // multiply-adds per output column: steps 3 and 5 (c^2 each), step 4 (s c)
-    const double per_col = cplx * ((sym ? 1.0 : 2.0) * c * c + (double)s * c);
-    const int w = (int)std::max<int64_t>(1, std::min<int64_t>(s, (int64_t)(kSmallLevelTaskFma / per_col)));
-    const int64_t rb = H.rows_ptr[K], b0 = H.rows_blk[rb], bl = H.rows_blk[rb + c - 1];
-    const int64_t seg = H.blk_rel[bl] + (c - H.blk_pb[bl]) - H.blk_rel[b0];
-    const size_t b = small_level_smem(h->dtype, (int)c, (int)s, w, (int)(bl - b0 + 1), (int)seg);
-    if (b > kSmallLevelMaxSmem) return false;
-    smem = std::max(smem, b);
-    fma_max = std::max(fma_max, per_col * w);
-    flops += 2.0 * per_col * s * nb;
-    bytes += (double)h->esize * nb * (c * c + 4.0 * c * s + 2.0 * s * s);
-    for (int64_t b2 = 0; b2 < nb; b2++)
-      for (int64_t j0 = 0; j0 < s; j0 += w)
-        tasks.push_back({(int)b2, (int)K, (int)j0, (int)std::min<int64_t>(w, s - j0)});
+    const int64_t s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
+    if (c == 0 || cu == 0) continue;
+    flops += 2.0 * cplx * ((sym ? 1.0 : 2.0) * c * cu * s + (double)s * s * cu) * nb;
+    bytes += (double)h->esize * nb * (c * cu + 4.0 * c * s + 2.0 * s * s);
+    for (int side = 0; side < (sym ? 1 : 2); side++) {
+      const int64_t M = side ? c : cu;
+      const int64_t nr = ceil_div(M, ceil_div(M, kLevelTile));
+      const int64_t nw = ceil_div(s, ceil_div(s, kLevelTile));
+      for (int64_t j = 0; j < s; j += nw)
+        for (int64_t r = 0; r < M; r += nr) {
+          const LevelTask t = {H.sn_offset[K], H.rows_ptr[K],
+                               H.general ? H.urows_ptr[K] : H.rows_ptr[K], (int)K, (int)c, (int)cu,
+                               (int)s, (int)r, (int)std::min(nr, M - r), (int)j,
+                               (int)std::min(nw, s - j), side, 0};
+          smem = std::max(smem, small_level_smem(h->dtype, t));
+          tasks.push_back(t);
+        }
+    }
   }
   if (tasks.empty()) return false;
-  // the largest task alone on an SM, or the level's multiply-adds spread
-  // over all 152 SMs, whichever is longer
-  const double t_fused = std::max(fma_max, flops / 2.0 / 152.0) / 2.0 / 2.07e9;
-  const double t_launches = 3 * 15e-6 + flops / 1e12;
-  if (t_fused >= t_launches) return false;
+  auto cost = [](const LevelTask& t) {
+    return (int64_t)t.nr * t.nw * (t.side ? t.cu : t.c + t.s);
+  };
+  std::stable_sort(tasks.begin(), tasks.end(),
+                   [&](const LevelTask& x, const LevelTask& y) { return cost(x) > cost(y); });
   Step st;
   st.kind = ST_SMALL_LEVEL;
   st.cfg = (int)smem;
@@ -1906,27 +1908,28 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
         add_ozaki_level(h, P, grp, nb, (int)lev, max_cursor);
         continue;
       }
-      if (schedule == PSELINV_SCHED_LEVEL && !H.general && add_small_level(h, P, grp, nb, (int)lev))
-        continue;
+      // with one structure empty (a general pattern) the other panel of Ainv is
+      // zero (steps 3 and 5 sum over the empty one); nothing else after D_K
+      std::vector<CopySeg> zsegs;
+      for (int64_t b = 0; b < nb && H.general; b++)
+        for (int64_t K : grp) {
+          const int64_t s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
+          if ((c == 0) == (cu == 0)) continue;
+          const size_t so = ((size_t)b * H.storage + H.sn_offset[K]) * es;
+          zsegs.push_back({nullptr, h->ainv + so + (size_t)s * s * es,
+                           (c + cu) * s * (int64_t)(es / 8)});
+        }
+      add_zero_step(P, zsegs, (int)lev);
+      if (schedule == PSELINV_SCHED_LEVEL && add_small_level(h, P, grp, nb, (int)lev)) continue;
       std::vector<SnTask> gt;
       std::vector<int64_t> gofs;
       std::vector<GemmDesc> main, dg;
-      std::vector<CopySeg> mirror, zsegs;
+      std::vector<CopySeg> mirror;
       int64_t goff = 0;
       for (int64_t b = 0; b < nb; b++)
         for (int64_t K : grp) {
           const int64_t s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
-          if (c == 0 || cu == 0) {
-            // nothing after D_K; with one structure empty (a general
-            // pattern) the other panel of Ainv is zero (steps 3 and 5 sum
-            // over the empty one)
-            if (c + cu > 0) {
-              const size_t so = ((size_t)b * H.storage + H.sn_offset[K]) * es;
-              zsegs.push_back({nullptr, h->ainv + so + (size_t)s * s * es,
-                               (c + cu) * s * (int64_t)(es / 8)});
-            }
-            continue;
-          }
+          if (c == 0 || cu == 0) continue;
           const int64_t g0 = goff;
           goff += c * cu;
           h->scratch_high = std::max(h->scratch_high, (size_t)goff * es);
@@ -1962,7 +1965,6 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
           dg.push_back(make_desc(h->nf + (sym ? lo : uo), h->ainv + lo, h->ainv + so, s, s, c, c, c,
                                  s, 1, 0, -1.0, 1.0, 1));
         }
-      add_zero_step(P, zsegs, (int)lev);
       if (gt.empty()) continue;
       Step g;
       g.kind = ST_GATHER;
@@ -2116,8 +2118,9 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
       launch_zero((const CopySeg*)(a + s.tasks), s.n, s.grid, st);
       break;
     case ST_SMALL_LEVEL:
-      launch_small_level(h->dtype, h->S, h->ainv, h->nf, (const SnTask*)(a + s.tasks), s.n,
-                         (size_t)s.cfg, h->opts.symmetric != 0, st);
+      launch_small_level(h->dtype, h->S, h->ainv, h->nf, (const LevelTask*)(a + s.tasks), s.n,
+                         (int)h->nbatch, (size_t)s.cfg,
+                         h->opts.symmetric != 0 && !h->H.general, st);
       break;
     case ST_GSLICE:
       launch_gslice(h->dtype, h->S, h->ainv, (const SliceDesc*)(a + s.descs),
@@ -2448,7 +2451,6 @@ int pselinv_factor(pselinv_t h, int dtype, int64_t nbatch, const void* values, v
     CK(cudaMalloc(&h->outstage, (size_t)h->H.nnz * es + 256));
     CK(cudaMalloc(&h->rcmax, (size_t)nbatch * 2 * h->H.n * 8 + 256));
     CK(prepare_dense_kernels());
-    CK(prepare_map_kernels());
     CK(prepare_ozaki_kernels());
     h->slices = h->opts.slices <= 0 ? 6 : std::min(6, std::max(4, (int)h->opts.slices));
   }

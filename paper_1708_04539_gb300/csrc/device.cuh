@@ -359,23 +359,27 @@ int fp64_peak_grid(int sms);
 double launch_fp64_peak(double* out, int grid, int iters, cudaStream_t st);
 // one-time kernel attributes
 cudaError_t prepare_dense_kernels();
+// Algorithm 1 steps 3-5 of an FP64 level in one launch (nothing of G is
+// stored), a CTA per task and instance: rows r0 .. r0 + nr - 1,
+// columns j0 .. j0 + nw - 1 of step 3's (side 0, with step 4) or step 5's
+// (side 1) output of supernode K; off = sn_off[K], rl = rows_ptr[K], ru =
+// urows_ptr[K] (rows_ptr[K] unless the pattern is general).  nr and nw are
+// at most kLevelTile; smem is the largest small_level_smem of the tasks.
+// D_K must already be in the diagonal blocks of store.
+struct LevelTask {
+  int64_t off, rl, ru;
+  int K, c, cu, s, r0, nr, j0, nw, side, pad;
+};
+constexpr int kLevelK = 32, kLevelTile = 16, kLevelThreads = 128;  // contraction chunk, tile, CTA
+size_t small_level_smem(int dtype, const LevelTask& t);
+void launch_small_level(int dtype, const SymDev& S, void* store, const void* nf,
+                        const LevelTask* tasks, int ntasks, int nbatch, size_t smem,
+                        int sym, cudaStream_t st);
 // G_K = Ainv(R_K, R_K) gathered from `store` into out + gofs[task]
 // tasks {inst, K, tile_p, tile_q} (32 x 32 tiles).  With mofs != null
 // (real data only), the row and column maxima of |G_K| are also accumulated
 // (atomicMax on the bit patterns) into maxbase + mofs[task] (rows, c
 // entries) and maxbase + mofs[task] + c (columns).
-// Algorithm 1 steps 3-5 of a level of narrow supernodes in one launch, a
-// CTA per task {inst, K, j0, w} (c > 0; columns j0 .. j0 + w - 1 of the
-// supernode's outputs) with G, Lhat, Uhat^T and w columns of Ainv(C,K) in
-// `smem` bytes of shared memory (at most kSmallLevelMaxSmem, see
-// small_level_smem); D_K must already be in the diagonal blocks of store
-constexpr size_t kSmallLevelMaxSmem = 160 * 1024;
-constexpr int kSmallLevelMaxC = 128;
-// nblk blocks in R_K, seg relative indices of R_K's blocks
-size_t small_level_smem(int dtype, int c, int s, int w, int nblk, int seg);
-cudaError_t prepare_map_kernels();
-void launch_small_level(int dtype, const SymDev& S, void* store, const void* nf, const SnTask* tasks,
-                        int ntasks, size_t smem, int sym, cudaStream_t st);
 void launch_gather(int dtype, const SymDev& S, const void* store, void* out,
                    const int64_t* gofs, const SnTask* tasks, int ntasks, cudaStream_t st,
                    const int64_t* mofs = nullptr, unsigned long long* maxbase = nullptr);

@@ -5,6 +5,8 @@
 // extraction of the selected entries (Algorithm 1 step 6, Theorem 2).
 #include "device.cuh"
 
+#include <type_traits>
+
 namespace pselinv {
 
 namespace {
@@ -536,109 +538,262 @@ __global__ void __launch_bounds__(kThreads) trace_final_kernel(const T* __restri
   if (threadIdx.x == 0) *out = red[0];
 }
 
-// Algorithm 1 steps 3-5 of an FP64 level of narrow supernodes in one
-// launch.  A task {inst, K, j0, w} owns columns j0 .. j0 + w - 1 of the
-// supernode's outputs: G = Ainv(R_K, R_K) is gathered into shared memory
-// (leading dimension ldg = c | 1, so that the transposed reads of step 5
-// spread over the banks) with Lhat and Uhat^T (c x s); then Ainv(C,K) = -G
-// Lhat and Ainv(K,C)^T = -G^T Uhat^T for those columns into the panels (for
-// a symmetric A the second is a copy of the first) and Ainv_KK(:, j) = D_K(:,
-// j) - Uhat Ainv(C,K)(:, j) onto the diagonal block (D_K written there by
-// the normalisation).  Dot products over c from shared memory; the tasks
-// of a supernode write disjoint columns, so no atomics.
+// Algorithm 1 steps 3-5 of an FP64 level in one launch: nothing of G is
+// stored.  A task owns the tile [r0, r0 + nr) x [j0, j0 + nw) of one
+// supernode's outputs.
+//   side 0 (step 3): X = -G(r, :) Lhat(:, j) into Ainv(R_U, K), and step 4's
+//     share of these rows, Ainv_KK(:, j) -= Uhat(:, r) X, atomically (D_K
+//     written there by the normalisation);
+//   side 1 (step 5): -G(:, r)^T Uhat^T(:, j) into Ainv(K, R_L)^T.
+// A symmetric A has side 0 only and writes its tile to both panels.  The
+// contraction runs in chunks of kLevelK, software pipelined: while a chunk is
+// multiplied, the next one's entries of G are on their way from the
+// ancestors' blocks (storage bases per position, as in scatter_sub_kernel) and
+// the bases of the one after.  Entries of G stored along r are read with
+// lanes along r, the others with lanes along k; most chunks hold only one
+// kind.  Tiles of few outputs split the contraction over `kg` groups of
+// threads.
+// Small levels are bound by latency (launch, task, bases, relative index,
+// value, then the chain of FP64 operations at 64 cycles each), larger ones by
+// the FP64 pipe (17 cycles per warp operation and SM, 1.18 TFLOP/s: 24^3
+// upwind's levels of 700 Mflop run at 1.06).  Tiles of 32 x 16 and 32 x 32 with 256
+// threads were slower at every size (five 2D grids: 2.38, 2.56, 2.81 ms), without
+// the pipelining 2.66; a kernel that held all of G of a supernode took 2.45 with
+// the levels that did not fit on the product launches (sweep 3.67 -> 2.92).
+// Five CTAs per SM (95 registers) against four: 3.76 / 3.96 ms on 24^3 upwind;
+// complex values spill at five.
 template <typename T>
-__global__ void __launch_bounds__(kThreads)
-small_level_kernel(SymDev S, T* store, const T* __restrict__ nf, const SnTask* __restrict__ tasks,
-                   int ntasks, int sym) {
+__global__ void __launch_bounds__(kLevelThreads, sizeof(T) == 8 ? 5 : 4)
+small_level_kernel(SymDev S, T* store, const T* __restrict__ nf, const LevelTask* __restrict__ tasks,
+                   int nbatch, int sym) {
+  constexpr int NT = kLevelThreads, TP = kLevelTile;
+  constexpr int NG = TP * kLevelK / NT, NB = NG, NC = TP * TP / NT;
   extern __shared__ __align__(16) unsigned char small_smem[];
-  for (int t = blockIdx.x; t < ntasks; t += gridDim.x) {
-    const SnTask task = tasks[t];
-    const int K = task.K, j0 = task.a, w = task.b;
-    const int c = S.sn_c[K], s = S.sn_width[K];
-    const int ldg = c | 1;
-    const int64_t rb = S.rows_ptr[K];
-    const int64_t base = (int64_t)task.inst * S.storage;
-    const int64_t so = base + S.sn_off[K], lo = so + (int64_t)s * s, uo = lo + (int64_t)c * s;
-    // index tables of R_K's blocks (consecutive block ids b0 ..): the local
-    // block of every position, the supernode's relative-index segment, and
-    // per block the storage offset, width and |R| of its supernode and the
-    // start of its relative indices within the segment
-    const int b0 = S.rows_blk[rb], nblk = S.rows_blk[rb + c - 1] - b0 + 1;
-    const int64_t rel0 = S.blk_rel[b0];
-    const int seg = (int)(S.blk_rel[b0 + nblk - 1] + (c - S.blk_pb[b0 + nblk - 1]) - rel0);
-    int64_t* m_off = reinterpret_cast<int64_t*>(small_smem);
-    int* m_s = reinterpret_cast<int*>(m_off + nblk);
-    int* m_c = m_s + nblk;
-    int* m_base = m_c + nblk;
-    int* lblk = m_base + nblk;
-    int* rel = lblk + c;
-    const size_t ibytes = ((size_t)nblk * 20 + (size_t)(c + seg) * 4 + 15) & ~size_t(15);
-    T* G = reinterpret_cast<T*>(small_smem + ibytes);
-    T* Lh = G + (int64_t)ldg * c;
-    T* Uh = Lh + (int64_t)c * s;
-    T* X = Uh + (int64_t)c * s;  // c x w: Ainv(C,K)(:, j0 .. j0 + w - 1)
-    for (int l = threadIdx.x; l < nblk; l += blockDim.x) {
-      const int J = S.blk_sn[b0 + l];
-      m_off[l] = S.sn_off[J];
-      m_s[l] = S.sn_width[J];
-      m_c[l] = S.sn_c[J];
-      m_base[l] = (int)(S.blk_rel[b0 + l] - rel0) - S.blk_pb[b0 + l];
-    }
-    for (int p = threadIdx.x; p < c; p += blockDim.x) lblk[p] = S.rows_blk[rb + p] - b0;
-    for (int i = threadIdx.x; i < seg; i += blockDim.x) rel[i] = S.relidx[rel0 + i];
-    for (int e = threadIdx.x; e < c * s; e += blockDim.x) {
-      Lh[e] = nf[lo + e];
-      if (!sym) Uh[e] = nf[uo + e];
-    }
-    __syncthreads();
-    // G = Ainv(R_K, R_K): the slot of (p, q) as in map_slot, from the tables
-    const T* src = store + base;
-    for (int e = threadIdx.x; e < c * c; e += blockDim.x) {
-      const int p = e % c, q = e / c;
-      T v = sc_zero(T());
-      if (S.check) {
-        if (!map_in_range(S, rb, p, q))
-          set_error(S.err, DEV_CHECK, K);
-        else
-          v = src[map_slot(S, rb, p, q)];
-      } else {
-        const int lp = lblk[p], lq = lblk[q], l = lp < lq ? lp : lq;
-        const int rp = rel[m_base[l] + p], rq = rel[m_base[l] + q];
-        const int64_t sJ = m_s[l], cJ = m_c[l];
-        int64_t slot;
-        if (lp == lq)
-          slot = m_off[l] + rp + rq * sJ;
-        else if (lp > lq)
-          slot = m_off[l] + sJ * sJ + rp + rq * cJ;
-        else
-          slot = m_off[l] + sJ * sJ + cJ * sJ + rq + rp * cJ;
-        v = src[slot];
+  __shared__ int64_t rdiag[TP], rpan[TP], rrel[TP];
+  __shared__ int64_t kdiag[2][kLevelK], kpan[2][kLevelK], krel[2][kLevelK];
+  __shared__ int rsn[TP], ksn[2][kLevelK];
+  const LevelTask t = tasks[blockIdx.x];
+  const int tid = threadIdx.x;
+  const int nr = t.nr, nw = t.nw, s = t.s;
+  const bool side = t.side != 0;
+  const int kt = side ? t.cu : t.c;  // length of the contraction
+  const int kc = min(kt, kLevelK), ldr = nr | 1, ldw = nw | 1, si = min(s, kLevelK);
+  T* const sG = reinterpret_cast<T*>(small_smem);  // [k][r]
+  T* const sB = sG + kc * ldr;                     // [k][j]
+  T* const sU = sB + kc * ldw;                     // [i][r]
+  T* const sX = sU + si * ldr;                     // [j][r], and the partial sums of kg groups
+  const unsigned mr = (65536u + nr - 1) / nr;      // e / nr = e mr >> 16 for e < 2048
+  // bases of the positions of R_U (rows of G) and R_L (its columns): of the
+  // tile's r and of the contraction's k
+  const int64_t* const g_kpan = side ? S.row_pan + t.ru : S.col_pan + t.rl;
+  const int64_t* const g_krel = side ? S.row_rel + t.ru : S.col_rel + t.rl;
+  const int32_t* const g_ksn = side ? S.row_sn + t.ru : S.col_sn + t.rl;
+  const int O = nr * nw;
+  const int kg = O * 2 <= NT ? min(min(NT / O, 8), kt) : 1;
+  const int g = kg > 1 ? tid / O : 0;
+  // outputs of the warp's threads (uniform over the warp: out-of-range lanes
+  // repeat the last output)
+  const int wbase = tid & ~31;
+  const int cnt = kg > 1 ? (g < kg) : (wbase < O ? (O - wbase + NT - 1) / NT : 0);
+  int er[NC], ej[NC];
+#pragma unroll
+  for (int i = 0; i < NC; i++) {
+    const int e = min((kg > 1 ? tid - g * O : tid) + i * NT, O - 1);
+    ej[i] = (int)(e * mr >> 16);
+    er[i] = e - ej[i] * nr;
+  }
+  for (int inst = blockIdx.y; inst < nbatch; inst += gridDim.y) {
+    const int64_t base = (int64_t)inst * S.storage;
+    const T* const src = store + base;
+    const int64_t so = base + t.off, lo = so + (int64_t)s * s, uo = lo + (int64_t)t.c * s;
+    const T* const B = nf + (side ? uo : lo) + (int64_t)t.j0 * kt;
+    const T* const U4 = nf + (sym ? lo : uo) + t.r0;
+    const int ld4 = t.cu;
+    int64_t t_diag = 0, t_pan = 0, t_rel = 0;
+    int t_sn = 0;
+    T breg[NB], va[NG], vb[NG];  // vb: entries stored along k
+    unsigned have = 0;           // entries of va (bits 0 ..) and vb (bits 16 ..) in flight
+    auto load_bases = [&](int k0) {
+      const int k = k0 + tid;
+      if (tid >= kc || k >= kt) return;
+      t_pan = g_kpan[k];
+      t_rel = g_krel[k];
+      t_sn = g_ksn[k];
+      if (!side) t_diag = S.col_diag[t.rl + k];
+    };
+    auto store_bases = [&](int buf) {
+      if (tid >= kc) return;
+      kpan[buf][tid] = t_pan;
+      krel[buf][tid] = t_rel;
+      ksn[buf][tid] = t_sn;
+      kdiag[buf][tid] = t_diag;
+    };
+    auto load_b = [&](int k0) {
+      const int kn = min(kc, kt - k0);
+      const unsigned mk = (65536u + kn - 1) / kn;
+#pragma unroll
+      for (int i = 0; i < NB; i++) {
+        const int e = tid + i * NT, j = (int)(e * mk >> 16), k = e - j * kn;
+        if (j < nw) breg[i] = B[k0 + k + (int64_t)j * kt];
       }
-      G[p + q * ldg] = v;
-    }
-    __syncthreads();
-    // steps 3 and 5
-    for (int e = threadIdx.x; e < c * w; e += blockDim.x) {
-      const int p = e % c, j = j0 + e / c;
-      T a = sc_zero(T()), b = sc_zero(T());
-      for (int q = 0; q < c; q++) {
-        a = fma_s(G[p + q * ldg], Lh[q + j * c], a);
-        if (!sym) b = fma_s(G[q + p * ldg], Uh[q + j * c], b);
+    };
+    // the chunk's entries of G into registers: (r, k) is stored with r's block
+    // (contiguous along k) or with k's (contiguous along r)
+    auto slot_of = [&](bool with_r, int r, int k, int k0, int buf) -> int64_t {
+      const int64_t ri = with_r ? rrel[r] + k0 + k : krel[buf][k] + t.r0 + r;
+      if (S.check && (ri < 0 || ri >= S.relidx_size)) return -1;
+      const bool dg = rsn[r] == ksn[buf][k];
+      return (with_r ? (dg ? rdiag[r] : rpan[r]) : (dg ? kdiag[buf][k] : kpan[buf][k])) +
+             S.relidx[ri];
+    };
+    auto gather = [&](int k0, int buf) {
+      const int kn = min(kc, kt - k0), n = nr * kn;
+      const unsigned mk = (65536u + kn - 1) / kn;
+      // positions ascend with the supernodes: side 0 stores (r, k) with r where
+      // k's supernode is the later one, side 1 where it is not the earlier one
+      const int rf = rsn[0], rl = rsn[nr - 1], kf = ksn[buf][0], kl = ksn[buf][kn - 1];
+      const bool any_r = side ? rf <= kl : kl > rf, any_k = side ? rl > kf : kf <= rl;
+      int64_t slot[2 * NG];
+      have = 0;
+#pragma unroll
+      for (int u = 0; u < 2 * NG; u++) {
+        const bool with_r = u >= NG;
+        slot[u] = -1;
+        if (with_r ? !any_r : !any_k) continue;
+        const int e = tid + (u % NG) * NT;
+        if (e >= n) continue;
+        const int hi = (int)(e * (with_r ? mk : mr) >> 16), lw = e - hi * (with_r ? kn : nr);
+        const int r = with_r ? hi : lw, k = with_r ? lw : hi;
+        const int a = rsn[r], b = ksn[buf][k];
+        if ((side ? a <= b : b > a) != with_r) continue;
+        slot[u] = slot_of(with_r, r, k, k0, buf);
+        if (S.check && (slot[u] < 0 || slot[u] >= S.storage)) {
+          set_error(S.err, DEV_CHECK, t.K);
+          slot[u] = 0;
+        }
+        have |= 1u << (with_r ? 16 + u - NG : u);
       }
-      a = scale_s(a, -1.0);
-      X[e] = a;
-      store[lo + p + (int64_t)j * c] = a;
-      store[uo + p + (int64_t)j * c] = sym ? a : scale_s(b, -1.0);
+#pragma unroll
+      for (int u = 0; u < NG; u++) {
+        if (slot[u] >= 0) va[u] = src[slot[u]];
+        if (slot[NG + u] >= 0) vb[u] = src[slot[NG + u]];
+      }
+    };
+    load_bases(0);
+    load_b(0);
+    if (tid < nr) {
+      rpan[tid] = (side ? S.col_pan + t.rl : S.row_pan + t.ru)[t.r0 + tid];
+      rrel[tid] = (side ? S.col_rel + t.rl : S.row_rel + t.ru)[t.r0 + tid];
+      rsn[tid] = (side ? S.col_sn + t.rl : S.row_sn + t.ru)[t.r0 + tid];
+      if (side) rdiag[tid] = S.col_diag[t.rl + t.r0 + tid];
     }
+    if (!side)
+      for (int e = tid; e < nr * si; e += NT) {
+        const int i = (int)(e * mr >> 16), r = e - i * nr;
+        sU[i * ldr + r] = U4[r + (int64_t)i * ld4];
+      }
+    store_bases(0);
     __syncthreads();
-    // step 4 (symmetric A: Uhat^T = Lhat)
-    const T* A4 = sym ? Lh : Uh;
-    for (int e = threadIdx.x; e < s * w; e += blockDim.x) {
-      const int i = e % s, jj = e / s;
-      T a = sc_zero(T());
-      for (int q = 0; q < c; q++) a = fma_s(A4[q + i * c], X[q + jj * c], a);
-      T* d = store + so + i + (int64_t)(j0 + jj) * s;
-      *d = sub_s(*d, a);
+    gather(0, 0);
+    load_bases(kc);
+    T acc[NC];
+#pragma unroll
+    for (int i = 0; i < NC; i++) acc[i] = sc_zero(T());
+    for (int k0 = 0, buf = 0; k0 < kt; k0 += kc, buf ^= 1) {
+      const int kn = min(kc, kt - k0);
+      const unsigned mk = (65536u + kn - 1) / kn;
+#pragma unroll
+      for (int i = 0; i < NB; i++) {
+        const int e = tid + i * NT, j = (int)(e * mk >> 16), k = e - j * kn;
+        if (j < nw) sB[k * ldw + j] = breg[i];
+      }
+#pragma unroll
+      for (int u = 0; u < NG; u++) {
+        const int e = tid + u * NT;
+        if (have >> u & 1) {
+          const int k = (int)(e * mr >> 16), r = e - k * nr;
+          sG[k * ldr + r] = va[u];
+        }
+        if (have >> (16 + u) & 1) {
+          const int r = (int)(e * mk >> 16), k = e - r * kn;
+          sG[k * ldr + r] = vb[u];
+        }
+      }
+      store_bases(buf ^ 1);
+      __syncthreads();
+      if (k0 + kc < kt) {
+        gather(k0 + kc, buf ^ 1);
+        load_b(k0 + kc);
+        load_bases(k0 + 2 * kc);
+      }
+      auto dots = [&](auto count) {
+        constexpr int C = decltype(count)::value;
+        const T* pg = sG + g * ldr;
+        const T* pb = sB + g * ldw;
+#pragma unroll 4
+        for (int k = g; k < kn; k += kg) {
+#pragma unroll
+          for (int i = 0; i < C; i++) acc[i] = fma_s(pg[er[i]], pb[ej[i]], acc[i]);
+          pg += kg * ldr;
+          pb += kg * ldw;
+        }
+      };
+      if (cnt == 1) dots(std::integral_constant<int, 1>());
+      else if (cnt == 2) dots(std::integral_constant<int, 2>());
+      __syncthreads();
+    }
+    if (kg > 1) {
+      if (g < kg) sX[tid] = acc[0];
+      __syncthreads();
+      if (tid < O)
+        for (int i = 1; i < kg; i++) acc[0] = add_s(acc[0], sX[i * O + tid]);
+      __syncthreads();
+    }
+    {
+      const int ldo = side ? t.c : t.cu;
+      T* out = store + (side != (S.general != 0) ? uo : lo) + t.r0 + (int64_t)t.j0 * ldo;
+      T* out2 = store + uo + t.r0 + (int64_t)t.j0 * ldo;
+#pragma unroll
+      for (int i = 0; i < NC; i++) {
+        const int e = tid + i * NT;
+        if (e >= O) break;
+        const int j = (int)(e * mr >> 16), r = e - j * nr;
+        const T x = scale_s(acc[i], -1.0);
+        out[r + (int64_t)j * ldo] = x;
+        if (sym) out2[r + (int64_t)j * ldo] = x;
+        sX[j * ldr + r] = x;
+      }
+    }
+    if (!side) {
+      // step 4: i0 .. i0 + in - 1 of the diagonal block's rows at a time
+      for (int i0 = 0; i0 < s; i0 += si) {
+        const int in = min(si, s - i0);
+        if (i0 > 0) {
+          __syncthreads();
+          for (int e = tid; e < nr * in; e += NT) {
+            const int i = (int)(e * mr >> 16), r = e - i * nr;
+            sU[i * ldr + r] = U4[r + (int64_t)(i0 + i) * ld4];
+          }
+        }
+        __syncthreads();
+        const unsigned mi = (65536u + in - 1) / in;
+        const int n4 = in * nw, rg = n4 * 2 <= NT ? min(min(NT / n4, 4), nr) : 1;
+        T* const D = store + so + i0 + (int64_t)t.j0 * s;
+        for (int e4 = tid; e4 < n4 * rg; e4 += NT) {
+          const int grp = rg > 1 ? e4 / n4 : 0, e = e4 - grp * n4;
+          const int j = (int)(e * mi >> 16), i = e - j * in;
+          T a = sc_zero(T()), b = sc_zero(T());
+          const T* pu = sU + i * ldr;
+          const T* px = sX + j * ldr;
+          int r = grp;
+          for (; r + rg < nr; r += 2 * rg) {
+            a = fma_s(pu[r], px[r], a);
+            b = fma_s(pu[r + rg], px[r + rg], b);
+          }
+          if (r < nr) a = fma_s(pu[r], px[r], a);
+          atomic_add_s(D + i + (int64_t)j * s, scale_s(add_s(a, b), -1.0));
+        }
+      }
     }
     __syncthreads();
   }
@@ -663,30 +818,26 @@ void launch_scatter_values(int dtype, const SymDev& S, const void* values, void*
         S, (const cdouble*)values, (cdouble*)store, total);
 }
 
-size_t small_level_smem(int dtype, int c, int s, int w, int nblk, int seg) {
-  const size_t ibytes = ((size_t)nblk * 20 + (size_t)(c + seg) * 4 + 15) & ~size_t(15);
-  return ibytes + (size_t)((int64_t)(c | 1) * c + 2 * (int64_t)c * s + (int64_t)c * w) *
-                      (dtype == DT_F64 ? 8 : 16);
+size_t small_level_smem(int dtype, const LevelTask& t) {
+  const int kt = t.side ? t.cu : t.c, kc = kt < kLevelK ? kt : kLevelK, si = t.s < kLevelK ? t.s : kLevelK;
+  const int ldr = t.nr | 1, ldw = t.nw | 1;
+  // the partial sums of kg <= 8 groups (at most 256 of them) share the tile X
+  const int part = 8 * t.nr * t.nw < 256 ? 8 * t.nr * t.nw : 256;
+  const int x = ldr * t.nw > part ? ldr * t.nw : part;
+  return (size_t)(kc * ldr + kc * ldw + si * ldr + x) * (dtype == DT_F64 ? 8 : 16);
 }
 
-cudaError_t prepare_map_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(small_level_kernel<double>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kSmallLevelMaxSmem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(small_level_kernel<cdouble>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallLevelMaxSmem);
-}
-
-void launch_small_level(int dtype, const SymDev& S, void* store, const void* nf, const SnTask* tasks,
-                        int ntasks, size_t smem, int sym, cudaStream_t st) {
+void launch_small_level(int dtype, const SymDev& S, void* store, const void* nf,
+                        const LevelTask* tasks, int ntasks, int nbatch, size_t smem, int sym,
+                        cudaStream_t st) {
   if (ntasks <= 0) return;
+  const dim3 grid((unsigned)ntasks, (unsigned)(nbatch < 65535 ? nbatch : 65535));
   if (dtype == DT_F64)
-    small_level_kernel<double><<<ntasks, kThreads, smem, st>>>(S, (double*)store, (const double*)nf,
-                                                               tasks, ntasks, sym);
+    small_level_kernel<double><<<grid, kLevelThreads, smem, st>>>(
+        S, (double*)store, (const double*)nf, tasks, nbatch, sym);
   else
-    small_level_kernel<cdouble><<<ntasks, kThreads, smem, st>>>(S, (cdouble*)store,
-                                                                (const cdouble*)nf, tasks, ntasks, sym);
+    small_level_kernel<cdouble><<<grid, kLevelThreads, smem, st>>>(
+        S, (cdouble*)store, (const cdouble*)nf, tasks, nbatch, sym);
 }
 
 void launch_gather(int dtype, const SymDev& S, const void* store, void* out, const int64_t* gofs,
