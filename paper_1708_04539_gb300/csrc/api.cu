@@ -64,7 +64,7 @@ enum StepKind {
 
 struct Step {
   StepKind kind;
-  int cfg = 0;    // GEMM: kernel config; LU_PANEL: line groups of a task; SLICE: 1 maxima pass;
+  int cfg = 0;    // GEMM: kernel config; LU_PANEL: lines of a task; SLICE: 1 maxima pass;
                   // OZGEMM: slices; SMALL_LEVEL: shared-memory bytes of a CTA
   int n = 0;      // tasks / segments
   int n2 = 0;     // GSLICE: ordinary slice tasks after the n G tiles; LU_PANEL: 1 panel solves
@@ -666,26 +666,33 @@ int choose_small_tile(int dtype, const std::vector<GemmDesc>& descs) {
   return tiles < 2 * 152 ? GEMM_16x16 : GEMM_32x32;
 }
 
-// One launch of panel tasks (32 lines each).  More than two per SM: tasks of
-// 32 kLuGroups lines, so that the pivot block is factored less often (from one
-// per SM on: 40^3 upwind factorisation 12.45 against 12.1 ms).
-void add_panel_step(Plan& P, const std::vector<LuTask>& tasks, int level, bool solve) {
+// Bulk Schur work (in the 36 us of 2 M entries) from which the LU panels beside
+// it keep to 32 lines a task: they share the SMs that its sliced products leave
+// (8^3 x 64 DG solve 50.0 ms with fewer lines everywhere, 49.0 so; 40^3 upwind,
+// below it, 16.4 against 16.1)
+constexpr double kCrowdedBulk = 8.0;
+
+// One launch of panel tasks (given with 32 lines each).  More than two per SM:
+// tasks of 32 kLuGroups lines, so that the pivot block is factored less often
+// (from one per SM on: 40^3 upwind factorisation 12.45 against 12.1 ms).  Where
+// 16 or 8 lines a task still leave one task per SM: that many, with two or four
+// lanes a line, as the lines' instructions share the pivot block's schedulers.
+void add_panel_step(Plan& P, const std::vector<LuTask>& tasks, int level, bool solve, bool crowded) {
   if (tasks.empty()) return;
   Step d;
   d.kind = ST_LU_PANEL;
   d.n2 = solve ? 1 : 0;  // narrow supernodes: their panels' rows are among the lines
-  d.cfg = tasks.size() > 2 * 152 ? kLuGroups : 1;
+  const size_t n = tasks.size();
+  d.cfg = n > 2 * 152 ? 32 * kLuGroups : crowded || n > 152 / 2 ? 32 : n > 152 / 4 ? 16 : 8;
   d.level = level;
-  if (d.cfg == 1) {
-    d.n = (int)tasks.size();
-    d.tasks = P.push(tasks);
-  } else {
-    std::vector<LuTask> grouped;
-    for (const LuTask& t : tasks)
-      if (t.line0 % (32 * kLuGroups) == 0) grouped.push_back(t);
-    d.n = (int)grouped.size();
-    d.tasks = P.push(grouped);
+  std::vector<LuTask> out;
+  for (const LuTask& t : tasks) {
+    if (t.line0 % std::max(32, d.cfg) != 0) continue;
+    for (int l = 0; l < 32; l += std::min(32, d.cfg))
+      out.push_back({t.inst, t.K, t.j0, t.line0 + l});
   }
+  d.n = (int)out.size();
+  d.tasks = P.push(out);
   P.steps.push_back(d);
 }
 
@@ -838,7 +845,10 @@ int build_factor_plan(pselinv_ctx* h) {
   //   inverse_ready: this level's inverses; bulk_ready: the level below's rest.
   // Both are waited for by the next main-stream step that is not an LU panel
   // (a later event of the same stream stands for an earlier one).
+  // crowded: that rest takes longer than the LU beside it and its sliced
+  // products leave few SMs.
   int inverse_ready = -1, bulk_ready = -1;
+  bool crowded = false;
   auto wait_pending = [&](size_t from) {
     for (size_t i = from; i < P.steps.size() && (inverse_ready >= 0 || bulk_ready >= 0); i++)
       if (P.steps[i].side == 0) {
@@ -953,7 +963,7 @@ int build_factor_plan(pselinv_ctx* h) {
     if (bulk_ready >= 0 && !panels.empty()) {
       // panels of narrow supernodes take updates of the rest: behind it
       const size_t first = P.steps.size();
-      add_panel_step(P, solving, (int)lev, true);
+      add_panel_step(P, solving, (int)lev, true, crowded);
       if (P.steps.size() > first) {
         P.steps.back().side = 2;
         bulk_ready = event((int)lev, kEvSolved);
@@ -980,7 +990,7 @@ int build_factor_plan(pselinv_ctx* h) {
                                   (int)w, (int)s, (int)s, (int)s, 0, 0, -1.0, 1.0));
         }
       }
-      add_panel_step(P, panels, (int)lev, !split);
+      add_panel_step(P, panels, (int)lev, !split, bulk_ready >= 0 && crowded);
       if (wide.empty()) wait_pending(at);  // (panel solves among them)
       at = P.steps.size();
       if (!wide.empty()) {  // side stream: block row p of the inverses, inner products of p + 1
@@ -1059,6 +1069,7 @@ int build_factor_plan(pselinv_ctx* h) {
         wide_next = wide_next || H.sn_width[H.hlevel_sn[i]] > 2 * kLuPanel;
     const double bulk = split ? (double)entries * (dt == DT_F64 ? 1.0 : 2.0) * (ldlt ? 0.5 : 1.0) / 2e6
                               : ops * 16.0 / 152.0 / 72e3;
+    crowded = split && bulk >= kCrowdedBulk;
     if (!H.general && wide_next && bulk >= 1.0) {
       size_t last = P.steps.size() - 1;  // the operands are there after the last main step
       while (last > 0 && P.steps[last].side != 0) last--;

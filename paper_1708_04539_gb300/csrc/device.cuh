@@ -183,7 +183,7 @@ struct SnTask {
   int inst, K, a, b;
 };
 
-// panel step of the diagonal LU: 32-column panels, tasks of 32 or
+// panel step of the diagonal LU: 32-column panels, tasks of 8, 16, 32 or
 // 32 kLuGroups lines (see lu_panel_kernel)
 constexpr int kLuPanel = 32;
 constexpr int kLuGroups = 3;
@@ -344,12 +344,11 @@ size_t trace_partial_bytes();
 // value scatter (A's entries into the storage of every instance)
 void launch_scatter_values(int dtype, const SymDev& S, const void* values, void* store,
                            int nbatch, cudaStream_t st);
-// one panel step of the blocked diagonal LU (one CTA per task; groups = 1 or
-// kLuGroups: 32 or 32 kLuGroups lines per task; solve: narrow supernodes'
-// panels too; sym: symmetric values), and the factored pivot blocks into the
+// one panel step of the blocked diagonal LU (one CTA per task of `lines` = 8,
+// 16, 32 or 32 kLuGroups lines; solve: narrow supernodes' panels too; sym: symmetric values), and the factored pivot blocks into the
 // storage
 void launch_lu_panel(int dtype, const SymDev& S, void* store, void* winv, void* piv,
-                     const LuTask* tasks, int ntasks, int groups, bool solve, bool sym,
+                     const LuTask* tasks, int ntasks, int lines, bool solve, bool sym,
                      cudaStream_t st);
 void launch_unpack_pivots(int dtype, const SymDev& S, void* store, const void* piv, int nbatch,
                           cudaStream_t st);

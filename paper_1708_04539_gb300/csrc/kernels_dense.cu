@@ -9,6 +9,7 @@
 // it saturates the FP64 pipe with a 16x16 thread grid and 4x4 (real) or
 // 2x2 (complex) outputs per thread.
 #include <algorithm>
+#include <type_traits>
 
 #include "device.cuh"
 
@@ -159,8 +160,14 @@ gemm_kernel(const GemmDesc* __restrict__ descs, const GemmTask* __restrict__ tas
 // updates column k + 1, computes its reciprocal and the scaled column of L;
 // the others apply step k to the columns behind it and publish row k + 1,
 // column k + 2 and the lines' entries k + 1.
-// Bound: the pivot chain (five dependent FP64 operations and a barrier per
-// column) and, about as long, the FP64 pipe.
+// P > 1: 32 / P lines a team and P lanes a line, columns dealt over 3 P lanes.  The
+// lines' instructions share three schedulers with the pivot block's (a wide
+// block's 32 lines: 22 FP64 instructions a warp in the first step), and a launch
+// of a few blocks leaves most SMs idle: 8 lines a task there, 16 where 8 would
+// give more than one task per SM (256 wide block, one panel: real 25.1 -> 22.0 us,
+// complex 57 -> 49; 127^2 grid solve 1.93 -> 1.77 ms, 40^3 upwind 16.9 -> 16.1).
+// Bound: the pivot chain (three dependent FP64 operations, a reciprocal and a
+// barrier per column) and, about as long, the FP64 pipe.
 template <typename T>
 __device__ __forceinline__ T shfl_t(T v, int src);
 template <>
@@ -171,18 +178,34 @@ template <>
 __device__ __forceinline__ cdouble shfl_t(cdouble v, int src) {
   return {__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src)};
 }
-// 1 / d: the approximate reciprocal (relative error e below 2^-19) and one
-// third-order step r (1 + e + e^2) of the Householder family, three dependent
-// operations against about nine of a division; within 2^-52 of 1 / d over
-// 10^8 random mantissas.  Numbers near the ends of the range, zeros and
-// non-finite ones take the division.
+// 1 / d in integers, as the pivot chain waits for it and an FP64 instruction
+// takes 64 to 133 cycles there (three of them: 27.1 us a panel of a wide block;
+// this: 25.1).  y = Y 2^-24: the FP32 reciprocal of the mantissa's
+// leading bits; its residual e = 1 - m y (|e| < 2^-21, units 2^-76) is exact,
+// and y (1 + e + e^2) is one third-order step of the Householder family, off by
+// e^3 < 2^-63; then rounded to nearest.  Half a unit of the last place and 2^-62
+// over 3 10^7 random and near-power-of-two mantissas with y moved by a unit
+// either way.  Numbers near the ends of the range, zeros and non-finite ones
+// take the division.
 __device__ __forceinline__ double rcp_s(double d) {
-  const int e = (__double2hiint(d) >> 20) & 0x7FF;
-  if (e < 64 || e > 1982) return 1.0 / d;
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  const double h = fma(-d, r, 1.0);
-  return fma(r, fma(h, h, h), r);
+  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+  const uint32_t E = (hi >> 20) & 0x7FFu;
+  if (E < 64u || E > 1982u) return 1.0 / d;
+  float yf;
+  asm("rcp.approx.ftz.f32 %0, %1;"
+      : "=f"(yf)
+      : "f"(__uint_as_float(0x3F800000u | (((hi << 3) | (lo >> 29)) & 0x7FFFFFu))));
+  yf = fminf(fmaxf(yf, 0.5f), 0.99999994f);
+  const uint32_t Y = (__float_as_uint(yf) & 0x7FFFFFu) | 0x800000u;
+  const uint64_t M = ((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
+  const int64_t e = -(int64_t)(M * Y);  // 2^76 - M Y, which fits 64 bits
+  const int64_t eh = (int32_t)(e >> 32);
+  const int64_t c = e + ((eh * eh) >> 12);
+  const int64_t yc = (int64_t)(int32_t)(c >> 32) * (int64_t)Y +
+                     (int64_t)(((uint64_t)(uint32_t)c * Y) >> 32);  // units 2^-68
+  const uint64_t r = ((uint64_t)Y << 40) + (uint64_t)(yc >> 4);       // units 2^-64
+  const uint64_t bits = ((uint64_t)(2044u - E) << 52) + (r >> 11) + ((r >> 10) & 1u);
+  return __longlong_as_double((long long)(bits | ((uint64_t)(hi & 0x80000000u) << 32)));
 }
 __device__ __forceinline__ cdouble rcp_s(cdouble b) {
   const int ex = (__double2hiint(b.x) >> 20) & 0x7FF, ey = (__double2hiint(b.y) >> 20) & 0x7FF;
@@ -197,16 +220,19 @@ __device__ __forceinline__ cdouble fnma_s(cdouble a, cdouble b, cdouble c) {
 }
 
 constexpr int kLuW = kLuPanel;  // panel width
-template <typename T, int G>
+// lines of a task: G teams of 32 / P lines, P lanes a line
+template <int G, int P>
+constexpr int kLuLines = 32 / P * G;
+template <typename T, int G, int P>
 __global__ void __launch_bounds__(128 * (G + 1))
 lu_panel_kernel(SymDev S, T* store, T* winv, T* piv, const LuTask* __restrict__ tasks, int solve,
                 int sym) {
-  constexpr int kThr = 128 * (G + 1);
+  constexpr int kThr = 128 * (G + 1), kLines = kLuLines<G, P>;
   extern __shared__ __align__(16) unsigned char lu_smem[];
   T(*Dd)[kLuW + 1] = reinterpret_cast<T(*)[kLuW + 1]>(lu_smem);  // A11, then the rows of U11
   T(*Ls)[kLuW + 1] = Dd + kLuW;                                  // scaled columns of L11
   T(*X)[kLuW + 1] = Ls + kLuW;                                   // lines (unscaled)
-  T* R = reinterpret_cast<T*>(X + 32 * G);                       // reciprocals of the pivots
+  T* R = reinterpret_cast<T*>(X + kLines);                       // reciprocals of the pivots
   T(*Cn)[kLuW] = reinterpret_cast<T(*)[kLuW]>(R + kLuW);         // the chain's next column
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int team = warp >> 2, q = (warp & 3) - 1;  // q = -1: the chain (warp 0) or idle
@@ -235,8 +261,8 @@ lu_panel_kernel(SymDev S, T* store, T* winv, T* piv, const LuTask* __restrict__ 
   }
   // lines: lanes along the lines (contiguous), except the columns of U12 of a
   // wide block, contiguous along k
-  for (int e = tid; e < 32 * G * kLuW; e += kThr) {
-    const int i = e % (32 * G), k = e / (32 * G), l = task.line0 + i;
+  for (int e = tid; e < kLines * kLuW; e += kThr) {
+    const int i = e % kLines, k = e / kLines, l = task.line0 + i;
     if (l >= nlines || k >= w) {
       X[i][k] = sc_zero(T());
     } else if (l < nl) {
@@ -249,16 +275,11 @@ lu_panel_kernel(SymDev S, T* store, T* winv, T* piv, const LuTask* __restrict__ 
     }
   }
   if (!narrow)
-    for (int e = tid; e < 32 * G * kLuW; e += kThr) {
+    for (int e = tid; e < kLines * kLuW; e += kThr) {
       const int k = e & 31, i = e >> 5, l = task.line0 + i;
       if (l >= nl && l < nl + nu && k < w) X[i][k] = Ub[(l - nl) * us + k * uk];
     }
   __syncthreads();
-  const int row = team == 0 ? lane : 32 * (team - 1) + lane;  // row of Dd or of X
-  // a line's multiplier and coefficients: L lines (and unit rows) x_k r_k and
-  // row k of U11, U lines (and unit columns) x_k and column k of L11
-  const int line = task.line0 + row;
-  const bool is_l = team > 0 && (line < nl || (line >= nl + nu && line < nl + nu + w));
   if (warp == 0) {
     T v = Dd[lane][0], l = sc_zero(T());
     for (int k = 0; k < w; k++) {
@@ -275,83 +296,107 @@ lu_panel_kernel(SymDev S, T* store, T* winv, T* piv, const LuTask* __restrict__ 
       }
       __syncthreads();
     }
-  } else if (q < 0 || (team > 0 && task.line0 + 32 * (team - 1) >= nlines)) {
+  } else if (q < 0 || (team > 0 && task.line0 + 32 / P * (team - 1) >= nlines)) {
     for (int k = 0; k < w; k++) __syncthreads();  // a scheduler's spare warp, or no lines left
   } else {
-    constexpr int kCols = (kLuW + 2) / 3;
     const T* sm = reinterpret_cast<const T*>(lu_smem);
-    const bool from_u = team == 0 || is_l;  // coefficients from the rows of U11
-    const int cbase = from_u ? 0 : kLuW * (kLuW + 1);
-    const int cj = from_u ? 1 : kLuW + 1, ck = from_u ? kLuW + 1 : 1;  // strides along j and k
-    const bool warp_l = __any_sync(0xffffffffu, is_l);
-    // a[jj] holds column 3 (t + jj) + q in round t (columns past the panel hold
-    // values nobody uses)
-    T a[kCols];
+    constexpr int kEither = 0, kPivot = 1, kLine = 2;
+    // the pivot block's warps (one lane a row), a team's (PL lanes a line), or
+    // both from one loop: complex values at one lane a line, whose two copies
+    // would be slower (pole solve 17.0 against 16.8 ms; real values the other way
+    // round: 8^3 x 64 DG 48.95 against 49.3)
+    auto eliminate = [&](auto who, auto lanes) {
+      constexpr int kWho = decltype(who)::value;
+      const bool piv = kWho == kEither ? team == 0 : kWho == kPivot;
+      constexpr int PL = decltype(lanes)::value;
+      constexpr int kCyc = 3 * PL, kCols = (kLuW + kCyc - 1) / kCyc;
+      // row of Dd or of X; first column (columns qq, qq + kCyc, ...)
+      const int row = piv ? lane : 32 / PL * (team - 1) + lane % (32 / PL);
+      const int qq = q + 3 * (lane / (32 / PL));
+      // a line's multiplier and coefficients: L lines (and unit rows) x_k r_k
+      // and row k of U11, U lines (and unit columns) x_k and column k of L11
+      const int line = task.line0 + row;
+      const bool is_l = !piv && (line < nl || (line >= nl + nu && line < nl + nu + w));
+      const bool from_u = piv || is_l;  // coefficients from the rows of U11
+      const int cbase = from_u ? 0 : kLuW * (kLuW + 1);
+      const int cj = from_u ? 1 : kLuW + 1, ck = from_u ? kLuW + 1 : 1;  // strides along j and k
+      const bool warp_l = __any_sync(0xffffffffu, is_l);
+      // a[jj] holds column kCyc (t + jj) + qq in round t (columns past the panel
+      // hold values nobody uses)
+      T a[kCols];
 #pragma unroll
-    for (int jj = 0; jj < kCols; jj++) {
-      const int j = min(3 * jj + q, kLuW - 1);
-      a[jj] = team == 0 ? Dd[row][j] : X[row][j];
-    }
-    const int nr = (w + 2) / 3;
-    for (int t = 0; t < nr; t++) {
-      const int nj = nr - t;  // columns of this warp still in the panel
-#pragma unroll
-      for (int kk = 0; kk < 3; kk++) {
-        const int k = 3 * t + kk;
-        if (k >= w) break;
-        __syncthreads();  // row k of U11, column k of L11, r_k and x_k are in place
-        // (rows <= k of the pivot block are final and published: their lanes run along)
-        T m = team == 0 ? Ls[lane][k] : X[row][k];
-        if (warp_l) {
-          const T ml = mul_s(m, R[k]);
-          if (is_l) m = ml;
-        }
-        const T* cp = sm + cbase + (3 * t + q) * cj + k * ck;
-        // team 0 publishes column k + 2 for the chain (which has column k + 1
-        // itself), the lines their entry k + 1
-        const int ahead = team == 0 ? 2 : 1;
-        if (q - kk >= ahead) {
-          a[0] = fnma_s(m, cp[0], a[0]);
-          if (q - kk == ahead) {
-            if (team == 0) Cn[k & 1][lane] = a[0];
-            else X[row][k + 1] = a[0];
-          }
-        }
-        if (nj > 1 && q + 3 - kk >= ahead) {
-          a[1] = fnma_s(m, cp[3 * cj], a[1]);
-          if (q + 3 - kk == ahead) {
-            if (team == 0) Cn[k & 1][lane] = a[1];
-            else X[row][k + 1] = a[1];
-          }
-        }
-        // (jumps out: a predicated-off FP64 instruction still takes its 64 cycles)
-#pragma unroll
-        for (int jj = 2; jj < kCols; jj++) {
-          if (jj >= nj) break;
-          a[jj] = fnma_s(m, cp[3 * jj * cj], a[jj]);
-        }
-        if (team == 0 && lane == k + 1) {  // row k + 1 of U11 right of its diagonal is final
-#pragma unroll
-          for (int jj = 0; jj < kCols; jj++) {
-            const int j = 3 * (t + jj) + q;
-            if (jj < nj && j > k + 1) Dd[k + 1][j] = a[jj];
-          }
-        }
+      for (int jj = 0; jj < kCols; jj++) {
+        const int j = min(kCyc * jj + qq, kLuW - 1);
+        a[jj] = piv ? Dd[row][j] : X[row][j];
       }
+      const int nr = (w + kCyc - 1) / kCyc;
+      for (int t = 0; t < nr; t++) {
+        const int nj = nr - t;  // columns of this lane still in the panel
 #pragma unroll
-      for (int jj = 0; jj + 1 < kCols; jj++) a[jj] = a[jj + 1];
+        for (int kk = 0; kk < kCyc; kk++) {
+          const int k = kCyc * t + kk;
+          if (k >= w) break;
+          __syncthreads();  // row k of U11, column k of L11, r_k and x_k are in place
+          // (rows <= k of the pivot block are final and published: their lanes run along)
+          T m = piv ? Ls[lane][k] : X[row][k];
+          if (warp_l) {
+            const T ml = mul_s(m, R[k]);
+            if (is_l) m = ml;
+          }
+          const T* cp = sm + cbase + (kCyc * t + qq) * cj + k * ck;
+          // the pivot block's warps publish column k + 2 for the chain (which
+          // has column k + 1 itself), the lines their entry k + 1
+          const int ahead = piv ? 2 : 1;
+          if (qq - kk >= ahead) {
+            a[0] = fnma_s(m, cp[0], a[0]);
+            if (qq - kk == ahead) {
+              if (piv) Cn[k & 1][lane] = a[0];
+              else X[row][k + 1] = a[0];
+            }
+          }
+          if (nj > 1 && qq + kCyc - kk >= ahead) {
+            a[1] = fnma_s(m, cp[kCyc * cj], a[1]);
+            if (qq + kCyc - kk == ahead) {
+              if (piv) Cn[k & 1][lane] = a[1];
+              else X[row][k + 1] = a[1];
+            }
+          }
+          // (jumps out: a predicated-off FP64 instruction still takes its 64 cycles)
+#pragma unroll
+          for (int jj = 2; jj < kCols; jj++) {
+            if (jj >= nj) break;
+            a[jj] = fnma_s(m, cp[kCyc * jj * cj], a[jj]);
+          }
+          if (piv && lane == k + 1) {  // row k + 1 of U11 right of its diagonal is final
+#pragma unroll
+            for (int jj = 0; jj < kCols; jj++) {
+              const int j = kCyc * (t + jj) + qq;
+              if (jj < nj && j > k + 1) Dd[k + 1][j] = a[jj];
+            }
+          }
+        }
+#pragma unroll
+        for (int jj = 0; jj + 1 < kCols; jj++) a[jj] = a[jj + 1];
+      }
+    };
+    using One = std::integral_constant<int, 1>;
+    if constexpr (P == 1 && sizeof(T) == 16) {
+      eliminate(std::integral_constant<int, kEither>(), One());
+    } else {
+      if (team == 0) eliminate(std::integral_constant<int, kPivot>(), One());
+      else eliminate(std::integral_constant<int, kLine>(), std::integral_constant<int, P>());
     }
   }
   __syncthreads();
   if (task.line0 == 0) {
-    T* P = piv + ((int64_t)task.inst * S.n + S.sn_first[K] + j0) * kLuW;
+    T* Pv = piv + ((int64_t)task.inst * S.n + S.sn_first[K] + j0) * kLuW;
     for (int e = tid; e < w * w; e += kThr) {
       const int i = e % w, j = e / w;
-      P[i + j * kLuW] = i <= j ? Dd[i][j] : Ls[i][j];
+      Pv[i + j * kLuW] = i <= j ? Dd[i][j] : Ls[i][j];
     }
   }
-  for (int e = tid; e < 32 * G * kLuW; e += kThr) {
-    const int i = e % (32 * G), k = e / (32 * G), l = task.line0 + i;
+  for (int e = tid; e < kLines * kLuW; e += kThr) {
+    const int i = e % kLines, k = e / kLines, l = task.line0 + i;
     if (l >= nlines || k >= w) continue;
     const T x = X[i][k];
     if (l < nl) {
@@ -368,7 +413,7 @@ lu_panel_kernel(SymDev S, T* store, T* winv, T* piv, const LuTask* __restrict__ 
     }
   }
   if (!narrow)
-    for (int e = tid; e < 32 * G * kLuW; e += kThr) {
+    for (int e = tid; e < kLines * kLuW; e += kThr) {
       const int k = e & 31, i = e >> 5, l = task.line0 + i;
       if (l >= nl && l < nl + nu && k < w) Ub[(l - nl) * us + k * uk] = X[i][k];
     }
@@ -556,29 +601,41 @@ void launch_gemm(int dtype, int cfg, const GemmDesc* descs, const GemmTask* task
 }
 
 namespace {
-template <typename T, int G>
+template <typename T, int G, int P>
 constexpr int lu_smem_bytes() {
-  return (int)sizeof(T) * ((2 + G) * kLuW * (kLuW + 1) + 3 * kLuW);
+  return (int)sizeof(T) * ((2 * kLuW + kLuLines<G, P>) * (kLuW + 1) + 3 * kLuW);
 }
-template <typename T, int G>
+template <typename T, int G, int P>
 void lu_launch_t(const SymDev& S, void* store, void* winv, void* piv, const LuTask* tasks,
                  int ntasks, bool solve, bool sym, cudaStream_t st) {
-  lu_panel_kernel<T, G><<<ntasks, 128 * (G + 1), lu_smem_bytes<T, G>(), st>>>(
+  lu_panel_kernel<T, G, P><<<ntasks, 128 * (G + 1), lu_smem_bytes<T, G, P>(), st>>>(
       S, (T*)store, (T*)winv, (T*)piv, tasks, solve ? 1 : 0, sym ? 1 : 0);
+}
+template <typename T>
+void lu_dispatch_t(const SymDev& S, void* store, void* winv, void* piv, const LuTask* tasks,
+                   int ntasks, int lines, bool solve, bool sym, cudaStream_t st) {
+  switch (lines) {
+    case 8: lu_launch_t<T, 1, 4>(S, store, winv, piv, tasks, ntasks, solve, sym, st); break;
+    case 16: lu_launch_t<T, 1, 2>(S, store, winv, piv, tasks, ntasks, solve, sym, st); break;
+    case 32: lu_launch_t<T, 1, 1>(S, store, winv, piv, tasks, ntasks, solve, sym, st); break;
+    default: lu_launch_t<T, kLuGroups, 1>(S, store, winv, piv, tasks, ntasks, solve, sym, st); break;
+  }
+}
+template <typename T, int G, int P>
+cudaError_t lu_prepare_t() {
+  return cudaFuncSetAttribute(lu_panel_kernel<T, G, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              lu_smem_bytes<T, G, P>());
 }
 }  // namespace
 
 void launch_lu_panel(int dtype, const SymDev& S, void* store, void* winv, void* piv,
-                     const LuTask* tasks, int ntasks, int groups, bool solve, bool sym,
+                     const LuTask* tasks, int ntasks, int lines, bool solve, bool sym,
                      cudaStream_t st) {
   if (ntasks <= 0) return;
-  if (dtype == DT_F64) {
-    if (groups == 1) lu_launch_t<double, 1>(S, store, winv, piv, tasks, ntasks, solve, sym, st);
-    else lu_launch_t<double, kLuGroups>(S, store, winv, piv, tasks, ntasks, solve, sym, st);
-  } else {
-    if (groups == 1) lu_launch_t<cdouble, 1>(S, store, winv, piv, tasks, ntasks, solve, sym, st);
-    else lu_launch_t<cdouble, kLuGroups>(S, store, winv, piv, tasks, ntasks, solve, sym, st);
-  }
+  if (dtype == DT_F64)
+    lu_dispatch_t<double>(S, store, winv, piv, tasks, ntasks, lines, solve, sym, st);
+  else
+    lu_dispatch_t<cdouble>(S, store, winv, piv, tasks, ntasks, lines, solve, sym, st);
 }
 
 void launch_unpack_pivots(int dtype, const SymDev& S, void* store, const void* piv, int nbatch,
@@ -595,13 +652,9 @@ void launch_unpack_pivots(int dtype, const SymDev& S, void* store, const void* p
 }
 
 cudaError_t prepare_dense_kernels() {
-  const cudaError_t e = cudaFuncSetAttribute(lu_panel_kernel<cdouble, 1>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             lu_smem_bytes<cdouble, 1>());
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(lu_panel_kernel<cdouble, kLuGroups>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              lu_smem_bytes<cdouble, kLuGroups>());
+  cudaError_t e = lu_prepare_t<cdouble, 1, 1>();
+  if (e == cudaSuccess) e = lu_prepare_t<cdouble, kLuGroups, 1>();
+  return e;
 }
 
 namespace {

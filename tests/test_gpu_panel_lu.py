@@ -80,6 +80,25 @@ def test_many_instances(torch, s, complex_values):
 
 
 @pytest.mark.parametrize("kind", ["real", "complex", "symmetric"])
+@pytest.mark.parametrize("s", [20, 70])
+@pytest.mark.parametrize("nb", [9, 20])
+def test_lanes_per_line(torch, kind, s, nb):
+    """Launches whose lines take two lanes or one (one instance: four), with
+    ragged last panels and line groups."""
+    import paper_1708_04539_gb300 as ps
+    n = s + 45
+    ii, jj = np.meshgrid(np.arange(n), np.arange(n), indexing="ij")
+    p = gen.problems._finish_small(n, ii.reshape(-1), jj.reshape(-1), 970 + s, kind == "complex",
+                                   f"dense_{n}", s, symmetric_values=kind == "symmetric")
+    p.values = np.ascontiguousarray(p.values[None, :] * np.linspace(0.5, 2.0, nb)[:, None])
+    h = ps.SelInv.from_problem(p, symmetric=kind == "symmetric", check_level=1)
+    h.factor(torch.from_numpy(p.values).cuda())
+    h.selinv()
+    check(p, h, [0, nb - 1])
+    h.close()
+
+
+@pytest.mark.parametrize("kind", ["real", "complex", "symmetric"])
 def test_large_schur_tiles(torch, kind):
     """Levels with enough Schur work for 32 x 32 tiles and a K split: ragged
     tiles (133 rows) over supernodes of 90 columns, 24 instances."""
