@@ -67,7 +67,8 @@ struct Step {
   int cfg = 0;    // GEMM: kernel config; LU_PANEL: lines of a task; SLICE: 1 maxima pass;
                   // OZGEMM: slices; SMALL_LEVEL: shared-memory bytes of a CTA
   int n = 0;      // tasks / segments
-  int n2 = 0;     // GSLICE: ordinary slice tasks after the n G tiles; LU_PANEL: 1 panel solves
+  int n2 = 0;     // GSLICE: ordinary slice tasks after the n G tiles; LU_PANEL: 1 panel solves;
+                  // OZGEMM: 1 outputs subtracted from the ancestors' blocks
   int grid = 0;
   size_t tasks = 0, descs = 0, offs = 0, offs2 = 0;  // byte offsets into the plan arena
   void* ptr = nullptr;                    // memset target / store
@@ -788,6 +789,43 @@ void add_inverse_row(pselinv_ctx* h, Plan& P, const std::vector<SnTask>& wide,
   for (size_t k = first; k < P.steps.size(); k++) P.steps[k].side = 1;
 }
 
+// Whether tile (m, n) (128 x 64) of a product of supernode K has an entry whose
+// row is in its column's supernode or later (SCHUR_COLS; rows m of the tile are
+// positions p of R_K, columns n positions q), or in an earlier one (SCHUR_ROWS:
+// m = q, n = p); positions ascend with the supernodes.
+bool schur_tile(const HostSym& H, int64_t K, int part, int64_t m, int64_t n) {
+  auto sn = [&](int64_t p) {
+    return H.sup_of[(size_t)H.rows[(size_t)std::min(H.rows_ptr[K] + p, H.rows_ptr[K + 1] - 1)]];
+  };
+  return part == SCHUR_ROWS ? sn(n) < sn(m + 127) : sn(m + 127) >= sn(n);
+}
+
+// Whether a level's six-slice Schur products are subtracted from the ancestors by
+// their own epilogue instead of stored and scattered by another launch.  The two
+// operand orders cover tiles on the block diagonal twice, so it is a question
+// of how much that adds: levels with at most 15% more tiles gain (10^3 x 64 DG,
+// c = 7000, s = 256, 1% more: 1813 -> 1676 us; 40^3 upwind, c = 1450, s = 177, 14%:
+// 166 and 167), others lose (c = 808, 25%: 203 -> 223; c = 269, 64%: 174 -> 258).
+// Complex values keep the scatter, which adds both parts of an entry at once: the
+// real and the imaginary product are tasks of their own (30^3 complex 27-point
+// solve, every level: 17.1 against 18.1 ms).  Symmetric values: the lower
+// triangle only, no tile twice.
+bool scatters_products(const pselinv_ctx* h, int lev, bool lower) {
+  const HostSym& H = h->H;
+  if (H.general || h->dtype != DT_F64) return false;
+  if (lower) return true;
+  int64_t plain = 0, both = 0;
+  for (int64_t i = H.hlevel_ptr[lev]; i < H.hlevel_ptr[lev + 1]; i++) {
+    const int64_t K = H.hlevel_sn[i], c = cK(H, K);
+    for (int64_t m = 0; m < c; m += 128)
+      for (int64_t n = 0; n < c; n += 64) {
+        plain++;
+        both += schur_tile(H, K, SCHUR_COLS, m, n) + schur_tile(H, K, SCHUR_ROWS, m, n);
+      }
+  }
+  return 100 * both <= 115 * plain;
+}
+
 constexpr double kEightMinFlops = 2e8;
 // events of a height level of the factorisation: one per panel (8 of 32
 // columns at most), and for its inverses, the operands and the bulk of its
@@ -882,6 +920,8 @@ int build_factor_plan(pselinv_ctx* h) {
     // sliced solves and Schur products: operands sliced from the level's scratch
     // after its FP64 region
     const bool split = mode[lev] != LV_FP64, eight = mode[lev] == LV_EIGHT;
+    // sliced Schur products subtracted from the ancestors as they are computed
+    const bool fused = mode[lev] == LV_SPLIT && scatters_products(h, (int)lev, ldlt);
     int64_t off = tbase, toff = 0;  // scalars into scratch
     int64_t smax = 0, entries = 0;
     double ops = 0;                 // FP64 warp operations of the Schur products
@@ -929,7 +969,7 @@ int build_factor_plan(pselinv_ctx* h) {
           }
         }
         const int64_t s0 = off;
-        if (split) off += c * cu;
+        if (split && !fused) off += c * cu;
         char* Sc = h->scratch + (size_t)s0 * es;
         const SchurProduct q{TL, TU, Sc, (int)c, (int)cu, (int)s, Lp, ldlt ? Lp : Up, Uinv, Linv};
         if (c > 0 && cu > 0) {
@@ -1019,6 +1059,28 @@ int build_factor_plan(pselinv_ctx* h) {
       add_ozaki_trsm(h, P, solves, (int)lev, align256((size_t)off * es), eight);
       add_ozaki_schur_slices(h, P, sprods, (int)lev, align256((size_t)off * es), eight, prods);
     }
+    const int per = dt == DT_F64 ? 1 : 2;  // real and imaginary products
+    const size_t nprods = prods.size();
+    if (fused) {
+      for (size_t d = 0; d < nprods; d++) {
+        OzDesc& g = prods[d];
+        const SnTask& t = sns[d / per];
+        g.C = (double*)(h->lu + (size_t)t.inst * H.storage * es);
+        g.alpha = -1.0;
+        g.K = t.K;
+        g.rb = H.rows_ptr[t.K];
+        g.scatter = ldlt ? SCHUR_LOWER : SCHUR_COLS;
+      }
+      for (size_t d = 0; d < nprods && !ldlt; d++) {
+        OzDesc g = prods[d];
+        std::swap(g.A, g.B);
+        std::swap(g.eA, g.eB);
+        std::swap(g.A_R64, g.B_R64);
+        std::swap(g.M, g.N);
+        g.scatter = SCHUR_ROWS;
+        prods.push_back(g);
+      }
+    }
     wait_pending(at);
     // Schur products and their scatter, of the corner tiles (part 1), of the
     // others (2) or all (0)
@@ -1026,19 +1088,28 @@ int build_factor_plan(pselinv_ctx* h) {
       return part == 0 || (part == 1) == (p0 < corner[(size_t)i] && q0 < corner[(size_t)i]);
     };
     auto add_schur = [&](int part) {
-      const int per = dt == DT_F64 ? 1 : 2;  // real and imaginary products
       if (!split) {
         add_schur_scatter(h, P, schur, (int)lev, ldlt,
                           [&](int d, int p0, int q0) { return in_part(part, d, p0, q0); });
         return;
       }
       const TileFilter keep = [&](int d, int tm, int tn) {
-        return in_part(part, d / per, tm * 128, tn * 64);
+        const int64_t m = tm * 128, n = tn * 64;
+        if (!fused) return in_part(part, d / per, m, n);
+        const OzDesc& g = prods[(size_t)d];
+        if (!schur_tile(H, g.K, g.scatter, m, n)) return false;
+        return g.scatter == SCHUR_ROWS ? in_part(part, (int)(d - nprods) / per, n, m)
+                                       : in_part(part, d / per, m, n);
       };
+      const size_t first = P.steps.size();
       if (eight)
         add_gemm8_step(P, prods, (int)lev, ldlt, keep);
       else  // K = s <= 256 is one exact chunk of six slices: no K split, no accumulation
         add_ozgemm_step(P, prods, h->slices, (int)lev, false, 1, 0, ldlt, keep);
+      if (fused) {
+        for (size_t i = first; i < P.steps.size(); i++) P.steps[i].n2 = 1;
+        return;
+      }
       std::vector<SnTask> gt;
       std::vector<int64_t> gofs;
       for (size_t i = 0; i < sns.size(); i++) {
@@ -2123,7 +2194,7 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
     case ST_OZGEMM:
       launch_ozaki_gemm(s.cfg, (const OzDesc*)(a + s.descs), (const OzTask*)(a + s.tasks), s.n,
                         h->derr, s.side == 0 ? 152 : s.side == 2 ? kBulkSms : s.n,
-                        h->opts.ozaki_a_tmem != 0, st);
+                        h->opts.ozaki_a_tmem != 0, s.n2 ? &h->S : nullptr, st);
       break;
     case ST_ZERO:
       launch_zero((const CopySeg*)(a + s.tasks), s.n, s.grid, st);

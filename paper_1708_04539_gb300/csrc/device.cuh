@@ -248,7 +248,14 @@ struct OzDesc {
   int half, swap_b, neg_half, cscale, coff;
   int tri;  // gemm8: op(B)(k, n) = 0 for k < n (1) or k > n (2)
   double alpha;
+  // Schur products subtracted from the ancestors as they are computed: C is the
+  // instance's storage, rb = rows_ptr[K]; outputs (p, q) with R_K[p] in R_K[q]'s
+  // supernode or later (SCHUR_COLS; m = p, n = q), of these p >= q only
+  // (SCHUR_LOWER), or in an earlier one (SCHUR_ROWS; m = q, n = p)
+  int scatter, K;
+  int64_t rb;
 };
+enum SchurPart { SCHUR_NONE = 0, SCHUR_COLS = 1, SCHUR_ROWS = 2, SCHUR_LOWER = 3 };
 struct OzTask {
   int d, tm, tn, ks;
 };
@@ -290,9 +297,10 @@ void launch_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, bo
                   cudaStream_t st);
 // max_grid: most CTAs of the launch (persistent beyond); a_tmem: the MMAs read
 // A from tensor memory (copied from the stage per K
-// half) instead of shared memory
+// half) instead of shared memory; sym: the outputs go to the ancestors' blocks
+// (OzDesc::scatter; shared-memory A only)
 void launch_ozaki_gemm(int S, const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
-                       int max_grid, bool a_tmem, cudaStream_t st);
+                       int max_grid, bool a_tmem, const SymDev* sym, cudaStream_t st);
 // Slices of operands with K <= 256 with their own row maxima (desc.maxbits
 // unused), `span` K blocks per task {d, row block, first K block}; and
 // products of eight slices, C = A op(B), tasks {d, tm, tn, 0}

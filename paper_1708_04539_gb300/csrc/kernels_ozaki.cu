@@ -745,10 +745,20 @@ __device__ __forceinline__ void task_range(const OzDesc& d, int ks, int& kb0, in
 // MMAs read A there, so shared memory serves each A tile once per K half
 // instead of once per slice pair; the 64-bit totals then live in shared
 // memory (64 KB after the ring) instead of tensor memory.
-template <int S, bool ATMEM>
+// SCATTER: the factorisation's Schur products, subtracted atomically from the
+// ancestors' blocks instead of stored and scattered by a launch of its own (a
+// level of 37.5 M entries, s = 256: 638 -> 577 us; 8^3 x 64 DG factorisation
+// 23.0 -> 21.2 ms).  Entries stored along the other index come from the product
+// of the swapped operands (see OzDesc), so that the lanes' atomics are
+// contiguous.  A lane holds what belongs to one of the 32 output columns (its
+// supernode, storage bases, exponent), loaded before the accumulators are
+// there, and hands it round: only the relative index is loaded per entry, 16 at a
+// time (a load chain per entry made the level 850 us).  Bound: the epilogue of
+// eight warps beside the MMAs of K <= 256.
+template <int S, bool ATMEM, bool SCATTER>
 __global__ void __launch_bounds__(kOzThreads, 1)
 ozaki_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ tasks, int ntasks,
-                  int* err) {
+                  int* err, const SymDev sym) {
   constexpr int kAB = S * 2 * kTileBytes;  // A part of a stage (128 rows)
   constexpr int kStage = S * 3 * kTileBytes;
   constexpr int kOzStages = oz_stages<S, ATMEM>();
@@ -960,6 +970,22 @@ ozaki_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ t
       const int r = task.tm * 128 + quarter * 32 + lane;
       const int nb = task.tn * 64 + hcol * 32;
       const int ea_row = r < dM ? dp->eA[r] : 0;
+      const int part = SCATTER ? dp->scatter : 0;
+      const int64_t rb = SCATTER ? dp->rb : 0;
+      const bool rows = part == SCHUR_ROWS;
+      // SCATTER: the supernode of the lane's row; of its column nb + lane the
+      // supernode, storage bases, relative-index base and exponent
+      int row_sn = 0, l_sn = 0, l_eb = 0;
+      long long l_rel = 0, l_pan = 0, l_diag = 0;
+      if (SCATTER) {
+        const int nl = min(nb + lane, dN - 1);
+        row_sn = sym.row_sn[rb + min(r, dM - 1)];
+        l_sn = sym.row_sn[rb + nl];
+        l_rel = (rows ? sym.row_rel : sym.col_rel)[rb + nl];
+        l_pan = (rows ? sym.row_pan : sym.col_pan)[rb + nl];
+        l_diag = sym.col_diag[rb + nl];
+        l_eb = eB[nl];
+      }
       for (int c = 0; c < nchunks; c++, q++) {
         if (!mbar_wait(smem_u32(&bar_acc_full), q & 1) || abort_flag) {
           ok = false;
@@ -1023,7 +1049,43 @@ ozaki_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ t
         for (int g2 = 0; g2 < 2; g2++) {
           uint32_t tv[32];
           if (!ATMEM) tmem_ld32(ttot + (uint32_t)(g2 * 32), tv);
-          if (r < dM) {
+          if (SCATTER) {
+            // the index loads of 16 outputs first, then their atomics; what belongs
+            // to an output's column comes from the lane that holds it
+            unsigned use = 0;
+            int rel[16];
+#pragma unroll
+            for (int j = 0; j < 16; j++) {
+              const int n = nb + g2 * 16 + j;
+              const int sn = __shfl_sync(0xffffffffu, l_sn, g2 * 16 + j);
+              int64_t ri = __shfl_sync(0xffffffffu, l_rel, g2 * 16 + j) + r;
+              bool ok = r < dM && n < dN && (rows ? sn < row_sn : sn <= row_sn) &&
+                        !(part == SCHUR_LOWER && r < n);
+              if (sym.check && ok && (ri < 0 || ri >= sym.relidx_size)) {
+                set_error(sym.err, DEV_CHECK, dp->K);
+                ok = false;
+              }
+              if (!ok) ri = 0;
+              rel[j] = __ldg(sym.relidx + ri);
+              use |= ok ? 1u << j : 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < 16; j++) {
+              const int sn = __shfl_sync(0xffffffffu, l_sn, g2 * 16 + j);
+              const long long pan = __shfl_sync(0xffffffffu, l_pan, g2 * 16 + j);
+              const long long dia = __shfl_sync(0xffffffffu, l_diag, g2 * 16 + j);
+              const int eb = __shfl_sync(0xffffffffu, l_eb, g2 * 16 + j);
+              const int64_t slot = (sn == row_sn ? dia : pan) + rel[j];
+              bool ok = use >> j & 1;
+              if (sym.check && ok && (slot < 0 || slot >= sym.storage)) {
+                set_error(sym.err, DEV_CHECK, dp->K);
+                ok = false;
+              }
+              const long long tt = (long long)(((unsigned long long)tv[2 * j + 1] << 32) | tv[2 * j]);
+              const double v = scaled_int_to_double(tt, ea + eb, neg);
+              if (ok) atomicAdd(Cp + slot * cscale + coff, v);
+            }
+          } else if (r < dM) {
 #pragma unroll
             for (int j = 0; j < 16; j++) {
               const int n = nb + g2 * 16 + j;
@@ -1334,16 +1396,19 @@ cudaError_t prepare_ozaki_kernels() {
   e = cudaFuncSetAttribute(gslice_kernel<cdouble, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)gslice_smem<cdouble>());
   if (e != cudaSuccess) return e;
-#define PSELINV_OZ_ATTR(S, AT)                                                               \
-  e = cudaFuncSetAttribute(ozaki_gemm_kernel<S, AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                           gemm_smem<S, AT>());                                                 \
+#define PSELINV_OZ_ATTR(S, AT, SC)                                                           \
+  e = cudaFuncSetAttribute(ozaki_gemm_kernel<S, AT, SC>,                                      \
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem<S, AT>());  \
   if (e != cudaSuccess) return e;
-  PSELINV_OZ_ATTR(4, false)
-  PSELINV_OZ_ATTR(5, false)
-  PSELINV_OZ_ATTR(6, false)
-  PSELINV_OZ_ATTR(4, true)
-  PSELINV_OZ_ATTR(5, true)
-  PSELINV_OZ_ATTR(6, true)
+  PSELINV_OZ_ATTR(4, false, false)
+  PSELINV_OZ_ATTR(5, false, false)
+  PSELINV_OZ_ATTR(6, false, false)
+  PSELINV_OZ_ATTR(4, true, false)
+  PSELINV_OZ_ATTR(5, true, false)
+  PSELINV_OZ_ATTR(6, true, false)
+  PSELINV_OZ_ATTR(4, false, true)
+  PSELINV_OZ_ATTR(5, false, true)
+  PSELINV_OZ_ATTR(6, false, true)
 #undef PSELINV_OZ_ATTR
   return cudaFuncSetAttribute(gemm8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               k8Stages * k8Stage);
@@ -1470,29 +1535,30 @@ void launch_gslice(int dtype, const SymDev& S, const void* store, const SliceDes
 }
 
 void launch_ozaki_gemm(int S, const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
-                       int max_grid, bool a_tmem, cudaStream_t st) {
+                       int max_grid, bool a_tmem, const SymDev* sym, cudaStream_t st) {
   if (ntasks <= 0) return;
   // one CTA fits an SM (shared memory and tensor memory): a persistent grid on
   // the critical stream (all SMs) and for the factorisation's bulk (most of
   // them); one task per CTA on the normalisation stream, so that its CTAs leave
   // SMs to the sweep between tasks
   const int grid = ntasks < max_grid ? ntasks : max_grid;
-#define PSELINV_OZ_LAUNCH(SS, AT)                                                        \
-  ozaki_gemm_kernel<SS, AT><<<grid, kOzThreads, gemm_smem<SS, AT>(), st>>>(descs, tasks, \
-                                                                          ntasks, err)
-  if (a_tmem) {
-    switch (S) {
-      case 4: PSELINV_OZ_LAUNCH(4, true); break;
-      case 5: PSELINV_OZ_LAUNCH(5, true); break;
-      default: PSELINV_OZ_LAUNCH(6, true); break;
-    }
-  } else {
-    switch (S) {
-      case 4: PSELINV_OZ_LAUNCH(4, false); break;
-      case 5: PSELINV_OZ_LAUNCH(5, false); break;
-      default: PSELINV_OZ_LAUNCH(6, false); break;
-    }
+#define PSELINV_OZ_LAUNCH(SS, AT, SC)                                            \
+  ozaki_gemm_kernel<SS, AT, SC><<<grid, kOzThreads, gemm_smem<SS, AT>(), st>>>(  \
+      descs, tasks, ntasks, err, sym ? *sym : SymDev{})
+#define PSELINV_OZ_SLICES(AT, SC)                  \
+  switch (S) {                                     \
+    case 4: PSELINV_OZ_LAUNCH(4, AT, SC); break;   \
+    case 5: PSELINV_OZ_LAUNCH(5, AT, SC); break;   \
+    default: PSELINV_OZ_LAUNCH(6, AT, SC); break;  \
   }
+  if (sym) {
+    PSELINV_OZ_SLICES(false, true)
+  } else if (a_tmem) {
+    PSELINV_OZ_SLICES(true, false)
+  } else {
+    PSELINV_OZ_SLICES(false, false)
+  }
+#undef PSELINV_OZ_SLICES
 #undef PSELINV_OZ_LAUNCH
 }
 

@@ -144,3 +144,35 @@ def test_factor_precision_switch(torch):
     with pytest.raises(ps.PselinvError):
         h.set_factor_precision(7)
     h.close()
+
+
+@pytest.mark.parametrize("kind,n,s,nb", [("real", 171, 43, 2), ("real", 1750, 255, 1),
+                                         ("complex", 333, 100, 2), ("symmetric", 333, 100, 2),
+                                         ("symmetric", 171, 43, 2)])
+def test_scattered_products(torch, kind, n, s, nb):
+    """Schur products subtracted from the ancestors as they are computed (wide
+    levels of real values; the others scatter them): ragged 128 x 64 tiles over
+    several ancestors, entries of all three kinds of block (diagonal, L panel, U^T
+    panel), maps checked."""
+    import paper_1708_04539_gb300 as ps
+    ii, jj = np.meshgrid(np.arange(n), np.arange(n), indexing="ij")
+    p = gen.problems._finish_small(n, ii.reshape(-1), jj.reshape(-1), 910 + s, kind == "complex",
+                                   f"dense_{n}", s, symmetric_values=kind == "symmetric")
+    vals = np.ascontiguousarray(p.values[None, :] * np.array([0.7, 1.6])[:nb, None])
+    h = ps.SelInv.from_problem(p, relax_pct=20, symmetric=kind == "symmetric", check_level=1,
+                               factor_precision=ps.PREC_OZAKI_FP16, factor_split_mflops=-1)
+    h.factor(torch.from_numpy(vals).cuda())
+    st = h.structure()
+    steps = h.profile(1)
+    scattered = {x["level"] for x in steps if x["kind"] == "ozaki_gemm"} - {
+        x["level"] for x in steps if x["kind"] == "scatter_sub"}
+    assert bool(scattered) == (kind != "complex")
+    h.factor(torch.from_numpy(vals).cuda())
+    sym, gi, oi, orows, ocols = sorted_against_oracle(st, p, 20)
+    for b in range(nb):
+        fac = h.get_selected(batch=b, layout=ps.LAYOUT_FACTORS)
+        f = oracle.lu(sym, p.colptr, p.rowind, vals[b])
+        ovals = np.concatenate([f.diag, f.low, f.up])[oi]
+        err = selected_error(fac[gi], ovals, orows, ocols, p.n)
+        assert err < TOL_FACTOR, (b, err)
+    h.close()
