@@ -105,8 +105,8 @@ typedef struct pselinv_opts {
                             products (exact FP32 accumulation, FP64 result) on the levels
                             whose Schur products reach factor_split_mflops (smaller levels
                             keep FP64 accuracy: FP64 products, or products of eight slices
-                            where the FP64 pipe would take longer); the diagonal LU, the triangular inverses and the scatter into the
-                            ancestors stay FP64 */
+                            where the FP64 pipe would take longer); the diagonal LU, the
+                            triangular inverses and the sums in the ancestors stay FP64 */
   int32_t factor_split_mflops; /* factor_precision = OZAKI_FP16: smallest Schur-product work
                             (MFLOP) of a level that goes split; 0 = default (200); < 0:
                             every level */
@@ -334,7 +334,8 @@ typedef struct pselinv_step_stat {
   int32_t param;  /* GEMM: kernel config (0 64x64, 1 32x32, 2 128x64 tiles, 3 row
                      panels); OZAKI_GEMM: K split;
                      else -1 */
-  int32_t side;   /* stream of the launch in a sweep: 0 main, 1 normalisation side stream */
+  int32_t side;   /* stream of the launch: 0 main, 1 side (normalisation, inverses), 2 the
+                     factorisation's bulk Schur products */
   double start_ms; /* which = 2: time from the start of the sweep until the launch's stream
                       reached it (its wait included); else 0 */
 } pselinv_step_stat;
@@ -344,7 +345,7 @@ enum pselinv_step_kind {
   PSELINV_STEP_GATHER = 3, PSELINV_STEP_SCATTER_SUB = 4, PSELINV_STEP_COPY = 5,
   PSELINV_STEP_MEMSET = 6, PSELINV_STEP_SCATTER_VALUES = 7, PSELINV_STEP_SLICE = 8,
   PSELINV_STEP_OZAKI_GEMM = 9, PSELINV_STEP_RECOMBINE = 10,
-  PSELINV_STEP_SMALL_LEVEL = 11, /* steps 3-5 of a level of narrow supernodes, one launch */
+  PSELINV_STEP_SMALL_LEVEL = 11, /* gather and steps 3-5 of an FP64 level, one launch */
   PSELINV_STEP_GATHER_SLICE = 12, /* split levels: Ainv_CC gathered and sliced in one pass
                                      (slices in both layouts, exponents from the running
                                      maxima), with the panels' maxima or slicing; Ainv_CC is

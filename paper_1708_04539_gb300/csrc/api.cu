@@ -826,7 +826,10 @@ bool scatters_products(const pselinv_ctx* h, int lev, bool lower) {
   return 100 * both <= 115 * plain;
 }
 
-constexpr double kEightMinFlops = 2e8;
+// FP64 work of a factorisation level from which its products are eight-slice ones
+// (40^3 upwind / 16 complex grids / symmetric 25^3 solve, ms: 200 MFLOP 16.05 / 8.55 /
+// 5.11, 100: 15.96 / 8.55 / 5.11, 50: 16.00 / 8.79 / 5.01)
+constexpr double kEightMinFlops = 1e8;
 // events of a height level of the factorisation: one per panel (8 of 32
 // columns at most), and for its inverses, the operands and the bulk of its
 // Schur products, and the solves of narrow supernodes on the bulk stream
@@ -858,7 +861,7 @@ int build_factor_plan(pselinv_ctx* h) {
   // precision of each level's products.  Split: opts.slices slices where the
   // Schur work pays for them; smaller levels keep FP64 accuracy, as products of
   // eight slices where the FP64 pipe would take longer than their four launches
-  // (200 MFLOP: 160 us)
+  // (100 MFLOP: 80 us)
   enum { LV_FP64, LV_SPLIT, LV_EIGHT };
   std::vector<int> mode((size_t)std::max(nlev, 0) + 1, LV_FP64);
   for (int lev = 0; lev < nlev && h->opts.factor_precision == PSELINV_PREC_OZAKI_FP16; lev++) {
