@@ -22,6 +22,7 @@
 #include "device.cuh"
 #include "internal.h"
 #include "pselinv.h"
+#include "schur_parts.h"
 
 using namespace pselinv;
 
@@ -1088,7 +1089,7 @@ int build_factor_plan(pselinv_ctx* h) {
     // Schur products and their scatter, of the corner tiles (part 1), of the
     // others (2) or all (0)
     auto in_part = [&](int part, int i, int64_t p0, int64_t q0) {
-      return part == 0 || (part == 1) == (p0 < corner[(size_t)i] && q0 < corner[(size_t)i]);
+      return schur_in_part(part, corner[(size_t)i], p0, q0);
     };
     auto add_schur = [&](int part) {
       if (!split) {
@@ -1097,7 +1098,7 @@ int build_factor_plan(pselinv_ctx* h) {
         return;
       }
       const TileFilter keep = [&](int d, int tm, int tn) {
-        const int64_t m = tm * 128, n = tn * 64;
+        const int64_t m = tm * kProductRows, n = tn * kProductCols;
         if (!fused) return in_part(part, d / per, m, n);
         const OzDesc& g = prods[(size_t)d];
         if (!schur_tile(H, g.K, g.scatter, m, n)) return false;
@@ -1119,7 +1120,7 @@ int build_factor_plan(pselinv_ctx* h) {
         const int64_t c = cK(H, sns[i].K), cu = cU(H, sns[i].K);
         for (int tq = 0; tq < ceil_div(cu, 32); tq++)
           for (int tp = ldlt ? tq : 0; tp < ceil_div(c, 32); tp++)
-            if (in_part(part, (int)i, tp * 32, tq * 32)) {
+            if (scatter_in_part(part, corner[i], tp, tq)) {
               gt.push_back({sns[i].inst, sns[i].K, tp, tq});
               gofs.push_back(sofs[i]);
             }
