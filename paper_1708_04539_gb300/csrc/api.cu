@@ -926,6 +926,13 @@ int build_factor_plan(pselinv_ctx* h) {
     const bool split = mode[lev] != LV_FP64, eight = mode[lev] == LV_EIGHT;
     // sliced Schur products subtracted from the ancestors as they are computed
     const bool fused = mode[lev] == LV_SPLIT && scatters_products(h, (int)lev, ldlt);
+    // a six-slice level with a supernode that has only one of R_L, R_U keeps all
+    // its panel solves in FP64
+    bool solves_fp64 = false;
+    for (int64_t i = l0; i < l1 && !eight; i++) {
+      const int64_t K = H.hlevel_sn[i];
+      solves_fp64 = solves_fp64 || (cK(H, K) == 0) != (cU(H, K) == 0);
+    }
     int64_t off = tbase, toff = 0;  // scalars into scratch
     int64_t smax = 0, entries = 0;
     double ops = 0;                 // FP64 warp operations of the Schur products
@@ -936,7 +943,8 @@ int build_factor_plan(pselinv_ctx* h) {
         // cu: rows of the U^T panel (c, or R_U(K))
         const int64_t K = H.hlevel_sn[i], s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
         smax = std::max(smax, s);
-        const bool oz = split && c > 0 && cu > 0;  // panel solves as sliced products
+        // panel solves as sliced products
+        const bool oz = split && c > 0 && cu > 0 && !solves_fp64;
         const bool narrow = s <= kLuPanel && !split;  // panel solves in the panel launch
         const int64_t w = std::min<int64_t>(s, kLuPanel);
         const int64_t lines = (narrow ? c + (ldlt ? 0 : cu) : 2 * (s - w)) + 2 * w;
