@@ -1122,9 +1122,10 @@ constexpr int gemm_smem() {
 // L_KK^{-1}, Uhat^T = U^T U_KK^{-T} of split levels, and the panel solves and
 // Schur products of the split factorisation's levels that are too small for
 // opts.slices slices.  Eight base-256 slices: 63 bits below each row's and
-// column's power of two and the 36 slice pairs with s + t <= 7, so an output
-// is off by some 2^-60 of
-// its row's and column's largest products.  Against correctly rounded exact
+// column's power of two 2^e and the 36 slice pairs with s + t <= 7, so that an
+// output of K terms is off by at most 9 K 2^-64 of 2^(e_row + e_column) (one unit
+// each from the two operands' digits, seven from the pairs left out), before the
+// one rounding to FP64.  Against correctly rounded exact
 // products of panels of 3D, 2D and DG matrices (s = 128) the relative error in
 // norm is 2e-18 to 2e-17; an FP64 sum's is 1.5e-16 to 2.8e-16.  (Base 128, 56
 // bits: up to 6e-16, from columns of Lhat far below their rows' largest
@@ -1339,11 +1340,16 @@ gemm8_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ tasks,
               const int n = nb + g2 * 16 + j;
               if (n < dN) {
                 const int eb = eB[n];
-                // the sum's top 63 bits, the rest as a sticky bit
+                // the sum (|sum| < 2^78) in 62 significant bits and a sticky bit: a
+                // small one (far below its row's and column's scale, or left by
+                // cancellation) keeps all of its bits
                 const long long top = hi[j] + (lo[j] >> 32);
                 const uint32_t rem = (uint32_t)lo[j];
-                const long long u = (top << 16) | (long long)(rem >> 16) | ((rem & 0xFFFFu) != 0);
-                double v = scaled_int_to_double(u, ea + eb - 70 + 16, false);
+                const int sh = max(0, 34 - __clzll(top ^ (top >> 63)));
+                const uint32_t lost = rem & ((1u << sh) - 1u);
+                const long long u = (long long)(((unsigned long long)top << (32 - sh)) |
+                                                (rem >> sh)) | (lost != 0);
+                double v = scaled_int_to_double(u, ea + eb - 70 + sh, false);
                 // exponent 1025: an infinity or a NaN in the row
                 if (ea > 1024 || eb > 1024) v = __longlong_as_double(0x7FF8000000000000ll);
                 double* cp = Cp + (r + (int64_t)n * ldc) * cscale + coff;

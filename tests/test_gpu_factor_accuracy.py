@@ -1,5 +1,5 @@
 """Accuracy of the split factorisation's products that are not six-slice ones:
-panel solves that stay on the FP64 pipe."""
+panel solves that stay on the FP64 pipe, and products of eight slices."""
 from __future__ import annotations
 
 import numpy as np
@@ -63,3 +63,45 @@ def test_one_sided_level_solves_in_fp64(torch, s, complex_values):
     ref, x = got[0][w], got[1][w]
     for part in (slice(0, s * (k - s)), slice(s * (k - s), None)):
         assert np.abs(x[part] - ref[part]).max() <= 8 * s * U64 * np.abs(ref[part]).max()
+
+
+@pytest.mark.parametrize("kind", ["real", "complex", "symmetric"])
+@pytest.mark.parametrize("s,c", [(33, 140), (64, 133), (65, 64), (256, 60)])
+def test_eight_slice_outputs_keep_their_bits(torch, kind, s, c):
+    """Panels over an identity block, so that the solved panels are A's own: every
+    row has entries of 1 and of 2^-20.  Their digits hold 63 bits below the
+    row's power of two (2 at most) and the other operand is one digit, so an entry
+    is off by at most 2^-63 and its own rounding."""
+    import paper_1708_04539_gb300 as ps
+    n = s + c
+    nb = int(1.2e8 / ((2.0 * c * c * s + 2.0 * c * s * s) * (4 if kind == "complex" else 1)
+                      * (0.5 if kind == "symmetric" else 1))) + 1
+    rng = np.random.default_rng(s)
+
+    def panel():
+        x = rng.uniform(0.5, 1, (c, s)) * np.where(rng.random((c, s)) < 0.2, 1.0, 2.0 ** -20)
+        return x + (1j * rng.uniform(-1, 1, (c, s)) * 2.0 ** -18 if kind == "complex" else 0)
+    low = panel()
+    up = low if kind == "symmetric" else panel()
+    a = np.zeros((n, n), dtype=low.dtype)
+    a[s:, :s], a[:s, s:] = low, up.T
+    a[:s, :s] = np.eye(s)
+    a[s:, s:] = 4.0 * n * np.eye(c)
+    colptr = np.arange(n + 1, dtype=np.int64) * n  # (the whole pattern, zeros too)
+    rowind = np.tile(np.arange(n, dtype=np.int64), n)
+    h = ps.SelInv(n, colptr, rowind, np.arange(n, dtype=np.int64), max_supernode=s,
+                  symmetric=kind == "symmetric", factor_precision=ps.PREC_OZAKI_FP16,
+                  factor_split_mflops=100000)
+    st = h.structure()
+    assert st["sn_width"][0] == s
+    h.factor(torch.from_numpy(np.tile(a.T.reshape(-1), (nb, 1))).cuda())
+    assert any(r["kind"] == "ozaki_gemm" and r["level"] == 0 for r in h.profile(1))
+    h.factor(torch.from_numpy(np.tile(a.T.reshape(-1), (nb, 1))).cuda())
+    for b in (0, nb - 1):
+        fac = h.get_selected(batch=b, layout=ps.LAYOUT_FACTORS)
+        o = st["sn_offset"][0] + s * s
+        for got, ref in ((fac[o:o + c * s], low), (fac[o + c * s:o + 2 * c * s], up)):
+            got = got.reshape(s, c).T
+            for x, r in ((got.real, ref.real), (got.imag, ref.imag)):
+                assert (np.abs(x - r) <= 2.0 ** -63 + U64 * np.abs(r)).all()
+    h.close()
