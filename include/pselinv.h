@@ -83,9 +83,13 @@ typedef struct pselinv_opts {
   int32_t host_only;     /* 1: pselinv_analyze makes no CUDA call (structure inspection only;
                             the handle then refuses pselinv_factor) */
   int32_t split_normalise; /* PREC_OZAKI_FP16 only.  0 (default): the normalisation (Lhat,
-                            Uhat^T, Algorithm 1 step 2) has FP64 accuracy (FP64 products, or
+                            Uhat^T, Algorithm 1 step 2) has FP64 accuracy: FP64 products, or
                             on split levels products of eight slices of 8 bits for supernodes
-                            wider than 32 columns), and D_K = U_KK^{-1} L_KK^{-1} stays in FP64
+                            wider than 32 columns, off by at most 1.2 K 2^-53 (K terms) of
+                            the largest output of their row; rows where the slices do not
+                            reach that far, and columns whose pivot is more than 2^7 out of
+                            line with the supernode's, are computed in FP64.  D_K =
+                            U_KK^{-1} L_KK^{-1} stays in FP64
                             like the triangular inverses and the final Ainv_KK combination; 1:
                             in split levels all three are products of opts.slices slices (one
                             more rounding stage) */
@@ -105,7 +109,8 @@ typedef struct pselinv_opts {
                             products (exact FP32 accumulation, FP64 result) on the levels
                             whose Schur products reach factor_split_mflops (smaller levels
                             keep FP64 accuracy: FP64 products, or products of eight slices
-                            where the FP64 pipe would take longer); the diagonal LU, the
+                            where the FP64 pipe would take longer, held to the same line
+                            as the normalisation's); the diagonal LU, the
                             triangular inverses and the sums in the ancestors stay FP64 */
   int32_t factor_split_mflops; /* factor_precision = OZAKI_FP16: smallest Schur-product work
                             (MFLOP) of a level that goes split; 0 = default (200); < 0:

@@ -60,7 +60,8 @@ enum StepKind {
   ST_UNPACK_PIVOTS,
   ST_PANEL_SLICE,
   ST_GEMM8,
-  ST_SCHUR_SCATTER
+  ST_SCHUR_SCATTER,
+  ST_GUARD8
 };
 
 struct Step {
@@ -72,7 +73,8 @@ struct Step {
                   // OZGEMM: 1 outputs subtracted from the ancestors' blocks
   int grid = 0;
   size_t tasks = 0, descs = 0, offs = 0, offs2 = 0;  // byte offsets into the plan arena
-  void* ptr = nullptr;                    // memset target / store
+  void* ptr = nullptr;                    // memset target / store; PANEL_SLICE: words to zero
+  int64_t words = 0;                      // PANEL_SLICE: how many
   void* ptr2 = nullptr;                   // second buffer
   size_t bytes = 0;
   double flops = 0;                       // useful flops of a GEMM step
@@ -500,7 +502,8 @@ size_t ozaki_norm_bytes(const HostSym& H, int64_t nb, size_t es) {
     size_t b = 512;
     for (int64_t i = H.level_ptr[d]; i < H.level_ptr[d + 1]; i++) {
       const int64_t K = H.level_sn[i], s = H.sn_width[K], c = std::max(cK(H, K), cU(H, K));
-      b += 2 * (parts * slice_bytes(s, s, S) + exps_bytes(s) + 512) + (size_t)(2 * c + 2 * s) * 8;
+      // (and the rows', columns' and products' maxima)
+      b += 2 * (parts * slice_bytes(s, s, S) + exps_bytes(s) + 512) + (size_t)(2 * c + 2 * s + 2) * 8;
       if (c > 0) b += 2 * (parts * slice_bytes(c, s, S) + exps_bytes(c) + 512);
     }
     mx = std::max(mx, b * (size_t)nb + 512);
@@ -564,10 +567,11 @@ size_t scratch_need(const HostSym& H, int64_t nb, size_t es) {
     for (int64_t i = H.hlevel_ptr[d]; i < H.hlevel_ptr[d + 1]; i++) {
       const int64_t K = H.hlevel_sn[i], s = H.sn_width[K], c = cK(H, K), cu = cU(H, K);
       f += (c + cu) * s + c * cu;
-      if (c > 0 && cu > 0)  // A_{C,K}, A_{K,C}^T, Uinv, Linv (the solves; then TL, TU)
+      // A_{C,K}, A_{K,C}^T, Uinv, Linv (the solves; then TL, TU) and the products' maxima
+      if (c > 0 && cu > 0)
         oz += parts * (slice_bytes(c, s, 8) + slice_bytes(cu, s, 8) + 2 * slice_bytes(s, s, 8)) +
               exps_bytes(c) + exps_bytes(cu) + 2 * exps_bytes(s) + 2048 +
-              (size_t)(c + cu + 2 * s) * 8;
+              (size_t)(c + cu + 2 * s + 2) * 8;
     }
     fmax = std::max(fmax, align256((size_t)(f * nb) * es) + oz * (size_t)nb + 512);
   }
@@ -649,13 +653,22 @@ struct SchurProduct {
 };
 void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
                     size_t base, bool eight);
+// eight-slice products: per product one GuardDesc and one (real) or two OzDescs,
+// which share its maxima (`words` in all, see GuardDesc)
+struct Products8 {
+  std::vector<OzDesc> prods;
+  std::vector<GuardDesc> guards;
+  unsigned* mx = nullptr;
+  size_t words = 0;
+};
 void add_ozaki_schur_slices(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
-                            size_t base, bool eight, std::vector<OzDesc>& out);
+                            size_t base, std::vector<OzDesc>& out);
+void add_schur_slices8(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
+                       size_t base, Products8 (&out)[2]);
 using TileFilter = std::function<bool(int, int, int)>;  // (descriptor, tile row, tile column)
 void add_ozgemm_step(Plan& P, std::vector<OzDesc>& descs, int S, int level, bool force_atomic,
                      int ks, int slot, bool lower_c, const TileFilter& keep);
-void add_gemm8_step(Plan& P, const std::vector<OzDesc>& prods, int lev, bool lower_c,
-                    const TileFilter& keep);
+void add_gemm8_step(Plan& P, const Products8& set, int lev, bool lower_c, const TileFilter& keep);
 
 // tile of the diagonal blocks' small products: 16 x 16 while 32 x 32 tiles
 // would leave SMs without a CTA (a 32 x 32 x 32 product takes an SM's FP64
@@ -955,8 +968,8 @@ int build_factor_plan(pselinv_ctx* h) {
         char* Up = Lp + (size_t)c * s * es;
         char* Linv = h->winv + (size_t)(b * h->w_stride + h->w_off[K]) * es;
         char* Uinv = Linv + (size_t)s * s * es;
-        // TL, TU: the solved panels, in place (narrow: by the panel step; split:
-        // the sliced products read copies), else in scratch and copied back
+        // TL, TU: the solved panels, in place (narrow: by the panel step; six
+        // slices: the products read copies), else in scratch and copied back
         char *TL = Lp, *TU = Up;
         if (s > kLuPanel) {
           wide.push_back({(int)b, (int)K, 0, 0});
@@ -966,15 +979,15 @@ int build_factor_plan(pselinv_ctx* h) {
           mirrored.push_back({(int)b, (int)K, 0, 0});
         }
         if (!narrow) {
-          if (!oz && (c > 0 || cu > 0)) {
+          if ((!oz || eight) && (c > 0 || cu > 0)) {
             TL = h->scratch + (size_t)off * es;
             TU = TL + (size_t)c * s * es;
             off += (c + cu) * s;
             // L = A U^-1, U^T = A^T L^-T: both B operands upper triangular
-            if (c > 0)
+            if (c > 0 && !oz)
               trsm.push_back(make_desc(Lp, Uinv, TL, c, s, s, c, s, c, 0, 0, 1.0, 0.0, 0, 1,
                                        GEMM_TRI_UPPER_B));
-            if (cu > 0)
+            if (cu > 0 && !oz)
               trsm.push_back(make_desc(ldlt ? Lp : Up, Linv, TU, cu, s, s, cu, s, cu, 0, 1, 1.0,
                                        0.0, 0, 1, GEMM_TRI_UPPER_B));
             segs.push_back({TL, Lp, (c + cu) * s});
@@ -1067,9 +1080,13 @@ int build_factor_plan(pselinv_ctx* h) {
     add_gemm_step(P, dt, choose_small_tile(dt, trsm) == GEMM_16x16 ? GEMM_16x16 : GEMM_ROWS, trsm,
                   (int)lev);
     std::vector<OzDesc> prods;
+    Products8 prods8[2];  // with the maxima of the corner's launch, and of the others'
     if (split) {
       add_ozaki_trsm(h, P, solves, (int)lev, align256((size_t)off * es), eight);
-      add_ozaki_schur_slices(h, P, sprods, (int)lev, align256((size_t)off * es), eight, prods);
+      if (eight)
+        add_schur_slices8(h, P, sprods, (int)lev, align256((size_t)off * es), prods8);
+      else
+        add_ozaki_schur_slices(h, P, sprods, (int)lev, align256((size_t)off * es), prods);
     }
     const int per = dt == DT_F64 ? 1 : 2;  // real and imaginary products
     const size_t nprods = prods.size();
@@ -1115,7 +1132,7 @@ int build_factor_plan(pselinv_ctx* h) {
       };
       const size_t first = P.steps.size();
       if (eight)
-        add_gemm8_step(P, prods, (int)lev, ldlt, keep);
+        add_gemm8_step(P, prods8[part == 2], (int)lev, ldlt, keep);
       else  // K = s <= 256 is one exact chunk of six slices: no K split, no accumulation
         add_ozgemm_step(P, prods, h->slices, (int)lev, false, 1, 0, ldlt, keep);
       if (fused) {
@@ -1255,8 +1272,9 @@ void add_slice_step(Plan& P, const std::vector<SliceDesc>& descs, int level, boo
 
 // Slices of operands with K <= 256, each task finding its rows' maxima: one
 // launch (see panel_slice_kernel).  Few row blocks: their K range is spread
-// over CTAs too.
-void add_panel_slice_step(Plan& P, const std::vector<SliceDesc>& descs, int level) {
+// over CTAs too.  zero: words set to zero beside it.
+void add_panel_slice_step(Plan& P, const std::vector<SliceDesc>& descs, int level,
+                          unsigned* zero = nullptr, size_t words = 0) {
   if (descs.empty()) return;
   int64_t blocks = 0;
   for (const SliceDesc& d : descs) blocks += d.R64;
@@ -1271,6 +1289,8 @@ void add_panel_slice_step(Plan& P, const std::vector<SliceDesc>& descs, int leve
   }
   Step st;
   st.kind = ST_PANEL_SLICE;
+  st.ptr = zero;
+  st.words = (int64_t)words;
   st.cfg = span;
   st.n = (int)tasks.size();
   st.descs = P.push(descs);
@@ -1458,13 +1478,38 @@ struct OzBuilder {
     d.coff = 1;
     out.push_back(d);
   }
+  // one eight-slice product (its maxima's place in the set as an offset for now)
+  void product8(Products8& set, const SliceDesc& a, const SliceDesc& b, char* C, int ldc, int M,
+                int N, int pivots = GUARD_NONE, const char* Uinv = nullptr) const {
+    const size_t first = set.prods.size();
+    product(set.prods, a, b, C, ldc, M, N, 1.0);
+    unsigned* const at = reinterpret_cast<unsigned*>(set.words * sizeof(unsigned));
+    for (size_t i = first; i < set.prods.size(); i++) set.prods[i].mx = at;
+    GuardDesc g{};
+    g.A = a.src; g.lda = a.ld; g.amode = a.mode; g.eA = a.exps;
+    g.B = b.src; g.ldb = b.ld; g.bmode = b.mode; g.eB = b.exps;
+    g.C = C; g.ldc = ldc; g.M = M; g.N = N; g.K = a.Kd; g.tri = b.tri;
+    g.mx = at;
+    g.pivots = pivots;
+    g.diag = Uinv;
+    set.guards.push_back(g);
+    set.words += 1 + (size_t)M;
+  }
+  // the maxima of a complete set
+  void place_maxima(Products8& set) {
+    char* const base = take(set.words * sizeof(unsigned));
+    set.mx = (unsigned*)base;
+    for (OzDesc& d : set.prods) d.mx = (unsigned*)(base + reinterpret_cast<size_t>(d.mx));
+    for (GuardDesc& g : set.guards) g.mx = (unsigned*)(base + reinterpret_cast<size_t>(g.mx));
+  }
 };
 
-// Products of eight slices (see gemm8_kernel), longest K ranges first;
-// lower_c: the tiles of C on or below its diagonal only
-void add_gemm8_step(Plan& P, const std::vector<OzDesc>& prods, int lev, bool lower_c,
-                    const TileFilter& keep) {
-  std::vector<OzTask> tasks;
+// Products of eight slices (see gemm8_kernel), longest K ranges first, and the
+// check of their tiles (guard8_kernel); lower_c: the tiles of C on or below its
+// diagonal only
+void add_gemm8_step(Plan& P, const Products8& set, int lev, bool lower_c, const TileFilter& keep) {
+  const std::vector<OzDesc>& prods = set.prods;
+  std::vector<OzTask> tasks, checks;
   double flops = 0, bytes = 0, all = 0;
   for (size_t d = 0; d < prods.size(); d++) {
     const OzDesc& g = prods[d];
@@ -1494,6 +1539,16 @@ void add_gemm8_step(Plan& P, const std::vector<OzDesc>& prods, int lev, bool low
   m.bytes = (size_t)(bytes * (keep ? (double)tasks.size() / all : 1.0));
   m.level = lev;
   P.steps.push_back(m);
+  const int per = set.guards.empty() ? 1 : (int)(prods.size() / set.guards.size());
+  for (const OzTask& t : tasks)
+    if (t.d % per == 0) checks.push_back({t.d / per, t.tm, t.tn, 0});
+  Step c;
+  c.kind = ST_GUARD8;
+  c.n = (int)checks.size();
+  c.descs = P.push(set.guards);
+  c.tasks = P.push(checks);
+  c.level = lev;
+  P.steps.push_back(c);
 }
 
 // Triangular solves of one factorisation level as sliced products (K = s):
@@ -1507,6 +1562,7 @@ void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& pr
   OzBuilder ob(h, base, eight ? kSlices8 : 0);
   std::vector<SliceDesc> sl;
   std::vector<OzDesc> out;
+  Products8 set;
   for (const SchurProduct& q : prods) {
     const SliceDesc al = ob.slice(q.AL, q.c, SLICE_ROWS, q.c, q.s);
     SliceDesc ub = ob.slice(q.Uinv, q.s, SLICE_COLS, q.s, q.s);
@@ -1520,12 +1576,18 @@ void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& pr
     sl.push_back(al);
     sl.push_back(ub);
     sl.push_back(lb);
-    ob.product(out, al, ub, q.TL, q.c, q.c, q.s, 1.0);
-    ob.product(out, au, lb, q.TU, q.cu, q.cu, q.s, 1.0);
+    if (eight) {
+      ob.product8(set, al, ub, q.TL, q.c, q.c, q.s);
+      ob.product8(set, au, lb, q.TU, q.cu, q.cu, q.s, GUARD_SCALED, q.Uinv);
+    } else {
+      ob.product(out, al, ub, q.TL, q.c, q.c, q.s, 1.0);
+      ob.product(out, au, lb, q.TU, q.cu, q.cu, q.s, 1.0);
+    }
   }
-  add_panel_slice_step(P, sl, lev);
+  if (eight) ob.place_maxima(set);
+  add_panel_slice_step(P, sl, lev, set.mx, set.words);
   if (eight)
-    add_gemm8_step(P, out, lev, false, nullptr);
+    add_gemm8_step(P, set, lev, false, nullptr);
   else
     add_ozgemm_step(P, out, h->slices, lev, false, 1, 0, false, nullptr);
 }
@@ -1534,8 +1596,8 @@ void add_ozaki_trsm(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& pr
 // TU (both by rows: A = TL, B = TU with K = s) in one launch, and the products
 // into the FP64 Sc blocks that the scatter subtracts.
 void add_ozaki_schur_slices(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
-                            size_t base, bool eight, std::vector<OzDesc>& out) {
-  OzBuilder ob(h, base, eight ? kSlices8 : 0);
+                            size_t base, std::vector<OzDesc>& out) {
+  OzBuilder ob(h, base);
   std::vector<SliceDesc> sl;
   for (const SchurProduct& q : prods) {
     const SliceDesc a = ob.slice(q.TL, q.c, SLICE_ROWS, q.c, q.s);
@@ -1545,6 +1607,28 @@ void add_ozaki_schur_slices(pselinv_ctx* h, Plan& P, const std::vector<SchurProd
     ob.product(out, a, b, q.Sc, q.c, q.c, q.cu, 1.0);
   }
   add_panel_slice_step(P, sl, lev);
+}
+// the same as eight-slice products, once with the maxima of the corner's launch
+// and once with the others'
+void add_schur_slices8(pselinv_ctx* h, Plan& P, const std::vector<SchurProduct>& prods, int lev,
+                       size_t base, Products8 (&out)[2]) {
+  OzBuilder ob(h, base, kSlices8);
+  std::vector<SliceDesc> sl;
+  Products8& set = out[0];
+  for (const SchurProduct& q : prods) {
+    const SliceDesc a = ob.slice(q.TL, q.c, SLICE_ROWS, q.c, q.s);
+    const SliceDesc b = ob.slice(q.TU, q.cu, SLICE_ROWS, q.cu, q.s);
+    sl.push_back(a);
+    sl.push_back(b);
+    ob.product8(set, a, b, q.Sc, q.c, q.c, q.cu);
+  }
+  const size_t words = set.words;
+  set.words *= 2;
+  ob.place_maxima(set);
+  add_panel_slice_step(P, sl, lev, set.mx, set.words);
+  out[1] = set;
+  for (OzDesc& d : out[1].prods) d.mx += words;
+  for (GuardDesc& g : out[1].guards) g.mx += words;
 }
 
 // Split-precision normalisation of one depth level (Algorithm 1 step 2 and
@@ -1622,7 +1706,7 @@ void add_sliced_normalize(pselinv_ctx* h, Plan& P, const std::vector<std::pair<i
   const size_t es = h->esize;
   OzBuilder ob(h, base, kSlices8);
   std::vector<SliceDesc> sl;
-  std::vector<OzDesc> prods;
+  Products8 set;
   for (const auto& bk : sns) {
     const int64_t b = bk.first, K = bk.second;
     const int s = (int)H.sn_width[K], c = (int)cK(H, K), cu = (int)cU(H, K);
@@ -1636,7 +1720,7 @@ void add_sliced_normalize(pselinv_ctx* h, Plan& P, const std::vector<std::pair<i
       const SliceDesc la = ob.slice(h->lu + lo, c, SLICE_ROWS, c, s);
       sl.push_back(lb);
       sl.push_back(la);
-      ob.product(prods, la, lb, h->nf + lo, c, c, s, 1.0);
+      ob.product8(set, la, lb, h->nf + lo, c, c, s, GUARD_INVERSE, Uinv);
     }
     if (cu > 0 && !h->opts.symmetric) {  // symmetric A: Uhat = Lhat^T, not needed
       SliceDesc ub = ob.slice(Uinv, s, SLICE_ROWS, s, s);  // Uinv(n, k)
@@ -1644,11 +1728,12 @@ void add_sliced_normalize(pselinv_ctx* h, Plan& P, const std::vector<std::pair<i
       const SliceDesc ua = ob.slice(h->lu + uo, cu, SLICE_ROWS, cu, s);
       sl.push_back(ub);
       sl.push_back(ua);
-      ob.product(prods, ua, ub, h->nf + uo, cu, cu, s, 1.0);
+      ob.product8(set, ua, ub, h->nf + uo, cu, cu, s);
     }
   }
-  add_panel_slice_step(P, sl, lev);
-  add_gemm8_step(P, prods, lev, false, nullptr);
+  ob.place_maxima(set);
+  add_panel_slice_step(P, sl, lev, set.mx, set.words);
+  add_gemm8_step(P, set, lev, false, nullptr);
 }
 
 // Merge the finished blocks of the supernodes `sns` (diagonal block, L and
@@ -2164,10 +2249,13 @@ void launch_step(pselinv_ctx* h, const Plan& P, const Step& s, cudaStream_t st) 
       break;
     case ST_PANEL_SLICE:
       launch_panel_slice((const SliceDesc*)(a + s.descs), (const SliceTask*)(a + s.tasks), s.n, s.cfg,
-                        st);
+                         (unsigned*)s.ptr, s.words, st);
       break;
     case ST_GEMM8:
       launch_gemm8((const OzDesc*)(a + s.descs), (const OzTask*)(a + s.tasks), s.n, h->derr, st);
+      break;
+    case ST_GUARD8:
+      launch_guard8(h->dtype, (const GuardDesc*)(a + s.descs), (const OzTask*)(a + s.tasks), s.n, st);
       break;
     case ST_UNPACK_PIVOTS:
       launch_unpack_pivots(h->dtype, h->S, h->lu, h->piv, (int)h->nbatch, st);
@@ -2853,7 +2941,7 @@ int pselinv_profile(pselinv_t h, int which, void* stream, pselinv_step_stat* out
                                 PSELINV_STEP_GATHER_SLICE, PSELINV_STEP_OUTPUT_MAXIMA,
                                 PSELINV_STEP_COPY, PSELINV_STEP_COPY,
                                 PSELINV_STEP_SLICE, PSELINV_STEP_OZAKI_GEMM,
-                                PSELINV_STEP_GEMM};
+                                PSELINV_STEP_GEMM, PSELINV_STEP_GEMM};
     out[i].kind = kinds[s.kind];
     out[i].level = s.level;
     out[i].tasks = s.n;

@@ -247,6 +247,7 @@ struct OzDesc {
   int A_R64, B_R64, K32, M, N, ldc, ksplit, atomic;
   int half, swap_b, neg_half, cscale, coff;
   int tri;  // gemm8: op(B)(k, n) = 0 for k < n (1) or k > n (2)
+  unsigned* mx;  // gemm8: maxima of the product's rows (see GuardDesc)
   double alpha;
   // Schur products subtracted from the ancestors as they are computed: C is the
   // instance's storage, rb = rows_ptr[K]; outputs (p, q) with R_K[p] in R_K[q]'s
@@ -259,6 +260,24 @@ enum SchurPart { SCHUR_NONE = 0, SCHUR_COLS = 1, SCHUR_ROWS = 2, SCHUR_LOWER = 3
 struct OzTask {
   int d, tm, tn, ks;
 };
+// One eight-slice product C = A op(B) as stored (modes as in SliceDesc, B by its
+// N side), and what gemm8 left in mx: [0] the largest exponent of its columns (+
+// kExpBias), then the largest |C| of the M rows (high words; either part of a
+// complex value).  pivots: GUARD_SCALED / GUARD_INVERSE, the products whose columns
+// carry the scale of the supernode's rows (U^T = A^T L^-T, column j like U_jj) or
+// its inverse (Lhat = L L^-1, like 1 / U_jj); diag is then U_KK^{-1} (N x N).
+enum GuardPivots { GUARD_NONE = 0, GUARD_SCALED = 1, GUARD_INVERSE = 2 };
+struct GuardDesc {
+  const void* A;
+  const void* B;
+  void* C;
+  const void* diag;
+  const int* eA;
+  const int* eB;
+  const unsigned* mx;
+  int lda, ldb, amode, bmode, ldc, M, N, K, tri, pivots;
+};
+constexpr int kExpBias = 8192;
 // One 64 x 64 tile (tp, tq) of G_K = Ainv(R_K, R_K) of instance `inst`,
 // sliced straight from the ancestors' blocks in `store`: dr / dc index the
 // SliceDescs of G by rows and by columns (R = Kd = c_K; their src is unused;
@@ -302,12 +321,16 @@ void launch_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, bo
 void launch_ozaki_gemm(int S, const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
                        int max_grid, bool a_tmem, const SymDev* sym, cudaStream_t st);
 // Slices of operands with K <= 256 with their own row maxima (desc.maxbits
-// unused), `span` K blocks per task {d, row block, first K block}; and
-// products of eight slices, C = A op(B), tasks {d, tm, tn, 0}
+// unused), `span` K blocks per task {d, row block, first K block}, with `nzero`
+// words at `zero` set to zero; products of eight slices, C = A op(B), tasks {d, tm,
+// tn, 0}; and their tiles checked, and computed in FP64 where the slices do not
+// reach far enough (GuardDesc, the same tasks)
 void launch_panel_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, int span,
-                       cudaStream_t st);
+                       unsigned* zero, int64_t nzero, cudaStream_t st);
 void launch_gemm8(const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,
                       cudaStream_t st);
+void launch_guard8(int dtype, const GuardDesc* descs, const OzTask* tasks, int ntasks,
+                   cudaStream_t st);
 void launch_zero(const CopySeg* segs, int nseg, int per_seg, cudaStream_t st);
 // a kernel whose only wait never completes: it gives up after budget_ns and
 // records DEV_TIMEOUT in err[0]

@@ -199,6 +199,15 @@ __device__ __forceinline__ void write_digits(const double (&x)[8], int e, int S,
     write_digits_s<4>(x, e, dst, slice_stride);
 }
 
+// Exponent of a row of an eight-slice operand: a row of zeros is marked, and a
+// subnormal maximum counts as out of range (1026, like an infinity or a NaN), so
+// that its products are computed in FP64
+constexpr int kZeroRow = -4000;
+__device__ __forceinline__ int exp_of_max8(unsigned long long bits) {
+  const int E = (int)(bits >> 52);
+  return bits == 0 ? kZeroRow : E == 0 ? 1026 : E - 1022;
+}
+
 // The eight balanced base-256 digits of the normalisation's operands, Q =
 // rint(x 2^{63 - e}), |Q| <= 2^63, from four exact floats of two digits each
 // (|a_s| <= 128).
@@ -257,8 +266,12 @@ __device__ __forceinline__ void write_digits8(const double (&x)[8], int e, __hal
 // the row block's diagonal.
 __global__ void __launch_bounds__(kSliceThreads)
 panel_slice_kernel(const SliceDesc* __restrict__ descs, const SliceTask* __restrict__ tasks,
-                  int ntasks, int span) {
+                  int ntasks, int span, unsigned* zero, int64_t nzero) {
   const int tid = threadIdx.x, ci = tid >> 3, rr = tid & 7;
+  // the products' maxima, which nobody reads or writes before the next launch
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + tid; i < nzero;
+       i += (int64_t)gridDim.x * blockDim.x)
+    zero[i] = 0;
   const int rl = (ci >> 2) * 8 + rr, kg = ci & 3;
   for (int t = blockIdx.x; t < ntasks; t += gridDim.x) {
     const SliceTask task = tasks[t];
@@ -273,7 +286,7 @@ panel_slice_kernel(const SliceDesc* __restrict__ descs, const SliceTask* __restr
     }
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 8));
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
-    const int e = r < d.R ? exp_of_max(m) : 0;
+    const int e = r < d.R ? (d.S == 8 ? exp_of_max8(m) : exp_of_max(m)) : 0;
     if (task.kc == 0 && kg == 0 && r < d.R) d.exps[r] = e;
     const int64_t slice_stride = (int64_t)d.R64 * d.K32 * (kTileBytes / 2);
     const int half = d.cplx ? d.K32 / 2 : d.K32;
@@ -1125,7 +1138,7 @@ constexpr int gemm_smem() {
 // column's power of two 2^e and the 36 slice pairs with s + t <= 7, so that an
 // output of K terms is off by at most 9 K 2^-64 of 2^(e_row + e_column) (one unit
 // each from the two operands' digits, seven from the pairs left out), before the
-// one rounding to FP64.  Against correctly rounded exact
+// one rounding to FP64; guard8_kernel holds that against the outputs.  Against correctly rounded exact
 // products of panels of 3D, 2D and DG matrices (s = 128) the relative error in
 // norm is 2e-18 to 2e-17; an FP64 sum's is 1.5e-16 to 2.8e-16.  (Base 128, 56
 // bits: up to 6e-16, from columns of Lhat far below their rows' largest
@@ -1304,6 +1317,8 @@ gemm8_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ tasks,
       const int r = task.tm * 128 + quarter * 32 + lane;
       const int nb = task.tn * 64 + hcol * 32;
       const int ea = r < dM ? dp->eA[r] : 0;
+      unsigned* __restrict__ mx = dp->mx;
+      unsigned row_max = 0;
       for (int c = 0; c < nchunks; c++, q++) {
         if (!mbar_wait(smem_u32(&bar_acc_full), q & 1) || abort_flag) {
           ok = false;
@@ -1334,32 +1349,41 @@ gemm8_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ tasks,
               asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_acc_empty))
                            : "memory");
           }
-          if (r < dM) {
 #pragma unroll
-            for (int j = 0; j < 16; j++) {
-              const int n = nb + g2 * 16 + j;
-              if (n < dN) {
-                const int eb = eB[n];
-                // the sum (|sum| < 2^78) in 62 significant bits and a sticky bit: a
-                // small one (far below its row's and column's scale, or left by
-                // cancellation) keeps all of its bits
-                const long long top = hi[j] + (lo[j] >> 32);
-                const uint32_t rem = (uint32_t)lo[j];
-                const int sh = max(0, 34 - __clzll(top ^ (top >> 63)));
-                const uint32_t lost = rem & ((1u << sh) - 1u);
-                const long long u = (long long)(((unsigned long long)top << (32 - sh)) |
-                                                (rem >> sh)) | (lost != 0);
-                double v = scaled_int_to_double(u, ea + eb - 70 + sh, false);
-                // exponent 1025: an infinity or a NaN in the row
-                if (ea > 1024 || eb > 1024) v = __longlong_as_double(0x7FF8000000000000ll);
-                double* cp = Cp + (r + (int64_t)n * ldc) * cscale + coff;
-                *cp = c == 0 ? v : *cp + v;
-              }
+          for (int j = 0; j < 16; j++) {
+            const int n = nb + g2 * 16 + j;
+            unsigned m = 0;
+            if (r < dM && n < dN) {
+              const int eb = eB[n];
+              // the sum (|sum| < 2^78) in 62 significant bits and a sticky bit: a
+              // small one (far below its row's and column's scale, or left by
+              // cancellation) keeps all of its bits
+              const long long top = hi[j] + (lo[j] >> 32);
+              const uint32_t rem = (uint32_t)lo[j];
+              const int sh = max(0, 34 - __clzll(top ^ (top >> 63)));
+              const uint32_t lost = rem & ((1u << sh) - 1u);
+              const long long u = (long long)(((unsigned long long)top << (32 - sh)) |
+                                              (rem >> sh)) | (lost != 0);
+              double v = scaled_int_to_double(u, ea + eb - 70 + sh, false);
+              // exponent above 1024: an infinity, a NaN or a subnormal maximum in the row
+              if (ea > 1024 || eb > 1024) v = __longlong_as_double(0x7FF8000000000000ll);
+              double* cp = Cp + (r + (int64_t)n * ldc) * cscale + coff;
+              if (c > 0) v += *cp;
+              *cp = v;
+              m = (unsigned)__double2hiint(v) & 0x7FFFFFFFu;
             }
+            if (c == nchunks - 1) row_max = max(row_max, m);
           }
           __syncwarp();  // converged again for the next tensor-memory load
         }
       }
+      if (!ok) break;
+      // the tile's share of the product's maxima (see guard8_kernel)
+      const int nl = nb + lane;
+      const unsigned eb_max =
+          __reduce_max_sync(0xffffffffu, nl < dN ? (unsigned)(eB[nl] + kExpBias) : 0u);
+      if (lane == 0 && eb_max) atomicMax(mx, eb_max);
+      if (r < dM) atomicMax(mx + 1 + r, row_max);
     }
     if (!ok) abort_flag = 1;
   }
@@ -1368,6 +1392,120 @@ gemm8_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ tasks,
   __syncthreads();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
+}
+
+// ---------------------------------------------------------------------------
+// Eight slices reach 63 bits below a row's (a column's) largest entry, an FP64
+// sum as far as its own terms go: where scales differ along the contraction (rows
+// or columns of A scaled inside a supernode, strong contrasts) an output can lie
+// far below the product of its row's and column's maxima, and the slices' fixed
+// error, 9 K 2^-64 2^(e_row + e_column), shows.  This kernel follows every gemm8
+// launch with the same tiles, and computes in FP64 from the stored operands
+//   rows whose largest output is more than 2^kGuardReach below their operand's
+//      largest entry times the largest of op(B): what stays is off by at most 1.2
+//      K 2^-53 of its row's largest output, what an FP64 sum of K terms of that size
+//      may lose;
+//   columns whose pivot is further than that from the supernode's largest (U^T
+//      = A^T L^-T) or smallest (Lhat = L L^-1), times the largest entry of the
+//      column of op(B): they carry the pivot's scale or its inverse, and a row
+//      of larger ones would hide them.
+// A column may also be small for lack of coupling (the first ones of a leaf domain
+// barely reach its boundary, 2^-40 on 2D grids and 27-point operators).  Its error
+// stays small against its rows and its pivot, and holding it against itself would
+// send a third of such levels to the FP64 pipe (30^3 complex 27-point solve 17 -> 33
+// ms).  On 3D operators rows reach 2^10 at most and pivots 2^4.
+// Non-finite outputs, and rows near the subnormal range, fail too.
+// Bound: a launch with nothing to do waits for one round of loads; otherwise the
+// FP64 pipe.
+// ---------------------------------------------------------------------------
+constexpr int kGuardReach = 7;
+constexpr int kGuardThreads = 256;
+
+// exponent of a non-negative high word as frexp gives it; far out for zeros,
+// numbers near the subnormal range and non-finite ones
+__device__ __forceinline__ int guard_exp(unsigned hi, int far) {
+  const int E = (int)(hi >> 20);
+  return E < 64 || E == 0x7FF ? far : E - 1022;
+}
+__device__ __forceinline__ unsigned abs_hi(double x) { return (unsigned)__double2hiint(x) & 0x7FFFFFFFu; }
+__device__ __forceinline__ unsigned abs_hi(cdouble x) { return max(abs_hi(x.x), abs_hi(x.y)); }
+
+template <typename T>
+__global__ void __launch_bounds__(kGuardThreads)
+guard8_kernel(const GuardDesc* __restrict__ descs, const OzTask* __restrict__ tasks) {
+  constexpr int kFar = 1 << 20;
+  __shared__ unsigned rows[4], cols[2];
+  __shared__ int extreme[kGuardThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const OzTask t = tasks[blockIdx.x];
+  const GuardDesc& d = descs[t.d];
+  const int M = d.M, N = d.N, m0 = t.tm * 128, n0 = t.tn * 64, pivots = d.pivots;
+  const int eb_max = (int)d.mx[0] - kExpBias;
+  if (eb_max == kZeroRow) return;  // op(B) is zero there
+  if (pivots != GUARD_NONE) {
+    // the largest of -e (GUARD_SCALED: the smallest inverse pivot) or e over U_KK^{-1}'s
+    // diagonal (N <= 256)
+    int e = -kFar;
+    if (tid < N) {
+      const int far = pivots == GUARD_SCALED ? -kFar : kFar;
+      const int q = guard_exp(abs_hi(((const T*)d.diag)[(int64_t)tid * (N + 1)]), far);
+      e = pivots == GUARD_SCALED ? -q : q;
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) extreme[warp] = e;
+    __syncthreads();
+  }
+  if (tid < 128) {
+    const int r = m0 + tid;
+    bool fails = false;
+    if (r < M && d.eA[r] != kZeroRow)
+      fails = d.eA[r] + eb_max - guard_exp(d.mx[1 + r], -kFar) > kGuardReach;
+    const unsigned b = __ballot_sync(0xffffffffu, fails);
+    if (lane == 0) rows[warp] = b;
+  } else if (tid < 192) {
+    const int n = n0 + tid - 128;
+    bool fails = false;
+    if (n < N && pivots != GUARD_NONE) {
+      int top = extreme[0];
+      for (int w = 1; w < kGuardThreads / 32; w++) top = max(top, extreme[w]);
+      const int far = pivots == GUARD_SCALED ? kFar : -kFar;
+      const int q = guard_exp(abs_hi(((const T*)d.diag)[(int64_t)n * (N + 1)]), far);
+      fails = top + (pivots == GUARD_SCALED ? q : -q) + d.eB[n] > kGuardReach;
+    }
+    const unsigned b = __ballot_sync(0xffffffffu, fails);
+    if (lane == 0) cols[warp - 4] = b;
+  }
+  __syncthreads();
+  const unsigned long long cmask = (unsigned long long)cols[1] << 32 | cols[0];
+  const unsigned long long rmask[2] = {(unsigned long long)rows[1] << 32 | rows[0],
+                                       (unsigned long long)rows[3] << 32 | rows[2]};
+  if ((cmask | rmask[0] | rmask[1]) == 0) return;
+  const T* __restrict__ A = (const T*)d.A;
+  const T* __restrict__ B = (const T*)d.B;
+  const int64_t ak = d.amode == SLICE_ROWS ? d.lda : 1, ar = d.amode == SLICE_ROWS ? 1 : d.lda;
+  const int64_t bk = d.bmode == SLICE_ROWS ? d.ldb : 1, bn = d.bmode == SLICE_ROWS ? 1 : d.ldb;
+  auto dot = [&](int r, int n) {  // (the zero triangle of op(B) is skipped)
+    const T* a = A + r * ar;
+    const T* b = B + n * bn;
+    const int k1 = d.tri == 2 ? n + 1 : d.K;
+    T acc = sc_zero(T());
+#pragma unroll 4
+    for (int k = d.tri == 1 ? n : 0; k < k1; k++) acc = fma_s(a[k * ak], b[k * bk], acc);
+    ((T*)d.C)[r + (int64_t)n * d.ldc] = acc;
+  };
+  // failing columns: lanes along the rows; then the failing rows' other columns
+  int i = 0;
+  for (unsigned long long m = cmask; m != 0; m &= m - 1, i ^= 1) {
+    const int r = m0 + (tid & 127);
+    if (i == tid >> 7 && r < M) dot(r, n0 + __ffsll((long long)m) - 1);
+  }
+  i = 0;
+  for (int h = 0; h < 2; h++)
+    for (unsigned long long m = rmask[h]; m != 0; m &= m - 1, i = (i + 1) & 3) {
+      const int n = tid & 63;
+      if (i == tid >> 6 && n0 + n < N && !(cmask >> n & 1))
+        dot(m0 + 64 * h + __ffsll((long long)m) - 1, n0 + n);
+    }
 }
 
 // Failure-path check: wait on an mbarrier that nothing will complete, with a
@@ -1421,10 +1559,19 @@ cudaError_t prepare_ozaki_kernels() {
 }
 
 void launch_panel_slice(const SliceDesc* descs, const SliceTask* tasks, int ntasks, int span,
-                       cudaStream_t st) {
+                       unsigned* zero, int64_t nzero, cudaStream_t st) {
   if (ntasks <= 0) return;
   const int grid = ntasks < 152 * 16 ? ntasks : 152 * 16;
-  panel_slice_kernel<<<grid, kSliceThreads, 0, st>>>(descs, tasks, ntasks, span);
+  panel_slice_kernel<<<grid, kSliceThreads, 0, st>>>(descs, tasks, ntasks, span, zero, nzero);
+}
+
+void launch_guard8(int dtype, const GuardDesc* descs, const OzTask* tasks, int ntasks,
+                   cudaStream_t st) {
+  if (ntasks <= 0) return;
+  if (dtype == DT_F64)
+    guard8_kernel<double><<<ntasks, kGuardThreads, 0, st>>>(descs, tasks);
+  else
+    guard8_kernel<cdouble><<<ntasks, kGuardThreads, 0, st>>>(descs, tasks);
 }
 
 void launch_gemm8(const OzDesc* descs, const OzTask* tasks, int ntasks, int* err,

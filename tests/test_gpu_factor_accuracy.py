@@ -1,9 +1,14 @@
-"""Accuracy of the split factorisation's products that are not six-slice ones:
-panel solves that stay on the FP64 pipe, and products of eight slices."""
+"""Accuracy of the split options' products that are not six-slice ones: panel
+solves that stay on the FP64 pipe, and products of eight slices, those of badly
+scaled operands included."""
 from __future__ import annotations
 
 import numpy as np
 import pytest
+
+import gen
+import oracle
+from helpers import selected_error
 
 pytestmark = pytest.mark.gpu
 
@@ -105,3 +110,111 @@ def test_eight_slice_outputs_keep_their_bits(torch, kind, s, c):
             for x, r in ((got.real, ref.real), (got.imag, ref.imag)):
                 assert (np.abs(x - r) <= 2.0 ** -63 + U64 * np.abs(r)).all()
     h.close()
+
+
+def scalings(kind, n, s, seed):
+    """Row and column scalings by powers of two, (rows, columns)."""
+    rng = np.random.default_rng(seed)
+    k = np.arange(n)
+    which, how = kind.split("-")
+    d = []
+    for x in ("rows", "cols"):
+        e = {"up": 40 * k // s, "down": 40 - 40 * k // s, "random": rng.integers(0, 41, n)}[how]
+        e = np.where(k < s, e - 20, 0)  # within the first supernode
+        d.append(np.ldexp(1.0, e if which in (x, "both") else 0 * e))
+    return d
+
+
+SCALINGS = ["rows-up", "rows-down", "rows-random", "cols-up", "cols-down", "cols-random",
+            "both-up", "both-down", "both-random"]
+
+
+@pytest.mark.parametrize("kind", ["real", "complex"])
+@pytest.mark.parametrize("scaling", SCALINGS)
+def test_scaled_factors(torch, kind, scaling):
+    """A level of eight-slice products whose first supernode's rows or columns are
+    scaled by powers of two: the FP64 factorisation would give exactly the scaled
+    factors, so they are held to the FP64 bound, 1e-12, with the scaling undone."""
+    import paper_1708_04539_gb300 as ps
+    from paper_1708_04539_gb300.binding import supernodal_coordinates
+    s, n, nb = 96, 96 + 133, 40 if kind == "real" else 12
+    ii, jj = np.meshgrid(np.arange(n), np.arange(n), indexing="ij")
+    p = gen.problems._finish_small(n, ii.reshape(-1), jj.reshape(-1), 70, kind == "complex",
+                                   f"dense_{n}", s)
+    d1, d2 = scalings(scaling, n, s, 3)
+    col = np.repeat(np.arange(n), np.diff(p.colptr))
+    vals = p.values * d1[p.rowind] * d2[col]
+    h = ps.SelInv.from_problem(p, factor_precision=ps.PREC_OZAKI_FP16, factor_split_mflops=100000)
+    h.factor(torch.from_numpy(np.tile(vals, (nb, 1))).cuda())
+    assert any(r["kind"] == "ozaki_gemm" for r in h.profile(1))
+    h.factor(torch.from_numpy(np.tile(vals, (nb, 1))).cuda())
+    sym = oracle.analyze(p, relax_pct=20)
+    orows, ocols = sym.lu_pattern()
+    grows, gcols = supernodal_coordinates(h.structure())
+    gi, oi = np.argsort(grows * n + gcols), np.argsort(orows * n + ocols)
+    f = oracle.lu(sym, p.colptr, p.rowind, p.values)
+    ref = np.concatenate([f.diag, f.low, f.up])
+    r, c = grows, gcols
+    undo = np.where(r > c, d1[c] / d1[r], 1.0 / (d1[r] * d2[c]))  # L, U
+    for b in (0, nb - 1):
+        got = h.get_selected(batch=b, layout=ps.LAYOUT_FACTORS) * undo
+        assert selected_error(got[gi], ref[oi], orows[oi], ocols[oi], n) < 1e-12
+    h.close()
+
+
+@pytest.mark.parametrize("kind", ["real", "complex"])
+@pytest.mark.parametrize("scaling", SCALINGS)
+def test_scaled_normalisation(torch, kind, scaling):
+    """The same for the split sweep, whose six-slice products see nothing of a
+    scaling inside one supernode: 1e-11 with the scaling undone, as unscaled."""
+    import paper_1708_04539_gb300 as ps
+    from paper_1708_04539_gb300.binding import supernodal_coordinates
+    s, n = 96, 96 + 133
+    ii, jj = np.meshgrid(np.arange(n), np.arange(n), indexing="ij")
+    p = gen.problems._finish_small(n, ii.reshape(-1), jj.reshape(-1), 71, kind == "complex",
+                                   f"dense_{n}", s)
+    d1, d2 = scalings(scaling, n, s, 4)
+    col = np.repeat(np.arange(n), np.diff(p.colptr))
+    vals = p.values * d1[p.rowind] * d2[col]
+    h = ps.SelInv.from_problem(p)
+    nlev = int(h.structure()["nlevels"])
+    h.plan_set([(lev, 3, 0) for lev in range(nlev)], ps.PREC_OZAKI_FP16)
+    h.factor(torch.from_numpy(vals).cuda())
+    h.selinv(precision=ps.PREC_OZAKI_FP16)
+    sel = oracle.selected_inverse(p, relax_pct=20)
+    orows, ocols = sel.sym.lu_pattern()
+    grows, gcols = supernodal_coordinates(h.structure())
+    gi, oi = np.argsort(grows * n + gcols), np.argsort(orows * n + ocols)
+    got = h.get_selected(layout=ps.LAYOUT_SUPERNODAL) * (d2[grows] * d1[gcols])
+    h.close()
+    ref = sel.values_lu_order()
+    assert selected_error(got[gi], ref[oi], orows[oi], ocols[oi], n) < 1e-11
+
+
+@pytest.mark.parametrize("tiny", [2.0 ** -1060, 2.0 ** -1000, 0.0])
+def test_tiny_rows(torch, tiny):
+    """Rows of a panel at and below the end of the normal range, and of zeros: an
+    eight-slice level gives what the FP64 one gives, to its rounding."""
+    import paper_1708_04539_gb300 as ps
+    s, c, nb = 64, 133, 40
+    n = s + c
+    rng = np.random.default_rng(8)
+    a = rng.uniform(-1, 1, (n, n))
+    a[s + 5, :s] *= tiny
+    a[:s, s + 9] *= tiny
+    np.fill_diagonal(a, 2.0 * n)
+    colptr = np.arange(n + 1, dtype=np.int64) * n
+    rowind = np.tile(np.arange(n, dtype=np.int64), n)
+    got = []
+    for kw in ({}, {"factor_precision": ps.PREC_OZAKI_FP16, "factor_split_mflops": 100000}):
+        h = ps.SelInv(n, colptr, rowind, np.arange(n, dtype=np.int64), max_supernode=s, **kw)
+        st = h.structure()
+        h.factor(torch.from_numpy(np.tile(a.T.reshape(-1), (nb, 1))).cuda())
+        got.append(h.get_selected(batch=nb - 1, layout=ps.LAYOUT_FACTORS))
+        h.close()
+    o = st["sn_offset"][0] + s * s
+    for row, o in ((5, o), (9, o + c * s)):
+        x, ref = (g[o:o + c * s].reshape(s, c)[:, row] for g in got)
+        scale = max(np.abs(ref).max(), 0.0)
+        assert np.abs(x - ref).max() <= max(8 * s * U64 * scale, 4 * s * 2.0 ** -1074) * (tiny != 0)
+    assert np.isfinite(got[1]).all()
