@@ -1883,13 +1883,14 @@ void add_ozaki_level(pselinv_ctx* h, Plan& P, const std::vector<int64_t>& grp, i
 // largest K split of the normalisation's products
 constexpr int kNormMaxKsplit = 8;
 
-// K split of FP64 products: a task's chain of multiply-adds (row panels: 8 per
-// k, 64 cycles each) should not outlast a quarter of the launch's work spread
-// over the chip (16 cycles per warp operation and SM), so that a few tasks
-// more or less per scheduler do not show, down to chunks of 32.  Returns
-// whether any product is split (its chunks then add atomically).  24^3 upwind
-// sweep: step 4 of level 7 (24 MFLOP, K up to 500) 160 -> 41 us, steps 3 and 5
-// of level 2 (110 MFLOP, 384 tasks unsplit) 150 -> 119 us.
+// K split of the FP64 products of steps 3-5 (per-supernode schedule, and levels
+// too large for the fused launch, where it seldom splits): a task's chain of
+// multiply-adds (row panels: 8 per k, 64 cycles each) should not outlast a quarter
+// of the launch's work spread over the chip (16 cycles per warp operation and SM),
+// so that a few tasks more or less per scheduler do not show, down to chunks of
+// 32.  Returns whether any product is split (its chunks then add atomically).
+// Measured on level launches: 24 MFLOP of step 4, K up to 500, 160 -> 41 us; 110
+// MFLOP of steps 3 and 5, 384 tasks unsplit, 150 -> 119 us.
 bool split_fp64_products(std::vector<GemmDesc>& descs, int dtype) {
   const double cplx = dtype == DT_F64 ? 1.0 : 4.0;
   double ops = 0;
@@ -1909,13 +1910,16 @@ bool split_fp64_products(std::vector<GemmDesc>& descs, int dtype) {
 }
 
 // An FP64 level as one fused launch (gather and steps 3-5,
-// small_level_kernel); false for a level without off-diagonal blocks.  Every
-// FP64 level of the level schedule runs this way: against the gather and the
-// two K-split products it measured 8 / 27 us (a level of 0.01 Mflop), 37 / 76
-// (15), 171 / 162 (141), 739 / 837 (785), 6440 / 6700 (7600), over whole sweeps
-// 0.52 / 1.72 ms (one-way 90^2), 2.4 / 4.7 (five 2D grids), 3.8 / 4.7 (24^3 upwind),
-// 76.5 / 80.4 (40^3); only levels whose tasks just exceed a wave of 760 lose (up
-// to 14%, dif 30^3 level 4).  The longest tasks go first, so that the last wave
+// small_level_kernel); false for a level without off-diagonal blocks.  The
+// FP64 levels of the level schedule run this way up to kFusedMaxFlops: against the
+// gather and the two K-split products it measured 8 / 27 us (a level of 0.01
+// Mflop), 37 / 76 (15), 171 / 162 (141), 739 / 837 (785), 6440 / 6700 (7600), over
+// whole sweeps 0.52 / 1.72 ms (one-way 90^2), 2.4 / 4.7 (five 2D grids), 3.8 / 4.7
+// (24^3 upwind), 76.5 / 80.4 (40^3); levels whose tasks just exceed a wave of 760
+// lose (up to 14%, dif 30^3 level 4).  Beyond, G is gathered again for every 16
+// columns of a wide supernode: from 20 Gflop on the products are ahead by 0.5 to
+// 1% on most levels (8^3, 10^3, 12^3 x 64 DG sweeps 710 / 705, 3030 / 3001, 9720 /
+// 9631 ms with every level one way or the other; 704 and 3000 with this line).  The longest tasks go first, so that the last wave
 // is short (24^3 complex stencil: 3.25 -> 2.99 ms).
 bool add_small_level(pselinv_ctx* h, Plan& P, const std::vector<int64_t>& grp, int64_t nb, int lev) {
   const HostSym& H = h->H;
@@ -1973,6 +1977,8 @@ double level_product_flops(const pselinv_ctx* h, int lev) {
   }
   return lf * (double)h->nbatch * (h->dtype == DT_F64 ? 1.0 : 4.0);
 }
+// largest FP64 level that runs as one fused launch (see add_small_level)
+constexpr double kFusedMaxFlops = 2e10;
 
 int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
   const HostSym& H = h->H;
@@ -2099,7 +2105,9 @@ int build_selinv_plan(pselinv_ctx* h, int schedule, int precision) {
                            (c + cu) * s * (int64_t)(es / 8)});
         }
       add_zero_step(P, zsegs, (int)lev);
-      if (schedule == PSELINV_SCHED_LEVEL && add_small_level(h, P, grp, nb, (int)lev)) continue;
+      if (schedule == PSELINV_SCHED_LEVEL && level_product_flops(h, (int)lev) <= kFusedMaxFlops &&
+          add_small_level(h, P, grp, nb, (int)lev))
+        continue;
       std::vector<SnTask> gt;
       std::vector<int64_t> gofs;
       std::vector<GemmDesc> main, dg;
