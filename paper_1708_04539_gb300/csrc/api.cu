@@ -3128,11 +3128,14 @@ int pselinv_tune(pselinv_t h, int precision, int mode, pselinv_model_t model, vo
       rc = measure(0);
       if (rc != PSELINV_OK) return rc;
     }
-    // phase B: FP64 levels, tile shapes and row panels.  Only levels whose
+    // phase B: FP64 levels, tile shapes and row panels (one pass where these
+    // levels are fused launches, which have neither).  Only levels whose
     // products are small enough that FP64 could win are run in FP64 (a level
     // of kTuneFp64MaxFlops takes about 20 ms in FP64 and 1 ms split); the
     // others stay split at the default K split and keep that mode.
-    for (int v = 0; v < 4; v++) {
+    static_assert(kTuneFp64MaxFlops <= kFusedMaxFlops, "phase B's levels are fused launches");
+    const int shapes = sched == PSELINV_SCHED_PER_SUPERNODE ? 4 : 1;
+    for (int v = 0; v < shapes; v++) {
       for (int l = 0; l < nlev; l++) {
         if (level_product_flops(h, l) > kTuneFp64MaxFlops) {
           h->tuned.erase(std::make_tuple(precision, l, 1));
