@@ -2430,6 +2430,32 @@ void free_numeric(pselinv_ctx* h) {
   h->factored = h->inverted = false;
 }
 
+// buffers of `nbatch` instances of a value type
+int alloc_numeric(pselinv_ctx* h, int dtype, int64_t nbatch) {
+  const size_t es = dtype == PSELINV_F64 ? 8 : 16;
+  h->dtype = dtype;
+  h->nbatch = nbatch;
+  h->esize = es;
+  const size_t sbytes = (size_t)nbatch * h->H.storage * es + 256;
+  CK(cudaMalloc(&h->lu, sbytes));
+  CK(cudaMalloc(&h->nf, sbytes));
+  CK(cudaMalloc(&h->ainv, sbytes));
+  CK(cudaMemset(h->nf, 0, sbytes));
+  // zeros outside the triangles, which are never written
+  CK(cudaMalloc(&h->winv, (size_t)nbatch * h->w_stride * es + 256));
+  CK(cudaMemset(h->winv, 0, (size_t)nbatch * h->w_stride * es + 256));
+  CK(cudaMalloc(&h->piv, (size_t)nbatch * h->H.n * kLuPanel * es + 256));
+  h->scratch_bytes = scratch_need(h->H, nbatch, es);
+  CK(cudaMalloc(&h->scratch, h->scratch_bytes));
+  CK(cudaMalloc(&h->staging, (size_t)nbatch * h->H.nnz * es + 256));
+  CK(cudaMalloc(&h->outstage, (size_t)h->H.nnz * es + 256));
+  CK(cudaMalloc(&h->rcmax, (size_t)nbatch * 2 * h->H.n * 8 + 256));
+  CK(prepare_dense_kernels());
+  CK(prepare_ozaki_kernels());
+  h->slices = h->opts.slices <= 0 ? 6 : std::min(6, std::max(4, (int)h->opts.slices));
+  return PSELINV_OK;
+}
+
 // Common tail of the analyses: the input pattern (for the consumers), and
 // the device copy of the structure.
 int finish_analyze(pselinv_ctx* h, int64_t n, const int64_t* colptr, const int64_t* rowind,
@@ -2623,26 +2649,11 @@ int pselinv_factor(pselinv_t h, int dtype, int64_t nbatch, const void* values, v
   const size_t es = dtype == PSELINV_F64 ? 8 : 16;
   if (h->dtype != dtype || h->nbatch != nbatch) {
     free_numeric(h);
-    h->dtype = dtype;
-    h->nbatch = nbatch;
-    h->esize = es;
-    const size_t sbytes = (size_t)nbatch * h->H.storage * es + 256;
-    CK(cudaMalloc(&h->lu, sbytes));
-    CK(cudaMalloc(&h->nf, sbytes));
-    CK(cudaMalloc(&h->ainv, sbytes));
-    CK(cudaMemset(h->nf, 0, sbytes));
-    // zeros outside the triangles, which are never written
-    CK(cudaMalloc(&h->winv, (size_t)nbatch * h->w_stride * es + 256));
-    CK(cudaMemset(h->winv, 0, (size_t)nbatch * h->w_stride * es + 256));
-    CK(cudaMalloc(&h->piv, (size_t)nbatch * h->H.n * kLuPanel * es + 256));
-    h->scratch_bytes = scratch_need(h->H, nbatch, es);
-    CK(cudaMalloc(&h->scratch, h->scratch_bytes));
-    CK(cudaMalloc(&h->staging, (size_t)nbatch * h->H.nnz * es + 256));
-    CK(cudaMalloc(&h->outstage, (size_t)h->H.nnz * es + 256));
-    CK(cudaMalloc(&h->rcmax, (size_t)nbatch * 2 * h->H.n * 8 + 256));
-    CK(prepare_dense_kernels());
-    CK(prepare_ozaki_kernels());
-    h->slices = h->opts.slices <= 0 ? 6 : std::min(6, std::max(4, (int)h->opts.slices));
+    const int rc = alloc_numeric(h, dtype, nbatch);
+    if (rc != PSELINV_OK) {  // leave nothing that a later call would take for buffers
+      free_numeric(h);
+      return rc;
+    }
   }
   if (!h->factor_plan.built) {
     const int rc = build_factor_plan(h);
