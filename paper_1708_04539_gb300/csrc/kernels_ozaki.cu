@@ -1000,7 +1000,9 @@ ozaki_gemm_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ t
         l_eb = eB[nl];
       }
       for (int c = 0; c < nchunks; c++, q++) {
-        if (!mbar_wait(smem_u32(&bar_acc_full), q & 1) || abort_flag) {
+        // (one outcome for the warp: a lane that gave up alone would leave the others
+        // at the warp-wide loads below for good)
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_acc_full), q & 1) && !abort_flag)) {
           ok = false;
           break;
         }
@@ -1320,7 +1322,9 @@ gemm8_kernel(const OzDesc* __restrict__ descs, const OzTask* __restrict__ tasks,
       unsigned* __restrict__ mx = dp->mx;
       unsigned row_max = 0;
       for (int c = 0; c < nchunks; c++, q++) {
-        if (!mbar_wait(smem_u32(&bar_acc_full), q & 1) || abort_flag) {
+        // (one outcome for the warp: a lane that gave up alone would leave the others
+        // at the warp-wide loads below for good)
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_acc_full), q & 1) && !abort_flag)) {
           ok = false;
           break;
         }
