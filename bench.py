@@ -54,6 +54,8 @@ SAMPLE_TARGET_N = {1: 961, 2: 4000, 3: 2000, 4: 4000, 5: 2048}
 # smaller matrices of the same family whose tuner records train the cost model
 TRAIN_SIZES = {2: (20, 24, 28), 5: (8, 10, 12)}
 SLICES = 6
+SLICES_NORM = 8  # the normalisation of split levels, supernodes wider than NARROW
+NARROW = 32
 
 
 def parse(argv=None):
@@ -97,7 +99,8 @@ def parse(argv=None):
                     help="profiler runs: one factorisation and one sweep (plan from --plan-in, "
                          "or the untuned heuristic), nothing timed, no JSON line")
     ap.add_argument("--split-normalise", action="store_true",
-                    help="also slice the normalisation and D_K (by default they stay FP64)")
+                    help="the normalisation and D_K as products of --slices slices too (by "
+                         "default eight slices at FP64 accuracy, D_K in FP64)")
     ap.add_argument("--size", type=int, default=None,
                     help="grid side (elements per side for the DG operator; default: the "
                          "configuration's own; smaller for profiling captures)")
@@ -270,11 +273,17 @@ def measured_peaks():
 GEMM_TEMPLATES = {0: "64,64,16", 1: "32,32,16", 2: "128,64,8"}  # tile config -> BM,BN,BK (3: row panels)
 
 
+def kernel_kind(r):
+    """Kind of a launch record; the eight-slice products (no K split) apart."""
+    eight = r["kind"] == "ozaki_gemm" and r.get("param", -1) < 0
+    return "ozaki_gemm8" if eight else r["kind"]
+
+
 def roofline_from_profile(prof, slices, fp64_peak):
     """Roofline record of the kernel kind with the largest share of the step."""
     kinds = {}
     for r in prof:
-        k = kinds.setdefault(r["kind"], {"launches": 0, "ms": 0.0, "flops": 0.0, "bytes": 0.0})
+        k = kinds.setdefault(kernel_kind(r), {"launches": 0, "ms": 0.0, "flops": 0.0, "bytes": 0.0})
         k["launches"] += 1
         k["ms"] += r["ms"]
         k["flops"] += r["flops"]
@@ -288,14 +297,14 @@ def roofline_from_profile(prof, slices, fp64_peak):
     k = kinds[top]
     by_param = {}
     for r in prof:
-        if r["kind"] == top:
+        if kernel_kind(r) == top:
             by_param[r.get("param", -1)] = by_param.get(r.get("param", -1), 0.0) + r["ms"]
     main_param = max(by_param, key=by_param.get) if by_param else -1
     sec = k["ms"] * 1e-3
     peaks = measured_peaks()
     if top == "gemm":
         achieved = k["flops"] / sec / 1e12
-        if main_param == 3:  # row panels (the normalisation's triangular products)
+        if main_param == 3:  # row panels (triangular products of the normalisation, D_K)
             name, tkey = "rows_gemm_kernel<double> (FP64 DFMA)", "rows_gemm_kernel_f64"
         else:
             tile = GEMM_TEMPLATES.get(main_param, "?")
@@ -305,17 +314,20 @@ def roofline_from_profile(prof, slices, fp64_peak):
                "peak_source": "measured in this run: pselinv_measure_fp64_peak (FP64 FMA loop "
                               "on every SM; mma.sync f64 measured slower on GB300)",
                "traffic": traffic_from_profiles(tkey)}
-    elif top == "ozaki_gemm":
-        pairs = slices * (slices + 1) // 2
+    elif top in ("ozaki_gemm", "ozaki_gemm8"):
+        eight = top == "ozaki_gemm8"
+        sl = SLICES_NORM if eight else slices
+        pairs = sl * (sl + 1) // 2
         achieved = pairs * k["flops"] / sec / 1e12
         peak = float(peaks.get("bf16_tflops", 1925.5))
-        rec = {"bound": "tensor", "kernel": f"ozaki_gemm_kernel<{slices}> (tcgen05 kind::f16)",
+        name = "gemm8_kernel" if eight else f"ozaki_gemm_kernel<{slices}>"
+        rec = {"bound": "tensor", "kernel": f"{name} (tcgen05 kind::f16)",
                "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                "peak_source": "measured bf16 dense peak (MEASURED_PEAKS.json) x 1.0 nominal "
                               "fp16/bf16 ratio",
                "tensor_flops_per_fp64_flop": pairs,
                # captured with the default six slices
-               "traffic": traffic_from_profiles("ozaki_gemm") if slices == SLICES else None}
+               "traffic": traffic_from_profiles(top) if eight or slices == SLICES else None}
     else:
         achieved = k["bytes"] / sec / 1e9
         peak = float(peaks.get("hbm_gbs", 6778.7))
@@ -329,17 +341,19 @@ def roofline_from_profile(prof, slices, fp64_peak):
                  for n, v in kinds.items()}
 
 
-def path_roofline(st, cplx, nbatch, ms_step, fp64_peak, split, slices=SLICES):
+def path_roofline(st, cplx, nbatch, ms_step, fp64_peak, split, slices=SLICES,
+                  split_normalise=False):
     """Path-level roofline of one sweep from its level structure.
 
     Per supernode (width s, c = |R_K|, relaxed structure): products of steps
-    3-5 P = 4 c^2 s + 2 c s^2, FP64 normalisation and diagonal block
-    F = 2 c s^2 + 4/3 s^3, algorithmic bytes (c^2 + 2 (2 c s + s^2)) w (G read
+    3-5 P = 4 c^2 s + 2 c s^2, normalisation N = 2 c s^2, diagonal block
+    D = 4/3 s^3, algorithmic bytes (c^2 + 2 (2 c s + s^2)) w (G read
     once, panels read and written).  FP64 roofline of level l:
     min(P_fp64, AI_l x HBM) over all its flops; split roofline: the sliced
-    products at the tensor peak (21 slice products each) or HBM, whichever
-    is slower, plus F at the FP64 peak (S (S + 1) / 2 slice products for S
-    slices).  frac = roofline time / measured."""
+    products at the tensor peak (S (S + 1) / 2 slice products for S slices; N
+    of supernodes wider than NARROW at SLICES_NORM slices) or HBM, whichever is
+    slower, plus D and the narrow supernodes' N at the FP64 peak
+    (split_normalise: N and D at S slices).  frac = roofline time / measured."""
     peaks = measured_peaks()
     hbm = float(peaks.get("hbm_gbs", 6778.7)) * 1e9
     tensor = float(peaks.get("bf16_tflops", 1925.5)) * 1e12
@@ -350,25 +364,34 @@ def path_roofline(st, cplx, nbatch, ms_step, fp64_peak, split, slices=SLICES):
     c = np.diff(np.asarray(st["rows_ptr"])).astype(float)
     depth = np.asarray(st["sn_depth"])
     prod = (4 * c * c * width + 2 * c * width * width) * mult
-    norm = (2 * c * width * width + 4.0 / 3.0 * width ** 3) * mult
+    norm = 2 * c * width * width * mult
+    diag = 4.0 / 3.0 * width ** 3 * mult
+    wide = width > NARROW
     byts = (c * c + 2 * (2 * c * width + width * width)) * w * nbatch
     t64 = tsplit = 0.0
     pairs = slices * (slices + 1) // 2
+    pairs_norm = SLICES_NORM * (SLICES_NORM + 1) // 2
+    if split_normalise:
+        tensor_work, fp64_work = (prod + norm + diag) * pairs, 0.0 * prod
+    else:
+        tensor_work = prod * pairs + np.where(wide, norm * pairs_norm, 0.0)
+        fp64_work = diag + np.where(wide, 0.0, norm)
     for lev in range(int(st["nlevels"])):
         m = depth == lev
-        f, b = float((prod[m] + norm[m]).sum()), float(byts[m].sum())
+        f, b = float((prod[m] + norm[m] + diag[m]).sum()), float(byts[m].sum())
         if f <= 0:
             continue
         t64 += f / min(p64, f / b * hbm)
-        tsplit += max(float(prod[m].sum()) * pairs / tensor, b / hbm) + float(norm[m].sum()) / p64
+        tsplit += max(float(tensor_work[m].sum()) / tensor, b / hbm) + float(fp64_work[m].sum()) / p64
     sec = ms_step * 1e-3
     out = {"fp64_roofline_ms": t64 * 1e3, "frac_vs_fp64_roofline": t64 / sec,
            "definition": "sum over depth levels of flops_l / min(P_fp64, AI_l x HBM), over the "
                          "measured step (the split path may exceed 1)"}
     if split:
         out.update({"split_roofline_ms": tsplit * 1e3, "frac_vs_split_roofline": tsplit / sec,
-                    "split_definition": "per level max(21 x products / tensor peak, bytes / HBM) "
-                                        "+ FP64 normalisation / P_fp64, over the measured step"})
+                    "split_definition": "per level max(slice products of steps 3-5 and of the "
+                                        "normalisation / tensor peak, bytes / HBM) + FP64 rest "
+                                        "/ P_fp64, over the measured step"})
     return out
 
 
@@ -834,7 +857,8 @@ def run_ours(args):
     roofline, kinds = roofline_from_profile(prof, nslices, fp64_peak)
     if roofline is not None:
         roofline["path"] = path_roofline(st, cplx, nbatch, ms_per_step / 1.0, fp64_peak,
-                                         prec == ps.PREC_OZAKI_FP16, nslices)
+                                         prec == ps.PREC_OZAKI_FP16, nslices,
+                                         args.split_normalise)
     if args.dump_profile and rank == 0:
         with torch.cuda.stream(stream):
             fprof = [] if big else h.profile(1, stream=stream)
@@ -906,7 +930,9 @@ def run_ours(args):
                    "flops_per_matrix": flops / nbatch,
                    "flops_relaxed_structure": st["flops_selinv"] * (4.0 if cplx else 1.0),
                    "schedule": args.schedule, "cuda_graph": not args.no_graph,
-                   "normalisation": "split" if args.split_normalise else "fp64",
+                   "normalisation": "fp64" if args.precision == "fp64" else
+                                    "split" if args.split_normalise else
+                                    "8 slices at fp64 accuracy, D_K fp64",
                    "factor_schur_products": fprec_name,
                    "tuning": tuning, "tuning_seconds": tune_s,
                    "parallelism": "replicas" if world > 1 else "single",

@@ -337,20 +337,21 @@ typedef struct pselinv_step_stat {
   double bytes;   /* algorithmic bytes moved (operands read + results written) */
   double ms;      /* device time from CUDA events around the launch */
   int32_t param;  /* GEMM: kernel config (0 64x64, 1 32x32, 2 128x64 tiles, 3 row
-                     panels); OZAKI_GEMM: K split;
-                     else -1 */
+                     panels); OZAKI_GEMM: K split, -1 for products of eight
+                     slices; else -1 */
   int32_t side;   /* stream of the launch: 0 main, 1 side (normalisation, inverses), 2 the
                      factorisation's bulk Schur products */
   double start_ms; /* which = 2: time from the start of the sweep until the launch's stream
                       reached it (its wait included); else 0 */
 } pselinv_step_stat;
 
-enum pselinv_step_kind {
+enum pselinv_step_kind { /* (no launch reports TRI_INV or RECOMBINE any more) */
   PSELINV_STEP_GEMM = 0, PSELINV_STEP_TRI_INV = 1, PSELINV_STEP_DIAG_LU = 2,
   PSELINV_STEP_GATHER = 3, PSELINV_STEP_SCATTER_SUB = 4, PSELINV_STEP_COPY = 5,
   PSELINV_STEP_MEMSET = 6, PSELINV_STEP_SCATTER_VALUES = 7, PSELINV_STEP_SLICE = 8,
   PSELINV_STEP_OZAKI_GEMM = 9, PSELINV_STEP_RECOMBINE = 10,
-  PSELINV_STEP_SMALL_LEVEL = 11, /* gather and steps 3-5 of an FP64 level, one launch */
+  PSELINV_STEP_SMALL_LEVEL = 11, /* gather and steps 3-5 of an FP64 level, one launch
+                                    (level schedule, up to 20 Gflop of steps 3 and 5) */
   PSELINV_STEP_GATHER_SLICE = 12, /* split levels: Ainv_CC gathered and sliced in one pass
                                      (slices in both layouts, exponents from the running
                                      maxima), with the panels' maxima or slicing; Ainv_CC is

@@ -44,3 +44,29 @@ def test_aggregate_throughput_over_replicas():
     value, ms = bench.aggregate_throughput(7.5e13, 2000.0, 2, 4)
     assert ms == 1000.0
     assert abs(value - 4 * 7.5e13 / 1.0 / 1e9) < 1e-6
+
+
+def test_eight_slice_products_are_their_own_kernel():
+    """Launches without a K split (param -1) do 36 slice pairs and are not counted
+    with the six-slice kernel."""
+    recs = _records() + [{"kind": "ozaki_gemm", "ms": 9.0, "flops": 3e12, "bytes": 1e9, "param": -1}]
+    rec, kinds = bench.roofline_from_profile(recs, 6, 1.25)
+    assert rec["kernel"].startswith("gemm8_kernel") and rec["tensor_flops_per_fp64_flop"] == 36
+    assert abs(rec["achieved"] - 36 * 3e12 / 9e-3 / 1e12) < 1e-6 * rec["achieved"]
+    assert kinds["ozaki_gemm"]["launches"] == 2 and kinds["ozaki_gemm8"]["launches"] == 1
+
+
+def test_path_roofline_of_one_supernode():
+    """One level, two supernodes (64 columns over 100 rows, 16 over none): products
+    at 21 and the wide normalisation at 36 slice pairs on the tensor peak (or the
+    bytes at the copy rate), the diagonal blocks in FP64."""
+    st = {"sn_width": [64, 16], "rows_ptr": [0, 100, 100], "sn_depth": [0, 0], "nlevels": 1}
+    peaks = bench.measured_peaks()
+    tensor = float(peaks.get("bf16_tflops", 1925.5)) * 1e12
+    hbm = float(peaks.get("hbm_gbs", 6778.7)) * 1e9
+    prod, norm = 4 * 100 ** 2 * 64 + 2 * 100 * 64 ** 2, 2 * 100 * 64 ** 2
+    diag = 4 / 3 * (64 ** 3 + 16 ** 3)
+    byts = 8 * (100 ** 2 + 2 * (2 * 100 * 64 + 64 ** 2) + 2 * 16 ** 2)
+    out = bench.path_roofline(st, False, 1, 1.0, 1.25, True)
+    expect = max((21 * prod + 36 * norm) / tensor, byts / hbm) + diag / 1.25e12
+    assert abs(out["split_roofline_ms"] - expect * 1e3) < 1e-9 * expect * 1e3

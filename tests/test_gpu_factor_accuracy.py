@@ -218,3 +218,41 @@ def test_tiny_rows(torch, tiny):
         scale = max(np.abs(ref).max(), 0.0)
         assert np.abs(x - ref).max() <= max(8 * s * U64 * scale, 4 * s * 2.0 ** -1074) * (tiny != 0)
     assert np.isfinite(got[1]).all()
+
+
+@pytest.mark.parametrize("s,c", [(96, 133), (128, 65)])
+def test_eight_slice_schur_products(torch, s, c):
+    """Schur products over an identity block against exact sums: the first row of
+    the next supernode is the negated products (zeros before).  A term's digits and
+    left-out pairs err by 2^-64 (standard deviation, of the rows' powers of two, 1
+    here), K <= 128 of them, one exact chunk, by sqrt(K) as much; 16 standard
+    deviations and one rounding.  A slice less would show 2^-56 a term."""
+    from fractions import Fraction
+
+    import paper_1708_04539_gb300 as ps
+    n = s + c
+    nb = int(1.2e8 / (2.0 * c * c * s + 2.0 * c * s * s)) + 1
+    rng = np.random.default_rng(c)
+
+    def panel():
+        return rng.uniform(0.5, 1, (c, s)) * rng.choice([-1.0, 1.0], (c, s))
+    low, up = panel(), panel()
+    a = np.zeros((n, n))
+    a[s:, :s], a[:s, s:] = low, up.T
+    a[:s, :s] = np.eye(s)
+    a[s:, s:] = 4.0 * n * np.eye(c)
+    colptr = np.arange(n + 1, dtype=np.int64) * n
+    rowind = np.tile(np.arange(n, dtype=np.int64), n)
+    h = ps.SelInv(n, colptr, rowind, np.arange(n, dtype=np.int64), max_supernode=s,
+                  factor_precision=ps.PREC_OZAKI_FP16, factor_split_mflops=100000)
+    st = h.structure()
+    h.factor(torch.from_numpy(np.tile(a.T.reshape(-1), (nb, 1))).cuda())
+    fac = h.get_selected(batch=nb - 1, layout=ps.LAYOUT_FACTORS)
+    h.close()
+    w, o = int(st["sn_width"][1]), int(st["sn_offset"][1])
+    assert w > 1 and st["sn_first"][1] == s
+    row = fac[o:o + w * w].reshape(w, w).T[0]  # U of the second supernode, first row
+    tol = 16 * np.sqrt(s) * 2.0 ** -64
+    for q in range(1, w):
+        ref = -sum(Fraction(float(x)) * Fraction(float(y)) for x, y in zip(low[0], up[q]))
+        assert abs(Fraction(float(row[q])) - ref) <= tol + U64 * abs(float(ref)), q
