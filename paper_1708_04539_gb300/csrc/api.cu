@@ -638,10 +638,6 @@ void gemm_features<GemmDesc>(Step& st, const std::vector<GemmDesc>& descs, doubl
 // ---------------------------------------------------------------------------
 void add_copy_step(Plan& P, const std::vector<CopySeg>& segs, int level, size_t es);
 
-// trailing updates of the blocked diagonal LU (K = 32): 32 x 32 tiles (row
-// panels: 61.9 vs 60.9 ms for the 40^3 factorisation)
-constexpr int kLuUpdateCfg = GEMM_32x32;
-
 // one supernode's products of the factorisation: the triangular solves
 // TL = AL Uinv (AL = A_{C,K}, c x s) and TU = AU Linv^T (AU = A_{K,C}^T,
 // cu x s), and the Schur complement Sc = TL TU^T (c x cu, K = s); column
@@ -874,8 +870,8 @@ int build_factor_plan(pselinv_ctx* h) {
   const int nlev = (int)H.hlevel_ptr.size() - 1;
   // precision of each level's products.  Split: opts.slices slices where the
   // Schur work pays for them; smaller levels keep FP64 accuracy, as products of
-  // eight slices where the FP64 pipe would take longer than their four launches
-  // (100 MFLOP: 80 us)
+  // eight slices where the FP64 pipe would take longer than their launches
+  // (slicing, product and check, twice; 100 MFLOP: 80 us)
   enum { LV_FP64, LV_SPLIT, LV_EIGHT };
   std::vector<int> mode((size_t)std::max(nlev, 0) + 1, LV_FP64);
   for (int lev = 0; lev < nlev && h->opts.factor_precision == PSELINV_PREC_OZAKI_FP16; lev++) {
@@ -1774,7 +1770,7 @@ void add_outmax_step(pselinv_ctx* h, Plan& P, const std::vector<int64_t>& sns, i
 // One level (or one supernode) of the split-precision sweep: gather G,
 // slice G (by rows and by columns), Lhat and Uhat^T, sliced products for
 // steps 3 and 5, slice Ainv(C,K), sliced product for step 4 accumulated onto
-// D_K.  Scratch layout after the W region (byte offsets).
+// D_K.
 void add_ozaki_level(pselinv_ctx* h, Plan& P, const std::vector<int64_t>& grp, int64_t nb,
                      int lev, size_t& max_cursor) {
   const HostSym& H = h->H;
